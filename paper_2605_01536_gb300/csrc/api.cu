@@ -86,7 +86,7 @@ struct Staging {
                                                   std::to_string(device) + ")");
     }
     gwn_status alloc(void **p, size_t bytes) {
-        GWN_CUDA_TRY(cudaMallocAsync(p, bytes > 0 ? bytes : 16, s));
+        GWN_CUDA_TRY(dev_alloc(p, bytes > 0 ? bytes : 16, s));
         allocs[nalloc++] = *p;
         return GWN_OK;
     }
@@ -185,6 +185,7 @@ gwn_status gwn_mesh_create(const float *V, int64_t nv, const int32_t *F, int64_t
     cudaStream_t s = (cudaStream_t)stream;
     gwn_mesh *m = new gwn_mesh();
     cudaGetDevice(&m->device);
+    m->pool.hold(m->device);
     m->nv = nv;
     m->nt = nt;
     if (cfg) m->cfg = *cfg;
@@ -214,16 +215,16 @@ gwn_status gwn_mesh_create(const float *V, int64_t nv, const int32_t *F, int64_t
         return st;
     };
     cudaError_t e;
-    if ((e = cudaMalloc(&m->counters, kStatusBytes)) != cudaSuccess)
+    if ((e = dev_alloc(&m->counters, kStatusBytes, s)) != cudaSuccess)
         return fail(set_error(GWN_ERR_OOM, cudaGetErrorString(e)));
     cudaMemsetAsync(m->counters, 0, kStatusBytes, s);
-    if (nv > 0 && (e = cudaMalloc(&m->V, sizeof(float4) * nv)) != cudaSuccess)
+    if (nv > 0 && (e = dev_alloc(&m->V, sizeof(float4) * nv, s)) != cudaSuccess)
         return fail(set_error(GWN_ERR_OOM, cudaGetErrorString(e)));
-    if (nt > 0 && ((e = cudaMalloc(&m->F, sizeof(int32_t) * 3 * nt)) != cudaSuccess ||
-                   (e = cudaMalloc(&m->tri9, sizeof(float) * 9 * nt)) != cudaSuccess))
+    if (nt > 0 && ((e = dev_alloc(&m->F, sizeof(int32_t) * 3 * nt, s)) != cudaSuccess ||
+                   (e = dev_alloc(&m->tri9, sizeof(float) * 9 * nt, s)) != cudaSuccess))
         return fail(set_error(GWN_ERR_OOM, cudaGetErrorString(e)));
     unsigned long long *bad = nullptr;
-    if ((e = cudaMallocAsync(&bad, sizeof(unsigned long long) * 2, s)) != cudaSuccess)
+    if ((e = dev_alloc(&bad, sizeof(unsigned long long) * 2, s)) != cudaSuccess)
         return fail(set_error(GWN_ERR_OOM, cudaGetErrorString(e)));
     cudaMemsetAsync(bad, 0, sizeof(unsigned long long) * 2, s);
     float *vtmp = nullptr;
@@ -233,7 +234,7 @@ gwn_status gwn_mesh_create(const float *V, int64_t nv, const int32_t *F, int64_t
     if (nv > 0) {
         const float *vdev = V;
         if (vkind == 0) {
-            if ((e = cudaMallocAsync(&vtmp, sizeof(float) * 3 * nv, s)) != cudaSuccess)
+            if ((e = dev_alloc(&vtmp, sizeof(float) * 3 * nv, s)) != cudaSuccess)
                 return fail(set_error(GWN_ERR_OOM, cudaGetErrorString(e)));
             cudaMemcpyAsync(vtmp, V, sizeof(float) * 3 * nv, cudaMemcpyHostToDevice, s);
             vdev = vtmp;
@@ -265,7 +266,7 @@ gwn_status gwn_mesh_destroy(gwn_mesh *m) {
     cudaDeviceSynchronize();
     for (void *p : {(void *)m->V, (void *)m->F, (void *)m->tri9, (void *)m->bedges, (void *)m->bpts,
                     (void *)m->nodes, (void *)m->leaf_tri, (void *)m->counters, (void *)m->leaf_q, (void *)m->box})
-        if (p) cudaFree(p);
+        if (p) cudaFreeAsync(p, nullptr);
     surrogate_free(m->sur);
     delete m;
     return GWN_OK;
@@ -364,7 +365,7 @@ gwn_status gwn_query_chi_visits(const gwn_mesh *m, const float *q, int64_t n, in
     const void *qd = nullptr;
     void *cd = nullptr;
     unsigned long long *v = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&v, 2 * sizeof(unsigned long long), stg.s));
+    GWN_CUDA_TRY(dev_alloc(&v, 2 * sizeof(unsigned long long), stg.s));
     GWN_CUDA_TRY(cudaMemsetAsync(v, 0, 2 * sizeof(unsigned long long), stg.s));
     if ((st = stg.input(q, sizeof(float) * 3 * n, &qd)) == GWN_OK &&
         (st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK)
@@ -538,7 +539,7 @@ struct GridAxes {
         for (int32_t k = 1; k < nz; ++k)
             if (h[nx + ny + k] < h[nx + ny + k - 1])
                 return set_error(GWN_ERR_INVALID_ARG, "grid z coordinates must be non-decreasing");
-        GWN_CUDA_TRY(cudaMallocAsync(&d, sizeof(float) * h.size(), s));
+        GWN_CUDA_TRY(dev_alloc(&d, sizeof(float) * h.size(), s));
         GWN_CUDA_TRY(cudaMemcpyAsync(d, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice, s));
         GWN_CUDA_TRY(cudaStreamSynchronize(s));   // h goes out of scope
         return GWN_OK;

@@ -23,6 +23,7 @@ using namespace gwn;
 
 struct gwn_batch {
     int device = 0;
+    PoolRef pool;
     std::vector<const gwn_mesh *> meshes;
     std::vector<int64_t> q_off;
     int64_t total_q = 0;
@@ -256,6 +257,7 @@ gwn_status gwn_batch_create(const gwn_mesh *const *meshes, int32_t n_mesh, const
     if (n_mesh > 0) b->device = meshes[0]->device;
     else cudaGetDevice(&b->device);
     Guard g(b->device);
+    b->pool.hold(b->device);
     b->meshes.assign(meshes, meshes + n_mesh);
     b->q_off.assign(q_offsets, q_offsets + n_mesh + 1);
     if (n_mesh == 0) b->q_off.assign(1, 0);

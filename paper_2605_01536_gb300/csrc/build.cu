@@ -510,17 +510,17 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     m->nb = 0;
     m->npts = 0;
     m->nloops = 0;
-    if (m->bedges) { cudaFree(m->bedges); m->bedges = nullptr; }
-    if (m->bpts) { cudaFree(m->bpts); m->bpts = nullptr; }
+    if (m->bedges) { cudaFreeAsync(m->bedges, s); m->bedges = nullptr; }
+    if (m->bpts) { cudaFreeAsync(m->bpts, s); m->bpts = nullptr; }
     if (nh == 0) return GWN_OK;
     uint64_t *keys = nullptr, *seg_key = nullptr;
     uint32_t *vals = nullptr, *head = nullptr, *hscan = nullptr, *cnt = nullptr, *off = nullptr, *tot = nullptr;
     int32_t *mult = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&keys, sizeof(uint64_t) * nh, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&vals, sizeof(uint32_t) * nh, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&head, sizeof(uint32_t) * nh, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&hscan, sizeof(uint32_t) * nh, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&tot, sizeof(uint32_t) * 2, s));
+    GWN_CUDA_TRY(dev_alloc(&keys, sizeof(uint64_t) * nh, s));
+    GWN_CUDA_TRY(dev_alloc(&vals, sizeof(uint32_t) * nh, s));
+    GWN_CUDA_TRY(dev_alloc(&head, sizeof(uint32_t) * nh, s));
+    GWN_CUDA_TRY(dev_alloc(&hscan, sizeof(uint32_t) * nh, s));
+    GWN_CUDA_TRY(dev_alloc(&tot, sizeof(uint32_t) * 2, s));
     k_halfedge_keys<<<grid_for(nh, TB), TB, 0, s>>>(m->F, m->nt, m->nv, keys, vals);
     int bits = 1;
     while (bits < 64 && ((unsigned __int128)1 << bits) <= (unsigned __int128)m->nv * (unsigned __int128)m->nv) ++bits;
@@ -532,10 +532,10 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     GWN_CUDA_TRY(cudaMemcpyAsync(&nseg_h, tot, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     GWN_CUDA_TRY(cudaStreamSynchronize(s));
     const int64_t nseg = nseg_h;
-    GWN_CUDA_TRY(cudaMallocAsync(&mult, sizeof(int32_t) * nseg, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&seg_key, sizeof(uint64_t) * nseg, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&cnt, sizeof(uint32_t) * nseg, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&off, sizeof(uint32_t) * nseg, s));
+    GWN_CUDA_TRY(dev_alloc(&mult, sizeof(int32_t) * nseg, s));
+    GWN_CUDA_TRY(dev_alloc(&seg_key, sizeof(uint64_t) * nseg, s));
+    GWN_CUDA_TRY(dev_alloc(&cnt, sizeof(uint32_t) * nseg, s));
+    GWN_CUDA_TRY(dev_alloc(&off, sizeof(uint32_t) * nseg, s));
     GWN_CUDA_TRY(cudaMemsetAsync(mult, 0, sizeof(int32_t) * nseg, s));
     k_seg_sum<<<grid_for(nh, TB), TB, 0, s>>>(keys, vals, head, hscan, nh, mult, seg_key);
     k_abs<<<grid_for(nseg, TB), TB, 0, s>>>(mult, nseg, cnt);
@@ -545,7 +545,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     GWN_CUDA_TRY(cudaStreamSynchronize(s));
     m->nb = nb_h;
     if (m->nb > 0) {
-        GWN_CUDA_TRY(cudaMalloc(&m->bedges, sizeof(int32_t) * 2 * m->nb));
+        GWN_CUDA_TRY(dev_alloc(&m->bedges, sizeof(int32_t) * 2 * m->nb, s));
         k_emit_edges<<<grid_for(nseg, TB), TB, 0, s>>>(mult, seg_key, off, nseg, m->nv, m->bedges);
     }
     cudaFreeAsync(keys, s);
@@ -566,7 +566,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     if (m->cfg.chain_boundary < 0) {
         m->npts = 2 * nb;
         m->nloops = nb;
-        GWN_CUDA_TRY(cudaMalloc(&m->bpts, sizeof(float4) * m->npts));
+        GWN_CUDA_TRY(dev_alloc(&m->bpts, sizeof(float4) * m->npts, s));
         k_emit_unchained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, m->V, nb, m->bpts);
         cudaFreeAsync(tot, s);
         GWN_LAUNCH_CHECK("boundary points");
@@ -579,20 +579,20 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     int32_t *rnx[2] = {nullptr, nullptr};
     uint32_t *lsize = nullptr, *loff = nullptr;
     unsigned long long *nl = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&kin, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&idin, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&kout, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&idout, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&succ, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&kin, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&idin, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&kout, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&idout, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&succ, sizeof(uint32_t) * nb, s));
     for (int b = 0; b < 2; ++b) {
-        GWN_CUDA_TRY(cudaMallocAsync(&rep[b], sizeof(uint32_t) * nb, s));
-        GWN_CUDA_TRY(cudaMallocAsync(&nx[b], sizeof(uint32_t) * nb, s));
-        GWN_CUDA_TRY(cudaMallocAsync(&dist[b], sizeof(uint32_t) * nb, s));
-        GWN_CUDA_TRY(cudaMallocAsync(&rnx[b], sizeof(int32_t) * nb, s));
+        GWN_CUDA_TRY(dev_alloc(&rep[b], sizeof(uint32_t) * nb, s));
+        GWN_CUDA_TRY(dev_alloc(&nx[b], sizeof(uint32_t) * nb, s));
+        GWN_CUDA_TRY(dev_alloc(&dist[b], sizeof(uint32_t) * nb, s));
+        GWN_CUDA_TRY(dev_alloc(&rnx[b], sizeof(int32_t) * nb, s));
     }
-    GWN_CUDA_TRY(cudaMallocAsync(&lsize, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&loff, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&nl, sizeof(unsigned long long), s));
+    GWN_CUDA_TRY(dev_alloc(&lsize, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&loff, sizeof(uint32_t) * nb, s));
+    GWN_CUDA_TRY(dev_alloc(&nl, sizeof(unsigned long long), s));
     int vbits = 1;
     while (vbits < 32 && ((int64_t)1 << vbits) <= m->nv) ++vbits;
     k_edge_vertex_keys<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, nb, 1, kin, idin);
@@ -621,7 +621,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     {   // loops in the Morton order of their first points
         int *bnd = nullptr;
         const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
-        GWN_CUDA_TRY(cudaMallocAsync(&bnd, sizeof(init), s));
+        GWN_CUDA_TRY(dev_alloc(&bnd, sizeof(init), s));
         GWN_CUDA_TRY(cudaMemcpyAsync(bnd, init, sizeof(init), cudaMemcpyHostToDevice, s));
         k_edge_start_bounds<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, m->V, nb, bnd);
         // kin / idin / kout are free again: loop keys, representative ids, permuted sizes
@@ -641,7 +641,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     GWN_CUDA_TRY(cudaStreamSynchronize(s));
     m->npts = npts_h;
     m->nloops = (int64_t)nl_h;
-    GWN_CUDA_TRY(cudaMalloc(&m->bpts, sizeof(float4) * m->npts));
+    GWN_CUDA_TRY(dev_alloc(&m->bpts, sizeof(float4) * m->npts, s));
     k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, m->bpts);
     for (void *p : {(void *)kin, (void *)idin, (void *)kout, (void *)idout, (void *)succ, (void *)lsize,
                     (void *)loff, (void *)nl, (void *)tot})
@@ -657,14 +657,14 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
 }
 
 gwn_status build_box(gwn_mesh *m, cudaStream_t s) {
-    if (!m->box) GWN_CUDA_TRY(cudaMalloc(&m->box, sizeof(float) * 6));
+    if (!m->box) GWN_CUDA_TRY(dev_alloc(&m->box, sizeof(float) * 6, s));
     if (m->nv == 0) {
         GWN_CUDA_TRY(cudaMemsetAsync(m->box, 0, sizeof(float) * 6, s));
         return GWN_OK;
     }
     int *bounds = nullptr;
     const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
-    GWN_CUDA_TRY(cudaMallocAsync(&bounds, sizeof(init), s));
+    GWN_CUDA_TRY(dev_alloc(&bounds, sizeof(init), s));
     GWN_CUDA_TRY(cudaMemcpyAsync(bounds, init, sizeof(init), cudaMemcpyHostToDevice, s));
     k_vertex_bounds<<<grid_for(m->nv, TB), TB, 0, s>>>(m->V, m->nv, bounds);
     k_bounds_to_box<<<1, 32, 0, s>>>(bounds, m->box);
@@ -681,15 +681,15 @@ static gwn_status build_tree(const gwn_mesh *m, int dims, const int *bounds, gwn
     uint32_t *codes = nullptr, *ids = nullptr;
     int32_t *left = nullptr, *right = nullptr, *parent = nullptr, *first = nullptr, *last = nullptr;
     unsigned *visits = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&codes, sizeof(uint32_t) * n, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&ids, sizeof(uint32_t) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&codes, sizeof(uint32_t) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&ids, sizeof(uint32_t) * n, s));
     const int64_t ni = n > 1 ? n - 1 : 1;
-    GWN_CUDA_TRY(cudaMallocAsync(&left, sizeof(int32_t) * ni, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&right, sizeof(int32_t) * ni, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&first, sizeof(int32_t) * ni, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&last, sizeof(int32_t) * ni, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&parent, sizeof(int32_t) * (2 * n - 1), s));
-    GWN_CUDA_TRY(cudaMallocAsync(&visits, sizeof(unsigned) * ni, s));
+    GWN_CUDA_TRY(dev_alloc(&left, sizeof(int32_t) * ni, s));
+    GWN_CUDA_TRY(dev_alloc(&right, sizeof(int32_t) * ni, s));
+    GWN_CUDA_TRY(dev_alloc(&first, sizeof(int32_t) * ni, s));
+    GWN_CUDA_TRY(dev_alloc(&last, sizeof(int32_t) * ni, s));
+    GWN_CUDA_TRY(dev_alloc(&parent, sizeof(int32_t) * (2 * n - 1), s));
+    GWN_CUDA_TRY(dev_alloc(&visits, sizeof(unsigned) * ni, s));
     GWN_CUDA_TRY(cudaMemsetAsync(parent, 0xff, sizeof(int32_t) * (2 * n - 1), s));
     GWN_CUDA_TRY(cudaMemsetAsync(visits, 0, sizeof(unsigned) * ni, s));
     k_morton<<<grid_for(n, TB), TB, 0, s>>>(m->V, m->F, n, bounds, dims, codes, ids);
@@ -717,8 +717,8 @@ static gwn_status build_tree(const gwn_mesh *m, int dims, const int *bounds, gwn
 constexpr int kTreeSamples = 4096;
 gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     const int64_t n = m->nt;
-    if (m->nodes) { cudaFree(m->nodes); m->nodes = nullptr; }
-    if (m->leaf_tri) { cudaFree(m->leaf_tri); m->leaf_tri = nullptr; }
+    if (m->nodes) { cudaFreeAsync(m->nodes, s); m->nodes = nullptr; }
+    if (m->leaf_tri) { cudaFreeAsync(m->leaf_tri, s); m->leaf_tri = nullptr; }
     m->nnodes = 0;
     if (n == 0) return GWN_OK;
     m->nnodes = 2 * n - 1;
@@ -728,21 +728,21 @@ gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     unsigned long long *visits = nullptr;
     auto cleanup = [&]() {
         for (int t = 0; t < 2; ++t) {
-            if (nodes[t]) cudaFree(nodes[t]);
-            if (leaf[t]) cudaFree(leaf[t]);
+            if (nodes[t]) cudaFreeAsync(nodes[t], s);
+            if (leaf[t]) cudaFreeAsync(leaf[t], s);
         }
     };
     for (int t = 0; t < 2; ++t) {
         cudaError_t e;
-        if ((e = cudaMalloc(&nodes[t], sizeof(gwn::BvhNode) * m->nnodes)) != cudaSuccess ||
-            (e = cudaMalloc(&leaf[t], sizeof(float4) * 3 * n)) != cudaSuccess) {
+        if ((e = dev_alloc(&nodes[t], sizeof(gwn::BvhNode) * m->nnodes, s)) != cudaSuccess ||
+            (e = dev_alloc(&leaf[t], sizeof(float4) * 3 * n, s)) != cudaSuccess) {
             cudaGetLastError();
             cleanup();
             return set_error(GWN_ERR_OOM, std::string("bvh: ") + cudaGetErrorString(e));
         }
     }
-    GWN_CUDA_TRY(cudaMallocAsync(&bounds, sizeof(int) * 6, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&visits, sizeof(unsigned long long) * 2, s));
+    GWN_CUDA_TRY(dev_alloc(&bounds, sizeof(int) * 6, s));
+    GWN_CUDA_TRY(dev_alloc(&visits, sizeof(unsigned long long) * 2, s));
     const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
     GWN_CUDA_TRY(cudaMemcpyAsync(bounds, init, sizeof(init), cudaMemcpyHostToDevice, s));
     GWN_CUDA_TRY(cudaMemsetAsync(visits, 0, sizeof(unsigned long long) * 2, s));
@@ -770,8 +770,8 @@ gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     m->nodes = nodes[keep];
     m->leaf_tri = leaf[keep];
     m->bvh_xy = keep == 1;
-    cudaFree(nodes[1 - keep]);
-    cudaFree(leaf[1 - keep]);
+    cudaFreeAsync(nodes[1 - keep], s);
+    cudaFreeAsync(leaf[1 - keep], s);
     GWN_LAUNCH_CHECK("bvh build");
     return GWN_OK;
 }

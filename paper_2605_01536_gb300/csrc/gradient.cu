@@ -197,7 +197,7 @@ gwn_status launch_gradient(const gwn_mesh *m, const float *q, int64_t n, float *
     chunks = std::min<int64_t>(chunks, 65535);
     const int64_t chunk_len = chunks > 1 ? (nedge_pts + chunks - 1) / chunks : nedge_pts;
     double *partial = nullptr;
-    if (chunks > 1) GWN_CUDA_TRY(cudaMallocAsync(&partial, sizeof(double) * 3 * chunks * n, s));
+    if (chunks > 1) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * 3 * chunks * n, s));
     {
         ProfScope prof("gradient", s);
         dim3 grid((unsigned)qblocks, (unsigned)chunks);

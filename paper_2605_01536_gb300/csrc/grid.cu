@@ -146,8 +146,8 @@ gwn_status launch_grid_chi(const gwn_mesh *m, const float *gx, int nx, const flo
     if (ncol == 0 || nz == 0) return GWN_OK;
     int32_t *overflow = nullptr;
     unsigned *n_over = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&overflow, sizeof(int32_t) * ncol, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&n_over, sizeof(unsigned), s));
+    GWN_CUDA_TRY(dev_alloc(&overflow, sizeof(int32_t) * ncol, s));
+    GWN_CUDA_TRY(dev_alloc(&n_over, sizeof(unsigned), s));
     cudaMemsetAsync(n_over, 0, sizeof(unsigned), s);
     {
         ProfScope prof("grid_chi", s);
@@ -177,7 +177,7 @@ gwn_status launch_classify_grid(const gwn_mesh *m, const float *gx, int nx, cons
     const int64_t n = (int64_t)nx * ny * nz;
     if (n == 0) return GWN_OK;
     int32_t *chi = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&chi, sizeof(int32_t) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, s));
     gwn_status st = launch_grid_chi(m, gx, nx, gy, ny, gz, nz, chi, s);
     if (st == GWN_OK && m->npts < 2) {
         k_chi_to_w<<<grid_for(n, 256), 256, 0, s>>>(chi, n, w, label);
@@ -186,10 +186,10 @@ gwn_status launch_classify_grid(const gwn_mesh *m, const float *gx, int nx, cons
         int32_t *list = nullptr;
         unsigned long long *len = nullptr;
         if ((st = [&]() -> gwn_status {
-                 GWN_CUDA_TRY(cudaMallocAsync(&pts, sizeof(float) * 3 * n, s));
-                 GWN_CUDA_TRY(cudaMallocAsync(&list, sizeof(int32_t) * n, s));
-                 GWN_CUDA_TRY(cudaMallocAsync(&len, sizeof(unsigned long long), s));
-                 if (!wt) GWN_CUDA_TRY(cudaMallocAsync(&wt, sizeof(float) * n, s));
+                 GWN_CUDA_TRY(dev_alloc(&pts, sizeof(float) * 3 * n, s));
+                 GWN_CUDA_TRY(dev_alloc(&list, sizeof(int32_t) * n, s));
+                 GWN_CUDA_TRY(dev_alloc(&len, sizeof(unsigned long long), s));
+                 if (!wt) GWN_CUDA_TRY(dev_alloc(&wt, sizeof(float) * n, s));
                  return GWN_OK;
              }()) == GWN_OK) {
             cudaMemsetAsync(len, 0, sizeof(unsigned long long), s);

@@ -54,6 +54,30 @@ struct DeviceScope {
                                                       cudaGetErrorString(e_));    \
     } while (0)
 
+// devmem.cu: stream-ordered device memory of the current device from the library's
+// pool (freed with cudaFreeAsync).  Every mesh, batch and parametric surface retains
+// the pool of its device while it lives; the last one's release gives it back.
+cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
+template <class T>
+cudaError_t dev_alloc(T **p, size_t bytes, cudaStream_t s) {
+    return dev_alloc_bytes(reinterpret_cast<void **>(p), bytes, s);
+}
+void pool_retain(int dev);
+void pool_release(int dev);
+struct PoolRef {
+    int dev = -1;
+    PoolRef() = default;
+    PoolRef(const PoolRef &) = delete;
+    PoolRef &operator=(const PoolRef &) = delete;
+    void hold(int d) {
+        dev = d;
+        pool_retain(d);
+    }
+    ~PoolRef() {
+        if (dev >= 0) pool_release(dev);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Device data of a mesh.
 // ---------------------------------------------------------------------------
@@ -98,6 +122,7 @@ constexpr size_t kStatusBytes = sizeof(unsigned long long) * CNT_SLOTS + 64;
 
 struct gwn_mesh {
     int device = 0;
+    gwn::PoolRef pool;
     int64_t nv = 0, nt = 0;
     gwn_config cfg{};
 

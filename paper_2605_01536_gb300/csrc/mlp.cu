@@ -717,7 +717,7 @@ static gwn_status build_band(gwn_mesh *m, cudaStream_t st) {
     const int64_t ncell = (int64_t)R * R * R, nwords = (ncell + 31) / 32;
     uint32_t *marked = nullptr, *band = nullptr;
     GWN_CUDA_TRY(cudaMalloc(&band, sizeof(uint32_t) * nwords));
-    GWN_CUDA_TRY(cudaMallocAsync(&marked, sizeof(uint32_t) * nwords, st));
+    GWN_CUDA_TRY(dev_alloc(&marked, sizeof(uint32_t) * nwords, st));
     cudaMemsetAsync(marked, 0, sizeof(uint32_t) * nwords, st);
     MlpDev P = mlp_dev(s);
     P.band_res = R;
@@ -904,11 +904,11 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
     int32_t *list = nullptr, *chi_all = nullptr;
     unsigned long long *len = nullptr;
     const bool chi_test = s->cfg.chi_tol >= 0.f;
-    GWN_CUDA_TRY(cudaMallocAsync(&list, sizeof(int32_t) * n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&len, sizeof(unsigned long long), st));
+    GWN_CUDA_TRY(dev_alloc(&list, sizeof(int32_t) * n, st));
+    GWN_CUDA_TRY(dev_alloc(&len, sizeof(unsigned long long), st));
     GWN_CUDA_TRY(cudaMemsetAsync(len, 0, sizeof(unsigned long long), st));
     if (chi_test) {
-        GWN_CUDA_TRY(cudaMallocAsync(&chi_all, sizeof(int32_t) * n, st));
+        GWN_CUDA_TRY(dev_alloc(&chi_all, sizeof(int32_t) * n, st));
         if (gwn_status r0 = launch_chi(m, q, n, chi_all, st)) {
             cudaFreeAsync(chi_all, st);
             cudaFreeAsync(list, st);
@@ -935,12 +935,12 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
         uint8_t *lf = nullptr;
         int32_t *cf = nullptr, *l2 = nullptr;
         unsigned long long *len2 = nullptr;
-        GWN_CUDA_TRY(cudaMallocAsync(&qf, sizeof(float) * 3 * nfb, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&wf, sizeof(float) * nfb, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&lf, nfb, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&cf, sizeof(int32_t) * nfb, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&l2, sizeof(int32_t) * nfb, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&len2, sizeof(unsigned long long), st));
+        GWN_CUDA_TRY(dev_alloc(&qf, sizeof(float) * 3 * nfb, st));
+        GWN_CUDA_TRY(dev_alloc(&wf, sizeof(float) * nfb, st));
+        GWN_CUDA_TRY(dev_alloc(&lf, nfb, st));
+        GWN_CUDA_TRY(dev_alloc(&cf, sizeof(int32_t) * nfb, st));
+        GWN_CUDA_TRY(dev_alloc(&l2, sizeof(int32_t) * nfb, st));
+        GWN_CUDA_TRY(dev_alloc(&len2, sizeof(unsigned long long), st));
         GWN_CUDA_TRY(cudaMemsetAsync(len2, 0, sizeof(unsigned long long), st));
         const unsigned g = grid_for((int64_t)nfb, 256);
         const int64_t nf = (int64_t)nfb;
@@ -976,7 +976,7 @@ gwn_status gwn_debug_tc_gemm(const void *A, const void *B, int32_t K, float *C, 
     if (K != 64 && K != 128) return set_error(GWN_ERR_INVALID_ARG, "K must be 64 or 128");
     cudaStream_t s = (cudaStream_t)stream;
     unsigned *err = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&err, sizeof(unsigned), s));
+    GWN_CUDA_TRY(dev_alloc(&err, sizeof(unsigned), s));
     GWN_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(unsigned), s));
     // operands plus slack so that every address a descriptor can form stays inside the allocation
     const size_t smem = (size_t)(128 + 64) * K * 2 + 32768;
@@ -1010,7 +1010,7 @@ gwn_status gwn_surrogate_train(gwn_mesh *m, const float *samples, const float *t
     if ((r = ensure_batch_buffers(s, nb)) != GWN_OK) return r;
     // input box of the samples
     int *box = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&box, sizeof(int) * 6, st));
+    GWN_CUDA_TRY(dev_alloc(&box, sizeof(int) * 6, st));
     const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
     GWN_CUDA_TRY(cudaMemcpyAsync(box, init, sizeof(init), cudaMemcpyHostToDevice, st));
     k_bbox<<<grid_for(n, 256), 256, 0, st>>>(samples, n, box);
@@ -1026,8 +1026,8 @@ gwn_status gwn_surrogate_train(gwn_mesh *m, const float *samples, const float *t
     float *tgt = const_cast<float *>(targets), *own = nullptr;
     if (!tgt) {
         int32_t *chi = nullptr;
-        GWN_CUDA_TRY(cudaMallocAsync(&own, sizeof(float) * n, st));
-        GWN_CUDA_TRY(cudaMallocAsync(&chi, sizeof(int32_t) * n, st));
+        GWN_CUDA_TRY(dev_alloc(&own, sizeof(float) * n, st));
+        GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, st));
         if ((r = launch_chi(m, samples, n, chi, st)) == GWN_OK)
             r = launch_boundary_sum_list(m, samples, n, chi, own, nullptr, false, nullptr, nullptr, st);
         cudaFreeAsync(chi, st);
@@ -1220,13 +1220,13 @@ gwn_status gwn_surrogate_calibrate(gwn_mesh *m, const float *samples, int64_t n,
     uint8_t *lab = nullptr;
     int32_t *chi = nullptr, *list = nullptr;
     unsigned long long *len = nullptr, *hist = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&w_hat, sizeof(float) * n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&w, sizeof(float) * n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&lab, n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&chi, sizeof(int32_t) * n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&list, sizeof(int32_t) * n, st));
-    GWN_CUDA_TRY(cudaMallocAsync(&len, sizeof(unsigned long long), st));
-    GWN_CUDA_TRY(cudaMallocAsync(&hist, sizeof(unsigned long long) * kCalibBins, st));
+    GWN_CUDA_TRY(dev_alloc(&w_hat, sizeof(float) * n, st));
+    GWN_CUDA_TRY(dev_alloc(&w, sizeof(float) * n, st));
+    GWN_CUDA_TRY(dev_alloc(&lab, n, st));
+    GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, st));
+    GWN_CUDA_TRY(dev_alloc(&list, sizeof(int32_t) * n, st));
+    GWN_CUDA_TRY(dev_alloc(&len, sizeof(unsigned long long), st));
+    GWN_CUDA_TRY(dev_alloc(&hist, sizeof(unsigned long long) * kCalibBins, st));
     cudaMemsetAsync(len, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * kCalibBins, st);
     cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFwd);

@@ -116,7 +116,7 @@ gwn_status order_query_list(const gwn_mesh *m, const float *q, int32_t *list, in
     if (n > (int64_t)0x7fffffff) return set_error(GWN_ERR_INVALID_ARG, "too many queries to order");
     ProfScope prof("query_order", s);
     uint32_t *keys = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&keys, sizeof(uint32_t) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&keys, sizeof(uint32_t) * n, s));
     k_list_morton<<<grid_for(n, TB), TB, 0, s>>>(q, list, n, m->box, keys);
     note_launches(1);
     gwn_status st = radix_sort_u32(keys, reinterpret_cast<uint32_t *>(list), n, kOrderBits, s);

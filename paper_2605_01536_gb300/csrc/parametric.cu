@@ -996,6 +996,7 @@ using namespace gwn;
 // curves of the union and their panel trees.
 struct gwn_param {
     int device = 0;
+    PoolRef pool;
     int np = 0, nc = 0;
     gwn_param_config cfg{};
     double *patches = nullptr;   // [np][4][4][3]
@@ -1130,7 +1131,7 @@ gwn_status stage_axes(const gwn_param *g, const float *x, int32_t nx, const floa
                       int32_t nz, float **d_out, cudaStream_t s) {
     const size_t total = (size_t)nx + ny + nz;
     float *d = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&d, sizeof(float) * std::max<size_t>(total, 1), s));
+    GWN_CUDA_TRY(dev_alloc(&d, sizeof(float) * std::max<size_t>(total, 1), s));
     *d_out = d;
     const float *src[3] = {x, y, z};
     const size_t len[3] = {(size_t)nx, (size_t)ny, (size_t)nz};
@@ -1209,6 +1210,7 @@ gwn_status gwn_param_create(const float *patches, int32_t np, const gwn_param_co
     if (gwn_status st = upload_tables(device)) return st;
     gwn_param *g = new gwn_param();
     g->device = device;
+    g->pool.hold(device);
     g->cfg = c;
     g->np = np;
     g->h_curves = extract_boundary(hp.data(), np);
@@ -1355,7 +1357,7 @@ gwn_status gwn_param_query(const gwn_param *g, const float *q, int64_t n, float 
     if (gwn_status st = check_device_ptrs(g->device, {q, w, chi_or_null}, "gwn_param_query")) return st;
     cudaStream_t s = (cudaStream_t)stream;
     int32_t *chi = chi_or_null;
-    if (!chi) GWN_CUDA_TRY(cudaMallocAsync(&chi, sizeof(int32_t) * n, s));
+    if (!chi) GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, s));
     {
         ProfScope prof("param_chi", s);
         k_param_chi<<<grid_for(n, kWarps), 32 * kWarps, 0, s>>>(q, n, g->patches, g->pinfo, g->np, g->pbox, g->same,
@@ -1395,7 +1397,7 @@ gwn_status gwn_param_query_grid(const gwn_param *g, const float *x, int32_t nx, 
     int32_t *chi = chi_or_null;
     if (gwn_status st = stage_axes(g, x, nx, y, ny, z, nz, &axes, s)) return st;
     const float *dx = axes, *dy = axes + nx, *dz = axes + nx + ny;
-    if (!chi) GWN_CUDA_TRY(cudaMallocAsync(&chi, sizeof(int32_t) * n, s));
+    if (!chi) GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, s));
     {
         ProfScope prof("param_grid_chi", s);
         const int64_t cols = (int64_t)nx * ny;

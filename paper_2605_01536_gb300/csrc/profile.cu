@@ -179,7 +179,7 @@ extern "C" gwn_status gwn_measure_pipe_peaks(double *ffma_per_s, double *ffma2_p
     *sm_count = sms;
     float *out = nullptr;
     const int blocks = sms * 8;   // 8 x 256 threads per SM: 64 warps
-    GWN_CUDA_TRY(cudaMallocAsync(&out, sizeof(float) * blocks, s));
+    GWN_CUDA_TRY(dev_alloc(&out, sizeof(float) * blocks, s));
     cudaEvent_t a, b;
     GWN_CUDA_TRY(cudaEventCreate(&a));
     GWN_CUDA_TRY(cudaEventCreate(&b));

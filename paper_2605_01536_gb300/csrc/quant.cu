@@ -65,12 +65,12 @@ int quant_exponent(double half_extent) {
 gwn_status setup_quant(gwn_mesh *m, cudaStream_t s) {
     QFrame f{};
     if (m->leaf_q) {
-        cudaFree(m->leaf_q);
+        cudaFreeAsync(m->leaf_q, s);
         m->leaf_q = nullptr;
     }
     if (m->cfg.quantize_bits == 30 && m->nt > 0) {
         int *box = nullptr;
-        GWN_CUDA_TRY(cudaMallocAsync(&box, sizeof(int) * 6, s));
+        GWN_CUDA_TRY(dev_alloc(&box, sizeof(int) * 6, s));
         const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
         GWN_CUDA_TRY(cudaMemcpyAsync(box, init, sizeof(init), cudaMemcpyHostToDevice, s));
         k_vertex_box<<<grid_for(m->nv, 256), 256, 0, s>>>(m->V, m->nv, box);
@@ -92,7 +92,7 @@ gwn_status setup_quant(gwn_mesh *m, cudaStream_t s) {
         f.scale = std::ldexp(1.0, -e);
         f.pad = (float)std::ldexp(1.0, e);
         int4 *lq = nullptr;
-        GWN_CUDA_TRY(cudaMalloc(&lq, sizeof(int4) * 3 * m->nt));
+        GWN_CUDA_TRY(dev_alloc(&lq, sizeof(int4) * 3 * m->nt, s));
         k_snap_leaves<<<grid_for(3 * m->nt, 256), 256, 0, s>>>(m->leaf_tri, 3 * m->nt, f, lq);
         m->leaf_q = lq;
         f.leaf_q = lq;

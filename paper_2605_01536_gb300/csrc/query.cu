@@ -1184,7 +1184,7 @@ static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, c
         if (partial_cap >= 0) {
             partial = partial_buf;
         } else {
-            GWN_CUDA_TRY(cudaMallocAsync(&partial, sizeof(double) * chunks * n, s));
+            GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * chunks * n, s));
             own = true;
         }
     }
@@ -1244,14 +1244,14 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
     if (n <= 0) return GWN_OK;
     const size_t words = (size_t)((n + 31) / 32);
     unsigned *listed = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&listed, sizeof(unsigned) * words, s));
+    GWN_CUDA_TRY(dev_alloc(&listed, sizeof(unsigned) * words, s));
     GWN_CUDA_TRY(cudaMemsetAsync(listed, 0, sizeof(unsigned) * words, s));
     // without a caller list (no labels wanted), queries whose cancelling terms
     // overflow the kernel's queue still need their FP64 re-evaluation
     const bool own_list = list == nullptr;
     if (own_list) {
-        GWN_CUDA_TRY(cudaMallocAsync(&list, sizeof(int32_t) * n, s));
-        GWN_CUDA_TRY(cudaMallocAsync(&list_len, sizeof(unsigned long long), s));
+        GWN_CUDA_TRY(dev_alloc(&list, sizeof(int32_t) * n, s));
+        GWN_CUDA_TRY(dev_alloc(&list_len, sizeof(unsigned long long), s));
         GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     }
     gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1, s);
@@ -1378,7 +1378,7 @@ gwn_status launch_direct(const gwn_mesh *m, const float *q, int64_t n, float *w,
     chunks = std::min<int64_t>(chunks, 65535);
     const int64_t chunk_len = (m->nt + chunks - 1) / chunks;
     double *partial = nullptr;
-    if (chunks > 1) GWN_CUDA_TRY(cudaMallocAsync(&partial, sizeof(double) * chunks * n, s));
+    if (chunks > 1) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * chunks * n, s));
     {
         ProfScope prof("direct_sum", s);
         dim3 grid((unsigned)qblocks, (unsigned)chunks);

@@ -150,9 +150,9 @@ gwn_status radix_sort_impl(K *keys, uint32_t *vals, int64_t n, int bits, cudaStr
     const int64_t ncounts = (int64_t)ntiles * 256;
     K *k2 = nullptr;
     uint32_t *v2 = nullptr, *counts = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&k2, sizeof(K) * n, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&v2, sizeof(uint32_t) * n, s));
-    GWN_CUDA_TRY(cudaMallocAsync(&counts, sizeof(uint32_t) * ncounts, s));
+    GWN_CUDA_TRY(dev_alloc(&k2, sizeof(K) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&v2, sizeof(uint32_t) * n, s));
+    GWN_CUDA_TRY(dev_alloc(&counts, sizeof(uint32_t) * ncounts, s));
     K *kin = keys, *kout = k2;
     uint32_t *vin = vals, *vout = v2;
     gwn_status st = GWN_OK;
@@ -192,7 +192,7 @@ gwn_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint
         return GWN_OK;
     }
     uint32_t *sums = nullptr;
-    GWN_CUDA_TRY(cudaMallocAsync(&sums, sizeof(uint32_t) * nchunks, s));
+    GWN_CUDA_TRY(dev_alloc(&sums, sizeof(uint32_t) * nchunks, s));
     k_chunk_sums<<<(unsigned)nchunks, SCAN_THREADS, 0, s>>>(in, n, sums);
     note_launches(2);   // with k_chunk_scan
     gwn_status st = exclusive_scan_u32(sums, sums, nchunks, nullptr, s);
