@@ -265,7 +265,9 @@ gwn_status gwn_mesh_destroy(gwn_mesh *m) {
     DeviceGuard g(m->device);
     cudaDeviceSynchronize();
     for (void *p : {(void *)m->V, (void *)m->F, (void *)m->tri9, (void *)m->bedges, (void *)m->bpts,
-                    (void *)m->nodes, (void *)m->leaf_tri, (void *)m->counters, (void *)m->leaf_q, (void *)m->box})
+                    (void *)m->nodes, (void *)m->leaf_tri, (void *)m->counters, (void *)m->leaf_q, (void *)m->box,
+                    (void *)m->far_nodes, (void *)m->far_pts, (void *)m->far_coef,
+                    (void *)m->far_roots})
         if (p) cudaFreeAsync(p, nullptr);
     surrogate_free(m->sur);
     delete m;
@@ -411,7 +413,7 @@ gwn_status gwn_query_batch(const gwn_mesh *m, const float *q, int64_t n, float *
                                 stg.s)) == GWN_OK &&
             (st = launch_chi(m, (const float *)qs, n, (int32_t *)cs, stg.s)) == GWN_OK &&
             (st = launch_boundary_sum_list(m, (const float *)qs, n, (const int32_t *)cs, (float *)ws, nullptr, false,
-                                           nullptr, nullptr, stg.s)) == GWN_OK &&
+                                           nullptr, nullptr, SumOrder::kSpatial, stg.s)) == GWN_OK &&
             (st = scatter_f32((const float *)ws, (const uint32_t *)perm, n, (float *)wd, stg.s)) == GWN_OK)
             st = scatter_i32((const int32_t *)cs, (const uint32_t *)perm, n, chi ? (int32_t *)cd : nullptr, stg.s);
         return stg.finish(st);
@@ -419,7 +421,7 @@ gwn_status gwn_query_batch(const gwn_mesh *m, const float *q, int64_t n, float *
     if ((st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK &&
         (st = launch_chi(m, (const float *)qd, n, (int32_t *)cd, stg.s)) == GWN_OK)
         st = launch_boundary_sum_list(m, (const float *)qd, n, (const int32_t *)cd, (float *)wd, nullptr, false,
-                                      nullptr, nullptr, stg.s);
+                                      nullptr, nullptr, SumOrder::kSpatial, stg.s);
     return stg.finish(st);
 }
 
@@ -467,7 +469,7 @@ gwn_status gwn_classify(const gwn_mesh *m, const float *q, int64_t n, uint8_t *l
         if ((st = launch_chi(m, (const float *)qs, n, (int32_t *)cd, stg.s)) == GWN_OK &&
             (st = launch_boundary_sum_list(m, (const float *)qs, n, (const int32_t *)cd, (float *)ws,
                                            (uint8_t *)ls, true, (int32_t *)list, (unsigned long long *)len,
-                                           stg.s)) == GWN_OK)
+                                           SumOrder::kSpatial, stg.s)) == GWN_OK)
             st = launch_fp64_fix_list(m, (const float *)qs, (const int32_t *)cd, (float *)ws, (uint8_t *)ls,
                                       (const int32_t *)list, (const unsigned long long *)len, stg.s);
         if (st == GWN_OK && ordered &&

@@ -13,6 +13,7 @@
 // LBVH (replaces the paper's Embree BVH, Sec. 5): 30-bit Morton codes of the
 // triangle centroids, radix sort, Karras' binary radix tree (Karras 2012),
 // bottom-up box refit, and depth-first escape links for stackless traversal.
+#include "farfield.cuh"
 #include "gwn_internal.cuh"
 #include "traverse.cuh"
 
@@ -151,7 +152,7 @@ __global__ void k_loop_sizes(const uint32_t *__restrict__ rep, const uint32_t *_
 __global__ void k_emit_chained(const int32_t *__restrict__ edges, const uint32_t *__restrict__ rep,
                                const uint32_t *__restrict__ dist, const uint32_t *__restrict__ loop_off,
                                const float4 *__restrict__ V, int64_t nb, int64_t npts,
-                               float4 *__restrict__ pts) {
+                               float4 *__restrict__ pts, uint2 *__restrict__ ends /* or NULL */) {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nb) return;
     uint32_t r = rep[e];
@@ -163,10 +164,12 @@ __global__ void k_emit_chained(const int32_t *__restrict__ edges, const uint32_t
     float4 p = V[edges[2 * e]];
     p.w = 1.0f;
     pts[base + pos] = p;
+    if (ends) ends[base + pos] = make_uint2(base, base + len);   // the loop's first and closing points
     if (e == (int64_t)r) {   // closing point: back to the loop's first vertex
         float4 c = V[edges[2 * e]];
         c.w = 0.0f;
         pts[base + len] = c;
+        if (ends) ends[base + len] = make_uint2(base, base + len);
     }
 }
 
@@ -188,7 +191,7 @@ __global__ void k_emit_unchained(const int32_t *__restrict__ edges, const float4
 __global__ void k_edge_start_bounds(const int32_t *__restrict__ edges, const float4 *__restrict__ V, int64_t nb,
                                     int *__restrict__ bounds /* 6: min xyz, max xyz (ordered ints) */);
 __global__ void k_loop_keys(const uint32_t *__restrict__ rep, const int32_t *__restrict__ edges,
-                            const float4 *__restrict__ V, int64_t nb, const int *__restrict__ bounds,
+                            const float4 *__restrict__ V, int64_t nb, const int *__restrict__ bounds, int hilbert,
                             uint32_t *__restrict__ keys, uint32_t *__restrict__ ids);
 
 __global__ void k_gather_sizes(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ size, int64_t nb,
@@ -291,17 +294,30 @@ __global__ void k_edge_start_bounds(const int32_t *__restrict__ edges, const flo
     }
 }
 
-// key of a loop's representative edge: the Morton code of its start point;
-// every other edge sorts after all loops (bit 30)
+// 30-bit Hilbert key in the cube over the bounds
+__device__ __forceinline__ uint32_t hilbert30(float x, float y, float z, const int *__restrict__ bounds) {
+    const float c[3] = {x, y, z};
+    float ext = 0.f;
+    for (int k = 0; k < 3; ++k) ext = fmaxf(ext, from_ordered_key(bounds[3 + k]) - from_ordered_key(bounds[k]));
+    uint32_t q[3];
+    for (int k = 0; k < 3; ++k) {
+        const float u = ext > 0.f ? (c[k] - from_ordered_key(bounds[k])) / ext : 0.f;
+        q[k] = min((uint32_t)(fminf(fmaxf(u, 0.f), 1.f) * 1024.0f), 1023u);
+    }
+    return hilbert_key(q[0], q[1], q[2], 10);
+}
+
+// key of a loop's representative edge: the Morton code or Hilbert key of its start
+// point; every other edge sorts after all loops (bit 30)
 __global__ void k_loop_keys(const uint32_t *__restrict__ rep, const int32_t *__restrict__ edges,
-                            const float4 *__restrict__ V, int64_t nb, const int *__restrict__ bounds,
+                            const float4 *__restrict__ V, int64_t nb, const int *__restrict__ bounds, int hilbert,
                             uint32_t *__restrict__ keys, uint32_t *__restrict__ ids) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nb) return;
     uint32_t key = 1u << 30;
     if (rep[e] == (uint32_t)e) {
         const float4 p = V[edges[2 * e]];
-        key = morton30(p.x, p.y, p.z, bounds);
+        key = hilbert ? hilbert30(p.x, p.y, p.z, bounds) : morton30(p.x, p.y, p.z, bounds);
     }
     keys[e] = key;
     ids[e] = (uint32_t)e;
@@ -512,6 +528,12 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     m->nloops = 0;
     if (m->bedges) { cudaFreeAsync(m->bedges, s); m->bedges = nullptr; }
     if (m->bpts) { cudaFreeAsync(m->bpts, s); m->bpts = nullptr; }
+    if (m->far_nodes) { cudaFreeAsync(m->far_nodes, s); m->far_nodes = nullptr; }
+    if (m->far_pts) { cudaFreeAsync(m->far_pts, s); m->far_pts = nullptr; }
+    if (m->far_coef) { cudaFreeAsync(m->far_coef, s); m->far_coef = nullptr; }
+    if (m->far_roots) { cudaFreeAsync(m->far_roots, s); m->far_roots = nullptr; }
+    m->far_nn = 0;
+    m->far_nroots = 0;
     if (nh == 0) return GWN_OK;
     uint64_t *keys = nullptr, *seg_key = nullptr;
     uint32_t *vals = nullptr, *head = nullptr, *hscan = nullptr, *cnt = nullptr, *off = nullptr, *tot = nullptr;
@@ -618,20 +640,23 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     }
     uint32_t *distf = dist[cd];
     k_loop_sizes<<<grid_for(nb, TB), TB, 0, s>>>(repf, distf, nb, lsize);
-    {   // loops in the Morton order of their first points
-        int *bnd = nullptr;
-        const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
-        GWN_CUDA_TRY(dev_alloc(&bnd, sizeof(init), s));
-        GWN_CUDA_TRY(cudaMemcpyAsync(bnd, init, sizeof(init), cudaMemcpyHostToDevice, s));
-        k_edge_start_bounds<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, m->V, nb, bnd);
-        // kin / idin / kout are free again: loop keys, representative ids, permuted sizes
-        k_loop_keys<<<grid_for(nb, TB), TB, 0, s>>>(repf, m->bedges, m->V, nb, bnd, kin, idin);
-        if ((st = radix_sort_u32(kin, idin, nb, 31, s)) != GWN_OK) return st;
+    int *bnd = nullptr;
+    const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
+    GWN_CUDA_TRY(dev_alloc(&bnd, sizeof(init), s));
+    GWN_CUDA_TRY(cudaMemcpyAsync(bnd, init, sizeof(init), cudaMemcpyHostToDevice, s));
+    k_edge_start_bounds<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, m->V, nb, bnd);
+    // the loops' offsets in the order of their first points on the curve (kin, idin
+    // and kout are free again: loop keys, representative ids, permuted sizes)
+    auto order_loops = [&](int hilbert) -> gwn_status {
+        k_loop_keys<<<grid_for(nb, TB), TB, 0, s>>>(repf, m->bedges, m->V, nb, bnd, hilbert, kin, idin);
+        gwn_status r = radix_sort_u32(kin, idin, nb, 31, s);
+        if (r != GWN_OK) return r;
         k_gather_sizes<<<grid_for(nb, TB), TB, 0, s>>>(idin, lsize, nb, kout);
-        if ((st = exclusive_scan_u32(kout, kout, nb, tot, s)) != GWN_OK) return st;
+        if ((r = exclusive_scan_u32(kout, kout, nb, tot, s)) != GWN_OK) return r;
         k_scatter_offsets<<<grid_for(nb, TB), TB, 0, s>>>(idin, kout, nb, loff);
-        cudaFreeAsync(bnd, s);
-    }
+        return GWN_OK;
+    };
+    if ((st = order_loops(0)) != GWN_OK) return st;
     GWN_CUDA_TRY(cudaMemsetAsync(nl, 0, sizeof(unsigned long long), s));
     k_count_heads<<<grid_for(nb, TB), TB, 0, s>>>(repf, nb, nl);
     uint32_t npts_h = 0;
@@ -642,7 +667,18 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     m->npts = npts_h;
     m->nloops = (int64_t)nl_h;
     GWN_CUDA_TRY(dev_alloc(&m->bpts, sizeof(float4) * m->npts, s));
-    k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, m->bpts);
+    k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, m->bpts, nullptr);
+    if (m->npts >= kFarMinPoints) {
+        float4 *fpts = nullptr;
+        uint2 *ends = nullptr;
+        GWN_CUDA_TRY(dev_alloc(&fpts, sizeof(float4) * m->npts, s));
+        GWN_CUDA_TRY(dev_alloc(&ends, sizeof(uint2) * m->npts, s));
+        if ((st = order_loops(1)) != GWN_OK) return st;
+        k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, fpts, ends);
+        st = build_far(m, fpts, ends, s);
+        cudaFreeAsync(ends, s);
+    }
+    cudaFreeAsync(bnd, s);
     for (void *p : {(void *)kin, (void *)idin, (void *)kout, (void *)idout, (void *)succ, (void *)lsize,
                     (void *)loff, (void *)nl, (void *)tot})
         cudaFreeAsync(p, s);
@@ -652,6 +688,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
         cudaFreeAsync(dist[b], s);
         cudaFreeAsync(rnx[b], s);
     }
+    if (st != GWN_OK) return st;
     GWN_LAUNCH_CHECK("boundary chaining");
     return GWN_OK;
 }

@@ -194,7 +194,7 @@ gwn_status launch_classify_grid(const gwn_mesh *m, const float *gx, int nx, cons
              }()) == GWN_OK) {
             cudaMemsetAsync(len, 0, sizeof(unsigned long long), s);
             k_grid_points<<<grid_for(n, 256), 256, 0, s>>>(gx, nx, gy, ny, gz, n, pts);
-            if ((st = launch_boundary_sum_list(m, pts, n, chi, wt, label, true, list, len, s)) == GWN_OK)
+            if ((st = launch_boundary_sum_list(m, pts, n, chi, wt, label, true, list, len, SumOrder::kCaller, s)) == GWN_OK)
                 st = launch_fp64_fix_list(m, pts, chi, wt, label, list, len, s);
         }
         for (void *p : {(void *)pts, (void *)list, (void *)len}) if (p) cudaFreeAsync(p, s);

@@ -114,6 +114,7 @@ enum CounterSlot {
 enum ErrorBits { ERR_TRAVERSAL_LIMIT = 1 };
 
 struct Surrogate;   // mlp.cu
+struct FarNode;     // farfield.cuh
 
 // bytes of a mesh's device status block: the counters and the fixed-point frame
 constexpr size_t kStatusBytes = sizeof(unsigned long long) * CNT_SLOTS + 64;
@@ -145,6 +146,13 @@ struct gwn_mesh {
                                                // fixed-point frame (quant.cuh), kStatusBytes in all
     int4 *leaf_q = nullptr;                    // [3 nt] snapped leaf triangles (quantize_bits = 30)
     float *box = nullptr;                      // [6] vertex box: min x, y, z, max x, y, z (after the build)
+    gwn::FarNode *far_nodes = nullptr;         // boundary hierarchy (farfield.cuh), or NULL: summed directly
+    float4 *far_pts = nullptr;                 // [npts] the chained points in the hierarchy's loop order
+    float *far_coef = nullptr;                 // [far_nn][kFarCoef] its expansions
+    int64_t far_nn = 0;
+    int32_t *far_roots = nullptr;              // [far_nroots + 1] the subtrees that cover the boundary, in preorder
+    int far_nroots = 0;
+    double far_cost = 0.0;                     // its mean cost per query, in FP32 operations
     gwn::Surrogate *sur = nullptr;             // optional learned surrogate (mlp.cu)
 };
 
@@ -165,6 +173,9 @@ gwn_status order_queries(const gwn_mesh *m, const float *q, int64_t n, uint32_t 
 gwn_status order_query_list(const gwn_mesh *m, const float *q, int32_t *list, int64_t n, cudaStream_t s);
 gwn_status scatter_f32(const float *in, const uint32_t *perm, int64_t n, float *out, cudaStream_t s);
 gwn_status scatter_i32(const int32_t *in, const uint32_t *perm, int64_t n, int32_t *out, cudaStream_t s);
+gwn_status gather_i32(const int32_t *in, const uint32_t *perm, int64_t n, int32_t *out, cudaStream_t s);
+// list entries (at most n, *len of them on the device) i -> perm[i]
+gwn_status map_list(int32_t *list, const unsigned long long *len, int64_t n, const uint32_t *perm, cudaStream_t s);
 gwn_status scatter_u8(const uint8_t *in, const uint32_t *perm, int64_t n, uint8_t *out, cudaStream_t s);
 // batches at least this large are evaluated in Morton order
 constexpr int64_t kOrderMinQueries = 16384;
@@ -183,14 +194,30 @@ gwn_status launch_chi_visits(const gwn_mesh *m, const float *q, int64_t n, int32
                              unsigned long long *visits, cudaStream_t s);
 // boundary-curve sum + combine; with classify, labels and appends queries within
 // the margin to list (length counter list_len, zeroed by the caller)
+enum class SumOrder {
+    kSpatial,   // a large batch is in spatial order: it may take the boundary hierarchy
+    kCaller,    // any order: ordered here first if it takes the hierarchy
+    kDirect,    // the direct sum (the surrogate's training labels: the same bits, so the same network)
+};
 gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi,
                                     float *w, uint8_t *label, bool classify, int32_t *list,
-                                    unsigned long long *list_len, cudaStream_t s);
+                                    unsigned long long *list_len, SumOrder order, cudaStream_t s);
 // FP64 re-evaluation of the listed queries (rewrites w and label)
 gwn_status launch_fp64_fix_list(const gwn_mesh *m, const float *q, const int32_t *chi, float *w,
                                 uint8_t *label, const int32_t *list, const unsigned long long *list_len,
                                 cudaStream_t s);
 gwn_status launch_direct(const gwn_mesh *m, const float *q, int64_t n, float *w, cudaStream_t s);
+// bsum_far.cu: the same sums over the boundary hierarchy.  far_pays: whether a call
+// with n queries takes it; listed etc. as for the direct sum
+bool far_pays(const gwn_mesh *m, int64_t n);
+gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
+                               uint8_t *label, bool classify, bool running, int32_t *list,
+                               unsigned long long *list_len, unsigned *listed, double *partial_buf,
+                               int64_t partial_cap, cudaStream_t s);
+// query.cu: w = chi + (sum over chunks, in order) / 2pi of partial [chunks][n], then the labels
+void launch_boundary_combine(const double *partial, int64_t n, int chunks, const int32_t *chi, float *w,
+                             uint8_t *label, bool classify, float margin, int32_t *list,
+                             unsigned long long *list_len, unsigned *listed, cudaStream_t s);
 // quant.cu: the fixed-point frame of the mesh (quantize_bits), written into the
 // status block; bits = 0 (exact FP32 predicates) unless configured
 gwn_status setup_quant(gwn_mesh *m, cudaStream_t s);

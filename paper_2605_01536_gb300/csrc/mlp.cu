@@ -951,7 +951,7 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
             if (chi_test) k_gather_i32<<<g, 256, 0, st>>>(chi_all, list, len, cf);
         }
         if (r == GWN_OK && (r = chi_test ? GWN_OK : launch_chi(m, qf, nf, cf, st)) == GWN_OK &&
-            (r = launch_boundary_sum_list(m, qf, nf, cf, wf, lf, true, l2, len2, st)) == GWN_OK &&
+            (r = launch_boundary_sum_list(m, qf, nf, cf, wf, lf, true, l2, len2, SumOrder::kSpatial, st)) == GWN_OK &&
             (r = launch_fp64_fix_list(m, qf, cf, wf, lf, l2, len2, st)) == GWN_OK)
             k_scatter_wl<<<g, 256, 0, st>>>(list, len, wf, lf, w, label);
         for (void *p : {(void *)qf, (void *)wf, (void *)lf, (void *)cf, (void *)l2, (void *)len2}) cudaFreeAsync(p, st);
@@ -1029,7 +1029,7 @@ gwn_status gwn_surrogate_train(gwn_mesh *m, const float *samples, const float *t
         GWN_CUDA_TRY(dev_alloc(&own, sizeof(float) * n, st));
         GWN_CUDA_TRY(dev_alloc(&chi, sizeof(int32_t) * n, st));
         if ((r = launch_chi(m, samples, n, chi, st)) == GWN_OK)
-            r = launch_boundary_sum_list(m, samples, n, chi, own, nullptr, false, nullptr, nullptr, st);
+            r = launch_boundary_sum_list(m, samples, n, chi, own, nullptr, false, nullptr, nullptr, SumOrder::kDirect, st);
         cudaFreeAsync(chi, st);
         if (r != GWN_OK) return r;
         tgt = own;
@@ -1236,7 +1236,7 @@ gwn_status gwn_surrogate_calibrate(gwn_mesh *m, const float *samples, int64_t n,
                                                nullptr, 0.f, s->err);
     gwn_status r;
     if ((r = launch_chi(m, samples, n, chi, st)) == GWN_OK &&
-        (r = launch_boundary_sum_list(m, samples, n, chi, w, lab, true, list, len, st)) == GWN_OK &&
+        (r = launch_boundary_sum_list(m, samples, n, chi, w, lab, true, list, len, SumOrder::kCaller, st)) == GWN_OK &&
         (r = launch_fp64_fix_list(m, samples, chi, w, lab, list, len, st)) == GWN_OK)
         k_calib_hist<<<grid_for(n, 256), 256, 0, st>>>(mlp_dev(s), samples, w_hat, lab, chi, s->cfg.chi_tol, n,
                                                        hist);

@@ -17,16 +17,13 @@
 
 #include "gwn_internal.cuh"
 #include "predicates.cuh"
-#include "atan_poly.cuh"
-#include "fp32x2.cuh"
+#include "bterms.cuh"
 #include "traverse.cuh"
 
 namespace gwn {
 
 namespace {
 
-constexpr double kInv2Pi = 0.15915494309189533577;
-constexpr float kPiF = 3.14159265358979f;
 
 // Launched in blocks of 128 threads (compiled for up to 256): finer tails than
 // 256 (measured 5.6% faster on 2M soup8 queries, bit-identical).
@@ -89,206 +86,6 @@ __global__ void __launch_bounds__(256) k_chi_visits(const float *__restrict__ q,
     }
 }
 
-// ------------------------------------------------------ boundary terms ----
-
-// atan2 for the hot loops: octant reduction to t = min/max in [0, 1], then
-// atan(t) = t P(t^2) with the minimax polynomial of atan_poly.cuh (fitted by
-// fit_atan.py), then the octant is undone.  Branch-free.  Callers never pass
-// (0, 0).  The larger magnitude is clamped to the smallest normal float only
-// to keep the approximate reciprocal finite; every operand the kernels pass is
-// a normal number (an accepted group product is at least (4.9e-5)^8 ~ 3e-35),
-// so the clamp never changes a result.
-constexpr float kFltMin = 1.17549435e-38f;
-__device__ __forceinline__ float fast_atan2(float y, float x) {
-    const float ax = fabsf(x), ay = fabsf(y);
-    const float mx = fmaxf(fmaxf(ax, ay), kFltMin), mn = fminf(ax, ay);
-    const float t = mn * sfu_rcp(mx);
-    const float s = t * t;
-    float r = gwn_atan_poly(s) * t;
-    r = ay > ax ? 1.57079632679489662f - r : r;
-    r = x < 0.f ? 3.14159265358979324f - r : r;
-    return copysignf(r, y);
-}
-
-// Unit vector from the query to a boundary point, kept as (A_x, A_y, H) with
-// H = 1 - A_z computed without cancellation: (A_x^2 + A_y^2) / (1 + A_z) when
-// A_z > 0.  The point coincident with the query gives (0, 0, 0).  With two such
-// vectors A, B the van Oosterom-Strackee numerator and denominator of
-// Area(A, B, x1) / 2 for x1 = (0, 0, -1) are
-//   n = A.(B x x1) = A_y B_x - A_x B_y,
-//   d = 1 + A.B + A.x1 + B.x1 = H_a H_b + A_x B_x + A_y B_y.
-struct PointRel {
-    float ax, ay, h;
-};
-
-// Limit of atan2(n, d) for the edge (u, v) when u lies exactly on the query's
-// vertical ray (u - q = (0, 0, h), h > 0): the perturbed unit vector to u is
-// (-e1/h, -e2/h, 1), so n ~ e1 r_y - e2 r_x and d ~ -e1 r_x - e2 r_y with
-// r = v - q; hence atan2(r_y, -r_x), and for r_y = 0 the e2 order gives -pi
-// (r_x > 0) or 0 (r_x < 0).
-__device__ __forceinline__ float apex_angle(float rx, float ry, bool &degenerate) {
-    if (ry != 0.f) return atan2f(ry, -rx);
-    if (rx > 0.f) return -kPiF;
-    if (rx < 0.f) return 0.f;
-    degenerate = true;
-    return 0.f;
-}
-
-// Rare path of one edge term: n = d = 0 (a boundary vertex straight above the
-// query, or the query on the edge), or d <= 0 with |n| within its rounding
-// bound (the atan2 branch cut, where the sign of n is the exact perturbed sign
-// of the 2-D edge classification, Supp. S2.1).
-__device__ __noinline__ float edge_angle_slow(float4 Pa, float4 Pb, float qx, float qy, float qz, float n, float d,
-                                               unsigned long long *counters) {
-    if (n == 0.f && d == 0.f) {
-        const float ax = Pa.x - qx, ay = Pa.y - qy, az = Pa.z - qz;
-        const float bx = Pb.x - qx, by = Pb.y - qy, bz = Pb.z - qz;
-        bool deg = false;
-        float t;
-        const bool a_up = ax == 0.f && ay == 0.f, b_up = bx == 0.f && by == 0.f;
-        if (a_up && !b_up && az > 0.f) {
-            t = apex_angle(bx, by, deg);
-        } else if (b_up && !a_up && bz > 0.f) {
-            t = -apex_angle(ax, ay, deg);
-        } else {
-            deg = true;
-            t = 0.f;
-        }
-        atomicAdd(&counters[deg ? CNT_DEGENERATE : CNT_APEX], 1ull);
-        return t;
-    }
-    atomicAdd(&counters[CNT_EXACT_BRANCH], 1ull);
-    const int s = branch_sos(qx, qy, Pa.x, Pa.y, Pb.x, Pb.y, counters);   // n ~ -classification
-    const float mag = fabsf(n);
-    return atan2f(s > 0 ? -mag : mag, d);
-}
-
-// One edge term atan2(n, d).  |n - n_exact| <= ~4u (|A_y B_x| + |A_x B_y|) + the
-// rounding of the unit vectors; 1e-6 (|A_y B_x| + |A_x B_y|) + 1e-30 covers it
-// with margin, so outside that band the FP32 sign of n is the exact one.
-__device__ __forceinline__ float edge_term(float n, float d, const PointRel &A, const PointRel &B, float4 Pa,
-                                           float4 Pb, float qx, float qy, float qz, unsigned long long *counters) {
-    if (d <= 0.f && fabsf(n) <= fmaf(1e-6f, fabsf(A.ay * B.ax) + fabsf(A.ax * B.ay), 1e-30f))
-        return edge_angle_slow(Pa, Pb, qx, qy, qz, n, d, counters);
-    return fast_atan2(n, d);
-}
-
-struct PointRel2 {
-    float2 ax, ay, h;
-};
-
-// point_rel for two queries (nqx, nqy, nqz hold minus the query coordinates).
-// H = 1 - A_z without a select: with g = 1 + |A_z|, hh = (A_x^2 + A_y^2) / g
-// equals 1 - |A_z| (no cancellation), and H = hh + (|A_z| - A_z).
-__device__ __forceinline__ PointRel2 point_rel2(float4 P, float2 nqx, float2 nqy, float2 nqz) {
-    const float2 dx = add2(bc2(P.x), nqx), dy = add2(bc2(P.y), nqy), dz = add2(bc2(P.z), nqz);
-    const float2 s = fma2(dx, dx, mul2(dy, dy));
-    const float2 r2 = add2(fma2(dz, dz, s), bc2(1e-37f));    // > 0 even for a coincident point
-    const float2 inv = make_float2(sfu_rsqrt(r2.x), sfu_rsqrt(r2.y));
-    PointRel2 r;
-    r.ax = mul2(dx, inv);
-    r.ay = mul2(dy, inv);
-    const float2 az = mul2(dz, inv);
-    const float2 aaz = make_float2(fabsf(az.x), fabsf(az.y));
-    const float2 g = add2(bc2(1.0f), aaz);
-    const float2 hh = mul2(mul2(mul2(s, inv), inv), make_float2(sfu_rcp(g.x), sfu_rcp(g.y)));
-    r.h = add2(hh, add2(aaz, neg2(az)));
-    return r;
-}
-
-
-// fast_atan2 for two (y, x) pairs at once
-__device__ __forceinline__ float2 fast_atan2_2(float2 y, float2 x) {
-    const float axx = fabsf(x.x), axy = fabsf(x.y), ayx = fabsf(y.x), ayy = fabsf(y.y);
-    const float mxx = fmaxf(fmaxf(axx, ayx), kFltMin), mxy = fmaxf(fmaxf(axy, ayy), kFltMin);
-    const float2 t = mul2(make_float2(fminf(axx, ayx), fminf(axy, ayy)), make_float2(sfu_rcp(mxx), sfu_rcp(mxy)));
-    const float2 s = mul2(t, t);
-    float2 p = bc2(GWN_ATAN_C8);
-    p = fma2(p, s, bc2(GWN_ATAN_C7));
-    p = fma2(p, s, bc2(GWN_ATAN_C6));
-    p = fma2(p, s, bc2(GWN_ATAN_C5));
-    p = fma2(p, s, bc2(GWN_ATAN_C4));
-    p = fma2(p, s, bc2(GWN_ATAN_C3));
-    p = fma2(p, s, bc2(GWN_ATAN_C2));
-    p = fma2(p, s, bc2(GWN_ATAN_C1));
-    p = fma2(p, s, bc2(GWN_ATAN_C0));
-    const float2 r = mul2(p, t);
-    // undo the octant reduction: r -> A + B r with (A, B) from (|y| > |x|, x < 0)
-    const bool fx1 = ayx > axx, fy1 = ayy > axy, fx2 = x.x < 0.f, fy2 = x.y < 0.f;
-    const float2 A = make_float2(fx1 ? 1.57079632679489662f : (fx2 ? 3.14159265358979324f : 0.f),
-                                 fy1 ? 1.57079632679489662f : (fy2 ? 3.14159265358979324f : 0.f));
-    const float2 B = make_float2((fx1 != fx2) ? -1.f : 1.f, (fy1 != fy2) ? -1.f : 1.f);
-    const float2 o = fma2(B, r, A);
-    return make_float2(copysignf(o.x, y.x), copysignf(o.y, y.y));
-}
-
-// Terms are grouped GROUP edges at a time: each term's (d + i n) is multiplied
-// into a running product, one atan2 per group.  The product's argument equals
-// the sum of the accepted angles as long as it never passes +-pi, which either
-// of two acceptance tests guarantees:
-// - per term (the default for sparse boundaries): |n| < tan(pi/GROUP) d -
-//   kAccept, each angle below pi/8 in magnitude, so 8 of them sum to less
-//   than pi.  The test depends on the term alone, off the product's chain.
-// - running (dense boundaries, where many terms are steep: on random soups
-//   2.5% fail the per-term test, 0.35% this one): d > kMinD and the product
-//   with the term keeps a positive real part.  By induction the argument
-//   stays in (-pi/2, pi/2): an accepted angle is below pi/2 in magnitude
-//   (d > 0), so the new argument lies in (-pi, pi), and a positive real part
-//   puts it in (-pi/2, pi/2).  Rounding can only matter where the real part is
-//   near zero, an argument near +-pi/2, where atan2 is continuous.  The test
-//   sits on the product's chain (compare, then select), which costs 9% where
-//   nearly every term passes either test.
-// Both margins keep every accepted factor's modulus above 4.9e-5, so a product
-// of 8 factors of modulus at most 4 neither underflows nor overflows.  A term
-// that is not accepted (an edge seen steeply from the query, the atan2 branch
-// cut, a vertex straight above) leaves the product unchanged and takes its own
-// atan2, with the exact branch-cut sign and apex limit where they apply.
-constexpr int GROUP = 8;
-constexpr float kTanGroup = 0.41f;     // < tan(pi/8) = 0.41421
-constexpr float kAccept = 2e-5f;
-constexpr float kMinD = 5e-5f;
-
-template <int KP>
-struct BsumState {
-    float2 re[KP], im[KP], part[KP], comp[KP];
-};
-
-// part + x as an unevaluated sum part + comp (Knuth's TwoSum, error folded into
-// comp): keeps the FP32 running sum of group angles accurate to about one
-// rounding however many groups a tile holds.
-__device__ __forceinline__ void two_sum_acc2(float2 &part, float2 &comp, float2 x) {
-    const float2 s = add2(part, x);
-    const float2 bv = add2(s, neg2(part));
-    const float2 av = add2(s, neg2(bv));
-    const float2 err = add2(add2(part, neg2(av)), add2(x, neg2(bv)));
-    comp = add2(comp, err);
-    part = s;
-}
-
-__device__ __forceinline__ void two_sum_acc(float &part, float &comp, float x) {
-    const float s = part + x;
-    const float bv = s - part;
-    const float av = s - bv;
-    comp += (part - av) + (x - bv);
-    part = s;
-}
-
-// Load the block's queries: thread t holds queries base + t + k * blockDim.x,
-// k < 2 KP, as KP float2 pairs of negated coordinates (NaN past n).
-template <int KP>
-__device__ __forceinline__ void load_query_pairs(const float *__restrict__ q, int64_t base, int64_t n,
-                                                 float2 (&nqx)[KP], float2 (&nqy)[KP], float2 (&nqz)[KP]) {
-#pragma unroll
-    for (int k = 0; k < 2 * KP; ++k) {
-        const int64_t idx = base + (int64_t)k * blockDim.x;
-        const bool ok = idx < n;
-        const float nan = __int_as_float(0x7fc00000);
-        const float x = ok ? -q[3 * idx] : nan, y = ok ? -q[3 * idx + 1] : nan, z = ok ? -q[3 * idx + 2] : nan;
-        if (k & 1) { nqx[k >> 1].y = x; nqy[k >> 1].y = y; nqz[k >> 1].y = z; }
-        else       { nqx[k >> 1].x = x; nqy[k >> 1].x = y; nqz[k >> 1].x = z; }
-    }
-}
-
 // Boundary terms of the edges starting at points [e_begin, e_end) for the
 // block's 2 KP queries per thread, added to the thread's FP64 accumulators in
 // shared memory, s_acc[k * blockDim.x + threadIdx.x] (touched once per tile, so
@@ -296,225 +93,6 @@ __device__ __forceinline__ void load_query_pairs(const float *__restrict__ q, in
 // block streams the chained points through shared memory (tile + 1 points);
 // point j carries flag w = 1 when an edge runs from it to point j+1.  Every
 // thread of the block must call it.
-// Deferred fallback terms (the batched kernel's variant).  Where many terms
-// fail the group test (dense soups: about 1 in 40), nearly every warp-edge has
-// some failing lane, and computing the failing terms in place runs the scalar
-// path once per query slot with most lanes idle.  Instead each warp appends its
-// failing (query, edge) pairs to a queue in shared memory, entry
-// j << 7 | k << 5 | lane (edge j of the tile, query slot k of that lane), and
-// drains it with all 32 lanes once it holds 32 KQ entries and at the end of
-// every tile.  Drained terms are added to per-query 64-bit fixed-point sums
-// (units of 2^-40 rad) with integer atomics: exact, so the result does not
-// depend on the order of the drain.
-constexpr float kFixScale = 0x1p40f;
-
-// Scalar twins of point_rel2 and edge_nd2: the same operations in the same
-// order with explicit rounding (no contraction), so a drained term is computed
-// from bit-identical n and d to the ones the group test saw.  Near n = d = 0
-// (an apex seen almost head-on) atan2 is ill-conditioned enough that another
-// rounding of the unit vectors moves the term by ~1e-5 rad.
-__device__ __forceinline__ PointRel point_rel_twin(float4 P, float qx, float qy, float qz) {
-    const float dx = __fadd_rn(P.x, -qx), dy = __fadd_rn(P.y, -qy), dz = __fadd_rn(P.z, -qz);
-    const float s = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
-    const float r2 = __fadd_rn(__fmaf_rn(dz, dz, s), 1e-37f);
-    const float inv = sfu_rsqrt(r2);
-    PointRel r;
-    r.ax = __fmul_rn(dx, inv);
-    r.ay = __fmul_rn(dy, inv);
-    const float az = __fmul_rn(dz, inv);
-    const float aaz = fabsf(az);
-    const float g = __fadd_rn(1.0f, aaz);
-    const float hh = __fmul_rn(__fmul_rn(__fmul_rn(s, inv), inv), sfu_rcp(g));
-    r.h = __fadd_rn(hh, __fadd_rn(aaz, -az));
-    return r;
-}
-
-// Ill-conditioned terms: |d + i n| < 2^-6 H_a H_b.  A term's FP32 rounding
-// error is a few units of rounding of the products that make up n and d,
-// whose size is about H_a H_b where the term is ill-conditioned (the unit
-// vectors to the edge's ends nearly opposite: the query close to the edge),
-// divided by |d + i n|; below 2^-6 H_a H_b the amplification exceeds 64 and
-// the term is recomputed in FP64 from the FP32 inputs, where the differences
-// to the query are exact.  |d + i n|^2 = 2 (1 + A.B) H_a H_b for unit A, B, so
-// this needs 1 + A.B < H_a H_b / 8192: A and B within 1/45 rad of opposite.
-// The hot loop tests it (paired, the same arithmetic) only in warps near the
-// boundary tile, and keeps such terms out of the group products.
-constexpr float kCancel = 0x1p-6f;
-__device__ __forceinline__ bool cancels(float n, float d, float ha, float hb) {
-    const float t = kCancel * (ha * hb);
-    return fmaf(n, n, d * d) < t * t;
-}
-__device__ double edge_angle64(float4 Pa, float4 Pb, float qx, float qy, float qz,
-                               const unsigned long long *counters);
-
-// The FP64 evaluation does not run inside the edge loop: its registers would
-// crowd the loop's (a call to it from there cost 9% of the kernel).  A
-// cancelling term found in the loop is put on a per-warp queue in shared
-// memory, entry j << 7 | k << 5 | lane (edge j of the tile, query slot k of that
-// lane), and the warp evaluates the queue in FP64 after the tile's edges, where
-// the loop's registers are free; the results go to per-query 64-bit
-// fixed-point sums (units of 2^-40 rad) with integer atomics, exact and
-// independent of the order.  A queue that is full (more than kCancelCap such
-// terms for one warp in one tile) lists the query for a full FP64
-// re-evaluation instead (k_fp64_fix), once per query (the listed bits).
-constexpr int kCancelCap = 64;
-constexpr double kFixUnit = 0x1p-40;
-constexpr double kFixScale64 = 0x1p40;
-
-struct CancelQ {
-    unsigned *queue;            // this warp's queue, kCancelCap entries
-    int *count;                 // this warp's entry count
-    long long *fix;             // fixed-point sums, fix[k blockDim.x + t]
-    const float *q;             // the block's queries: slot k of thread t at q[3 (t + k blockDim.x)]
-    int64_t qbase;              // caller's index of the block's query slot 0 of thread 0 (for the list)
-    int32_t *list;              // queries for a full FP64 re-evaluation (NULL: count the term as
-    unsigned long long *list_len;   //  an FP32 one and record it in CNT_CANCEL_OVERFLOW)
-    unsigned *listed;           // one bit per query: already listed
-};
-
-// Put query idx on the FP64 re-evaluation list unless it is there already.
-__device__ __forceinline__ void list_query(int64_t idx, int32_t *list, unsigned long long *list_len,
-                                           unsigned *listed) {
-    const unsigned bit = 1u << (idx & 31);
-    if (atomicOr(&listed[idx >> 5], bit) & bit) return;
-    list[atomicAdd(list_len, 1ull)] = (int32_t)idx;
-}
-
-// Queue a cancelling term; false when the queue is full and the query has been
-// listed for a full FP64 re-evaluation (or there is no list).
-__device__ __forceinline__ bool cancel_enqueue(const CancelQ &cq, int j, int k, int lane) {
-    const int slot = atomicAdd(cq.count, 1);
-    if (slot < kCancelCap) {
-        cq.queue[slot] = (unsigned)j << 7 | (unsigned)k << 5 | (unsigned)lane;
-        return true;
-    }
-    if (cq.list) list_query(cq.qbase + (threadIdx.x & ~31) + lane + (int64_t)k * blockDim.x, cq.list, cq.list_len,
-                            cq.listed);
-    return false;
-}
-
-// FP64 evaluation of this warp's queued terms (points of the staged tile); all
-// 32 lanes of the warp call it, with the loop's registers out of use.
-__device__ __noinline__ void cancel_drain(const CancelQ &cq, const float4 *s_pts, unsigned long long *counters) {
-    __syncwarp();
-    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    const int count = min(*cq.count, kCancelCap);
-    for (int r = lane; r < count; r += 32) {
-        const unsigned e = cq.queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
-        const int local = owner + k * (int)blockDim.x;
-        const double t = edge_angle64(s_pts[j], s_pts[j + 1], cq.q[3 * local], cq.q[3 * local + 1],
-                                      cq.q[3 * local + 2], counters);
-        atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
-                  (unsigned long long)__double2ll_rn(t * kFixScale64));
-    }
-    if (lane == 0 && count > 0) atomicAdd(&counters[CNT_CANCEL], (unsigned long long)count);
-    __syncwarp();
-    if (lane == 0) *cq.count = 0;
-    __syncwarp();
-}
-
-// A term that failed the group test and does not cancel, from the n and d the
-// test saw.  Out of line: it runs for a few terms in a thousand, and inlined its
-// registers would crowd the group loop.
-__device__ __noinline__ float fallback_term(float n, float d, PointRel a, PointRel b, float4 Pa, float4 Pb, float qx,
-                                            float qy, float qz, unsigned long long *counters) {
-    return edge_term(n, d, a, b, Pa, Pb, qx, qy, qz, counters);
-}
-
-struct BsumDefer {
-    const float *q;            // the block's queries: query slot k of thread t at q[3 (t + k blockDim.x)]
-    unsigned *queue;           // this warp's queue, 64 KQ entries
-    long long *fix;            // fixed-point sums, fix[k blockDim.x + t]
-};
-
-// The deferred terms of the batched kernel, drained by all 32 lanes.  With
-// Cond, a term whose d cancels goes on the cancellation queue (FP64 after the
-// tile) instead; if that is full it is taken in FP32 and counted.
-template <bool Cond>
-__device__ __noinline__ void bsum_drain(const unsigned *queue, int count, const float4 *s_pts, const float *q,
-                                        long long *fix, CancelQ cq, unsigned long long *counters) {
-    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    for (int r = lane; r < count; r += 32) {
-        const unsigned e = queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
-        const int local = owner + k * (int)blockDim.x;
-        const float4 Pa = s_pts[j], Pb = s_pts[j + 1];
-        const float qx = q[3 * local], qy = q[3 * local + 1], qz = q[3 * local + 2];
-        const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
-        const float n = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
-        const float d = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
-        if (Cond && cancels(n, d, A.h, B.h)) {
-            const int slot = atomicAdd(cq.count, 1);
-            if (slot < kCancelCap) {
-                cq.queue[slot] = (unsigned)j << 7 | (unsigned)k << 5 | (unsigned)(e & 31u);
-                continue;
-            }
-            if (cq.list) list_query(cq.qbase + local, cq.list, cq.list_len, cq.listed);
-            else atomicAdd(&counters[CNT_CANCEL_OVERFLOW], 1ull);
-        }
-        const float t = edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
-        atomicAdd(reinterpret_cast<unsigned long long *>(fix + (k * (int)blockDim.x + owner)),
-                  (unsigned long long)__float2ll_rn(t * kFixScale));
-    }
-    __syncwarp();
-}
-
-// Box of the staged tile's points (points 0..cnt) widened on every side by a
-// tenth of its longest edge, into box[0..5] = (min x, max x, min y, max y,
-// min z, max z) for every thread of the block.  An ill-conditioned term,
-// |d + i n| < H_a H_b / 64, has |d + i n|^2 = 2 (1 + A.B) H_a H_b below
-// (H_a H_b)^2 / 4096, so 1 + A.B < H_a H_b / 8192 <= 4.9e-4 (H_a H_b <= 4): the
-// edge subtends an angle within 0.032 rad of pi, which puts the query within
-// 0.032 L of the edge (L its length).  A tenth of the longest edge leaves a
-// factor of three for rounding.  Contains barriers: every thread of the block
-// must call it.
-__device__ __noinline__ void tile_box(const float4 *s_pts, int cnt, float *box) {
-    __shared__ float s_red[8][8];   // up to 8 warps x (3 minima, 3 maxima, edge length^2)
-    float v[7] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY, 0.f};
-    for (int i = threadIdx.x; i <= cnt; i += blockDim.x) {
-        const float4 P = s_pts[i];
-        v[0] = fminf(v[0], P.x); v[1] = fminf(v[1], P.y); v[2] = fminf(v[2], P.z);
-        v[3] = fmaxf(v[3], P.x); v[4] = fmaxf(v[4], P.y); v[5] = fmaxf(v[5], P.z);
-        if (i < cnt && P.w != 0.f) {
-            const float4 Q = s_pts[i + 1];
-            const float dx = Q.x - P.x, dy = Q.y - P.y, dz = Q.z - P.z;
-            v[6] = fmaxf(v[6], dx * dx + dy * dy + dz * dz);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = fminf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-#pragma unroll
-        for (int k = 3; k < 7; ++k) v[k] = fmaxf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-    }
-    const int warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int k = 0; k < 7; ++k) s_red[warp][k] = v[k];
-    }
-    __syncthreads();
-    float r[7];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) r[k] = s_red[0][k];
-    for (int w = 1; w < nwarps; ++w) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) r[k] = fminf(r[k], s_red[w][k]);
-#pragma unroll
-        for (int k = 3; k < 7; ++k) r[k] = fmaxf(r[k], s_red[w][k]);
-    }
-    __syncthreads();   // s_red is reused by the next tile
-    const float L = 0.1f * sqrtf(r[6]);
-    box[0] = r[0] - L; box[1] = r[3] + L;
-    box[2] = r[1] - L; box[3] = r[4] + L;
-    box[4] = r[2] - L; box[5] = r[5] + L;
-}
-
-__device__ __forceinline__ bool in_box(const float *b, float x, float y, float z) {
-    return x >= b[0] && x <= b[1] && y >= b[2] && y <= b[3] && z >= b[4] && z <= b[5];
-}
-
 template <int KP, bool Defer = false, bool Cond = false, bool Running = false>
 __device__ __forceinline__ void bsum_accumulate(const float4 *__restrict__ pts, int64_t e_begin, int64_t e_end,
                                                 int tile, float4 *s_pts, const float2 (&nqx)[KP],
@@ -894,90 +472,6 @@ __global__ void k_boundary_combine(const double *__restrict__ partial, int64_t n
     }
 }
 
-// --------------------------------------------------- FP64 re-evaluation ----
-
-__device__ double apex_angle64(double rx, double ry, bool &degenerate) {
-    if (ry != 0.0) return atan2(ry, -rx);
-    if (rx > 0.0) return -3.14159265358979323846;
-    if (rx < 0.0) return 0.0;
-    degenerate = true;
-    return 0.0;
-}
-
-__device__ double edge_angle64(float4 Pa, float4 Pb, float qx, float qy, float qz,
-                               const unsigned long long *counters) {
-    const double ax = (double)Pa.x - qx, ay = (double)Pa.y - qy, az = (double)Pa.z - qz;
-    const double bx = (double)Pb.x - qx, by = (double)Pb.y - qy, bz = (double)Pb.z - qz;
-    const double sa = ax * ax + ay * ay, sb = bx * bx + by * by;
-    const double la = sqrt(sa + az * az), lb = sqrt(sb + bz * bz);
-    const double ha = az > 0.0 ? sa / (la + az) : la - az;
-    const double hb = bz > 0.0 ? sb / (lb + bz) : lb - bz;
-    const double n = ay * bx - ax * by;
-    const double d = ha * hb + ax * bx + ay * by;
-    if (n == 0.0 && d == 0.0) {
-        bool deg = false;
-        if (ax == 0.0 && ay == 0.0 && ha == 0.0 && !(bx == 0.0 && by == 0.0)) return apex_angle64(bx, by, deg);
-        if (bx == 0.0 && by == 0.0 && hb == 0.0 && !(ax == 0.0 && ay == 0.0)) return -apex_angle64(ax, ay, deg);
-        return 0.0;
-    }
-    if (d < 0.0) {
-        const int s = branch_sos(qx, qy, Pa.x, Pa.y, Pb.x, Pb.y, counters);
-        return atan2(s > 0 ? -fabs(n) : fabs(n), d);
-    }
-    return atan2(n, d);
-}
-
-
-// FP64 boundary sum of one query over the edges that start at points
-// [j0, j1) of a chained point stream, for the re-evaluation kernels.  FP64 runs
-// at 1/64 of the FP32 rate here, so the terms are grouped like the FP32 path:
-// each point's unnormalised relative vector (l, and h = l - z without
-// cancellation) is formed once and shared by its two edges, and a term with
-// 0 < |n| / d < 0.41 (angle below pi/8) is multiplied into a complex product,
-// one atan2 per 8 edges.  1e-30 < d < 1e30 keeps a product of 8 such factors
-// inside the FP64 range whatever the coordinates' scale.  Every other term
-// (steep, on the branch cut, degenerate) is edge_angle64's, exactly as before.
-__device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64_t j1, float qx, float qy, float qz,
-                               const unsigned long long *counters) {
-    if (j0 >= j1) return 0.0;
-    double acc = 0.0, re = 1.0, im = 0.0;
-    int g = 0;
-    float4 P = pts[j0];
-    double ax = (double)P.x - qx, ay = (double)P.y - qy, az = (double)P.z - qz;
-    double sa = ax * ax + ay * ay;
-    double la = sqrt(sa + az * az);
-    double ha = az > 0.0 ? sa / (la + az) : la - az;
-    for (int64_t j = j0; j < j1; ++j) {
-        const float4 Q = pts[j + 1];
-        const double bx = (double)Q.x - qx, by = (double)Q.y - qy, bz = (double)Q.z - qz;
-        const double sb = bx * bx + by * by, lb = sqrt(sb + bz * bz);
-        const double hb = bz > 0.0 ? sb / (lb + bz) : lb - bz;
-        if (P.w != 0.f) {
-            const double n = ay * bx - ax * by, d = ha * hb + ax * bx + ay * by;
-            if (d > 1e-30 && d < 1e30 && fabs(n) < 0.41 * d) {
-                const double r = re * d - im * n;
-                im = re * n + im * d;
-                re = r;
-            } else {
-                acc += edge_angle64(P, Q, qx, qy, qz, counters);
-            }
-            if (++g == GROUP) {
-                acc += atan2(im, re);
-                re = 1.0;
-                im = 0.0;
-                g = 0;
-            }
-        }
-        P = Q;
-        ax = bx;
-        ay = by;
-        az = bz;
-        ha = hb;
-    }
-    if (g > 0) acc += atan2(im, re);
-    return acc;
-}
-
 // One block per listed query (grid-stride over the list): FP64 boundary sum,
 // fixed-order block reduction, then w and the label are rewritten.
 __global__ void __launch_bounds__(256) k_fp64_fix(const float *__restrict__ q, const float4 *__restrict__ pts,
@@ -1156,6 +650,14 @@ gwn_status launch_chi_visits(const gwn_mesh *m, const float *q, int64_t n, int32
     return GWN_OK;
 }
 
+void launch_boundary_combine(const double *partial, int64_t n, int chunks, const int32_t *chi, float *w,
+                             uint8_t *label, bool classify, float margin, int32_t *list,
+                             unsigned long long *list_len, unsigned *listed, cudaStream_t s) {
+    k_boundary_combine<<<grid_for(n, 256), 256, 0, s>>>(partial, n, chunks, chi, w, label, classify ? 1 : 0, margin,
+                                                        list, list_len, listed);
+    note_launches(1);
+}
+
 template <int KP, bool Cond = false, bool Running = false>
 static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                  uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
@@ -1174,7 +676,10 @@ static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, c
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // split the boundary into chunks when the query tiles alone cannot fill the GPU
     int64_t chunks = (8 * (int64_t)(sms > 0 ? sms : 148) + qblocks - 1) / qblocks;
-    chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (nedge_pts + 2 * tile - 1) / (2 * tile)));
+    // (a chunk of 128 points still pays for its partial sums: 64 queries against
+    // 9.8k edges take 47 us instead of 200 us with chunks of 1024 points)
+    const int64_t min_chunk = n < kOrderMinQueries ? std::min<int64_t>(128, 2 * tile) : 2 * tile;
+    chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (nedge_pts + min_chunk - 1) / min_chunk));
     if (partial_cap >= 0) chunks = std::min<int64_t>(chunks, partial_cap / n);   // caller-provided room
     chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, 65535));
     const int64_t chunk_len = chunks > 1 ? (nedge_pts + chunks - 1) / chunks : std::max<int64_t>(nedge_pts, 1);
@@ -1194,9 +699,7 @@ static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, c
                                                                       margin, list, list_len, listed, m->counters);
     note_launches(1);
     if (partial) {
-        k_boundary_combine<<<grid_for(n, 256), 256, 0, s>>>(partial, n, (int)chunks, chi, w, label,
-                                                            classify ? 1 : 0, margin, list, list_len, listed);
-        note_launches(1);
+        launch_boundary_combine(partial, n, (int)chunks, chi, w, label, classify, margin, list, list_len, listed, s);
         if (own) cudaFreeAsync(partial, s);
     }
     GWN_LAUNCH_CHECK("k_boundary_sum");
@@ -1218,10 +721,13 @@ static bool group_test_running(const gwn_mesh *m) {
 // needed when partial_cap < 0.
 static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                   uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                  unsigned *listed, double *partial_buf, int64_t partial_cap, cudaStream_t s) {
+                                  unsigned *listed, double *partial_buf, int64_t partial_cap, bool ordered,
+                                  cudaStream_t s) {
     const int kq = m->cfg.queries_per_thread > 0 ? m->cfg.queries_per_thread : 4;
     ProfScope prof("boundary_sum", s);
     const bool running = group_test_running(m);
+    if (ordered && far_pays(m, n))
+        return launch_boundary_far(m, q, n, chi, w, label, classify, running, list, list_len, listed, partial_buf, partial_cap, s);
 #define GWN_BSUM(KP, C, R) \
     launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, partial_cap, s)
     if (m->cfg.fp64_cancel >= 0) {   // the default: cancelling terms in FP64
@@ -1240,8 +746,33 @@ static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, 
 
 gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                     uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                    cudaStream_t s) {
+                                    SumOrder order, cudaStream_t s) {
     if (n <= 0) return GWN_OK;
+    if (order == SumOrder::kCaller && far_pays(m, n)) {
+        // the hierarchy wants neighbours in a warp: evaluate in spatial order, scatter back
+        uint32_t *keys = nullptr, *perm = nullptr;
+        float *qs = nullptr, *ws = nullptr;
+        int32_t *cs = nullptr;
+        uint8_t *ls = nullptr;
+        gwn_status st = [&]() -> gwn_status {
+            GWN_CUDA_TRY(dev_alloc(&keys, sizeof(uint32_t) * n, s));
+            GWN_CUDA_TRY(dev_alloc(&perm, sizeof(uint32_t) * n, s));
+            GWN_CUDA_TRY(dev_alloc(&qs, sizeof(float) * 3 * n, s));
+            GWN_CUDA_TRY(dev_alloc(&ws, sizeof(float) * n, s));
+            GWN_CUDA_TRY(dev_alloc(&cs, sizeof(int32_t) * n, s));
+            if (label) GWN_CUDA_TRY(dev_alloc(&ls, n, s));
+            return GWN_OK;
+        }();
+        if (st == GWN_OK && (st = order_queries(m, q, n, keys, perm, qs, s)) == GWN_OK &&
+            (st = gather_i32(chi, perm, n, cs, s)) == GWN_OK &&
+            (st = launch_boundary_sum_list(m, qs, n, cs, ws, ls, classify, list, list_len, SumOrder::kSpatial, s)) == GWN_OK &&
+            (st = scatter_f32(ws, perm, n, w, s)) == GWN_OK && (st = scatter_u8(ls, perm, n, label, s)) == GWN_OK &&
+            list)
+            st = map_list(list, list_len, n, perm, s);
+        for (void *p : {(void *)keys, (void *)perm, (void *)qs, (void *)ws, (void *)cs, (void *)ls})
+            if (p) cudaFreeAsync(p, s);
+        return st;
+    }
     const size_t words = (size_t)((n + 31) / 32);
     unsigned *listed = nullptr;
     GWN_CUDA_TRY(dev_alloc(&listed, sizeof(unsigned) * words, s));
@@ -1254,7 +785,8 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
         GWN_CUDA_TRY(dev_alloc(&list_len, sizeof(unsigned long long), s));
         GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     }
-    gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1, s);
+    gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1,
+                                    order == SumOrder::kSpatial, s);
     if (st == GWN_OK && own_list) st = launch_fp64_fix_list(m, q, chi, w, nullptr, list, list_len, s);
     cudaFreeAsync(listed, s);
     if (own_list) {
@@ -1280,7 +812,7 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
                                                                         m->counters);
     GWN_LAUNCH_CHECK("k_chi");
     gwn_status st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial,
-                                    partial ? partial_cap : 0, s);
+                                    partial ? partial_cap : 0, false, s);
     if (st != GWN_OK) return st;
     return launch_fp64_fix_list(m, q, chi_tmp, w, label, list, list_len, s);
 }
