@@ -63,6 +63,9 @@ int sm_count(int dev) {
     return sms > 0 ? sms : 148;
 }
 
+// Whether the mesh's triangle loops are summed as triangles in a batch.
+bool batch_split(const gwn_mesh *m) { return m->n_tri_loops > 0; }
+
 void drop_graph(gwn_batch *b) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     b->gexec = nullptr;
@@ -74,6 +77,7 @@ void drop_graph(gwn_batch *b) {
 // With qcap > 0 only the first qcap queries of each mesh get tiles (the
 // autotuner's timing subsample).
 gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, int64_t qcap = 0) {
+    tile = std::max(tile, 64);   // room for triangle loops, 5 points each
     const int T = 512 * kp;
     std::vector<BatchTile> tiles;
     std::vector<BatchItem> items;
@@ -82,8 +86,11 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
         const gwn_mesh *m = b->meshes[mi];
         const int64_t q0 = b->q_off[mi];
         const int64_t nq = qcap > 0 ? std::min<int64_t>(qcap, b->q_off[mi + 1] - q0) : b->q_off[mi + 1] - q0;
-        const int64_t nedge_pts = m->npts > 0 ? m->npts - 1 : 0;
-        const int64_t nchunks = nedge_pts > 0 ? (nedge_pts + chunk - 1) / chunk : 0;
+        const bool split = batch_split(m);
+        const int64_t npts = split ? m->n_rest : m->npts, ntri = split ? m->n_tri_loops : 0;
+        const int64_t nedge_pts = npts > 0 ? npts - 1 : 0;
+        const int64_t nchunks = (nedge_pts + chunk - 1) / chunk;
+        const int64_t tchunk = std::max(chunk / 8, 1), ntchunks = (ntri + tchunk - 1) / tchunk;
         const double chi_unit = 40.0 + 8.0 * std::log2((double)m->nt + 2.0);   // ~ one traversal in point terms
         // the autotuner's subsample: whole tiles spread evenly over the mesh's
         // (spatially ordered) queries, so that it samples the whole domain
@@ -96,11 +103,16 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
             tl.mesh = (int32_t)mi;
             tl.q_begin = q0 + t0;
             tl.q_count = (int32_t)std::min<int64_t>(T, nq_all - t0);
-            tl.n_items = (int32_t)(1 + nchunks);
+            tl.n_items = (int32_t)(1 + nchunks + ntchunks);
             const int32_t ti = (int32_t)tiles.size();
             tiles.push_back(tl);
             items.push_back(BatchItem{ti, 0, 0, 0});
             cost.push_back(chi_unit * tl.q_count);
+            for (int64_t c = 0; c < ntchunks; ++c) {   // a triangle costs about two points
+                const int64_t p0 = c * tchunk, p1 = std::min<int64_t>(ntri, p0 + tchunk);
+                items.push_back(BatchItem{ti, 2, p0, p1});
+                cost.push_back(2.0 * (double)(p1 - p0) * (double)T);
+            }
             for (int64_t c = 0; c < nchunks; ++c) {
                 const int64_t p0 = c * chunk, p1 = std::min<int64_t>(nedge_pts, p0 + chunk);
                 items.push_back(BatchItem{ti, 1, p0, p1});
@@ -274,7 +286,9 @@ gwn_status gwn_batch_create(const gwn_mesh *const *meshes, int32_t n_mesh, const
     std::vector<BatchMesh> md(std::max(n_mesh, 1));
     for (int i = 0; i < n_mesh; ++i) {
         const gwn_mesh *m = meshes[i];
-        md[i] = BatchMesh{m->nodes, m->leaf_tri, m->bpts, m->nnodes, m->npts, m->counters, m->box};
+        const bool split = batch_split(m);
+        md[i] = BatchMesh{m->nodes, m->leaf_tri, m->bpts, m->tri_loops, split ? m->rest_pts : m->bpts,
+                          split ? m->n_rest : m->npts, m->nnodes, m->npts, m->counters, m->box};
     }
     cudaError_t e;
     if ((e = cudaMalloc(&b->d_meshes, sizeof(BatchMesh) * md.size())) != cudaSuccess ||

@@ -519,6 +519,268 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
     return acc;
 }
 
+// ------------------------------------------------------- triangle loops ----
+//
+// A loop of three edges a -> b -> c bounds the triangle T = (a, b, c), and its
+// three antipodal terms sum to (Eq. 9 for T alone)
+//   2 pi S_T = atan2(det, den) - 2 pi cross(q, T),
+// half T's solid angle (van Oosterom-Strackee) minus the signed crossing of the
+// ray with T.  One such term costs 43 paired operations against 3 edges of about 60
+// each (random soups, whose every loop is a triangle, and small holes), and its
+// rounding is relative to the triangle's solid angle, not to the edges' steep angles.
+// With unit vectors A, B, C toward the vertices, N the triangle's normal vector:
+//   den = 1 + A.B + A.C + B.C,  det = (a . N) / (|a| |b| |c|).
+// The term enters the group product if 0.41 den - |det| > 0.05: its angle is below
+// pi/8 (8 factors stay below pi), away from the cut at +-pi, and den > 0.12 bounds
+// the amplification of rounding.  Otherwise (the query within about an edge's length)
+// it takes its own atan2 or, close to T, its three edges' terms.  A ray that meets the
+// triangle's box takes the crossing predicate; every other ray misses T.  Both are
+// deferred like the batched kernel's failing terms: about 3% of a warp's triangles have
+// such a lane (random soup, 100k queries), and done in place, with most lanes idle,
+// they cost more than all the rest.  Measured, edges -> triangles: soup8's direct sum with
+// 2M queries 383 -> 212 ms; 3,000 random triangles with 20k queries 0.83 -> 0.43 ms (2.0
+// ms with the terms done in place), 20,000 with 50k 6.6 -> 3.0 ms; the maximum error
+// against FP64 on soup8 1.3e-6 -> 5.2e-7.  Bound by the FP32 pipe (74 issue slots a term).
+struct __align__(16) TriLoop {
+    float4 a, b, c;   // the vertices; a.w = max z
+    float4 n;         // (b - a) x (c - a)
+    float4 box;       // min x, max x, min y, max y
+};
+static_assert(sizeof(TriLoop) == 80, "TriLoop must be 80 bytes");
+constexpr float kTriAccept = 0.05f;
+
+// The exact predicate, where the FP32 filter of tri_cross cannot decide.
+__device__ __noinline__ int tri_cross_exact(const TriLoop &T, float qx, float qy, float qz,
+                                            unsigned long long *counters) {
+    return tri_crossing(make_float3(qx, qy, qz), make_float3(T.a.x, T.a.y, T.a.z), make_float3(T.b.x, T.b.y, T.b.z),
+                        make_float3(T.c.x, T.c.y, T.c.z), &counters[CNT_EXACT_EDGE], &counters[CNT_EXACT_PLANE]);
+}
+
+// Signed crossing of the ray of a query inside the triangle's box.  The signs of the
+// three projected edge functions and of the plane side are those of the exact values
+// where they exceed 1e-6 of the sum of their products' magnitudes (16 units of
+// rounding; at most 4 to 6 occur).  *vertex is set when the query coincides with a
+// vertex (the term is then degenerate: its edges decide).
+__device__ __forceinline__ int tri_cross(const TriLoop &T, float qx, float qy, float qz, bool *vertex,
+                                         unsigned long long *counters) {
+    const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy, bz = T.b.z - qz,
+                cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
+    *vertex = (ax == 0.f && ay == 0.f && az == 0.f) || (bx == 0.f && by == 0.f && bz == 0.f) ||
+              (cx == 0.f && cy == 0.f && cz == 0.f);
+    const float p0 = ax * by, m0 = ay * bx, p1 = bx * cy, m1 = by * cx, p2 = cx * ay, m2 = cy * ax;
+    const float e0 = p0 - m0, e1 = p1 - m1, e2 = p2 - m2;
+    const bool clear = fabsf(e0) > fmaf(1e-6f, fabsf(p0) + fabsf(m0), 1e-30f) &&
+                       fabsf(e1) > fmaf(1e-6f, fabsf(p1) + fabsf(m1), 1e-30f) &&
+                       fabsf(e2) > fmaf(1e-6f, fabsf(p2) + fabsf(m2), 1e-30f);
+    if (clear) {
+        if ((e0 > 0.f) != (e1 > 0.f) || (e0 > 0.f) != (e2 > 0.f)) return 0;
+        const float nx = ax * T.n.x, ny = ay * T.n.y, nz = az * T.n.z, side = nx + ny + nz;
+        if (fabsf(side) > fmaf(1e-6f, fabsf(nx) + fabsf(ny) + fabsf(nz), 1e-30f))
+            return (side > 0.f) == (e0 > 0.f) ? (e0 > 0.f ? 1 : -1) : 0;
+    }
+    return tri_cross_exact(T, qx, qy, qz, counters);
+}
+
+__device__ __forceinline__ float4 tri_vertex(const TriLoop &T, int e) { return e == 0 ? T.a : e == 1 ? T.b : T.c; }
+
+// The three edge terms of triangle j (of the staged tile) for query slot k of a lane
+// (the block's query local); ill-conditioned ones go on the warp's FP64 queue (entry
+// 3 j + edge), or list the query when that is full.
+__device__ __noinline__ float tri_edges(const TriLoop &T, int j, int k, int lane, int local, float qx, float qy, float qz, const CancelQ &cq,
+                                        unsigned long long *counters) {
+    float sum = 0.f;
+    for (int e = 0; e < 3; ++e) {
+        const float4 Pa = tri_vertex(T, e), Pb = tri_vertex(T, e == 2 ? 0 : e + 1);
+        const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
+        const float n = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
+        const float d = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
+        if (cancels(n, d, A.h, B.h)) {
+            const int slot = atomicAdd(cq.count, 1);
+            if (slot < kCancelCap) {
+                cq.queue[slot] = (unsigned)(3 * j + e) << 7 | (unsigned)k << 5 | (unsigned)lane;
+                continue;
+            }
+            if (cq.list) list_query(cq.qbase + local, cq.list, cq.list_len, cq.listed);
+            else atomicAdd(&counters[CNT_CANCEL_OVERFLOW], 1ull);
+        }
+        sum += edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
+    }
+    return sum;
+}
+
+// FP64 evaluation of the warp's queued edges of the staged triangles (cancel_drain).
+__device__ __noinline__ void tri_drain(const CancelQ &cq, const TriLoop *s_tri, unsigned long long *counters) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
+    const int count = min(*cq.count, kCancelCap);
+    for (int r = lane; r < count; r += 32) {
+        const unsigned e = cq.queue[r];
+        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
+        const int local = owner + k * (int)blockDim.x, ed = j % 3;
+        const TriLoop &T = s_tri[j / 3];
+        const double t = edge_angle64(tri_vertex(T, ed), tri_vertex(T, ed == 2 ? 0 : ed + 1), cq.q[3 * local],
+                                      cq.q[3 * local + 1], cq.q[3 * local + 2], counters);
+        atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
+                  (unsigned long long)__double2ll_rn(t * kFixScale64));
+    }
+    if (lane == 0 && count > 0) atomicAdd(&counters[CNT_CANCEL], (unsigned long long)count);
+    __syncwarp();
+    if (lane == 0) *cq.count = 0;
+    __syncwarp();
+}
+
+// The warp's deferred triangle terms, drained by all 32 lanes: entry
+// fail << 31 | triangle of the tile << 7 | query slot << 5 | lane.  fail: the term is not
+// in the group product.  Sums go to the fixed-point accumulators (order-independent).
+__device__ __noinline__ void tri_deferred(const unsigned *queue, int count, const TriLoop *s_tri, const CancelQ &cq,
+                                          unsigned long long *counters) {
+    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
+    for (int r = lane; r < count; r += 32) {
+        const unsigned e = queue[r];
+        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7 & 0xffffffu);
+        const bool fail = e >> 31;
+        const int local = owner + k * (int)blockDim.x;
+        const float qx = cq.q[3 * local], qy = cq.q[3 * local + 1], qz = cq.q[3 * local + 2];
+        const TriLoop &T = s_tri[j];
+        bool edges = false;
+        const bool inbox = qx >= T.box.x && qx <= T.box.y && qy >= T.box.z && qy <= T.box.w && qz <= T.a.w;
+        const int cr = inbox ? tri_cross(T, qx, qy, qz, &edges, counters) : 0;
+        float t = 0.f;
+        if (fail && !edges) {   // a well-conditioned angle away from the cut takes its own atan2
+            const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy,
+                        bz = T.b.z - qz, cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
+            const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az), ib = sfu_rsqrt(bx * bx + by * by + bz * bz),
+                        ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz);
+            const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
+                              (bx * cx + by * cy + bz * cz) * (ib * ic);
+            const float det = (ax * T.n.x + ay * T.n.y + az * T.n.z) * (ia * ib * ic);
+            if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
+            else edges = true;
+        }
+        const double sum = edges ? (double)tri_edges(T, j, k, (int)(e & 31u), local, qx, qy, qz, cq, counters)
+                                 : (double)t - 6.28318530717958647693 * cr;
+        if (sum != 0.0)
+            atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
+                      (unsigned long long)__double2ll_rn(sum * kFixScale64));
+    }
+    __syncwarp();
+}
+
+// Terms of triangle loops [t_begin, t_end) for the block's 2 KP queries per thread,
+// added to s_acc as in bsum_accumulate (which the caller runs after this, for the
+// other loops); s_tri holds cap triangles, queue 64 KQ entries of this warp.  Every
+// thread of the block must call it.
+template <int KP>
+__device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris, int64_t t_begin, int64_t t_end, int cap,
+                                               TriLoop *s_tri, const float2 (&nqx)[KP], const float2 (&nqy)[KP],
+                                               const float2 (&nqz)[KP], double *s_acc, unsigned long long *counters,
+                                               const CancelQ &cq, unsigned *queue) {
+    constexpr int KQ = 2 * KP;
+    if (t_begin >= t_end) return;
+#pragma unroll
+    for (int k = 0; k < KQ; ++k) cq.fix[k * blockDim.x + threadIdx.x] = 0;
+    if ((threadIdx.x & 31) == 0) *cq.count = 0;
+    __syncwarp();
+    float2 re[KP], im[KP], part[KP], comp[KP];
+    int q_count = 0;   // entries in the warp's queue
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+        re[k] = bc2(1.f);
+        im[k] = bc2(0.f);
+        part[k] = comp[k] = bc2(0.f);
+    }
+    int g = 0;
+    auto close = [&]() {
+#pragma unroll
+        for (int k = 0; k < KP; ++k) {
+            two_sum_acc2(part[k], comp[k], fast_atan2_2(im[k], re[k]));
+            re[k] = bc2(1.f);
+            im[k] = bc2(0.f);
+        }
+        g = 0;
+    };
+    for (int64_t t0 = t_begin; t0 < t_end; t0 += cap) {
+        const int cnt = (int)min((int64_t)cap, t_end - t0);
+        __syncthreads();
+        const float4 *src = reinterpret_cast<const float4 *>(tris + t0);
+        for (int i = threadIdx.x; i < 5 * cnt; i += blockDim.x) reinterpret_cast<float4 *>(s_tri)[i] = __ldg(src + i);
+        __syncthreads();
+        for (int j = 0; j < cnt; ++j) {
+            const float4 a = s_tri[j].a, b = s_tri[j].b, c = s_tri[j].c, N = s_tri[j].n, bx = s_tri[j].box;
+            unsigned fail = 0, inbox = 0;
+            float2 den[KP], det[KP];
+#pragma unroll
+            for (int k = 0; k < KP; ++k) {
+                const float2 ax = add2(bc2(a.x), nqx[k]), ay = add2(bc2(a.y), nqy[k]), az = add2(bc2(a.z), nqz[k]);
+                const float2 px = add2(bc2(b.x), nqx[k]), py = add2(bc2(b.y), nqy[k]), pz = add2(bc2(b.z), nqz[k]);
+                const float2 cx = add2(bc2(c.x), nqx[k]), cy = add2(bc2(c.y), nqy[k]), cz = add2(bc2(c.z), nqz[k]);
+                // (1e-37: a coincident vertex gives a finite reciprocal length)
+                const float2 la = fma2(ax, ax, fma2(ay, ay, fma2(az, az, bc2(1e-37f))));
+                const float2 lb = fma2(px, px, fma2(py, py, fma2(pz, pz, bc2(1e-37f))));
+                const float2 lc = fma2(cx, cx, fma2(cy, cy, fma2(cz, cz, bc2(1e-37f))));
+                const float2 ia = make_float2(sfu_rsqrt(la.x), sfu_rsqrt(la.y)), ib = make_float2(sfu_rsqrt(lb.x), sfu_rsqrt(lb.y)),
+                             ic = make_float2(sfu_rsqrt(lc.x), sfu_rsqrt(lc.y));
+                const float2 ab = fma2(ax, px, fma2(ay, py, mul2(az, pz)));
+                const float2 ac = fma2(ax, cx, fma2(ay, cy, mul2(az, cz)));
+                const float2 bc = fma2(px, cx, fma2(py, cy, mul2(pz, cz)));
+                const float2 iab = mul2(ia, ib);
+                den[k] = fma2(ab, iab, fma2(mul2(ac, ia), ic, fma2(mul2(bc, ib), ic, bc2(1.f))));
+                const float2 dn = fma2(ax, bc2(N.x), fma2(ay, bc2(N.y), mul2(az, bc2(N.z))));
+                det[k] = mul2(dn, mul2(iab, ic));
+                // a NaN (a padding query past n) counts as accepted: its sum is never read
+                const float2 v = fma2(bc2(kTanGroup), den[k], neg2(make_float2(fabsf(det[k].x), fabsf(det[k].y))));
+                fail |= (v.x <= kTriAccept ? 1u : 0u) << (2 * k) | (v.y <= kTriAccept ? 2u : 0u) << (2 * k);
+                inbox |= (-nqx[k].x >= bx.x && -nqx[k].x <= bx.y && -nqy[k].x >= bx.z && -nqy[k].x <= bx.w && -nqz[k].x <= a.w ? 1u : 0u) << (2 * k) |
+                         (-nqx[k].y >= bx.x && -nqx[k].y <= bx.y && -nqy[k].y >= bx.z && -nqy[k].y <= bx.w && -nqz[k].y <= a.w ? 2u : 0u) << (2 * k);
+            }
+            // near the triangle, or below its box (every lane of the warp is here)
+            if (__any_sync(0xffffffffu, fail | inbox)) {
+                const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+#pragma unroll
+                for (int k = 0; k < KQ; ++k) {
+                    const bool mine = (fail | inbox) >> k & 1u;
+                    const unsigned m = __ballot_sync(0xffffffffu, mine);
+                    if (mine)
+                        queue[q_count + __popc(m & below)] = (fail >> k & 1u) << 31 | (unsigned)j << 7 | (unsigned)k << 5 | lane;
+                    q_count += __popc(m);
+                }
+                if (q_count >= 32 * KQ) {
+                    __syncwarp();
+                    tri_deferred(queue, q_count, s_tri, cq, counters);
+                    q_count = 0;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < KP; ++k) {
+                const bool fx = fail >> (2 * k) & 1u, fy = fail >> (2 * k + 1) & 1u;
+                const float2 fd = make_float2(fx ? 1.f : den[k].x, fy ? 1.f : den[k].y);
+                const float2 fn = make_float2(fx ? 0.f : det[k].x, fy ? 0.f : det[k].y);
+                const float2 r = fma2(re[k], fd, neg2(mul2(im[k], fn)));
+                im[k] = fma2(re[k], fn, mul2(im[k], fd));
+                re[k] = r;
+            }
+            if (++g == GROUP) close();
+        }
+        if (g > 0) close();
+        __syncwarp();
+        if (q_count > 0) {   // the entries index this tile's triangles
+            tri_deferred(queue, q_count, s_tri, cq, counters);
+            q_count = 0;
+        }
+        if (*cq.count > 0) tri_drain(cq, s_tri, counters);
+#pragma unroll
+        for (int k = 0; k < KP; ++k) {
+            s_acc[(2 * k) * blockDim.x + threadIdx.x] += (double)part[k].x + (double)comp[k].x;
+            s_acc[(2 * k + 1) * blockDim.x + threadIdx.x] += (double)part[k].y + (double)comp[k].y;
+            part[k] = comp[k] = bc2(0.f);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < KQ; ++k)
+        s_acc[k * blockDim.x + threadIdx.x] += (double)cq.fix[k * blockDim.x + threadIdx.x] * kFixUnit;
+}
+
 }  // namespace
 
 }  // namespace gwn

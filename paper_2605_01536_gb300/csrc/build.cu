@@ -13,6 +13,8 @@
 // LBVH (replaces the paper's Embree BVH, Sec. 5): 30-bit Morton codes of the
 // triangle centroids, radix sort, Karras' binary radix tree (Karras 2012),
 // bottom-up box refit, and depth-first escape links for stackless traversal.
+#include <algorithm>
+
 #include "farfield.cuh"
 #include "gwn_internal.cuh"
 #include "traverse.cuh"
@@ -152,7 +154,7 @@ __global__ void k_loop_sizes(const uint32_t *__restrict__ rep, const uint32_t *_
 __global__ void k_emit_chained(const int32_t *__restrict__ edges, const uint32_t *__restrict__ rep,
                                const uint32_t *__restrict__ dist, const uint32_t *__restrict__ loop_off,
                                const float4 *__restrict__ V, int64_t nb, int64_t npts,
-                               float4 *__restrict__ pts, uint2 *__restrict__ ends /* or NULL */) {
+                               float4 *__restrict__ pts, uint2 *__restrict__ ends) {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nb) return;
     uint32_t r = rep[e];
@@ -164,12 +166,12 @@ __global__ void k_emit_chained(const int32_t *__restrict__ edges, const uint32_t
     float4 p = V[edges[2 * e]];
     p.w = 1.0f;
     pts[base + pos] = p;
-    if (ends) ends[base + pos] = make_uint2(base, base + len);   // the loop's first and closing points
+    ends[base + pos] = make_uint2(base, base + len);   // the loop's first and closing points
     if (e == (int64_t)r) {   // closing point: back to the loop's first vertex
         float4 c = V[edges[2 * e]];
         c.w = 0.0f;
         pts[base + len] = c;
-        if (ends) ends[base + len] = make_uint2(base, base + len);
+        ends[base + len] = make_uint2(base, base + len);
     }
 }
 
@@ -208,10 +210,50 @@ __global__ void k_scatter_offsets(const uint32_t *__restrict__ ids, const uint32
     loop_off[ids[i]] = off[i];
 }
 
-__global__ void k_count_heads(const uint32_t *__restrict__ rep, int64_t nb, unsigned long long *count) {
+// count[0]: loops, count[1]: of them with three edges
+__global__ void k_count_heads(const uint32_t *__restrict__ rep, const uint32_t *__restrict__ dist, int64_t nb,
+                              unsigned long long *count) {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nb) return;
-    if (rep[e] == (uint32_t)e) atomicAdd(count, 1ull);
+    const bool head = e < nb && rep[e] == (uint32_t)e;
+    const unsigned heads = __ballot_sync(0xffffffffu, head), tris = __ballot_sync(0xffffffffu, head && dist[e] == 2u);
+    if ((threadIdx.x & 31) == 0 && heads) {
+        atomicAdd(count, (unsigned long long)__popc(heads));
+        if (tris) atomicAdd(count + 1, (unsigned long long)__popc(tris));
+    }
+}
+
+// 1 at the first point of every loop of three edges (ends: per point the first and
+// closing point of its loop)
+__global__ void k_tri_heads(const uint2 *__restrict__ ends, int64_t npts, uint32_t *__restrict__ head) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= npts) return;
+    head[i] = ends[i].x == (uint32_t)i && ends[i].y - ends[i].x == 3u;
+}
+
+// Splits the chained points into triangle loops (5 float4 each, TriLoop) and the points
+// of the other loops; before: the triangle loops that start before each point (each
+// takes four points)
+__global__ void k_split_loops(const float4 *__restrict__ pts, const uint2 *__restrict__ ends,
+                              const uint32_t *__restrict__ before, int64_t npts, float4 *__restrict__ tri,
+                              float4 *__restrict__ rest) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= npts) return;
+    if (ends[i].y - ends[i].x != 3u) {
+        rest[i - 4 * (int64_t)before[i]] = pts[i];
+        return;
+    }
+    if (ends[i].x != (uint32_t)i) return;
+    float4 a = pts[i], b = pts[i + 1], c = pts[i + 2], *T = tri + 5 * (int64_t)before[i];
+    const double ux = (double)b.x - a.x, uy = (double)b.y - a.y, uz = (double)b.z - a.z;
+    const double vx = (double)c.x - a.x, vy = (double)c.y - a.y, vz = (double)c.z - a.z;
+    a.w = fmaxf(a.z, fmaxf(b.z, c.z));
+    b.w = c.w = 0.f;
+    T[0] = a;
+    T[1] = b;
+    T[2] = c;
+    T[3] = make_float4((float)(uy * vz - uz * vy), (float)(uz * vx - ux * vz), (float)(ux * vy - uy * vx), 0.f);
+    T[4] = make_float4(fminf(a.x, fminf(b.x, c.x)), fmaxf(a.x, fmaxf(b.x, c.x)), fminf(a.y, fminf(b.y, c.y)),
+                       fmaxf(a.y, fmaxf(b.y, c.y)));
 }
 
 // ------------------------------------------------------------------ BVH ----
@@ -528,6 +570,9 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     m->nloops = 0;
     if (m->bedges) { cudaFreeAsync(m->bedges, s); m->bedges = nullptr; }
     if (m->bpts) { cudaFreeAsync(m->bpts, s); m->bpts = nullptr; }
+    if (m->tri_loops) { cudaFreeAsync(m->tri_loops, s); m->tri_loops = nullptr; }
+    if (m->rest_pts) { cudaFreeAsync(m->rest_pts, s); m->rest_pts = nullptr; }
+    m->n_tri_loops = m->n_rest = 0;
     if (m->far_nodes) { cudaFreeAsync(m->far_nodes, s); m->far_nodes = nullptr; }
     if (m->far_pts) { cudaFreeAsync(m->far_pts, s); m->far_pts = nullptr; }
     if (m->far_coef) { cudaFreeAsync(m->far_coef, s); m->far_coef = nullptr; }
@@ -614,7 +659,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     }
     GWN_CUDA_TRY(dev_alloc(&lsize, sizeof(uint32_t) * nb, s));
     GWN_CUDA_TRY(dev_alloc(&loff, sizeof(uint32_t) * nb, s));
-    GWN_CUDA_TRY(dev_alloc(&nl, sizeof(unsigned long long), s));
+    GWN_CUDA_TRY(dev_alloc(&nl, 2 * sizeof(unsigned long long), s));
     int vbits = 1;
     while (vbits < 32 && ((int64_t)1 << vbits) <= m->nv) ++vbits;
     k_edge_vertex_keys<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, nb, 1, kin, idin);
@@ -657,27 +702,40 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
         return GWN_OK;
     };
     if ((st = order_loops(0)) != GWN_OK) return st;
-    GWN_CUDA_TRY(cudaMemsetAsync(nl, 0, sizeof(unsigned long long), s));
-    k_count_heads<<<grid_for(nb, TB), TB, 0, s>>>(repf, nb, nl);
+    GWN_CUDA_TRY(cudaMemsetAsync(nl, 0, 2 * sizeof(unsigned long long), s));
+    k_count_heads<<<grid_for(nb, TB), TB, 0, s>>>(repf, distf, nb, nl);
     uint32_t npts_h = 0;
-    unsigned long long nl_h = 0;
+    unsigned long long nl_h[2] = {0, 0};
     GWN_CUDA_TRY(cudaMemcpyAsync(&npts_h, tot, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    GWN_CUDA_TRY(cudaMemcpyAsync(&nl_h, nl, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    GWN_CUDA_TRY(cudaMemcpyAsync(nl_h, nl, sizeof(nl_h), cudaMemcpyDeviceToHost, s));
     GWN_CUDA_TRY(cudaStreamSynchronize(s));
     m->npts = npts_h;
-    m->nloops = (int64_t)nl_h;
+    m->nloops = (int64_t)nl_h[0];
+    uint2 *ends = nullptr;
     GWN_CUDA_TRY(dev_alloc(&m->bpts, sizeof(float4) * m->npts, s));
-    k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, m->bpts, nullptr);
+    GWN_CUDA_TRY(dev_alloc(&ends, sizeof(uint2) * m->npts, s));
+    k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, m->bpts, ends);
+    const int64_t ntri = (int64_t)nl_h[1];
+    if (6 * ntri >= nb && m->cfg.quantize_bits == 0) {   // at least half of the edges
+        uint32_t *before = nullptr;
+        m->n_tri_loops = ntri;
+        m->n_rest = m->npts - 4 * ntri;
+        GWN_CUDA_TRY(dev_alloc(&before, sizeof(uint32_t) * m->npts, s));
+        GWN_CUDA_TRY(dev_alloc(&m->tri_loops, 5 * sizeof(float4) * ntri, s));
+        GWN_CUDA_TRY(dev_alloc(&m->rest_pts, sizeof(float4) * std::max<int64_t>(m->n_rest, 1), s));
+        k_tri_heads<<<grid_for(m->npts, TB), TB, 0, s>>>(ends, m->npts, before);
+        if ((st = exclusive_scan_u32(before, before, m->npts, nullptr, s)) != GWN_OK) return st;
+        k_split_loops<<<grid_for(m->npts, TB), TB, 0, s>>>(m->bpts, ends, before, m->npts, m->tri_loops, m->rest_pts);
+        cudaFreeAsync(before, s);
+    }
     if (m->npts >= kFarMinPoints) {
         float4 *fpts = nullptr;
-        uint2 *ends = nullptr;
         GWN_CUDA_TRY(dev_alloc(&fpts, sizeof(float4) * m->npts, s));
-        GWN_CUDA_TRY(dev_alloc(&ends, sizeof(uint2) * m->npts, s));
         if ((st = order_loops(1)) != GWN_OK) return st;
         k_emit_chained<<<grid_for(nb, TB), TB, 0, s>>>(m->bedges, repf, distf, loff, m->V, nb, m->npts, fpts, ends);
         st = build_far(m, fpts, ends, s);
-        cudaFreeAsync(ends, s);
     }
+    cudaFreeAsync(ends, s);
     cudaFreeAsync(bnd, s);
     for (void *p : {(void *)kin, (void *)idin, (void *)kout, (void *)idout, (void *)succ, (void *)lsize,
                     (void *)loff, (void *)nl, (void *)tot})

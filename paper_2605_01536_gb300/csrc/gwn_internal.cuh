@@ -146,6 +146,10 @@ struct gwn_mesh {
                                                // fixed-point frame (quant.cuh), kStatusBytes in all
     int4 *leaf_q = nullptr;                    // [3 nt] snapped leaf triangles (quantize_bits = 30)
     float *box = nullptr;                      // [6] vertex box: min x, y, z, max x, y, z (after the build)
+    // the boundary as the direct sum reads it: loops of three edges as triangles (TriLoop,
+    // bterms.cuh) and the chained points of the other loops; NULL, 0: bpts as a whole
+    float4 *tri_loops = nullptr, *rest_pts = nullptr;
+    int64_t n_tri_loops = 0, n_rest = 0;
     gwn::FarNode *far_nodes = nullptr;         // boundary hierarchy (farfield.cuh), or NULL: summed directly
     float4 *far_pts = nullptr;                 // [npts] the chained points in the hierarchy's loop order
     float *far_coef = nullptr;                 // [far_nn][kFarCoef] its expansions
@@ -245,7 +249,9 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
 struct BatchMesh {
     const BvhNode *nodes;
     const float4 *tri;
-    const float4 *pts;
+    const float4 *pts;   // all boundary points (FP64 re-evaluation)
+    const float4 *tri_loops, *rest_pts;   // the boundary as the direct sum reads it
+    int64_t n_rest;
     int64_t nnodes;
     int64_t npts;
     unsigned long long *counters;
@@ -262,10 +268,10 @@ struct BatchTile {      // up to 512 * KP queries of one mesh
     int32_t q_count;
     int32_t pad;
 };
-struct BatchItem {      // kind 0: crossing numbers of the tile; 1: boundary chunk
+struct BatchItem {      // kind 0: crossing numbers of the tile; 1: points, 2: triangle loops of the boundary
     int32_t tile;
     int32_t kind;
-    int64_t p_begin, p_end;   // edge start points of the chunk
+    int64_t p_begin, p_end;   // edge start points, or triangle loops, of the chunk
 };
 // list / list_len / listed: queries whose cancelling boundary terms overflow the
 // kernel's queue, for launch_batch_fp64_fix (listed: zeroed bits, one per query)

@@ -298,6 +298,7 @@ constexpr int kBsumThreads = 128;
 template <int KP, bool Cond = false, bool Running = false>
 __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *__restrict__ q, int64_t n,
                                                       const float4 *__restrict__ pts, int64_t npts, int tile,
+                                                      const TriLoop *__restrict__ tris, int64_t ntri,
                                                       int64_t chunk_len, double *__restrict__ partial,
                                                       const int32_t *__restrict__ chi, float *__restrict__ w,
                                                       uint8_t *__restrict__ label, int classify, float margin,
@@ -313,11 +314,15 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
     constexpr int KQ = 2 * KP;
     const int64_t qblock = (int64_t)blockIdx.x * blockDim.x * KQ;
     const int64_t base = qblock + threadIdx.x;
-    const int64_t e_begin = (int64_t)blockIdx.y * chunk_len;
-    const int64_t e_end = min(npts - 1, e_begin + chunk_len);   // edge start points
+    // chunk of the boundary: the triangle loops, two units each, then the edge start points
+    const int64_t c0 = (int64_t)blockIdx.y * chunk_len, c1 = c0 + chunk_len;
+    const int64_t e_begin = max((int64_t)0, c0 - 2 * ntri);
+    const int64_t e_end = min(npts - 1, c1 - 2 * ntri);
     CancelQ cq{};
+    unsigned *tri_queue = nullptr;   // with triangle loops, after the counts: per warp 64 KQ entries
     if constexpr (Cond) {
         const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+        tri_queue = reinterpret_cast<unsigned *>(s_acc + 2 * KQ * blockDim.x) + nwarps * (kCancelCap + 1) + warp * 64 * KQ;
         cq.fix = reinterpret_cast<long long *>(s_acc + KQ * blockDim.x);
         unsigned *queues = reinterpret_cast<unsigned *>(cq.fix + KQ * blockDim.x);
         cq.queue = queues + warp * kCancelCap;
@@ -332,6 +337,9 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
     load_query_pairs<KP>(q, base, n, nqx, nqy, nqz);
 #pragma unroll
     for (int k = 0; k < KQ; ++k) s_acc[k * blockDim.x + threadIdx.x] = 0.0;
+    if constexpr (Cond)
+        tri_accumulate<KP>(tris, min(ntri, c0 / 2), min(ntri, c1 / 2), (tile + 1) / 5, reinterpret_cast<TriLoop *>(s_pts),
+                           nqx, nqy, nqz, s_acc, counters, cq, tri_queue);
     bsum_accumulate<KP, false, Cond, Running>(pts, e_begin, e_end, tile, s_pts, nqx, nqy, nqz, s_acc, counters, cq);
     double acc[KQ];
 #pragma unroll
@@ -354,10 +362,11 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
 }
 
 // Bytes of k_boundary_sum's dynamic shared memory.
-static size_t bsum_smem(int kp, int tile, bool cond) {
+static size_t bsum_smem(int kp, int tile, bool cond, bool tris) {
     const size_t kq = 2 * (size_t)kp, threads = kBsumThreads;
     size_t b = sizeof(float4) * (tile + 1) + sizeof(double) * kq * threads;
     if (cond) b += sizeof(long long) * kq * threads + (sizeof(unsigned) * kCancelCap + sizeof(int)) * (threads / 32);
+    if (tris) b += sizeof(unsigned) * 64 * kq * (threads / 32);
     return b;
 }
 
@@ -432,7 +441,12 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
             load_query_pairs<KP>(dq.q, threadIdx.x, tl.q_count, nqx, nqy, nqz);
 #pragma unroll
             for (int k = 0; k < KQ; ++k) s_acc[k * blockDim.x + threadIdx.x] = 0.0;
-            bsum_accumulate<KP, true, true, true>(mh.pts, wi.p_begin, wi.p_end, tile_pts, s_pts, nqx, nqy, nqz, s_acc,
+            if (wi.kind == 2)
+                tri_accumulate<KP>(reinterpret_cast<const TriLoop *>(mh.tri_loops), wi.p_begin, wi.p_end,
+                                   (tile_pts + 1) / 5, reinterpret_cast<TriLoop *>(s_pts), nqx, nqy, nqz, s_acc,
+                                   mh.counters, cq, dq.queue);
+            else
+                bsum_accumulate<KP, true, true, true>(mh.rest_pts, wi.p_begin, wi.p_end, tile_pts, s_pts, nqx, nqy, nqz, s_acc,
                                             mh.counters, cq, dq);
 #pragma unroll
             for (int k = 0; k < KQ; ++k) {
@@ -661,28 +675,35 @@ void launch_boundary_combine(const double *partial, int64_t n, int chunks, const
 template <int KP, bool Cond = false, bool Running = false>
 static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                  uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                 unsigned *listed, double *partial_buf, int64_t partial_cap, cudaStream_t s) {
+                                 unsigned *listed, double *partial_buf, int64_t partial_cap, bool plain,
+                                 cudaStream_t s) {
     const int tile = m->cfg.boundary_tile > 0 ? m->cfg.boundary_tile : 512;
-    const size_t smem = bsum_smem(KP, tile, Cond);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_boundary_sum<KP, Cond, Running>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
     const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
     const int64_t per_block = kBsumThreads * 2 * KP;
     const int64_t qblocks = (n + per_block - 1) / per_block;
-    const int64_t nedge_pts = m->npts > 0 ? m->npts - 1 : 0;
+    // triangle loops as one term each (tri_accumulate; the FP64 test of their edges needs Cond)
+    const bool split = Cond && !plain && m->n_tri_loops > 0 && tile >= 64;
+    const float4 *pts = split ? m->rest_pts : m->bpts;
+    const int64_t npts = split ? m->n_rest : m->npts, ntri = split ? m->n_tri_loops : 0;
+    const int64_t nedge_pts = (npts > 0 ? npts - 1 : 0) + 2 * ntri;
+    const size_t smem = bsum_smem(KP, tile, Cond, ntri > 0);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_boundary_sum<KP, Cond, Running>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // split the boundary into chunks when the query tiles alone cannot fill the GPU
-    int64_t chunks = (8 * (int64_t)(sms > 0 ? sms : 148) + qblocks - 1) / qblocks;
+    // (with triangle loops finer: their near terms make blocks uneven)
+    int64_t chunks = ((ntri > 0 ? 48 : 8) * (int64_t)(sms > 0 ? sms : 148) + qblocks - 1) / qblocks;
     // (a chunk of 128 points still pays for its partial sums: 64 queries against
     // 9.8k edges take 47 us instead of 200 us with chunks of 1024 points)
-    const int64_t min_chunk = n < kOrderMinQueries ? std::min<int64_t>(128, 2 * tile) : 2 * tile;
+    const int64_t min_chunk = n < kOrderMinQueries || ntri > 0 ? std::min<int64_t>(128, 2 * tile) : 2 * tile;
     chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (nedge_pts + min_chunk - 1) / min_chunk));
     if (partial_cap >= 0) chunks = std::min<int64_t>(chunks, partial_cap / n);   // caller-provided room
     chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, 65535));
-    const int64_t chunk_len = chunks > 1 ? (nedge_pts + chunks - 1) / chunks : std::max<int64_t>(nedge_pts, 1);
+    int64_t chunk_len = chunks > 1 ? (nedge_pts + chunks - 1) / chunks : std::max<int64_t>(nedge_pts, 1);
+    if (ntri > 0) chunk_len += chunk_len & 1;   // whole triangles
     double *partial = nullptr;
     bool own = false;
     if (chunks > 1) {
@@ -694,8 +715,9 @@ static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, c
         }
     }
     dim3 grid((unsigned)qblocks, (unsigned)chunks);
-    k_boundary_sum<KP, Cond, Running><<<grid, kBsumThreads, smem, s>>>(q, n, m->bpts, m->npts, tile, chunk_len,
-                                                                      partial, chi, w, label, classify ? 1 : 0,
+    k_boundary_sum<KP, Cond, Running><<<grid, kBsumThreads, smem, s>>>(q, n, pts, npts, tile,
+                                                                      reinterpret_cast<const TriLoop *>(m->tri_loops),
+                                                                      ntri, chunk_len, partial, chi, w, label, classify ? 1 : 0,
                                                                       margin, list, list_len, listed, m->counters);
     note_launches(1);
     if (partial) {
@@ -722,14 +744,14 @@ static bool group_test_running(const gwn_mesh *m) {
 static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                   uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
                                   unsigned *listed, double *partial_buf, int64_t partial_cap, bool ordered,
-                                  cudaStream_t s) {
+                                  bool plain, cudaStream_t s) {
     const int kq = m->cfg.queries_per_thread > 0 ? m->cfg.queries_per_thread : 4;
     ProfScope prof("boundary_sum", s);
     const bool running = group_test_running(m);
     if (ordered && far_pays(m, n))
         return launch_boundary_far(m, q, n, chi, w, label, classify, running, list, list_len, listed, partial_buf, partial_cap, s);
 #define GWN_BSUM(KP, C, R) \
-    launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, partial_cap, s)
+    launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, partial_cap, plain, s)
     if (m->cfg.fp64_cancel >= 0) {   // the default: cancelling terms in FP64
         const bool small = kq == 1 || kq == 2;   // 8 queries per thread: the queue holds 2-bit slots
         if (running) return small ? GWN_BSUM(1, true, true) : GWN_BSUM(2, true, true);
@@ -786,7 +808,7 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
         GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     }
     gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1,
-                                    order == SumOrder::kSpatial, s);
+                                    order == SumOrder::kSpatial, order == SumOrder::kDirect, s);
     if (st == GWN_OK && own_list) st = launch_fp64_fix_list(m, q, chi, w, nullptr, list, list_len, s);
     cudaFreeAsync(listed, s);
     if (own_list) {
@@ -812,7 +834,7 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
                                                                         m->counters);
     GWN_LAUNCH_CHECK("k_chi");
     gwn_status st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial,
-                                    partial ? partial_cap : 0, false, s);
+                                    partial ? partial_cap : 0, false, false, s);
     if (st != GWN_OK) return st;
     return launch_fp64_fix_list(m, q, chi_tmp, w, label, list, list_len, s);
 }
