@@ -91,7 +91,6 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
         const int64_t nedge_pts = npts > 0 ? npts - 1 : 0;
         const int64_t nchunks = (nedge_pts + chunk - 1) / chunk;
         const int64_t tchunk = std::max(chunk / 8, 1), ntchunks = (ntri + tchunk - 1) / tchunk;
-        const double chi_unit = 40.0 + 8.0 * std::log2((double)m->nt + 2.0);   // ~ one traversal in point terms
         // the autotuner's subsample: whole tiles spread evenly over the mesh's
         // (spatially ordered) queries, so that it samples the whole domain
         const int64_t nq_all = b->q_off[mi + 1] - q0;
@@ -103,11 +102,18 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
             tl.mesh = (int32_t)mi;
             tl.q_begin = q0 + t0;
             tl.q_count = (int32_t)std::min<int64_t>(T, nq_all - t0);
-            tl.n_items = (int32_t)(1 + nchunks + ntchunks);
+            const int64_t nchi = (tl.q_count + 255) / 256;   // one query per thread
+            tl.n_items = (int32_t)(nchi + nchunks + ntchunks);
             const int32_t ti = (int32_t)tiles.size();
             tiles.push_back(tl);
-            items.push_back(BatchItem{ti, 0, 0, 0});
-            cost.push_back(chi_unit * tl.q_count);
+            // The walks are serial chains of up to thousands of loads that leave the FP32
+            // pipe idle: they go first, one round each, and the boundary items beside and
+            // after them fill the pipe (24 uneven meshes: 17.6 -> 12.5 ms against one item
+            // per tile in the order of an estimated cost).
+            for (int64_t c = 0; c < nchi; ++c) {
+                items.push_back(BatchItem{ti, 0, 256 * c, std::min<int64_t>(tl.q_count, 256 * (c + 1))});
+                cost.push_back(1e30);
+            }
             for (int64_t c = 0; c < ntchunks; ++c) {   // a triangle costs about two points
                 const int64_t p0 = c * tchunk, p1 = std::min<int64_t>(ntri, p0 + tchunk);
                 items.push_back(BatchItem{ti, 2, p0, p1});

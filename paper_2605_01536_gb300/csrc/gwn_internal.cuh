@@ -271,7 +271,7 @@ struct BatchTile {      // up to 512 * KP queries of one mesh
 struct BatchItem {      // kind 0: crossing numbers of the tile; 1: points, 2: triangle loops of the boundary
     int32_t tile;
     int32_t kind;
-    int64_t p_begin, p_end;   // edge start points, or triangle loops, of the chunk
+    int64_t p_begin, p_end;   // queries of the tile, edge start points, or triangle loops
 };
 // list / list_len / listed: queries whose cancelling boundary terms overflow the
 // kernel's queue, for launch_batch_fp64_fix (listed: zeroed bits, one per query)

@@ -402,9 +402,9 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
             // the crossing numbers of the tile: in exact mode the warp walks
             // together (bvh_walk_up_warp), so every lane takes every round
             const bool fixed = qframe(mh.counters)->bits != 0;
-            for (int base = 0; base < tl.q_count; base += blockDim.x) {
-                const int i = base + (int)threadIdx.x;
-                const bool active = i < tl.q_count;
+            for (int64_t base = wi.p_begin; base < wi.p_end; base += blockDim.x) {
+                const int64_t i = base + threadIdx.x;
+                const bool active = i < wi.p_end;
                 const int64_t g = tl.q_begin + (active ? i : 0);
                 const float3 p = active ? make_float3(q[3 * g], q[3 * g + 1], q[3 * g + 2]) : make_float3(0.f, 0.f, 0.f);
                 int c = 0;
