@@ -267,7 +267,7 @@ gwn_status gwn_mesh_destroy(gwn_mesh *m) {
     for (void *p : {(void *)m->V, (void *)m->F, (void *)m->tri9, (void *)m->bedges, (void *)m->bpts,
                     (void *)m->nodes, (void *)m->leaf_tri, (void *)m->counters, (void *)m->leaf_q, (void *)m->box,
                     (void *)m->far_nodes, (void *)m->far_pts, (void *)m->far_coef,
-                    (void *)m->far_roots, (void *)m->tri_loops, (void *)m->rest_pts})
+                    (void *)m->far_gcoef, (void *)m->far_roots, (void *)m->tri_loops, (void *)m->rest_pts})
         if (p) cudaFreeAsync(p, nullptr);
     surrogate_free(m->sur);
     delete m;

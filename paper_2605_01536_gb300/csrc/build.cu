@@ -575,6 +575,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     m->n_tri_loops = m->n_rest = 0;
     if (m->far_nodes) { cudaFreeAsync(m->far_nodes, s); m->far_nodes = nullptr; }
     if (m->far_pts) { cudaFreeAsync(m->far_pts, s); m->far_pts = nullptr; }
+    if (m->far_gcoef) { cudaFreeAsync(m->far_gcoef, s); m->far_gcoef = nullptr; }
     if (m->far_coef) { cudaFreeAsync(m->far_coef, s); m->far_coef = nullptr; }
     if (m->far_roots) { cudaFreeAsync(m->far_roots, s); m->far_roots = nullptr; }
     m->far_nn = 0;

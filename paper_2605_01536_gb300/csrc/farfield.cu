@@ -172,7 +172,23 @@ __global__ void __launch_bounds__(Threads) k_far_geom(FarShape sh, int64_t t0, c
     nd.skip = (int32_t)far_before(sh, past);
     nd.begin = a;
     nd.count = b - a;
-    nd.pad0 = nd.pad1 = 0;
+    // the gradient's radius: bound E / r^(P+3) (P+1)(P+2) / (1-y)^3 <= kFarGradEps / ext
+    auto gbound = [&](float x) {
+        const float g = 1.f / (1.f - 1.f / x);
+        return e * exp2f(-(P + 3) * log2f(x)) * ((P + 1) * (P + 2)) * g * g * g;
+    };
+    const float geps = ext > 0.f ? kFarGradEps * (s / ext) : 0.f;
+    lo = 1.5f;
+    hi = 16384.f;
+    if (gbound(lo) <= geps) hi = lo;
+    else
+        for (int it = 0; it < 30; ++it) {
+            const float mid = sqrtf(lo * hi);
+            if (gbound(mid) <= geps) hi = mid;
+            else lo = mid;
+        }
+    nd.r2grad = use && hi < 16384.f ? (hi * s) * (hi * s) * 1.0001f : INFINITY;
+    nd.gpad = ext * 0x1p-7f;
     nd.nchord = 0;
     nd.ch[0] = nd.ch[1] = nd.ch[2] = nd.ch[3] = 0;
     if (a_mid) {   // the piece of a loop that began before a
@@ -420,6 +436,51 @@ __global__ void k_far_pack(FarShape sh, const Cplx *__restrict__ raw, float *__r
     }
 }
 
+// Packed coefficients of the gradient in preorder (layout in farfield.cuh), component
+// by component, with -(1/4pi) for w, the basis constants and the phase folded in; the
+// unit of length stays with the kernel.  With a = M_l^(m-1), b = M_l^(m+1):
+//   d/dx: Re[conj(a - b) I_(l+1)^m], d/dy: Re[conj(i (a + b)) I_(l+1)^m],
+//   d/dz: Re[conj(-2 M_l^m) I_(l+1)^m]  (m >= 1; for m = 0 half of each).
+__global__ void k_far_pack_grad(FarShape sh, const Cplx *__restrict__ raw, float *__restrict__ gcoef) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int kPer = kFarP + kFarGradCols;   // (l, m) entries of a component
+    if (t >= sh.total * kPer) return;
+    const int k = (int)(t % kPer);
+    int lev;
+    int64_t i;
+    far_level_of(sh, t / kPer, lev, i);
+    const Cplx *M = raw + (t / kPer) * kFarRaw;
+    int m = 0, l;   // degree of the gradient's entry
+    if (k < kFarP) {
+        l = k + 2;
+    } else {
+        m = 1;
+        while (far_grad_col(m + 1) <= k - kFarP) ++m;
+        l = far_grad_first(m) + (k - kFarP - far_grad_col(m));
+    }
+    const int L = l - 1;   // degree of the moment
+    auto mom = [&](int mm) -> Cplx { return mm > L ? Cplx{0.f, 0.f} : M[far_idx(L, mm)]; };
+    float f = -0.0795774715f;
+    for (int j = 2 * l - 1; j > 1; j -= 2) f *= (float)j;
+    if (m & 1) f = -f;
+    float *out = gcoef + far_preorder(sh, lev, i) * kFarGradCoef;
+    constexpr int kComp = kFarGradCoef / 3;
+    if (m == 0) {
+        out[k] = -f * mom(1).r;
+        out[kComp + k] = -f * mom(1).i;
+        out[2 * kComp + k] = -f * mom(0).r;
+    } else {
+        const Cplx a = mom(m - 1), b = mom(m + 1), c = mom(m);
+        const int at = kFarP + 2 * (k - kFarP);
+        out[at] = f * (a.r - b.r);
+        out[at + 1] = f * (a.i - b.i);
+        out[kComp + at] = -f * (a.i + b.i);
+        out[kComp + at + 1] = f * (a.r + b.r);
+        out[2 * kComp + at] = -2.f * f * c.r;
+        out[2 * kComp + at + 1] = -2.f * f * c.i;
+    }
+}
+
 // Preorder index of each node of level l, and of the end.
 __global__ void k_far_roots(FarShape sh, int l, int32_t *__restrict__ roots) {
     const int64_t i = threadIdx.x, n = far_level_count(sh, l);
@@ -504,7 +565,9 @@ gwn_status build_far(gwn_mesh *m, float4 *pts, const uint2 *ends, cudaStream_t s
         k_far_leaf_moments<<<grid_for(sh.nleaf, 2), 64, 0, s>>>(sh, nodes, pts, raw);
         for (int l = 1; l <= sh.top; ++l)
             k_far_up<<<grid_for(far_level_count(sh, l), 2), 64, 0, s>>>(sh, l, nodes, pts, raw);
+        GWN_CUDA_TRY(dev_alloc(&m->far_gcoef, sizeof(float) * kFarGradCoef * sh.total, s));
         k_far_pack<<<grid_for(sh.total * kFarRaw, 256), 256, 0, s>>>(sh, raw, coef);
+        k_far_pack_grad<<<grid_for(sh.total * (kFarP + kFarGradCols), 256), 256, 0, s>>>(sh, raw, m->far_gcoef);
         cudaFreeAsync(raw, s);
         m->far_pts = pts;
         m->far_nodes = nodes;

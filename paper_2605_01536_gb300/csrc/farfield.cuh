@@ -39,6 +39,8 @@ constexpr int kFarRaw = (kFarP + 1) * (kFarP + 2) / 2;    // complex moments (l,
 constexpr int kFarCoef = kFarP * (kFarP + 2);             // packed real coefficients (80)
 constexpr float kFarEps = 1e-7f;                          // truncation bound of one expansion, in w
 constexpr int kFarLeaf = 16;                              // target points of a leaf (at most twice that)
+constexpr float kFarGradEps = 2e-6f;                      // truncation bound of one gradient, times the box's side
+constexpr int kFarGradCoef = 3 * (kFarP + 2 * (kFarP * (kFarP + 3) / 2));   // 288: x, y, z
 constexpr double kFarWorth = 0.6;                         // kept below this share of the direct sum's cost
 constexpr int kFarMinPoints = 1024;                       // no hierarchy below this many points
 constexpr int kFarRoots = 64;                             // subtrees a walk may be split into (at most)
@@ -50,7 +52,8 @@ struct __align__(16) FarNode {
     float xmin, xmax, ymin, ymax;       // box of the points: the ray test (with a small margin)
     float zmax, inv_s;                  // its top; 1 / radius, the expansion's unit of length
     int32_t skip, nchord;               // next node after the subtree; chords (0 to 2)
-    int32_t begin, count, pad0, pad1;   // the points whose edges the node covers
+    int32_t begin, count;               // the points whose edges the node covers
+    float r2grad, gpad;                 // the gradient's: |q - c|^2 > r2grad, the ray outside the box widened by gpad
     int32_t ch[4];                      // chords ch[0] -> ch[1], ch[2] -> ch[3] (point indices)
 };
 static_assert(sizeof(FarNode) == 80, "FarNode must be 80 bytes");
@@ -66,6 +69,18 @@ __host__ __device__ constexpr float far_beta(int l, int m) {
 __host__ __device__ constexpr int far_idx(int l, int m) { return l * (l + 1) / 2 + m; }
 // first packed coefficient of column m >= 1
 __host__ __device__ constexpr int far_col(int m) { return kFarP + (m - 1) * (2 * kFarP + 2 - m); }
+
+// The gradient of an expansion is one of degrees 2..P+1 in the same basis for each
+// component (derivatives of I_l^m are I_(l+1)^(m-1..m+1)): P real coefficients for
+// m = 0, then (re, im) for m = 1..P+1, l = max(m, 2)..P+1.
+__host__ __device__ constexpr int far_grad_first(int m) { return m < 2 ? 2 : m; }   // lowest degree of column m
+__host__ __device__ constexpr int far_grad_col(int m) {   // first entry (complex) of column m >= 1, after column 0
+    int c = 0;
+    for (int k = 1; k < m; ++k) c += kFarP + 2 - far_grad_first(k);
+    return c;
+}
+constexpr int kFarGradCols = far_grad_col(kFarP + 2);   // 44 complex entries
+static_assert(kFarGradCoef == 3 * (kFarP + 2 * kFarGradCols), "gradient coefficients");
 
 // Position of cell (x, y, z), 2^bits cells per axis, on the Hilbert curve (Skilling
 // 2004, "Programming the Hilbert curve").  Neighbours on the curve are neighbours in

@@ -153,6 +153,7 @@ struct gwn_mesh {
     gwn::FarNode *far_nodes = nullptr;         // boundary hierarchy (farfield.cuh), or NULL: summed directly
     float4 *far_pts = nullptr;                 // [npts] the chained points in the hierarchy's loop order
     float *far_coef = nullptr;                 // [far_nn][kFarCoef] its expansions
+    float *far_gcoef = nullptr;                // [far_nn][kFarGradCoef] their gradients
     int64_t far_nn = 0;
     int32_t *far_roots = nullptr;              // [far_nroots + 1] the subtrees that cover the boundary, in preorder
     int far_nroots = 0;

@@ -118,3 +118,24 @@ def test_far_queries_at_the_boundary(gwn):
     ok = ref["flags"] == 0
     assert np.array_equal(chi.cpu().numpy()[sel], ref["chi"])
     assert np.max(np.abs(w.cpu().numpy()[sel].astype(np.float64) - ref["w_antipodal"])[ok]) <= TOL
+
+
+@pytest.mark.parametrize("name", ["rim5000", "mixed", "soup6"])
+def test_far_gradient(gwn, name):
+    """Algorithm 3's FP32 bound (test_gpu_gradient.py) plus the truncation of the expansions: at most
+    2e-6 / box side each, of random sign over some hundreds of them."""
+    V, F = MESHES[name]()
+    rng = np.random.default_rng(4)
+    ext = float((V.max(0) - V.min(0)).max())
+    n = 17_001
+    Q = np.concatenate([gen.queries_uniform_bbox(V, n // 2, rng), gen.queries_near_surface(V, F, n - n // 2, rng, 1e-3)])
+    q = torch.from_numpy(Q).cuda()
+    with gwn.Mesh(V, F) as m:
+        g = m.gradient(q)
+        perm = torch.randperm(n, device="cuda")
+        assert torch.equal(m.gradient(q[perm].contiguous()), g[perm])
+    sel = rng.choice(n, 500, replace=False)
+    ref, a, c, fl = oracle.gradient(V, oracle.boundary(F, len(V)), Q[sel])
+    ok = fl == 0
+    tol = 2.0 ** -24 * (128.0 * c + 128.0 * a) + 3e-5 / ext
+    assert not (ok[:, None] & (np.abs(g.cpu().numpy()[sel].astype(np.float64) - ref) > tol[:, None])).any()
