@@ -401,7 +401,7 @@ gwn_status gwn_query_batch(const gwn_mesh *m, const float *q, int64_t n, float *
     if ((st = stg.input(q, sizeof(float) * 3 * n, &qd)) != GWN_OK ||
         (st = stg.output(w, sizeof(float) * n, &wd)) != GWN_OK)
         return stg.finish(st);
-    if (n >= kOrderMinQueries) {   // in the queries' Morton order, scattered back
+    if (n >= kOrderMinQueries) {   // in spatial order, scattered back
         void *keys = nullptr, *perm = nullptr, *qs = nullptr, *ws = nullptr, *cs = nullptr;
         if ((st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK &&
             (st = stg.alloc(&keys, sizeof(uint32_t) * n)) == GWN_OK &&
@@ -413,9 +413,9 @@ gwn_status gwn_query_batch(const gwn_mesh *m, const float *q, int64_t n, float *
                                 stg.s)) == GWN_OK &&
             (st = launch_chi(m, (const float *)qs, n, (int32_t *)cs, stg.s)) == GWN_OK &&
             (st = launch_boundary_sum_list(m, (const float *)qs, n, (const int32_t *)cs, (float *)ws, nullptr, false,
-                                           nullptr, nullptr, SumOrder::kSpatial, stg.s)) == GWN_OK &&
-            (st = scatter_f32((const float *)ws, (const uint32_t *)perm, n, (float *)wd, stg.s)) == GWN_OK)
-            st = scatter_i32((const int32_t *)cs, (const uint32_t *)perm, n, chi ? (int32_t *)cd : nullptr, stg.s);
+                                           nullptr, nullptr, SumOrder::kSpatial, stg.s)) == GWN_OK)
+            st = scatter_results((const uint32_t *)perm, n, (const float *)ws, (float *)wd, (const int32_t *)cs,
+                                 chi ? (int32_t *)cd : nullptr, nullptr, nullptr, stg.s);
         return stg.finish(st);
     }
     if ((st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK &&
@@ -446,7 +446,7 @@ gwn_status gwn_classify(const gwn_mesh *m, const float *q, int64_t n, uint8_t *l
     }
     const bool ordered = n >= kOrderMinQueries;
     void *keys = nullptr, *perm = nullptr, *qs = nullptr, *ws = nullptr, *ls = nullptr;
-    if (ordered) {   // in the queries' Morton order, scattered back
+    if (ordered) {   // in spatial order, scattered back
         if (w_or_null && (st = stg.output(w_or_null, sizeof(float) * n, &wd)) != GWN_OK) return stg.finish(st);
         if ((st = stg.alloc(&keys, sizeof(uint32_t) * n)) != GWN_OK ||
             (st = stg.alloc(&perm, sizeof(uint32_t) * n)) != GWN_OK ||
@@ -472,9 +472,9 @@ gwn_status gwn_classify(const gwn_mesh *m, const float *q, int64_t n, uint8_t *l
                                            SumOrder::kSpatial, stg.s)) == GWN_OK)
             st = launch_fp64_fix_list(m, (const float *)qs, (const int32_t *)cd, (float *)ws, (uint8_t *)ls,
                                       (const int32_t *)list, (const unsigned long long *)len, stg.s);
-        if (st == GWN_OK && ordered &&
-            (st = scatter_u8((const uint8_t *)ls, (const uint32_t *)perm, n, (uint8_t *)ld, stg.s)) == GWN_OK)
-            st = scatter_f32((const float *)ws, (const uint32_t *)perm, n, (float *)wd, stg.s);
+        if (st == GWN_OK && ordered)
+            st = scatter_results((const uint32_t *)perm, n, (const float *)ws, (float *)wd, nullptr, nullptr,
+                                 (const uint8_t *)ls, (uint8_t *)ld, stg.s);
     }
     return stg.finish(st);
 }

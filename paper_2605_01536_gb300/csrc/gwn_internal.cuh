@@ -168,12 +168,18 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s);
 gwn_status build_bvh(gwn_mesh *m, cudaStream_t s);
 gwn_status build_box(gwn_mesh *m, cudaStream_t s);   // m->box from the vertices
 
-// order.cu: Morton order of a query batch in the mesh's box (keys, perm: [n]
-// scratch; qs: [3 n] the queries in that order), and the scatter of results
-// back to the caller's order (out[perm[i]] = in[i]; out NULL: nothing)
-gwn_status order_queries(const gwn_mesh *m, const float *q, int64_t n, uint32_t *keys, uint32_t *perm, float *qs,
+// order.cu: spatial order of a query batch in the mesh's box (rank, perm: [n]
+// scratch; qs: [3 n] the queries in that order), and the scatter of results back to
+// the caller's order (out[perm[i]] = in[i]; out NULL: nothing).  The _on form takes the
+// cell counts (order_cells_bytes(n)) from the caller and allocates nothing.
+size_t order_cells_bytes(int64_t n);
+gwn_status order_queries_on(const gwn_mesh *m, const float *q, int64_t n, uint32_t *rank, uint32_t *perm, float *qs,
+                            uint32_t *cells, cudaStream_t s);
+gwn_status order_queries(const gwn_mesh *m, const float *q, int64_t n, uint32_t *rank, uint32_t *perm, float *qs,
                          cudaStream_t s);
-// list: n indices into q, reordered by their queries' Morton codes (lists
+gwn_status scatter_results(const uint32_t *perm, int64_t n, const float *ws, float *w, const int32_t *cs, int32_t *chi,
+                           const uint8_t *ls, uint8_t *label, cudaStream_t s);
+// list: n indices into q, in their queries' order along the Hilbert curve (lists
 // shorter than kOrderMinQueries are left as they are)
 gwn_status order_query_list(const gwn_mesh *m, const float *q, int32_t *list, int64_t n, cudaStream_t s);
 gwn_status scatter_f32(const float *in, const uint32_t *perm, int64_t n, float *out, cudaStream_t s);
@@ -181,8 +187,7 @@ gwn_status scatter_i32(const int32_t *in, const uint32_t *perm, int64_t n, int32
 gwn_status gather_i32(const int32_t *in, const uint32_t *perm, int64_t n, int32_t *out, cudaStream_t s);
 // list entries (at most n, *len of them on the device) i -> perm[i]
 gwn_status map_list(int32_t *list, const unsigned long long *len, int64_t n, const uint32_t *perm, cudaStream_t s);
-gwn_status scatter_u8(const uint8_t *in, const uint32_t *perm, int64_t n, uint8_t *out, cudaStream_t s);
-// batches at least this large are evaluated in Morton order
+// batches at least this large are evaluated in spatial order
 constexpr int64_t kOrderMinQueries = 16384;
 
 // sort.cu: stable LSD radix sort of (key, value) pairs on the low `bits` bits.
@@ -242,7 +247,7 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
 // the classify sequence on caller-provided scratch; allocates nothing
 gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w,
                                       int32_t *chi_tmp, int32_t *list, unsigned long long *list_len,
-                                      unsigned *listed, double *partial, int64_t partial_cap, cudaStream_t s);
+                                      unsigned *listed, double *partial, int64_t partial_cap, bool far, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Batched evaluation of many meshes (one persistent launch over a work queue).

@@ -743,12 +743,12 @@ static bool group_test_running(const gwn_mesh *m) {
 // needed when partial_cap < 0.
 static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                   uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                  unsigned *listed, double *partial_buf, int64_t partial_cap, bool ordered,
+                                  unsigned *listed, double *partial_buf, int64_t partial_cap, bool far,
                                   bool plain, cudaStream_t s) {
     const int kq = m->cfg.queries_per_thread > 0 ? m->cfg.queries_per_thread : 4;
     ProfScope prof("boundary_sum", s);
     const bool running = group_test_running(m);
-    if (ordered && far_pays(m, n))
+    if (far)
         return launch_boundary_far(m, q, n, chi, w, label, classify, running, list, list_len, listed, partial_buf, partial_cap, s);
 #define GWN_BSUM(KP, C, R) \
     launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, partial_cap, plain, s)
@@ -788,8 +788,7 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
         if (st == GWN_OK && (st = order_queries(m, q, n, keys, perm, qs, s)) == GWN_OK &&
             (st = gather_i32(chi, perm, n, cs, s)) == GWN_OK &&
             (st = launch_boundary_sum_list(m, qs, n, cs, ws, ls, classify, list, list_len, SumOrder::kSpatial, s)) == GWN_OK &&
-            (st = scatter_f32(ws, perm, n, w, s)) == GWN_OK && (st = scatter_u8(ls, perm, n, label, s)) == GWN_OK &&
-            list)
+            (st = scatter_results(perm, n, ws, w, nullptr, nullptr, ls, label, s)) == GWN_OK && list)
             st = map_list(list, list_len, n, perm, s);
         for (void *p : {(void *)keys, (void *)perm, (void *)qs, (void *)ws, (void *)cs, (void *)ls})
             if (p) cudaFreeAsync(p, s);
@@ -808,7 +807,7 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
         GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     }
     gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1,
-                                    order == SumOrder::kSpatial, order == SumOrder::kDirect, s);
+                                    order == SumOrder::kSpatial && far_pays(m, n), order == SumOrder::kDirect, s);
     if (st == GWN_OK && own_list) st = launch_fp64_fix_list(m, q, chi, w, nullptr, list, list_len, s);
     cudaFreeAsync(listed, s);
     if (own_list) {
@@ -824,7 +823,8 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
 // into at most partial_cap / n point chunks; fewer than two means no split).
 gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w,
                                       int32_t *chi_tmp, int32_t *list, unsigned long long *list_len,
-                                      unsigned *listed, double *partial, int64_t partial_cap, cudaStream_t s) {
+                                      unsigned *listed, double *partial, int64_t partial_cap, bool far,
+                                      cudaStream_t s) {
     if (n <= 0) return GWN_OK;
     if (m->cfg.quantize_bits)
         k_chi<true><<<grid_for(n, kChiThreads), kChiThreads, 0, s>>>(q, n, m->nodes, m->nnodes, m->leaf_tri, chi_tmp,
@@ -834,7 +834,7 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
                                                                         m->counters);
     GWN_LAUNCH_CHECK("k_chi");
     gwn_status st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial,
-                                    partial ? partial_cap : 0, false, false, s);
+                                    partial ? partial_cap : 0, far, false, s);
     if (st != GWN_OK) return st;
     return launch_fp64_fix_list(m, q, chi_tmp, w, label, list, list_len, s);
 }

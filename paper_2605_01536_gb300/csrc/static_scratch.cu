@@ -9,6 +9,7 @@
 // from the stream-ordered allocator on every call; this entry point instead
 // uses one file-scope device array that every GPU loading the library holds
 // until the process exits.
+#include <algorithm>
 #include <mutex>
 
 #include "gwn_internal.cuh"
@@ -43,6 +44,42 @@ gwn_status scratch_address(int dev, unsigned char **out) {
 }
 
 
+// Queries per slice of an ordered call: 29.2 bytes of scratch each and 1 MiB of cell
+// counts (an order over fewer than 2^20 queries has at most 64^3 cells).
+constexpr int64_t kSlice = (int64_t(1) << 20) - 256;
+
+// layout: [counter | chi n x int32 | list n x int32 | w n x float | listed (n + 31) / 32 x uint32 |
+//          ordered: perm n x uint32 | queries n x 12 | label n | cell counts || FP64 partials ...]
+// (the ranks of the order share the crossing numbers' place)
+gwn_status run_slice(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w, bool ordered, bool far,
+                     unsigned char *base, cudaStream_t s) {
+    auto *len = reinterpret_cast<unsigned long long *>(base);
+    auto *chi = reinterpret_cast<int32_t *>(base + kHeader);
+    auto *list = chi + n;
+    float *ws = reinterpret_cast<float *>(list + n);
+    auto *listed = reinterpret_cast<unsigned *>(ws + n);
+    const size_t words = (size_t)((n + 31) / 32);
+    auto *perm = reinterpret_cast<uint32_t *>(listed + words);
+    float *qs = reinterpret_cast<float *>(perm + n);
+    auto *cells = reinterpret_cast<uint32_t *>(qs + 3 * n);
+    uint8_t *ls = reinterpret_cast<uint8_t *>(cells) + (ordered ? gwn::order_cells_bytes(n) : 0);
+    size_t used = ordered ? (size_t)(ls + n - base) : (size_t)(reinterpret_cast<unsigned char *>(perm) - base);
+    used = (used + 255) & ~size_t(255);
+    if (used > kScratchBytes) return gwn::set_error(GWN_ERR_INVALID_ARG, "gwn_classify_static: slice beyond the scratch");
+    double *partial = reinterpret_cast<double *>(base + used);
+    const int64_t partial_cap = (int64_t)((kScratchBytes - used) / sizeof(double));
+    GWN_CUDA_TRY(cudaMemsetAsync(len, 0, sizeof(unsigned long long), s));
+    GWN_CUDA_TRY(cudaMemsetAsync(listed, 0, sizeof(unsigned) * words, s));
+    if (!ordered)
+        return gwn::launch_classify_on_scratch(m, q, n, label, w ? w : ws, chi, list, len, listed, partial, partial_cap,
+                                               false, s);
+    gwn_status st = gwn::order_queries_on(m, q, n, reinterpret_cast<uint32_t *>(chi), perm, qs, cells, s);
+    if (st == GWN_OK)
+        st = gwn::launch_classify_on_scratch(m, qs, n, ls, ws, chi, list, len, listed, partial, partial_cap, far, s);
+    if (st == GWN_OK) st = gwn::scatter_results(perm, n, ws, w, nullptr, nullptr, ls, label, s);
+    return st;
+}
+
 }  // namespace
 
 extern "C" gwn_status gwn_classify_static(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label,
@@ -74,24 +111,12 @@ extern "C" gwn_status gwn_classify_static(const gwn_mesh *m, const float *q, int
         st = scratch_address(m->device, &base);
         if (st == GWN_OK) {
             cudaStream_t s = (cudaStream_t)stream;
-            // layout: [counter | chi n x int32 | list n x int32 | w n x float | listed (n + 31) / 32 x uint32 |
-            //          FP64 partials ...]
-            auto *len = reinterpret_cast<unsigned long long *>(base);
-            auto *chi = reinterpret_cast<int32_t *>(base + kHeader);
-            auto *list = chi + n;
-            float *w_tmp = reinterpret_cast<float *>(list + n);
-            auto *listed = reinterpret_cast<unsigned *>(w_tmp + n);
-            const size_t words = (size_t)((n + 31) / 32);
-            size_t used = kHeader + size_t(12) * size_t(n) + sizeof(unsigned) * words;
-            used = (used + 255) & ~size_t(255);
-            double *partial = reinterpret_cast<double *>(base + used);
-            const int64_t partial_cap = (int64_t)((kScratchBytes - used) / sizeof(double));
-            cudaError_t e = cudaMemsetAsync(len, 0, sizeof(unsigned long long), s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(listed, 0, sizeof(unsigned) * words, s);
-            if (e != cudaSuccess) st = gwn::set_error(GWN_ERR_CUDA, cudaGetErrorString(e));
-            else
-                st = gwn::launch_classify_on_scratch(m, q, n, label, w_or_null ? w_or_null : w_tmp, chi, list, len,
-                                                     listed, partial, partial_cap, s);
+            // Large calls run in spatial order like gwn_classify's, in slices that fit the
+            // scratch (an order over the slice serves as well); small ones as they come.
+            const bool ordered = n >= gwn::kOrderMinQueries, far = ordered && gwn::far_pays(m, n);
+            for (int64_t at = 0; at < n && st == GWN_OK; at += kSlice)
+                st = run_slice(m, q + 3 * at, std::min<int64_t>(kSlice, n - at), label + at,
+                               w_or_null ? w_or_null + at : nullptr, ordered, far, base, s);
         }
     }
     if (prev >= 0 && prev != m->device) cudaSetDevice(prev);
