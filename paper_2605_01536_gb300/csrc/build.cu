@@ -580,6 +580,7 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
     if (m->far_roots) { cudaFreeAsync(m->far_roots, s); m->far_roots = nullptr; }
     m->far_nn = 0;
     m->far_nroots = 0;
+    m->far_sum = false;
     if (nh == 0) return GWN_OK;
     uint64_t *keys = nullptr, *seg_key = nullptr;
     uint32_t *vals = nullptr, *head = nullptr, *hscan = nullptr, *cnt = nullptr, *off = nullptr, *tot = nullptr;

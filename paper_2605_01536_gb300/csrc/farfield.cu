@@ -575,6 +575,7 @@ gwn_status build_far(gwn_mesh *m, float4 *pts, const uint2 *ends, cudaStream_t s
         m->far_nn = sh.total;
         m->far_roots = roots;
         m->far_nroots = nroots;
+        m->far_sum = m->far_cost <= kFarWorth * direct_cost(m);
     } else {
         cudaFreeAsync(nodes, s);
         cudaFreeAsync(pts, s);

@@ -25,9 +25,12 @@
 // Degree 8 with leaves of 16 points: degrees 6 and 10 cost the same or more on soup8,
 // leaves of 32 points 10% more.  Loops in Hilbert order instead of Morton order: 30%
 // fewer expansions and 40% fewer near edges per query (no jumps inside a range).
-// The hierarchy is kept where its mean cost over sample points is at most kFarWorth
-// of the direct sum's (random soups of large triangles overlap everywhere and stay
-// with the direct sum; a 12k-point boundary of small holes is at 0.25).
+// The hierarchy is used where its mean cost over sample points is at most kFarWorth
+// of the direct sum's (a warp takes the union over its queries, 1.5 to 2 times the
+// mean).  Random soups of large triangles overlap everywhere and stay with the direct
+// sum; of small holes, 3.2k points (0.8 of the direct sum with triangle loops) are
+// faster directly (200k queries: 413 against 506 us), 12k points (0.26) are not (1491
+// against 831 us).
 #pragma once
 
 #include "gwn_internal.cuh"
@@ -41,7 +44,7 @@ constexpr float kFarEps = 1e-7f;                          // truncation bound of
 constexpr int kFarLeaf = 16;                              // target points of a leaf (at most twice that)
 constexpr float kFarGradEps = 2e-6f;                      // truncation bound of one gradient, times the box's side
 constexpr int kFarGradCoef = 3 * (kFarP + 2 * (kFarP * (kFarP + 3) / 2));   // 288: x, y, z
-constexpr double kFarWorth = 0.6;                         // kept below this share of the direct sum's cost
+constexpr double kFarWorth = 0.5;                         // used below this share of the direct sum's cost
 constexpr int kFarMinPoints = 1024;                       // no hierarchy below this many points
 constexpr int kFarRoots = 64;                             // subtrees a walk may be split into (at most)
 constexpr int kFarMinEdges = 10;                          // a leaf below this is summed directly

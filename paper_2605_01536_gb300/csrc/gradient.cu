@@ -378,7 +378,7 @@ gwn_status launch_gradient(const gwn_mesh *m, const float *q, int64_t n, float *
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 148;
-    if (far_pays(m, n)) {   // the boundary hierarchy, in spatial order
+    if (far_pays_gradient(m, n)) {   // the boundary hierarchy, in spatial order
         uint32_t *keys = nullptr, *perm = nullptr;
         float *qs = nullptr;
         double *partial = nullptr;

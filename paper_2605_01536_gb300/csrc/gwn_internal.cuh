@@ -158,6 +158,7 @@ struct gwn_mesh {
     int32_t *far_roots = nullptr;              // [far_nroots + 1] the subtrees that cover the boundary, in preorder
     int far_nroots = 0;
     double far_cost = 0.0;                     // its mean cost per query, in FP32 operations
+    bool far_sum = false;                      // it is worth using for the boundary sum (and always for the gradient)
     gwn::Surrogate *sur = nullptr;             // optional learned surrogate (mlp.cu)
 };
 
@@ -217,9 +218,15 @@ gwn_status launch_fp64_fix_list(const gwn_mesh *m, const float *q, const int32_t
                                 uint8_t *label, const int32_t *list, const unsigned long long *list_len,
                                 cudaStream_t s);
 gwn_status launch_direct(const gwn_mesh *m, const float *q, int64_t n, float *w, cudaStream_t s);
+// operations per query of the direct boundary sum: 28 a point, 60 a triangle loop
+inline double direct_cost(const gwn_mesh *m) {
+    return m->n_tri_loops > 0 ? 60.0 * (double)m->n_tri_loops + 28.0 * (double)m->n_rest : 28.0 * (double)m->npts;
+}
 // bsum_far.cu: the same sums over the boundary hierarchy.  far_pays: whether a call
-// with n queries takes it; listed etc. as for the direct sum
+// with n queries takes it for the boundary sum, far_pays_gradient for the gradient;
+// listed etc. as for the direct sum
 bool far_pays(const gwn_mesh *m, int64_t n);
+bool far_pays_gradient(const gwn_mesh *m, int64_t n);
 gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                uint8_t *label, bool classify, bool running, int32_t *list,
                                unsigned long long *list_len, unsigned *listed, double *partial_buf,
