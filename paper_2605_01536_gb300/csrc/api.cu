@@ -1,5 +1,6 @@
 // C ABI of the library (declared in include/gwn.h): argument checking, mesh
 // ingest and validation, host/device pointer staging, and call sequencing.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -518,7 +519,8 @@ namespace {
 // Validate a grid's axes (host or device arrays) and copy them to the device:
 // counts >= 0, at most 2^31 - 1 cells, finite coordinates, z non-decreasing.
 struct GridAxes {
-    float *d = nullptr;   // x | y | z on the device
+    float *d = nullptr;   // x | y | z | x sorted | y sorted | places of the sorted x | of the sorted y
+    GridDev dev{};
     int64_t n = 0;
     cudaStream_t s{};
     ~GridAxes() {
@@ -541,7 +543,23 @@ struct GridAxes {
         for (int32_t k = 1; k < nz; ++k)
             if (h[nx + ny + k] < h[nx + ny + k - 1])
                 return set_error(GWN_ERR_INVALID_ARG, "grid z coordinates must be non-decreasing");
+        // x and y in ascending order, with their places (the caller's order is free)
+        const size_t axes = h.size();
+        h.resize(axes + 2 * ((size_t)nx + ny));
+        float *xs = h.data() + axes, *ys = xs + nx;
+        int32_t *xi = reinterpret_cast<int32_t *>(ys + ny), *yi = xi + nx;
+        auto ascending = [](const float *a, int32_t len, float *sorted, int32_t *place) {
+            for (int32_t i = 0; i < len; ++i) place[i] = i;
+            if (!std::is_sorted(a, a + len))
+                std::stable_sort(place, place + len, [a](int32_t i, int32_t j) { return a[i] < a[j]; });
+            for (int32_t i = 0; i < len; ++i) sorted[i] = a[place[i]];
+        };
+        ascending(h.data(), nx, xs, xi);
+        ascending(h.data() + nx, ny, ys, yi);
         GWN_CUDA_TRY(dev_alloc(&d, sizeof(float) * h.size(), s));
+        const float *dxs = d + axes;
+        const int32_t *dxi = reinterpret_cast<const int32_t *>(dxs + nx + ny);
+        dev = GridDev{d, d + nx, d + nx + ny, dxs, dxs + nx, dxi, dxi + nx, nx, ny, nz};
         GWN_CUDA_TRY(cudaMemcpyAsync(d, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice, s));
         GWN_CUDA_TRY(cudaStreamSynchronize(s));   // h goes out of scope
         return GWN_OK;
@@ -567,7 +585,7 @@ gwn_status gwn_query_grid_chi(const gwn_mesh *m, const float *x, int32_t nx, con
     if (!chi) return set_error(GWN_ERR_INVALID_ARG, "chi is NULL");
     void *cd = nullptr;
     if ((st = stg.output(chi, sizeof(int32_t) * ax.n, &cd)) == GWN_OK)
-        st = launch_grid_chi(m, ax.d, nx, ax.d + nx, ny, ax.d + nx + ny, nz, (int32_t *)cd, stg.s);
+        st = launch_grid_chi(m, ax.dev, (int32_t *)cd, stg.s);
     return stg.finish(st);
 }
 
@@ -587,7 +605,7 @@ gwn_status gwn_classify_grid(const gwn_mesh *m, const float *x, int32_t nx, cons
     void *ld = nullptr, *wd = nullptr;
     if ((st = stg.output(label, ax.n, &ld)) == GWN_OK &&
         (st = stg.output(w_or_null, sizeof(float) * ax.n, &wd)) == GWN_OK)
-        st = launch_classify_grid(m, ax.d, nx, ax.d + nx, ny, ax.d + nx + ny, nz, (uint8_t *)ld, (float *)wd, stg.s);
+        st = launch_classify_grid(m, ax.dev, (uint8_t *)ld, (float *)wd, stg.s);
     return stg.finish(st);
 }
 

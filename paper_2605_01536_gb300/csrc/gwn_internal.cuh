@@ -238,12 +238,16 @@ void launch_boundary_combine(const double *partial, int64_t n, int chunks, const
 // quant.cu: the fixed-point frame of the mesh (quantize_bits), written into the
 // status block; bits = 0 (exact FP32 predicates) unless configured
 gwn_status setup_quant(gwn_mesh *m, cudaStream_t s);
-// grid.cu: ray reuse on a rectilinear grid (Supp. S3); axis arrays on the device,
-// gz non-decreasing; outputs indexed [(k ny + j) nx + i]
-gwn_status launch_grid_chi(const gwn_mesh *m, const float *gx, int nx, const float *gy, int ny, const float *gz,
-                           int nz, int32_t *chi, cudaStream_t s);
-gwn_status launch_classify_grid(const gwn_mesh *m, const float *gx, int nx, const float *gy, int ny, const float *gz,
-                                int nz, uint8_t *label, float *w, cudaStream_t s);
+// grid.cu: ray reuse on a rectilinear grid (Supp. S3); axes on the device, z
+// non-decreasing; xs, ys: x and y sorted, xi, yi: their entries' places in x and y;
+// outputs indexed [(k ny + j) nx + i]
+struct GridDev {
+    const float *x, *y, *z, *xs, *ys;
+    const int32_t *xi, *yi;
+    int nx, ny, nz;
+};
+gwn_status launch_grid_chi(const gwn_mesh *m, const GridDev &g, int32_t *chi, cudaStream_t s);
+gwn_status launch_classify_grid(const gwn_mesh *m, const GridDev &g, uint8_t *label, float *w, cudaStream_t s);
 // gradient.cu: grad w (float [n][3]) by Supp. S4, Algorithm 3
 gwn_status launch_gradient(const gwn_mesh *m, const float *q, int64_t n, float *grad, cudaStream_t s);
 // mlp.cu: the surrogate

@@ -49,3 +49,22 @@ def test_every_query_is_answered(mesh, n, spread):
                                         ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert rc == 0 and torch.equal(ls, lab)
     assert torch.max(torch.abs(ws - wc)).item() <= 1e-5
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(1, 1, 1), (33, 1, 5), (7, 40, 17), (130, 3, 16), (64, 70, 33)])
+def test_grid_rasterisation_on_any_axes(nx, ny, nz):
+    """Unsorted axes with repeated entries; triangles from smaller than a cell to the whole grid."""
+    import paper_2605_01536_gb300 as gwn
+    rng = np.random.default_rng(nx * ny)
+    small = gen.random_soup(300, rng)
+    V = np.concatenate([small.V, np.float32([[-9, -9, .3], [9, -9, .3], [0, 9, .9], [-1, -1, -1], [2, -1, -1], [-1, 2, 2]])])
+    F = np.concatenate([small.F, small.nv + np.array([[0, 1, 2], [3, 4, 5]], np.int32)])
+    axis = lambda n: rng.choice(np.linspace(-0.2, 1.2, 2 * n + 1), n).astype(np.float32)
+    x, y, z = axis(nx), axis(ny), np.sort(axis(nz))
+    Z, Y, X = np.meshgrid(z, y, x, indexing="ij")
+    P = torch.from_numpy(np.stack([X, Y, Z], -1).reshape(-1, 3).astype(np.float32)).cuda()
+    with gwn.Mesh(V, F) as m:
+        assert torch.equal(m.grid_chi(x, y, z).ravel(), m.chi(P))
+        lab, w = m.classify_grid(x, y, z, want_w=True)
+        ref_lab, ref_w = m.classify(P, want_w=True)
+    assert torch.equal(lab.ravel(), ref_lab) and torch.max(torch.abs(w.ravel() - ref_w)).item() <= 1e-5
