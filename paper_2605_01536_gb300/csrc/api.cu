@@ -39,21 +39,30 @@ __global__ void k_ingest_vertices(const float *__restrict__ V, int64_t nv, float
     out[i] = make_float4(x, y, z, 0.f);
 }
 
-__global__ void k_ingest_faces(const int32_t *__restrict__ F, int64_t nt, int64_t nv, const float4 *__restrict__ V,
-                               float *__restrict__ tri9, unsigned long long *bad) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nt) return;
-    int32_t a = F[3 * t], b = F[3 * t + 1], c = F[3 * t + 2];
-    if (a < 0 || b < 0 || c < 0 || a >= nv || b >= nv || c >= nv) {
-        atomicAdd(bad + 1, 1ull);
-        return;
+// One thread per face; the nine coordinates go out through shared memory, so that the
+// stores are whole lines (scattered 36-byte rows: 111 us for 642k faces).
+constexpr int kIngest = 128;
+__global__ void __launch_bounds__(kIngest) k_ingest_faces(const int32_t *__restrict__ F, int64_t nt, int64_t nv,
+                                                          const float4 *__restrict__ V, float *__restrict__ tri9,
+                                                          unsigned long long *bad) {
+    __shared__ float s_t[9 * kIngest];
+    const int64_t t0 = (int64_t)blockIdx.x * kIngest, t = t0 + threadIdx.x;
+    float *T = s_t + 9 * threadIdx.x;
+    bool out = false;
+    if (t < nt) {
+        const int32_t i[3] = {F[3 * t], F[3 * t + 1], F[3 * t + 2]};
+        out = i[0] < 0 || i[1] < 0 || i[2] < 0 || i[0] >= nv || i[1] >= nv || i[2] >= nv;
+        for (int k = 0; k < 3; ++k) {
+            const float4 p = out ? make_float4(0.f, 0.f, 0.f, 0.f) : V[i[k]];
+            T[3 * k] = p.x;
+            T[3 * k + 1] = p.y;
+            T[3 * k + 2] = p.z;
+        }
     }
-    const float4 P[3] = {V[a], V[b], V[c]};
-    for (int k = 0; k < 3; ++k) {
-        tri9[9 * t + 3 * k] = P[k].x;
-        tri9[9 * t + 3 * k + 1] = P[k].y;
-        tri9[9 * t + 3 * k + 2] = P[k].z;
-    }
+    if (out) atomicAdd(bad + 1, 1ull);
+    __syncthreads();
+    const int64_t n = min((int64_t)kIngest, nt - t0) * 9;
+    for (int64_t j = threadIdx.x; j < n; j += kIngest) tri9[9 * t0 + j] = s_t[j];
 }
 
 gwn_status check_mesh(const gwn_mesh *m) {
@@ -245,7 +254,7 @@ gwn_status gwn_mesh_create(const float *V, int64_t nv, const int32_t *F, int64_t
     if (nt > 0) {
         cudaMemcpyAsync(m->F, F, sizeof(int32_t) * 3 * nt, fkind > 0 ? cudaMemcpyDeviceToDevice
                                                                        : cudaMemcpyHostToDevice, s);
-        k_ingest_faces<<<grid_for(nt, TB), TB, 0, s>>>(m->F, nt, nv, m->V, m->tri9, bad);
+        k_ingest_faces<<<grid_for(nt, kIngest), kIngest, 0, s>>>(m->F, nt, nv, m->V, m->tri9, bad);
     }
     unsigned long long bad_h[2] = {0, 0};
     cudaMemcpyAsync(bad_h, bad, sizeof(bad_h), cudaMemcpyDeviceToHost, s);
