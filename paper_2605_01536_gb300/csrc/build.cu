@@ -17,7 +17,6 @@
 
 #include "farfield.cuh"
 #include "gwn_internal.cuh"
-#include "traverse.cuh"
 
 namespace gwn {
 
@@ -539,32 +538,33 @@ __global__ void k_morton(const float4 *__restrict__ V, const int32_t *__restrict
     ids[t] = (uint32_t)t;
 }
 
-// Node tests of the +z walks from nsample points spread uniformly over the
-// mesh's vertex box (a fixed hash sequence), summed into *visits: the cost the
-// two candidate trees are compared by.  Their leaves are the same triangles
-// (a triangle's leaf box admits the same rays in either tree), so the walks
-// differ only in the internal nodes they test.
-__device__ __forceinline__ float hash_unit(uint32_t x) {
-    x ^= x >> 16; x *= 0x7feb352du; x ^= x >> 15; x *= 0x846ca68bu; x ^= x >> 16;
-    return (float)(x >> 8) * (1.0f / 16777216.0f);
-}
-
-__global__ void k_tree_sample_visits(const gwn::BvhNode *__restrict__ nodes, int64_t nnodes,
-                                     const float *__restrict__ box, int nsample,
-                                     unsigned long long *__restrict__ counters,
-                                     unsigned long long *__restrict__ visits) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned nv = 0;
-    if (i < nsample) {
-        const float3 p = make_float3(box[0] + (box[3] - box[0]) * hash_unit(3u * i + 1u),
-                                     box[1] + (box[4] - box[1]) * hash_unit(3u * i + 2u),
-                                     box[2] + (box[5] - box[2]) * hash_unit(3u * i + 3u));
-        bvh_walk_up<false, true>(p, nodes, nnodes, nullptr, counters, [](int, float3, float3, float3) {}, 0.f, &nv,
-                                 false);
+// Expected node tests of the +z walk from a point uniform in the mesh's vertex box, the
+// cost the two candidate trees are compared by: a walk tests the root and both children
+// of every internal node it hits, it hits a node iff the point's xy lies in the node's
+// box and its z below the top (its ancestors' boxes contain it), and the three are
+// independent.  So the expectation is 1 + 2 sum over the internal nodes of (x share)
+// (y share) (z share); the sum goes to *cost.  (4,096 sampled walks, serial chains of
+// hundreds of loads, took 130 us a tree on soup7 and 530 us on 30,000 random triangles.)
+__global__ void __launch_bounds__(256) k_tree_cost(const gwn::BvhNode *__restrict__ nodes, int64_t ninternal,
+                                                   const float *__restrict__ box, double *__restrict__ cost) {
+    __shared__ double s_c[8];
+    const float ex = box[3] - box[0], ey = box[4] - box[1], ez = box[5] - box[2];
+    const float ix = ex > 0.f ? 1.f / ex : 0.f, iy = ey > 0.f ? 1.f / ey : 0.f, iz = ez > 0.f ? 1.f / ez : 0.f;
+    double c = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ninternal; i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(nodes + i));
+        const float zmax = __ldg(&nodes[i].zmax);
+        const float fx = ex > 0.f ? (b0.y - b0.x) * ix : 1.f, fy = ey > 0.f ? (b0.w - b0.z) * iy : 1.f,
+                    fz = ez > 0.f ? (zmax - box[2]) * iz : 1.f;
+        c += (double)(fx * fy) * fz;
     }
-    unsigned long long a = nv;
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(visits, a);
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((threadIdx.x & 31) == 0) s_c[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) c += s_c[w];
+        atomicAdd(cost, c);
+    }
 }
 
 __device__ __forceinline__ int delta(const uint32_t *codes, int64_t n, int64_t i, int64_t j) {
@@ -977,12 +977,10 @@ static gwn_status build_tree(const gwn_mesh *m, int dims, const int *bounds, gwn
 }
 
 // Both a tree over xyz Morton codes and one over xy codes (columns: the +z rays
-// of neighbouring queries share their paths) are built, and the one whose
-// walks from a fixed sample of points test fewer nodes (k_tree_sample_visits)
-// is kept.  Measured on the soup8 mesh: 57 instead of 99 node tests per query
-// for the xy tree; random soups of large overlapping triangles keep the xyz
-// tree, whose zmax bounds prune better there.
-constexpr int kTreeSamples = 4096;
+// of neighbouring queries share their paths) are built, and the one with fewer
+// expected node tests per walk (k_tree_cost) is kept.  On the soup8 mesh the xy tree
+// has 57 instead of 99 node tests per query; random soups of large overlapping
+// triangles keep the xyz tree, whose zmax bounds prune better there.
 gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     const int64_t n = m->nt;
     if (m->nodes) { cudaFreeAsync(m->nodes, s); m->nodes = nullptr; }
@@ -993,7 +991,7 @@ gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     gwn::BvhNode *nodes[2] = {nullptr, nullptr};
     float4 *leaf[2] = {nullptr, nullptr};
     int *bounds = nullptr;
-    unsigned long long *visits = nullptr;
+    double *cost = nullptr;
     auto cleanup = [&]() {
         for (int t = 0; t < 2; ++t) {
             if (nodes[t]) cudaFreeAsync(nodes[t], s);
@@ -1010,26 +1008,25 @@ gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
         }
     }
     GWN_CUDA_TRY(dev_alloc(&bounds, sizeof(int) * 6, s));
-    GWN_CUDA_TRY(dev_alloc(&visits, sizeof(unsigned long long) * 2, s));
+    GWN_CUDA_TRY(dev_alloc(&cost, sizeof(double) * 2, s));
     const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, (int)0x80000000, (int)0x80000000, (int)0x80000000};
     GWN_CUDA_TRY(cudaMemcpyAsync(bounds, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    GWN_CUDA_TRY(cudaMemsetAsync(visits, 0, sizeof(unsigned long long) * 2, s));
+    GWN_CUDA_TRY(cudaMemsetAsync(cost, 0, sizeof(double) * 2, s));
     k_centroid_bounds<<<std::min(grid_for(n, TB), kBoundsBlocks), TB, 0, s>>>(m->V, m->F, n, bounds);
     gwn_status st = GWN_OK;
     for (int t = 0; t < 2 && st == GWN_OK; ++t) {
         st = build_tree(m, t == 0 ? 3 : 2, bounds, nodes[t], leaf[t], s);
         if (st == GWN_OK)
-            k_tree_sample_visits<<<grid_for(kTreeSamples, TB), TB, 0, s>>>(nodes[t], m->nnodes, m->box, kTreeSamples,
-                                                                            m->counters, visits + t);
+            k_tree_cost<<<std::min(grid_for(n, TB), 608u), TB, 0, s>>>(nodes[t], n - 1, m->box, cost + t);
     }
-    unsigned long long cost_h[2] = {0, 0};
+    double cost_h[2] = {0.0, 0.0};
     if (st == GWN_OK) {
-        cudaError_t e = cudaMemcpyAsync(cost_h, visits, sizeof(cost_h), cudaMemcpyDeviceToHost, s);
+        cudaError_t e = cudaMemcpyAsync(cost_h, cost, sizeof(cost_h), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = set_error(GWN_ERR_CUDA, cudaGetErrorString(e));
     }
     cudaFreeAsync(bounds, s);
-    cudaFreeAsync(visits, s);
+    cudaFreeAsync(cost, s);
     if (st != GWN_OK) {
         cleanup();
         return st;

@@ -316,97 +316,103 @@ __global__ void __launch_bounds__(64) k_far_leaf_moments(FarShape sh, const FarN
     warp_store_moments(M, raw + i * kFarRaw, false);
 }
 
-// Moments of the nodes of level l > 0, one warp each: the children's moments
+// Moments of the nodes of level l > 0, one block each: the children's moments
 // translated to the node's centre,
 //   M_lm += sum_{l' <= l, m'} R_(l-l')^(m-m')(d) M_l'm',  d = the child's centre,
 // plus the closed polygons by which the children's chords differ from the node's.
-__global__ void __launch_bounds__(64) k_far_up(FarShape sh, int l, const FarNode *__restrict__ nodes,
-                                               const float4 *__restrict__ pts, Cplx *__restrict__ raw) {
-    __shared__ Cplx s_R[2][kFarRaw], s_M[2][kFarRaw];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 2 + warp;
-    const bool on = i < far_level_count(sh, l);
-    FarNode nd{};
-    Cplx acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-    int oL[2] = {0, 0}, oM[2] = {0, 0};   // this lane's (l, m) outputs: indices lane + 1, lane + 33
-    for (int h = 0; h < 2; ++h) {
-        const int k = lane + 1 + 32 * h;
-        int L = 1;
-        while (far_idx(L + 1, 0) <= k) ++L;
-        oL[h] = L;
-        oM[h] = k - far_idx(L, 0);
-    }
-    int chords = 0;
-    if (on) {
-        nd = nodes[far_preorder(sh, l, i)];
-        chords = nd.nchord;
-    }
-    for (int c = 0; c < 2; ++c) {
-        const int64_t ci = 2 * i + c;
-        bool have = on && ci < far_level_count(sh, l - 1);
-        __syncwarp();
-        if (have) have = nodes[far_preorder(sh, l - 1, ci)].count > 0;
-        if (have) {
-            const FarNode ch = nodes[far_preorder(sh, l - 1, ci)];
-            chords += ch.nchord;
-            const Cplx *cm = raw + (sh.off[l - 1] + ci) * kFarRaw;
-            const float ratio = ch.inv_s > 0.f ? nd.inv_s / ch.inv_s : 0.f;   // s_child / s
-            if (lane == 0) {
-                Cplx R[kFarRaw];
-                solid_regular<P>((ch.cx - nd.cx) * nd.inv_s, (ch.cy - nd.cy) * nd.inv_s, (ch.cz - nd.cz) * nd.inv_s, R);
+// The levels follow one another, so the latency of one node counts: thread (child,
+// output) sums one child's part of one moment, and the columns of R are made by one
+// thread each (one warp per node with R made by one lane: 24 us a level, now 7).
+constexpr int kUpThreads = 96;
+__global__ void __launch_bounds__(kUpThreads) k_far_up(FarShape sh, int l, const FarNode *__restrict__ nodes,
+                                                       const float4 *__restrict__ pts, Cplx *__restrict__ raw) {
+    __shared__ Cplx s_R[2][kFarRaw], s_M[2][kFarRaw], s_part[kFarRaw];
+    __shared__ int s_chords;
+    const int64_t i = blockIdx.x;
+    const FarNode *nd = nodes + far_preorder(sh, l, i);
+    const FarNode *ch[2] = {nullptr, nullptr};   // the children that have points
 #pragma unroll
-                for (int k = 0; k < kFarRaw; ++k) s_R[warp][k] = R[k];
-            }
-            for (int k = lane; k < kFarRaw; k += 32) {
-                int L = 0;
-                while (far_idx(L + 1, 0) <= k) ++L;
-                float f = ratio;
-                for (int t = 0; t < L; ++t) f *= ratio;
-                const Cplx v = cm[k];
-                s_M[warp][k] = k == 0 ? Cplx{0.f, 0.f} : Cplx{f * v.r, f * v.i};
-            }
+    for (int c = 0; c < 2; ++c)
+        if (2 * i + c < far_level_count(sh, l - 1)) {
+            const FarNode *p = nodes + far_preorder(sh, l - 1, 2 * i + c);
+            if (p->count > 0) ch[c] = p;
         }
-        __syncwarp();
-        if (have) {
-            for (int h = 0; h < 2; ++h) {
-                const int L = oL[h], m = oM[h];
-                if (L > P) continue;
-                for (int lp = 1; lp <= L; ++lp)
-                    for (int mp = max(-lp, m - (L - lp)); mp <= min(lp, m + (L - lp)); ++mp) {
-                        const int mr = m - mp;
-                        Cplx a = s_M[warp][far_idx(lp, abs(mp))], r = s_R[warp][far_idx(L - lp, abs(mr))];
-                        // X_l^(-m) = (-1)^m conj(X_l^m)
-                        if (mp < 0) a = (mp & 1) ? Cplx{-a.r, a.i} : Cplx{a.r, -a.i};
-                        if (mr < 0) r = (mr & 1) ? Cplx{-r.r, r.i} : Cplx{r.r, -r.i};
-                        const Cplx t = cmul(r, a);
-                        acc[h].r += t.r;
-                        acc[h].i += t.i;
-                    }
+    const int t = threadIdx.x;
+    if (t == 0) s_chords = nd->nchord + (ch[0] ? ch[0]->nchord : 0) + (ch[1] ? ch[1]->nchord : 0);
+    const float is = nd->inv_s;
+    if (t < 2 * (P + 1)) {   // column m of R at child c's centre
+        const int c = t / (P + 1), m = t % (P + 1);
+        if (ch[c]) {
+            const float x = (ch[c]->cx - nd->cx) * is, y = (ch[c]->cy - nd->cy) * is, z = (ch[c]->cz - nd->cz) * is,
+                        r2 = x * x + y * y + z * z;
+            Cplx a = {1.f, 0.f}, b = {0.f, 0.f};
+            for (int k = 1; k <= m; ++k) {
+                const float f = -0.5f / k;
+                a = cmul(a, {f * x, f * y});
+            }
+            s_R[c][far_idx(m, m)] = a;
+            for (int L = m + 1; L <= P; ++L) {
+                const float f = 1.f / (float)((L + m) * (L - m)), g = (2 * L - 1) * f * z, h = L == m + 1 ? 0.f : f * r2;
+                const Cplx n = {g * a.r - h * b.r, g * a.i - h * b.i};
+                b = a;
+                a = n;
+                s_R[c][far_idx(L, m)] = n;
             }
         }
     }
-    if (!on) return;
+    for (int k = t; k < 2 * kFarRaw; k += kUpThreads) {   // the children's moments in units of this node
+        const int c = k / kFarRaw, j = k % kFarRaw;
+        if (!ch[c] || j == 0) continue;
+        int L = 1;
+        while (far_idx(L + 1, 0) <= j) ++L;
+        const float ratio = ch[c]->inv_s > 0.f ? is / ch[c]->inv_s : 0.f;   // s_child / s
+        float f = ratio;
+        for (int q = 0; q < L; ++q) f *= ratio;
+        const Cplx v = raw[(sh.off[l - 1] + 2 * i + c) * kFarRaw + j];
+        s_M[c][j] = {f * v.r, f * v.i};
+    }
+    __syncthreads();
+    const int c = t / (kFarRaw - 1), o = 1 + t % (kFarRaw - 1);   // child, output
+    Cplx acc = {0.f, 0.f};
+    if (c < 2 && ch[c]) {
+        int L = 1;
+        while (far_idx(L + 1, 0) <= o) ++L;
+        const int m = o - far_idx(L, 0);
+        for (int lp = 1; lp <= L; ++lp)
+            for (int mp = max(-lp, m - (L - lp)); mp <= min(lp, m + (L - lp)); ++mp) {
+                const int mr = m - mp;
+                Cplx a = s_M[c][far_idx(lp, abs(mp))], r = s_R[c][far_idx(L - lp, abs(mr))];
+                // X_l^(-m) = (-1)^m conj(X_l^m)
+                if (mp < 0) a = (mp & 1) ? Cplx{-a.r, a.i} : Cplx{a.r, -a.i};
+                if (mr < 0) r = (mr & 1) ? Cplx{-r.r, r.i} : Cplx{r.r, -r.i};
+                const Cplx p = cmul(r, a);
+                acc.r += p.r;
+                acc.i += p.i;
+            }
+    }
+    if (c == 1) s_part[o] = acc;
+    __syncthreads();
     Cplx *out = raw + (sh.off[l] + i) * kFarRaw;
-    for (int h = 0; h < 2; ++h)
-        if (oL[h] <= P) out[lane + 1 + 32 * h] = acc[h];
-    if (chords == 0) return;   // warp-uniform
-    __syncwarp();
+    if (c == 0) out[o] = {acc.r + s_part[o].r, acc.i + s_part[o].i};
+    if (s_chords == 0) return;
+    __syncthreads();
+    if (t >= 32) return;
     Cplx M[kFarRaw];
 #pragma unroll
     for (int k = 0; k < kFarRaw; ++k) M[k] = {0.f, 0.f};
     // lanes 0-3: the children's chords (start -> end); 4, 5: the node's own, reversed
     int ja = -1, jb = -1;
-    if (lane < 4) {
-        const int64_t ci = 2 * i + (lane >> 1);
-        if (ci < far_level_count(sh, l - 1)) {
-            const FarNode &ch = nodes[far_preorder(sh, l - 1, ci)];
-            if ((lane & 1) < ch.nchord) { ja = ch.ch[2 * (lane & 1)]; jb = ch.ch[2 * (lane & 1) + 1]; }
+    if (t < 4) {
+        const FarNode *p = ch[t >> 1];
+        if (p && (t & 1) < p->nchord) {
+            ja = p->ch[2 * (t & 1)];
+            jb = p->ch[2 * (t & 1) + 1];
         }
-    } else if (lane < 6 && lane - 4 < nd.nchord) {
-        ja = nd.ch[2 * (lane - 4) + 1];
-        jb = nd.ch[2 * (lane - 4)];
+    } else if (t < 6 && t - 4 < nd->nchord) {
+        ja = nd->ch[2 * (t - 4) + 1];
+        jb = nd->ch[2 * (t - 4)];
     }
-    if (ja >= 0) edge_moments(rel_point(pts, ja, nd), rel_point(pts, jb, nd), M);
+    if (ja >= 0) edge_moments(rel_point(pts, ja, *nd), rel_point(pts, jb, *nd), M);
     warp_store_moments(M, out, true);
 }
 
@@ -564,7 +570,7 @@ gwn_status build_far(gwn_mesh *m, float4 *pts, const uint2 *ends, cudaStream_t s
         GWN_CUDA_TRY(dev_alloc(&coef, sizeof(float) * kFarCoef * sh.total, s));
         k_far_leaf_moments<<<grid_for(sh.nleaf, 2), 64, 0, s>>>(sh, nodes, pts, raw);
         for (int l = 1; l <= sh.top; ++l)
-            k_far_up<<<grid_for(far_level_count(sh, l), 2), 64, 0, s>>>(sh, l, nodes, pts, raw);
+            k_far_up<<<(unsigned)far_level_count(sh, l), kUpThreads, 0, s>>>(sh, l, nodes, pts, raw);
         GWN_CUDA_TRY(dev_alloc(&m->far_gcoef, sizeof(float) * kFarGradCoef * sh.total, s));
         k_far_pack<<<grid_for(sh.total * kFarRaw, 256), 256, 0, s>>>(sh, raw, coef);
         k_far_pack_grad<<<grid_for(sh.total * (kFarP + kFarGradCols), 256), 256, 0, s>>>(sh, raw, m->far_gcoef);
