@@ -411,6 +411,11 @@ gwn_status gwn_query_batch(const gwn_mesh *m, const float *q, int64_t n, float *
     if ((st = stg.input(q, sizeof(float) * 3 * n, &qd)) != GWN_OK ||
         (st = stg.output(w, sizeof(float) * n, &wd)) != GWN_OK)
         return stg.finish(st);
+    if (small_call(m, n)) {
+        if (!chi || (st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK)
+            st = launch_small(m, (const float *)qd, n, (float *)wd, (int32_t *)cd, nullptr, stg.s);
+        return stg.finish(st);
+    }
     if (n >= kOrderMinQueries) {   // in spatial order, scattered back
         void *keys = nullptr, *perm = nullptr, *qs = nullptr, *ws = nullptr, *cs = nullptr;
         if ((st = stg.output(chi, sizeof(int32_t) * n, &cd)) == GWN_OK &&
@@ -453,6 +458,11 @@ gwn_status gwn_classify(const gwn_mesh *m, const float *q, int64_t n, uint8_t *l
         // the gate needs w_hat somewhere even when the caller does not want w
         if ((st = stg.output(w_or_null, sizeof(float) * n, &wd)) != GWN_OK) return stg.finish(st);
         return stg.finish(classify_with_surrogate(m, (const float *)qd, n, (uint8_t *)ld, (float *)wd, stg.s));
+    }
+    if (small_call(m, n)) {
+        if (!w_or_null || (st = stg.output(w_or_null, sizeof(float) * n, &wd)) == GWN_OK)
+            st = launch_small(m, (const float *)qd, n, (float *)wd, nullptr, (uint8_t *)ld, stg.s);
+        return stg.finish(st);
     }
     const bool ordered = n >= kOrderMinQueries;
     void *keys = nullptr, *perm = nullptr, *qs = nullptr, *ws = nullptr, *ls = nullptr;

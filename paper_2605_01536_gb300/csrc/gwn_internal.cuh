@@ -201,6 +201,10 @@ gwn_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint
 
 // query.cu
 gwn_status launch_chi(const gwn_mesh *m, const float *q, int64_t n, int32_t *chi, cudaStream_t s);
+// a small call as one kernel: w, chi and label may be NULL (label: as gwn_classify)
+bool small_call(const gwn_mesh *m, int64_t n);
+gwn_status launch_small(const gwn_mesh *m, const float *q, int64_t n, float *w, int32_t *chi, uint8_t *label,
+                        cudaStream_t s);
 gwn_status launch_chi_visits(const gwn_mesh *m, const float *q, int64_t n, int32_t *chi,
                              unsigned long long *visits, cudaStream_t s);
 // boundary-curve sum + combine; with classify, labels and appends queries within

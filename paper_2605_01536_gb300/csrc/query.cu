@@ -28,6 +28,7 @@ namespace {
 // Launched in blocks of 128 threads (compiled for up to 256): finer tails than
 // 256 (measured 5.6% faster on 2M soup8 queries, bit-identical).
 constexpr int kChiThreads = 128;
+constexpr int64_t kSmallTris = 2048;   // leaves k_small tests one by one (64 per lane)
 
 // Fixed selects the predicate mode at compile time (the host knows the mesh's
 // quantize_bits), so the exact kernel carries none of the fixed-point code.
@@ -554,6 +555,81 @@ __global__ void __launch_bounds__(256) k_batch_fp64_fix(const BatchMesh *__restr
     }
 }
 
+// ------------------------------------------------------- small calls ----
+
+// A call of few queries against few boundary points, whole: one warp per query counts
+// the crossings (every leaf box by all lanes on a small mesh, else one lane walks the
+// tree), sums the edge terms lane by lane in FP64, and re-evaluates the sum in FP64 where
+// classify needs it.  The general path's kernels each leave the GPU nearly idle for a
+// serial chain (64 queries on a 36-edge boundary: crossings 22 us, boundary 20 us, FP64
+// check 4 us, with five allocations and two memsets); this is one launch of about 8 us
+// and no scratch.  Bound by latency: the chain of one warp.
+constexpr int kSmallThreads = 128;
+__global__ void __launch_bounds__(kSmallThreads) k_small(const float *__restrict__ q, int64_t n,
+                                                         const BvhNode *__restrict__ nodes, int64_t nnodes,
+                                                         const float4 *__restrict__ tri, const float4 *__restrict__ pts,
+                                                         int64_t npts, float *__restrict__ w, int32_t *__restrict__ chi,
+                                                         uint8_t *__restrict__ label, float margin,
+                                                         unsigned long long *__restrict__ counters) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const float qx = q[3 * i], qy = q[3 * i + 1], qz = q[3 * i + 2];
+    const float3 p = make_float3(qx, qy, qz);
+    const int64_t nt = (nnodes + 1) / 2;
+    int c = 0;
+    bool ok = true;
+    if (nt <= kSmallTris) {
+        for (int64_t t = lane; t < nt; t += 32) {
+            const float4 *np = reinterpret_cast<const float4 *>(nodes + (nt - 1) + t);   // leaf t of the tree
+            const float4 b0 = __ldg(np), b1 = __ldg(np + 1);
+            if (!(qx >= b0.x && qx <= b0.y && qy >= b0.z && qy <= b0.w && qz <= b1.x)) continue;
+            const float4 a = __ldg(tri + 3 * t), b = __ldg(tri + 3 * t + 1), d = __ldg(tri + 3 * t + 2);
+            c += tri_crossing(p, make_float3(a.x, a.y, a.z), make_float3(b.x, b.y, b.z), make_float3(d.x, d.y, d.z),
+                              &counters[CNT_EXACT_EDGE], &counters[CNT_EXACT_PLANE]);
+        }
+    } else if (lane == 0) {
+        ok = bvh_walk_up(p, nodes, nnodes, tri, counters, [&](int, float3 a, float3 b, float3 d) {
+            c += tri_crossing(p, a, b, d, &counters[CNT_EXACT_EDGE], &counters[CNT_EXACT_PLANE]);
+        });
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (!__all_sync(0xffffffffu, ok)) c = INT32_MIN;
+    double s = 0.0;
+    int cancelled = 0;
+    for (int64_t j = lane; j + 1 < npts; j += 32) {
+        const float4 Pa = __ldg(pts + j), Pb = __ldg(pts + j + 1);
+        if (Pa.w == 0.f) continue;
+        const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
+        const float en = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
+        const float ed = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
+        if (cancels(en, ed, A.h, B.h)) {
+            s += edge_angle64(Pa, Pb, qx, qy, qz, counters);
+            ++cancelled;
+        } else {
+            s += edge_term(en, ed, A, B, Pa, Pb, qx, qy, qz, counters);
+        }
+    }
+    cancelled = __reduce_add_sync(0xffffffffu, cancelled);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    double wv = (double)c + s * kInv2Pi;
+    if (label && fabs(wv - 0.5) <= (double)margin) {   // warp-uniform
+        s = 0.0;
+        for (int64_t j = lane; j + 1 < npts; j += 32) {
+            const float4 Pa = __ldg(pts + j);
+            if (Pa.w != 0.f) s += edge_angle64(Pa, __ldg(pts + j + 1), qx, qy, qz, counters);
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        wv = (double)c + s * kInv2Pi;
+        if (lane == 0) atomicAdd(&counters[CNT_FP64], 1ull);
+    }
+    if (lane != 0) return;
+    if (cancelled) atomicAdd(&counters[CNT_CANCEL], (unsigned long long)cancelled);
+    if (w) w[i] = (float)wv;
+    if (chi) chi[i] = c;
+    if (label) label[i] = wv > 0.5 ? 1 : 0;
+}
+
 // ------------------------------------------------------------- direct ----
 
 // Direct sum (Eq. 2, each area by Eq. 6): per triangle 2 atan2(det[a b c], l_a l_b l_c + (a.b) l_c
@@ -653,6 +729,26 @@ gwn_status launch_chi(const gwn_mesh *m, const float *q, int64_t n, int32_t *chi
         k_chi<false><<<grid_for(n, kChiThreads), kChiThreads, 0, s>>>(q, n, m->nodes, m->nnodes, m->leaf_tri, chi,
                                                                         m->counters);
     GWN_LAUNCH_CHECK("k_chi");
+    return GWN_OK;
+}
+
+// Few queries (a warp each), few points (a lane takes npts / 32 of them) and little
+// work in all: 2^20 terms of about 150 instructions are 4 us of the whole GPU.  Explicit
+// schedules and the plain FP32 or fixed-point forms keep the general path.
+bool small_call(const gwn_mesh *m, int64_t n) {
+    return n <= 4096 && m->npts <= 4096 && n * m->npts <= (int64_t(1) << 20) && m->cfg.quantize_bits == 0 &&
+           m->cfg.queries_per_thread == 0 && m->cfg.boundary_tile == 0 && m->cfg.group_test == 0 &&
+           m->cfg.fp64_cancel >= 0;
+}
+
+gwn_status launch_small(const gwn_mesh *m, const float *q, int64_t n, float *w, int32_t *chi, uint8_t *label,
+                        cudaStream_t s) {
+    if (n <= 0) return GWN_OK;
+    ProfScope prof("small_call", s);
+    const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
+    k_small<<<grid_for(32 * n, kSmallThreads), kSmallThreads, 0, s>>>(q, n, m->nodes, m->nnodes, m->leaf_tri, m->bpts,
+                                                                      m->npts, w, chi, label, margin, m->counters);
+    GWN_LAUNCH_CHECK("k_small");
     return GWN_OK;
 }
 

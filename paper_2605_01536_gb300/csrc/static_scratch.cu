@@ -109,7 +109,9 @@ extern "C" gwn_status gwn_classify_static(const gwn_mesh *m, const float *q, int
     } else {
         unsigned char *base = nullptr;
         st = scratch_address(m->device, &base);
-        if (st == GWN_OK) {
+        if (st == GWN_OK && gwn::small_call(m, n)) {
+            st = gwn::launch_small(m, q, n, w_or_null, nullptr, label, (cudaStream_t)stream);
+        } else if (st == GWN_OK) {
             cudaStream_t s = (cudaStream_t)stream;
             // Large calls run in spatial order like gwn_classify's, in slices that fit the
             // scratch (an order over the slice serves as well); small ones as they come.
