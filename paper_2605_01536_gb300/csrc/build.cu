@@ -1035,6 +1035,7 @@ gwn_status build_bvh(gwn_mesh *m, cudaStream_t s) {
     m->nodes = nodes[keep];
     m->leaf_tri = leaf[keep];
     m->bvh_xy = keep == 1;
+    m->walk_cost = 1.0 + 2.0 * cost_h[keep];
     cudaFreeAsync(nodes[1 - keep], s);
     cudaFreeAsync(leaf[1 - keep], s);
     GWN_LAUNCH_CHECK("bvh build");

@@ -140,6 +140,7 @@ struct gwn_mesh {
     int64_t nnodes = 0;
     gwn::BvhNode *nodes = nullptr;   // [2 nt - 1]
     float4 *leaf_tri = nullptr;      // [3 nt] triangles in BVH leaf order
+    double walk_cost = 0.0;          // expected node tests of a +z walk from a point of the box
     bool bvh_xy = false;             // the tree was built over xy Morton codes (columns), else xyz
 
     unsigned long long *counters = nullptr;   // status block: [CNT_SLOTS] counters, then the

@@ -51,6 +51,67 @@ __device__ __forceinline__ bool bvh_walk_up(float3 p, const BvhNode *__restrict_
     return true;
 }
 
+// The walk of one ray by the 32 lanes of a warp together: the subtrees still to visit
+// lie on a stack in shared memory and each round tests up to 32 of their roots.  A ray
+// that runs along a surface tests tens of thousands of nodes, and as one lane's chain of
+// dependent loads that takes milliseconds.  Items: node << 2 | follow; follow 1 adds the
+// node's escape link as an item of its own (the sibling of a left child), 2 the whole
+// chain of escape links (the rest of a depth-first walk that stands at the node).
+// on_leaf runs on the lane that tests the leaf; the leaves are those of bvh_walk_up.
+// Every lane must call it with the same arguments; stack: kFrontierCap entries of the warp.
+constexpr int kFrontierCap = 512;
+template <class OnLeaf>
+__device__ __forceinline__ bool bvh_frontier_warp(float3 p, int start, int follow, const BvhNode *__restrict__ nodes,
+                                                  int64_t nnodes, const float4 *__restrict__ tri,
+                                                  unsigned long long *__restrict__ counters,
+                                                  unsigned long long *stack, OnLeaf &&on_leaf) {
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int count = start >= 0 && start < nnodes ? 1 : 0;
+    if (lane == 0) stack[0] = (unsigned long long)start << 2 | (unsigned)follow;
+    __syncwarp();
+    int64_t budget = nnodes + 1;   // each node at most once
+    while (count > 0) {
+        // an item is replaced by at most two: near the stack's end one at a time, so that
+        // it grows by at most the tree's depth (below 64 levels, two items each)
+        const int k = count > kFrontierCap - 192 ? 1 : min(count, 32);
+        budget -= k;
+        if (budget < 0 || count > kFrontierCap - 2) {
+            if (lane == 0) atomicOr(&counters[CNT_ERROR], (unsigned long long)ERR_TRAVERSAL_LIMIT);
+            return false;
+        }
+        const bool mine = lane < k;
+        const unsigned long long item = mine ? stack[count - 1 - lane] : 0ull;
+        __syncwarp();
+        count -= k;
+        int child = -1, next = -1;
+        const int follows = (int)(item & 3u);
+        if (mine) {
+            const int node = (int)(item >> 2);
+            const float4 *np = reinterpret_cast<const float4 *>(nodes + node);
+            const float4 b0 = __ldg(np), b1 = __ldg(np + 1);
+            if (follows) next = __float_as_int(b1.z);
+            if (p.x >= b0.x && p.x <= b0.y && p.y >= b0.z && p.y <= b0.w && p.z <= b1.x) {
+                const int c = __float_as_int(b1.y);
+                if (__float_as_int(b1.w)) {
+                    const float4 a = __ldg(tri + 3 * (int64_t)c), bb = __ldg(tri + 3 * (int64_t)c + 1),
+                                 cc = __ldg(tri + 3 * (int64_t)c + 2);
+                    on_leaf(c, make_float3(a.x, a.y, a.z), make_float3(bb.x, bb.y, bb.z), make_float3(cc.x, cc.y, cc.z));
+                } else {
+                    child = c;
+                }
+            }
+        }
+        const unsigned mn = __ballot_sync(0xffffffffu, next >= 0), mc = __ballot_sync(0xffffffffu, child >= 0);
+        if (next >= 0) stack[count + __popc(mn & below)] = (unsigned long long)next << 2 | (follows == 2 ? 2u : 0u);
+        count += __popc(mn);
+        if (child >= 0) stack[count + __popc(mc & below)] = (unsigned long long)child << 2 | 1u;
+        count += __popc(mc);
+        __syncwarp();
+    }
+    return true;
+}
+
 // The walk of bvh_walk_up taken by the 32 lanes of a warp together, with the
 // leaves postponed so that the warp tests them in step: a lane that reaches a
 // hit leaf holds it and walks on; reaching a second one it stops; the warp
@@ -62,10 +123,16 @@ __device__ __forceinline__ bool bvh_walk_up(float3 p, const BvhNode *__restrict_
 // Each lane visits the same leaves in the same order as bvh_walk_up (on_leaf
 // gets the same calls), and its node budget counts the same visits.  Every
 // lane of the warp must call it; a lane without a query passes active = false.
-template <class OnLeaf>
+// Limited: a lane that has tested kWalkLimit nodes stops after the leaves it holds and
+// leaves the node it stands at in *rest (-1: done) for bvh_frontier_warp.
+constexpr int kWalkLimit = 192;
+template <bool Limited = false, class OnLeaf>
 __device__ __forceinline__ bool bvh_walk_up_warp(bool active, float3 p, const BvhNode *__restrict__ nodes,
                                                  int64_t nnodes, const float4 *__restrict__ tri,
-                                                 unsigned long long *__restrict__ counters, OnLeaf &&on_leaf) {
+                                                 unsigned long long *__restrict__ counters, OnLeaf &&on_leaf,
+                                                 int *rest = nullptr) {
+    int left = kWalkLimit;
+    if constexpr (Limited) *rest = -1;
     int node = active && nnodes > 0 ? 0 : -1;
     int held = -1, next = -1;   // the leaf to test next and the one after it
     int64_t budget = nnodes + 1;
@@ -88,6 +155,13 @@ __device__ __forceinline__ bool bvh_walk_up_warp(bool active, float3 p, const Bv
             continue;
         }
         if (!movable) continue;
+        if constexpr (Limited) {
+            if (--left < 0) {
+                *rest = node;
+                node = -1;
+                continue;
+            }
+        }
         if (--budget < 0 || node >= nnodes) {
             atomicOr(&counters[CNT_ERROR], (unsigned long long)ERR_TRAVERSAL_LIMIT);
             ok = false;
