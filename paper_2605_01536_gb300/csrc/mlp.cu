@@ -317,6 +317,16 @@ __global__ void __launch_bounds__(128) k_mlp_forward(
     if (warp == 0) tc::tmem_dealloc(tm, 64);
 }
 
+// eight BF16 values of a 16-byte chunk as FP32
+__device__ __forceinline__ void unpack_bf16(uint4 v, float *out) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        out[2 * i] = __uint_as_float(w[i] << 16);
+        out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+
 // delta_{l-1}[b][k] = (sum_n delta_l[b][n] W_l[n][k]) * (h_{l-1}[b][k] > 0), one
 // 128-row tile per CTA (layers 2..4, all 64 wide).  Also accumulates
 // grad b_l = sum_b delta_l[b][.].
@@ -338,10 +348,14 @@ __global__ void __launch_bounds__(128) k_mlp_back_dx(const __nv_bfloat16 *__rest
         const int nn = i / kHid, k = i % kHid;
         *reinterpret_cast<__nv_bfloat16 *>(sWt + tc::core_offset(k, nn, kHid)) = Wl[i];
     }
+    // the row in 16-byte loads (element by element: 64 loads a thread)
     float d[kHid];
 #pragma unroll
-    for (int j = 0; j < kHid; ++j) d[j] = valid ? __bfloat162float(Dl[row * kHid + j]) : 0.f;
-    store_row_bf16(sA, tid, d, kHid);
+    for (int kc = 0; kc < kHid / 8; ++kc) {
+        const uint4 v = valid ? __ldg(reinterpret_cast<const uint4 *>(Dl + row * kHid) + kc) : make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4 *>(sA + tc::core_offset(tid, kc * 8, kHid)) = v;
+        unpack_bf16(v, d + kc * 8);
+    }
     // grad of the bias of layer l
 #pragma unroll
     for (int j = 0; j < kHid; ++j) {
@@ -358,14 +372,15 @@ __global__ void __launch_bounds__(128) k_mlp_back_dx(const __nv_bfloat16 *__rest
     float out[kHid];
     const bool ok = mma_layer(tmem_base, sA, sWt, kHid, &bar, phase, out, err);
     if (ok && valid) {
-        float v[kHid];
-#pragma unroll
-        for (int j = 0; j < kHid; ++j) v[j] = __bfloat162float(Hprev[row * kHid + j]) > 0.f ? out[j] : 0.f;
 #pragma unroll
         for (int kc = 0; kc < kHid / 8; ++kc) {
+            float h[8];
+            unpack_bf16(__ldg(reinterpret_cast<const uint4 *>(Hprev + row * kHid) + kc), h);
             __nv_bfloat162 p[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(v[kc * 8 + 2 * i], v[kc * 8 + 2 * i + 1]);
+            for (int i = 0; i < 4; ++i)
+                p[i] = __floats2bfloat162_rn(h[2 * i] > 0.f ? out[kc * 8 + 2 * i] : 0.f,
+                                             h[2 * i + 1] > 0.f ? out[kc * 8 + 2 * i + 1] : 0.f);
             *reinterpret_cast<uint4 *>(Dprev + row * kHid + kc * 8) = *reinterpret_cast<uint4 *>(p);
         }
     }
@@ -377,19 +392,45 @@ __global__ void __launch_bounds__(128) k_mlp_back_dx(const __nv_bfloat16 *__rest
 // grad W_l[n][k] += sum_b delta_l[b][n] h_{l-1}[b][k] over a chunk of the batch:
 // D[k][n] (TMEM, 128 x 64; k < K_l, rows past K_l are zero padding) with
 // A[k][b] = h_{l-1}[b][k] and B[n][b] = delta_l[b][n] staged transposed, the
-// batch chunk as the reduction dimension (kChunkB rows per MMA chain).
+// batch chunk as the reduction dimension (kChunkB rows per MMA chain).  The four
+// layers run in one launch (blockIdx.y) once their deltas exist: a batch of 16,384 has
+// only 16 chunks of rows a layer.  Bound by the transposing stores to shared memory;
+// staged element by element and one layer at a time it took 96 us a layer (the whole
+// gradient of 16,384 samples 546 -> 158 us, of 65,536 696 -> 254; same bits).
 constexpr int kChunkB = 128;
-__global__ void __launch_bounds__(128) k_mlp_back_dw(const __nv_bfloat16 *__restrict__ Hprev, int Kl,
-                                                      const __nv_bfloat16 *__restrict__ Dl, int64_t nb,
-                                                      int64_t rows_per_cta, long long *__restrict__ gradW,
-                                                      unsigned *err) {
+struct DwLayers {
+    const __nv_bfloat16 *h[4], *d[4];   // h_{l-1} (the features for l = 1) and delta_l
+    int k[4], grad[4];                  // K_l and the offset of W_l's gradient
+};
+
+// Columns [8 kc, 8 kc + 8) of this thread's batch row (v) into the K-major matrix with the
+// batch along its rows' elements: neighbouring lanes exchange halves, so that each store
+// carries two batch entries of one row.
+__device__ __forceinline__ void stage_transposed(unsigned char *sM, int kc, int tid, uint4 v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const bool odd = tid & 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t o = __shfl_xor_sync(0xffffffffu, w[i], 1);
+        // even lanes: element 2 i of both rows; odd lanes: element 2 i + 1 of both
+        const uint32_t x = odd ? __byte_perm(o, w[i], 0x7632) : __byte_perm(w[i], o, 0x5410);
+        *reinterpret_cast<uint32_t *>(sM + tc::core_offset(kc * 8 + 2 * i + (odd ? 1 : 0), tid & ~1, kChunkB)) = x;
+    }
+}
+
+__global__ void __launch_bounds__(128) k_mlp_back_dw(DwLayers layers, int64_t nb, int64_t rows_per_cta,
+                                                      long long *__restrict__ grad, unsigned *err) {
     __shared__ __align__(1024) unsigned char sA[128 * kChunkB * 2];
     __shared__ __align__(1024) unsigned char sB[kHid * kChunkB * 2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, layer = blockIdx.y;
+    const __nv_bfloat16 *Hprev = layers.h[layer], *Dl = layers.d[layer];
+    const int Kl = layers.k[layer];
+    long long *gradW = grad + layers.grad[layer];
     if (warp == 0) tc::tmem_alloc(&tmem_base, 64);
     if (tid == 0) tc::mbar_init(&bar, 1);
+    for (int kc = Kl / 8; kc < 16; ++kc) stage_transposed(sA, kc, tid, make_uint4(0, 0, 0, 0));
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -398,17 +439,22 @@ __global__ void __launch_bounds__(128) k_mlp_back_dw(const __nv_bfloat16 *__rest
     const int64_t b0 = (int64_t)blockIdx.x * rows_per_cta, b1 = min(nb, b0 + rows_per_cta);
     bool first = true, ok = true;
     for (int64_t c0 = b0; c0 < b1 && ok; c0 += kChunkB) {
-        // stage: thread t owns batch column (c0 + t); writes its column of A (K_l rows) and B (64 rows)
+        // stage: thread t owns batch column (c0 + t) of A (K_l rows) and B (64 rows)
         const int64_t b = c0 + tid;
         const bool valid = b < b1;
-        for (int k = 0; k < 128; ++k) {
-            const __nv_bfloat16 hv = (valid && k < Kl) ? Hprev[b * Kl + k] : __float2bfloat16(0.f);
-            *reinterpret_cast<__nv_bfloat16 *>(sA + tc::core_offset(k, tid, kChunkB)) = hv;
+        const uint4 *hp = reinterpret_cast<const uint4 *>(Hprev + b * Kl), *dp = reinterpret_cast<const uint4 *>(Dl + b * kHid);
+        uint4 dv[8];
+#pragma unroll
+        for (int kc = 0; kc < 8; ++kc) dv[kc] = valid ? __ldg(dp + kc) : make_uint4(0, 0, 0, 0);
+        for (int k8 = 0; k8 < Kl / 8; k8 += 8) {
+            uint4 hv[8];
+#pragma unroll
+            for (int kc = 0; kc < 8; ++kc) hv[kc] = valid ? __ldg(hp + k8 + kc) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int kc = 0; kc < 8; ++kc) stage_transposed(sA, k8 + kc, tid, hv[kc]);
         }
-        for (int nn = 0; nn < kHid; ++nn) {
-            const __nv_bfloat16 dv = valid ? Dl[b * kHid + nn] : __float2bfloat16(0.f);
-            *reinterpret_cast<__nv_bfloat16 *>(sB + tc::core_offset(nn, tid, kChunkB)) = dv;
-        }
+#pragma unroll
+        for (int kc = 0; kc < 8; ++kc) stage_transposed(sB, kc, tid, dv[kc]);
         tc::fence_proxy_async_smem();
         tc::fence_before_sync();
         __syncthreads();
@@ -676,7 +722,7 @@ struct Surrogate {
     // training buffers
     int64_t cap_b = 0;
     int64_t *idx = nullptr;
-    __nv_bfloat16 *Xs = nullptr, *H = nullptr, *D[2] = {nullptr, nullptr};
+    __nv_bfloat16 *Xs = nullptr, *H = nullptr, *D[4] = {};
     // surface band of the gate
     uint32_t *band = nullptr;
     int band_res = 0;
@@ -687,7 +733,7 @@ void surrogate_free(Surrogate *s) {
     for (void *p : {(void *)s->params, (void *)s->m, (void *)s->v, (void *)s->grad, (void *)s->loss, (void *)s->gacc,
                     (void *)s->wbf,
                     (void *)s->err, (void *)s->idx, (void *)s->Xs, (void *)s->H, (void *)s->D[0], (void *)s->D[1],
-                    (void *)s->band})
+                    (void *)s->D[2], (void *)s->D[3], (void *)s->band})
         if (p) cudaFree(p);
     delete s;
 }
@@ -758,13 +804,13 @@ static gwn_status ensure_surrogate(gwn_mesh *m) {
 
 static gwn_status ensure_batch_buffers(Surrogate *s, int64_t nb) {
     if (nb <= s->cap_b) return GWN_OK;
-    for (void *p : {(void *)s->idx, (void *)s->Xs, (void *)s->H, (void *)s->D[0], (void *)s->D[1]})
+    for (void *p : {(void *)s->idx, (void *)s->Xs, (void *)s->H, (void *)s->D[0], (void *)s->D[1], (void *)s->D[2],
+                    (void *)s->D[3]})
         if (p) cudaFree(p);
     GWN_CUDA_TRY(cudaMalloc(&s->idx, sizeof(int64_t) * nb));
     GWN_CUDA_TRY(cudaMalloc(&s->Xs, sizeof(__nv_bfloat16) * nb * kIn));
     GWN_CUDA_TRY(cudaMalloc(&s->H, sizeof(__nv_bfloat16) * nb * kHid * 4));
-    GWN_CUDA_TRY(cudaMalloc(&s->D[0], sizeof(__nv_bfloat16) * nb * kHid));
-    GWN_CUDA_TRY(cudaMalloc(&s->D[1], sizeof(__nv_bfloat16) * nb * kHid));
+    for (auto &d : s->D) GWN_CUDA_TRY(cudaMalloc(&d, sizeof(__nv_bfloat16) * nb * kHid));
     s->cap_b = nb;
     return GWN_OK;
 }
@@ -785,21 +831,22 @@ static gwn_status mlp_fwd_bwd(Surrogate *s, const float *q, const float *target,
     const __nv_bfloat16 *Wbf[4] = {s->wbf, s->wbf + kHid * kIn, s->wbf + kHid * kIn + kHid * kHid,
                                    s->wbf + kHid * kIn + 2 * kHid * kHid};
     const int oW[4] = {oW1, oW2, oW3, oW4}, oB[4] = {oB1, oB2, oB3, oB4};
-    int cur = 0;
     const int64_t rows_per_cta = 1024;
     const unsigned dw_grid = (unsigned)((nb + rows_per_cta - 1) / rows_per_cta);
-    for (int l = 3; l >= 0; --l) {
+    DwLayers dw;
+    for (int l = 3; l >= 0; --l) {   // delta of layer l is in D[3 - l]
         const __nv_bfloat16 *Hprev = l == 0 ? s->Xs : s->H + (size_t)(l - 1) * nb * kHid;
-        const int Kl = l == 0 ? kIn : kHid;
-        k_mlp_back_dw<<<dw_grid, 128, 0, st>>>(Hprev, Kl, s->D[cur], nb, rows_per_cta, s->gacc + oW[l], s->err);
-        if (l > 0) {
-            k_mlp_back_dx<<<(unsigned)ntiles, 128, 0, st>>>(Wbf[l], s->D[cur], Hprev, nb, s->D[cur ^ 1],
+        dw.h[l] = Hprev;
+        dw.d[l] = s->D[3 - l];
+        dw.k[l] = l == 0 ? kIn : kHid;
+        dw.grad[l] = oW[l];
+        if (l > 0)
+            k_mlp_back_dx<<<(unsigned)ntiles, 128, 0, st>>>(Wbf[l], s->D[3 - l], Hprev, nb, s->D[4 - l],
                                                             s->gacc + oB[l], s->err);
-            cur ^= 1;
-        } else {
-            k_colsum64<<<(unsigned)ntiles, 128, 0, st>>>(s->D[cur], nb, s->gacc + oB[0]);
-        }
+        else
+            k_colsum64<<<(unsigned)ntiles, 128, 0, st>>>(s->D[3], nb, s->gacc + oB[0]);
     }
+    k_mlp_back_dw<<<dim3(dw_grid, 4), 128, 0, st>>>(dw, nb, rows_per_cta, s->gacc, s->err);
     k_grad_to_float<<<grid_for(kParams + 1, 256), 256, 0, st>>>(s->gacc, s->grad, s->loss);
     GWN_LAUNCH_CHECK("mlp forward/backward");
     return GWN_OK;
