@@ -796,21 +796,26 @@ __global__ void k_direct_reduce(const double *__restrict__ partial, int64_t n, i
 
 }  // namespace
 
-// Meshes whose walks k_chi may cut: above twice soup8's 57 expected node tests.
+// Where k_chi cuts walks: on meshes above twice soup8's 57 expected node tests, for calls
+// whose slowest walk holds the launch.  A warp of its own per long walk does more work in
+// all, so many queries are better left to fill the GPU.  Crossing counts on a 319k-triangle
+// height field, cut / whole: 1k queries 179 / 826 us, 16k 313 / 865, 32k 603 / 1020,
+// 100k 1265 / 1052, 1M 11.2 / 5.6 ms; on an 80k one 32k 454 / 434 us, 64k 366 / 259.
 constexpr double kLongWalk = 128.0;
-static bool long_walks(const gwn_mesh *m) {
-    return m->cfg.quantize_bits == 0 && m->walk_cost >= kLongWalk && m->nnodes > kWalkLimit;
+constexpr int64_t kLongWalkQueries = 32768;
+static bool long_walks(const gwn_mesh *m, int64_t n) {
+    return m->cfg.quantize_bits == 0 && m->walk_cost >= kLongWalk && m->nnodes > kWalkLimit && n <= kLongWalkQueries;
 }
 
 // rest_len, rest_q, rest_node: scratch for the long walks (a counter and n entries each),
-// used if long_walks(m)
+// used if long_walks(m, n)
 static gwn_status chi_on(const gwn_mesh *m, const float *q, int64_t n, int32_t *chi, unsigned long long *rest_len,
                          int32_t *rest_q, int32_t *rest_node, cudaStream_t s) {
     const unsigned blocks = grid_for(n, kChiThreads);
     if (m->cfg.quantize_bits) {
         k_chi<true, false><<<blocks, kChiThreads, 0, s>>>(q, n, m->nodes, m->nnodes, m->leaf_tri, chi, nullptr, nullptr,
                                                           nullptr, m->counters);
-    } else if (!long_walks(m)) {
+    } else if (!long_walks(m, n)) {
         k_chi<false, false><<<blocks, kChiThreads, 0, s>>>(q, n, m->nodes, m->nnodes, m->leaf_tri, chi, nullptr, nullptr,
                                                            nullptr, m->counters);
     } else {
@@ -829,7 +834,7 @@ static gwn_status chi_on(const gwn_mesh *m, const float *q, int64_t n, int32_t *
 gwn_status launch_chi(const gwn_mesh *m, const float *q, int64_t n, int32_t *chi, cudaStream_t s) {
     if (n <= 0) return GWN_OK;
     ProfScope prof("chi_traversal", s);
-    if (!long_walks(m)) return chi_on(m, q, n, chi, nullptr, nullptr, nullptr, s);
+    if (!long_walks(m, n)) return chi_on(m, q, n, chi, nullptr, nullptr, nullptr, s);
     unsigned long long *len = nullptr;
     GWN_CUDA_TRY(dev_alloc(&len, sizeof(unsigned long long) + 2 * sizeof(int32_t) * n, s));
     int32_t *rest_q = reinterpret_cast<int32_t *>(len + 1);
@@ -1031,7 +1036,7 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
     // (the FP64 list and w are free until the boundary sum: the long walks' list)
     gwn_status st = chi_on(m, q, n, chi_tmp, list_len, list, reinterpret_cast<int32_t *>(w), s);
     if (st != GWN_OK) return st;
-    if (long_walks(m)) GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
+    if (long_walks(m, n)) GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial, partial ? partial_cap : 0,
                          far, false, s);
     if (st != GWN_OK) return st;
