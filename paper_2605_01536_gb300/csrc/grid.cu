@@ -45,9 +45,8 @@ __device__ __forceinline__ int axis_bound(const float *__restrict__ a, int n, fl
 
 // One (triangle, column) test: the triangle's sign at the last cell it counts for.
 __device__ __forceinline__ void raster_test(const GridDev &g, float3 a, float3 b, float3 c, int si, int sj,
-                                            int32_t *__restrict__ diff, unsigned long long *__restrict__ counters) {
+                                            int32_t *__restrict__ diff, LocalCount ce, LocalCount cp) {
     const float px = __ldg(g.xs + si), py = __ldg(g.ys + sj);
-    unsigned long long *ce = &counters[CNT_EXACT_EDGE], *cp = &counters[CNT_EXACT_PLANE];
     const int s0 = edge_sos(px, py, a.x, a.y, b.x, b.y, ce);
     const int s1 = edge_sos(px, py, b.x, b.y, c.x, c.y, ce);
     if (s0 == 0 || s0 != s1) return;
@@ -110,6 +109,7 @@ __global__ void __launch_bounds__(kRasterThreads) k_grid_raster(GridDev g, const
     s_r[threadIdx.x][3] = incl - count;
     const int total = __shfl_sync(0xffffffffu, incl, 31);
     __syncwarp();
+    unsigned ce = 0, cp = 0;   // exact decisions
     for (int p = lane; p < total; p += 32) {
         int o = 0;   // the last triangle of the warp with at most p pairs before it
 #pragma unroll
@@ -119,8 +119,11 @@ __global__ void __launch_bounds__(kRasterThreads) k_grid_raster(GridDev g, const
         const float *T = s_t[w0 + o];
         const int q = p - r[3];
         raster_test(g, make_float3(T[0], T[1], T[2]), make_float3(T[3], T[4], T[5]), make_float3(T[6], T[7], T[8]),
-                    r[0] + q % r[2], r[1] + q / r[2], diff, counters);
+                    r[0] + q % r[2], r[1] + q / r[2], diff, LocalCount{&ce}, LocalCount{&cp});
     }
+    __syncwarp();
+    flush_count(ce, &counters[CNT_EXACT_EDGE]);
+    flush_count(cp, &counters[CNT_EXACT_PLANE]);
 }
 
 // The listed triangles: blocks (b, y) share triangle b's columns.
@@ -128,6 +131,7 @@ __global__ void __launch_bounds__(256) k_grid_big(GridDev g, const float4 *__res
                                                   const unsigned *__restrict__ n_big, int32_t *__restrict__ diff,
                                                   unsigned long long *__restrict__ counters) {
     const unsigned n = *n_big;
+    unsigned ce = 0, cp = 0;   // exact decisions
     for (unsigned k = blockIdx.x; k < n; k += gridDim.x) {
         const int64_t t = big[k];
         const float4 A = __ldg(tri + 3 * t), B = __ldg(tri + 3 * t + 1), C = __ldg(tri + 3 * t + 2);
@@ -138,8 +142,11 @@ __global__ void __launch_bounds__(256) k_grid_big(GridDev g, const float4 *__res
                   h = axis_bound(g.ys, g.ny, fmaxf(a.y, fmaxf(b.y, c.y)), true) - j0;
         const int64_t cols = (int64_t)w * h;
         for (int64_t q = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; q < cols; q += (int64_t)gridDim.y * blockDim.x)
-            raster_test(g, a, b, c, i0 + (int)(q % w), j0 + (int)(q / w), diff, counters);
+            raster_test(g, a, b, c, i0 + (int)(q % w), j0 + (int)(q / w), diff, LocalCount{&ce}, LocalCount{&cp});
     }
+    __syncwarp();
+    flush_count(ce, &counters[CNT_EXACT_EDGE]);
+    flush_count(cp, &counters[CNT_EXACT_PLANE]);
 }
 
 // Suffix sum up every column (one thread each, neighbouring columns in a warp): chi in

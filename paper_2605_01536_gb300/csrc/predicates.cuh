@@ -113,6 +113,7 @@ static __device__ __noinline__ int orient2d_exact32(float ax, float ay, float bx
     if (p1 == 0.f && d1 != 0.f && d2 != 0.f) ok = false;   // underflow to zero
     if (p2 == 0.f && d3 != 0.f && d4 != 0.f) ok = false;
     if (!ok) return 2;
+    if (e1 == 0.f && e2 == 0.f) return (p1 > p2) - (p1 < p2);   // a grid of few steps
     // Two-One-Diff(p1, e1, e2) = j + z0 + x0, then Two-One-Diff(j, z0, p2) = x3 + x2 + x1
     float i1, x0, j, z0, i2, x1, x3, x2;
     two_diff32(e1, e2, i1, x0);
@@ -125,20 +126,52 @@ static __device__ __noinline__ int orient2d_exact32(float ax, float ay, float bx
     return (x0 > 0.f) - (x0 < 0.f);
 }
 
+// Exact decisions are counted (gwn_counters): in a device counter, in a register, in a
+// warp's two shared words (no registers in the walk; the warp adds its sum once: the
+// degenerate precision workload, 500k queries, made 6.2M atomics on one address, half of
+// its crossing count), or not at all.
+struct LocalCount {
+    unsigned *n;
+};
+struct WarpCount {
+    unsigned *n;   // shared
+};
+__device__ __forceinline__ void count_exact(unsigned long long *c) {
+    if (c) atomicAdd(c, 1ull);
+}
+__device__ __forceinline__ void count_exact(LocalCount c) { ++*c.n; }
+__device__ __forceinline__ void count_exact(WarpCount c) { atomicAdd(c.n, 1u); }
+// every lane of the warp calls them
+__device__ __forceinline__ void flush_count(unsigned n, unsigned long long *counter) {
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(counter, (unsigned long long)n);
+}
+__device__ __forceinline__ void warp_count_begin(unsigned *w) {
+    if ((threadIdx.x & 31) < 2) w[threadIdx.x & 31] = 0;
+    __syncwarp();
+}
+__device__ __forceinline__ void warp_count_end(const unsigned *w, unsigned long long *counters) {
+    static_assert(CNT_EXACT_PLANE == CNT_EXACT_EDGE + 1, "the two words in this order");
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    if (lane < 2 && w[lane]) atomicAdd(&counters[CNT_EXACT_EDGE + lane], (unsigned long long)w[lane]);
+    __syncwarp();
+}
+
 __device__ __forceinline__ int sgn_diff(float a, float b) { return (a > b) - (a < b); }
 
 // Perturbed sign of the 2-D classification of q = (x, y) against the projected
 // edge p_i -> p_j:  (x + e1 - x_i)(y_i - y_j) + (y + e2 - y_i)(x_j - x_i), which
 // equals orient2d(p_i, p_j, q) plus the perturbation terms.  0 only when the
 // edge projects to a point.
-__device__ __forceinline__ int edge_sos(float x, float y, float xi, float yi, float xj, float yj,
-                                        unsigned long long *cnt) {
+template <class Count>
+__device__ __forceinline__ int edge_sos(float x, float y, float xi, float yi, float xj, float yj, Count cnt) {
     const float t1 = __fmul_rn(__fsub_rn(x, xi), __fsub_rn(yi, yj));
     const float t2 = __fmul_rn(__fsub_rn(y, yi), __fsub_rn(xj, xi));
     const float f = __fadd_rn(t1, t2);
     const float mag = fabsf(t1) + fabsf(t2);
     if (fabsf(f) > kFilter2 * mag && mag > kTiny) return f > 0.f ? 1 : -1;
-    if (cnt) atomicAdd(cnt, 1ull);
+    count_exact(cnt);
     int s = orient2d_exact32(xi, yi, xj, yj, x, y);
     if (s == 2) s = orient2d_exact(xi, yi, xj, yj, x, y);
     if (s) return s;
@@ -240,8 +273,8 @@ static __device__ __noinline__ int orient3d_exact32(float3 q, float3 a, float3 b
 // Perturbed sign of n . (a - q_eps), n = (b - a) x (c - a): the real part
 // det[a-q, b-q, c-q], then the e1, e2, e3 coefficients -n_x, -n_y, -n_z.
 // s_nz is the (already exact) sign of n_z.
-__device__ __forceinline__ int plane_sos(float3 q, float3 a, float3 b, float3 c, int s_nz,
-                                         unsigned long long *cnt) {
+template <class Count>
+__device__ __forceinline__ int plane_sos(float3 q, float3 a, float3 b, float3 c, int s_nz, Count cnt) {
     const float ux = __fsub_rn(a.x, q.x), uy = __fsub_rn(a.y, q.y), uz = __fsub_rn(a.z, q.z);
     const float vx = __fsub_rn(b.x, q.x), vy = __fsub_rn(b.y, q.y), vz = __fsub_rn(b.z, q.z);
     const float wx = __fsub_rn(c.x, q.x), wy = __fsub_rn(c.y, q.y), wz = __fsub_rn(c.z, q.z);
@@ -253,7 +286,7 @@ __device__ __forceinline__ int plane_sos(float3 q, float3 a, float3 b, float3 c,
     const float perm = fabsf(ux) * (fabsf(p1) + fabsf(p2)) + fabsf(uy) * (fabsf(p3) + fabsf(p4)) +
                        fabsf(uz) * (fabsf(p5) + fabsf(p6));
     if (fabsf(D) > kFilter3 * perm && perm > kTiny) return D > 0.f ? 1 : -1;
-    if (cnt) atomicAdd(cnt, 1ull);
+    count_exact(cnt);
     int s = orient3d_exact32(q, a, b, c);
     if (s == 2) s = orient3d_exact(q, a, b, c);
     if (s) return s;
@@ -270,8 +303,8 @@ __device__ __forceinline__ int plane_sos(float3 q, float3 a, float3 b, float3 c,
 // Signed crossing of the ray q_eps + t(0,0,1), t > 0, with triangle (a, b, c):
 // the common sign of the three perturbed edge classifications (= sign of n_z)
 // when the projected query is inside and the plane lies above it, else 0.
-__device__ __forceinline__ int tri_crossing(float3 q, float3 a, float3 b, float3 c,
-                                            unsigned long long *cnt_edge, unsigned long long *cnt_plane) {
+template <class Count>
+__device__ __forceinline__ int tri_crossing(float3 q, float3 a, float3 b, float3 c, Count cnt_edge, Count cnt_plane) {
     if (q.z >= fmaxf(a.z, fmaxf(b.z, c.z))) return 0;   // entirely at or below q_eps
     const int s0 = edge_sos(q.x, q.y, a.x, a.y, b.x, b.y, cnt_edge);
     const int s1 = edge_sos(q.x, q.y, b.x, b.y, c.x, c.y, cnt_edge);

@@ -106,7 +106,7 @@ __device__ __forceinline__ int branch_sos(float qx, float qy, float ax, float ay
         return edge_sos_q(qcoord(qx, qf->cx, qf->scale), qcoord(qy, qf->cy, qf->scale),
                           qcoord(ax, qf->cx, qf->scale), qcoord(ay, qf->cy, qf->scale),
                           qcoord(bx, qf->cx, qf->scale), qcoord(by, qf->cy, qf->scale));
-    return edge_sos(qx, qy, ax, ay, bx, by, nullptr);
+    return edge_sos(qx, qy, ax, ay, bx, by, (unsigned long long *)nullptr);
 }
 
 }  // namespace gwn

@@ -40,7 +40,7 @@ constexpr int64_t kSmallTris = 2048;   // leaves k_small tests one by one (64 pe
 // Where walks are short the test costs up to 13% (soup8, 57 nodes a walk), so it is
 // compiled in only for meshes whose expected walk is long.
 template <bool Fixed, bool Limited>
-__global__ void __launch_bounds__(256) k_chi(const float *__restrict__ q, int64_t n,
+__global__ void __launch_bounds__(256, 4) k_chi(const float *__restrict__ q, int64_t n,
                                              const BvhNode *__restrict__ nodes, int64_t nnodes,
                                              const float4 *__restrict__ tri, int32_t *__restrict__ chi,
                                              int32_t *__restrict__ rest_q, int32_t *__restrict__ rest_node,
@@ -52,14 +52,17 @@ __global__ void __launch_bounds__(256) k_chi(const float *__restrict__ q, int64_
         const float3 p = make_float3(q[3 * i], q[3 * i + 1], q[3 * i + 2]);
         chi[i] = chi_one_q(p, nodes, nnodes, tri, counters, qframe(counters));
     } else {   // the warp walks together (bvh_walk_up_warp): every lane stays to the end
+        __shared__ unsigned s_cnt[8][2];   // exact decisions of each warp
+        unsigned *cnt = s_cnt[threadIdx.x >> 5];
         const bool active = i < n;
         const float3 p = active ? make_float3(q[3 * i], q[3 * i + 1], q[3 * i + 2]) : make_float3(0.f, 0.f, 0.f);
         int c = 0, rest = -1;
+        warp_count_begin(cnt);
         const bool ok = bvh_walk_up_warp<Limited>(active, p, nodes, nnodes, tri, counters,
                                                   [&](int, float3 a, float3 b, float3 cc) {
-                                                      c += tri_crossing(p, a, b, cc, &counters[CNT_EXACT_EDGE],
-                                                                        &counters[CNT_EXACT_PLANE]);
+                                                      c += tri_crossing(p, a, b, cc, WarpCount{cnt}, WarpCount{cnt + 1});
                                                   }, &rest);
+        warp_count_end(cnt, counters);
         if (active) chi[i] = ok ? c : INT32_MIN;
         if (Limited && ok && rest >= 0) {
             const unsigned long long slot = atomicAdd(rest_len, 1ull);
@@ -77,17 +80,20 @@ __global__ void __launch_bounds__(128) k_chi_rest(const float *__restrict__ q, c
                                                   const unsigned long long *__restrict__ rest_len,
                                                   unsigned long long *__restrict__ counters) {
     __shared__ unsigned long long s_stack[4][kFrontierCap];
+    __shared__ unsigned s_cnt[4][2];   // exact decisions of each warp
+    unsigned *cnt = s_cnt[threadIdx.x >> 5];
     const unsigned long long len = *rest_len;
     for (unsigned long long k = (unsigned long long)blockIdx.x * 4 + (threadIdx.x >> 5); k < len;
          k += (unsigned long long)gridDim.x * 4) {
         const int64_t i = rest_q[k];
         const float3 p = make_float3(q[3 * i], q[3 * i + 1], q[3 * i + 2]);
         int c = 0;
+        warp_count_begin(cnt);
         const bool ok = bvh_frontier_warp(p, rest_node[k], 2, nodes, nnodes, tri, counters, s_stack[threadIdx.x >> 5],
                                           [&](int, float3 a, float3 b, float3 cc) {
-                                              c += tri_crossing(p, a, b, cc, &counters[CNT_EXACT_EDGE],
-                                                                &counters[CNT_EXACT_PLANE]);
+                                              c += tri_crossing(p, a, b, cc, WarpCount{cnt}, WarpCount{cnt + 1});
                                           });
+        warp_count_end(cnt, counters);
         c = __reduce_add_sync(0xffffffffu, c);
         if ((threadIdx.x & 31) == 0) chi[i] = ok ? chi[i] + c : INT32_MIN;
     }
@@ -427,6 +433,8 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
     extern __shared__ float4 s_pts[];
     __shared__ long long s_item;
     __shared__ int s_last;
+    __shared__ unsigned s_cnt[8][2];   // exact decisions of each warp
+    unsigned *cnt = s_cnt[threadIdx.x >> 5];
     constexpr int KQ = 2 * KP;
     while (true) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(head, 1ull);
@@ -447,14 +455,16 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
                 const int64_t g = tl.q_begin + (active ? i : 0);
                 const float3 p = active ? make_float3(q[3 * g], q[3 * g + 1], q[3 * g + 2]) : make_float3(0.f, 0.f, 0.f);
                 int c = 0;
+                warp_count_begin(cnt);
                 if (fixed) {
                     if (active) c = chi_one(p, mh.nodes, mh.nnodes, mh.tri, mh.counters);
                 } else {
                     const bool ok = bvh_walk_up_warp(active, p, mh.nodes, mh.nnodes, mh.tri, mh.counters,
                                                      [&](int, float3 a, float3 b, float3 cc) {
-                                                         c += tri_crossing(p, a, b, cc, &mh.counters[CNT_EXACT_EDGE],
-                                                                           &mh.counters[CNT_EXACT_PLANE]);
+                                                         c += tri_crossing(p, a, b, cc, WarpCount{cnt},
+                                                                           WarpCount{cnt + 1});
                                                      });
+                    warp_count_end(cnt, mh.counters);
                     if (!ok) c = INT32_MIN;
                 }
                 if (active) chi[g] = c;
