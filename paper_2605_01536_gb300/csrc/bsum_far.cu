@@ -374,26 +374,28 @@ bool far_pays(const gwn_mesh *m, int64_t n) {
     return m->far_sum && far_pays_gradient(m, n) && (double)n * direct_cost(m) >= 5e9;
 }
 
-gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
-                               uint8_t *label, bool classify, bool running, int32_t *list,
-                               unsigned long long *list_len, unsigned *listed, double *partial_buf,
-                               int64_t partial_cap, cudaStream_t s) {
-    const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
+// One walk is a serial chain of about 600 nodes: split it over the subtrees until there
+// are 320 blocks per SM (soup8, 200k queries: unsplit 4.0 ms, 16 parts 2.6, 64 parts 2.3;
+// 2M queries: 4 parts 11.4, 64 parts 11.5)
+int64_t far_parts(const gwn_mesh *m, int64_t n) {
     const int64_t blocks = (n + kFarThreads * 2 - 1) / (kFarThreads * 2);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // one walk is a serial chain of about 600 nodes: split it over the subtrees until
-    // there are 320 blocks per SM (soup8, 200k queries: unsplit 4.0 ms, 16 parts 2.6,
-    // 64 parts 2.3; 2M queries: 4 parts 11.4, 64 parts 11.5)
-    int64_t split = (320 * (int64_t)(sms > 0 ? sms : 148) + blocks - 1) / blocks;
-    split = std::max<int64_t>(1, std::min<int64_t>(split, m->far_nroots));
-    if (partial_cap >= 0) split = std::max<int64_t>(1, std::min<int64_t>(split, partial_cap / n));
-    double *partial = nullptr;
-    if (split > 1) {
-        if (partial_cap >= 0) partial = partial_buf;
-        else GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * split * n, s));
-    }
+    const int64_t parts = (320 * (int64_t)(sms > 0 ? sms : 148) + blocks - 1) / blocks;
+    return std::max<int64_t>(1, std::min<int64_t>(parts, m->far_nroots));
+}
+
+gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
+                               uint8_t *label, bool classify, bool running, int32_t *list,
+                               unsigned long long *list_len, unsigned *listed, double *partial_buf,
+                               int64_t call_n, cudaStream_t s) {
+    const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
+    const int64_t blocks = (n + kFarThreads * 2 - 1) / (kFarThreads * 2);
+    const int64_t split = far_parts(m, call_n);
+    double *partial = split > 1 ? partial_buf : nullptr;
+    const bool own = split > 1 && !partial_buf;
+    if (own) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * split * n, s));
     const dim3 grid((unsigned)blocks, (unsigned)split);
 #define GWN_FAR(R)                                                                                                    \
     k_boundary_far<R><<<grid, kFarThreads, 0, s>>>(q, n, m->far_nodes, m->far_roots, m->far_nroots, partial,           \
@@ -405,7 +407,7 @@ gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, con
     note_launches(1);
     if (partial) {
         launch_boundary_combine(partial, n, (int)split, chi, w, label, classify, margin, list, list_len, listed, s);
-        if (partial_cap < 0) cudaFreeAsync(partial, s);
+        if (own) cudaFreeAsync(partial, s);
     }
     GWN_LAUNCH_CHECK("k_boundary_far");
     return GWN_OK;

@@ -235,7 +235,10 @@ bool far_pays_gradient(const gwn_mesh *m, int64_t n);
 gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                uint8_t *label, bool classify, bool running, int32_t *list,
                                unsigned long long *list_len, unsigned *listed, double *partial_buf,
-                               int64_t partial_cap, cudaStream_t s);
+                               int64_t call_n, cudaStream_t s);
+// Parts a call of n queries splits the boundary into (partial sums: n doubles a part)
+int64_t far_parts(const gwn_mesh *m, int64_t n);
+int64_t boundary_parts(const gwn_mesh *m, int64_t n, bool far);
 // query.cu: w = chi + (sum over chunks, in order) / 2pi of partial [chunks][n], then the labels
 void launch_boundary_combine(const double *partial, int64_t n, int chunks, const int32_t *chi, float *w,
                              uint8_t *label, bool classify, float margin, int32_t *list,
@@ -263,7 +266,7 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
 // the classify sequence on caller-provided scratch; allocates nothing
 gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w,
                                       int32_t *chi_tmp, int32_t *list, unsigned long long *list_len,
-                                      unsigned *listed, double *partial, int64_t partial_cap, bool far, cudaStream_t s);
+                                      unsigned *listed, double *partial, int64_t call_n, bool far, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Batched evaluation of many meshes (one persistent launch over a work queue).

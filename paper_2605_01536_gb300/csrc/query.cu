@@ -889,50 +889,62 @@ void launch_boundary_combine(const double *partial, int64_t n, int chunks, const
     note_launches(1);
 }
 
+// The edges (with triangle loops apart: the other edges and two halves per triangle) that
+// the direct boundary sum splits into parts
+static bool split_triangles(const gwn_mesh *m, bool cond, bool plain) {
+    const int tile = m->cfg.boundary_tile > 0 ? m->cfg.boundary_tile : 512;
+    return cond && !plain && m->n_tri_loops > 0 && tile >= 64;
+}
+static int64_t edge_points(const gwn_mesh *m, bool split) {
+    const int64_t npts = split ? m->n_rest : m->npts;
+    return (npts > 0 ? npts - 1 : 0) + 2 * (split ? m->n_tri_loops : 0);
+}
+
+// Into how many parts a call of n queries splits them when the query tiles alone cannot
+// fill the GPU.  A function of the mesh and n only: a query's FP32 groups, and with them
+// the bits of w, follow it (the slices of gwn_classify_static pass the whole call's n).
+// 48 blocks per SM: a grid of 1.6 waves, 500k queries x 797 points, took 575 us instead of
+// 490, 100k queries 123 instead of 87, and near triangle loops make blocks uneven; the
+// surrogate's labels keep 8, and with it their bits.
+static int64_t direct_parts(const gwn_mesh *m, int64_t n, int kp, bool cond, bool plain) {
+    const int tile = m->cfg.boundary_tile > 0 ? m->cfg.boundary_tile : 512;
+    const int64_t per_block = kBsumThreads * 2 * kp, qblocks = (n + per_block - 1) / per_block;
+    const int64_t nedge_pts = edge_points(m, split_triangles(m, cond, plain));
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int64_t parts = ((plain ? 8 : 48) * (int64_t)(sms > 0 ? sms : 148) + qblocks - 1) / qblocks;
+    // (a part of 128 points still pays for its partial sums: 64 queries against
+    // 9.8k edges take 47 us instead of 200 us with parts of 1024 points)
+    const int64_t min_part = n < kOrderMinQueries || !plain ? std::min<int64_t>(128, 2 * tile) : 2 * tile;
+    parts = std::max<int64_t>(1, std::min<int64_t>(parts, (nedge_pts + min_part - 1) / min_part));
+    return std::min<int64_t>(parts, 65535);
+}
+
 template <int KP, bool Cond = false, bool Running = false>
 static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                  uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                 unsigned *listed, double *partial_buf, int64_t partial_cap, bool plain,
+                                 unsigned *listed, double *partial_buf, int64_t call_n, bool plain,
                                  cudaStream_t s) {
     const int tile = m->cfg.boundary_tile > 0 ? m->cfg.boundary_tile : 512;
     const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
     const int64_t per_block = kBsumThreads * 2 * KP;
     const int64_t qblocks = (n + per_block - 1) / per_block;
     // triangle loops as one term each (tri_accumulate; the FP64 test of their edges needs Cond)
-    const bool split = Cond && !plain && m->n_tri_loops > 0 && tile >= 64;
+    const bool split = split_triangles(m, Cond, plain);
     const float4 *pts = split ? m->rest_pts : m->bpts;
     const int64_t npts = split ? m->n_rest : m->npts, ntri = split ? m->n_tri_loops : 0;
-    const int64_t nedge_pts = (npts > 0 ? npts - 1 : 0) + 2 * ntri;
+    const int64_t nedge_pts = edge_points(m, split);
     const size_t smem = bsum_smem(KP, tile, Cond, ntri > 0);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_boundary_sum<KP, Cond, Running>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // split the boundary into chunks when the query tiles alone cannot fill the GPU
-    // (48 blocks per SM: a grid of 1.6 waves, 500k queries x 797 points, took 575 us instead
-    // of 490, 100k queries 123 instead of 87, and near triangle loops make blocks uneven;
-    // the surrogate's labels keep 8, and with it their bits)
-    int64_t chunks = ((plain ? 8 : 48) * (int64_t)(sms > 0 ? sms : 148) + qblocks - 1) / qblocks;
-    // (a chunk of 128 points still pays for its partial sums: 64 queries against
-    // 9.8k edges take 47 us instead of 200 us with chunks of 1024 points)
-    const int64_t min_chunk = n < kOrderMinQueries || !plain ? std::min<int64_t>(128, 2 * tile) : 2 * tile;
-    chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (nedge_pts + min_chunk - 1) / min_chunk));
-    if (partial_cap >= 0) chunks = std::min<int64_t>(chunks, partial_cap / n);   // caller-provided room
-    chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, 65535));
+    const int64_t chunks = direct_parts(m, call_n, KP, Cond, plain);
     int64_t chunk_len = chunks > 1 ? (nedge_pts + chunks - 1) / chunks : std::max<int64_t>(nedge_pts, 1);
     if (ntri > 0) chunk_len += chunk_len & 1;   // whole triangles
-    double *partial = nullptr;
-    bool own = false;
-    if (chunks > 1) {
-        if (partial_cap >= 0) {
-            partial = partial_buf;
-        } else {
-            GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * chunks * n, s));
-            own = true;
-        }
-    }
+    double *partial = chunks > 1 ? partial_buf : nullptr;
+    const bool own = chunks > 1 && !partial_buf;
+    if (own) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * chunks * n, s));
     dim3 grid((unsigned)qblocks, (unsigned)chunks);
     k_boundary_sum<KP, Cond, Running><<<grid, kBsumThreads, smem, s>>>(q, n, pts, npts, tile,
                                                                       reinterpret_cast<const TriLoop *>(m->tri_loops),
@@ -957,20 +969,20 @@ static bool group_test_running(const gwn_mesh *m) {
 }
 
 // The boundary sum with the scratch it needs provided: list (n entries), a
-// zeroed list_len and zeroed listed bits (n / 32 words, rounded up); the chunk
-// partials in partial_buf (room for partial_cap doubles), or allocated as
-// needed when partial_cap < 0.
+// zeroed list_len and zeroed listed bits (n / 32 words, rounded up); the parts' partial
+// sums in partial_buf (n times boundary_parts(m, call_n, far) doubles), or allocated as
+// needed when it is null.  call_n: the queries of the whole call.
 static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
                                   uint8_t *label, bool classify, int32_t *list, unsigned long long *list_len,
-                                  unsigned *listed, double *partial_buf, int64_t partial_cap, bool far,
+                                  unsigned *listed, double *partial_buf, int64_t call_n, bool far,
                                   bool plain, cudaStream_t s) {
     const int kq = m->cfg.queries_per_thread > 0 ? m->cfg.queries_per_thread : 4;
     ProfScope prof("boundary_sum", s);
     const bool running = group_test_running(m);
     if (far)
-        return launch_boundary_far(m, q, n, chi, w, label, classify, running, list, list_len, listed, partial_buf, partial_cap, s);
+        return launch_boundary_far(m, q, n, chi, w, label, classify, running, list, list_len, listed, partial_buf, call_n, s);
 #define GWN_BSUM(KP, C, R) \
-    launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, partial_cap, plain, s)
+    launch_bsum_kp<KP, C, R>(m, q, n, chi, w, label, classify, list, list_len, listed, partial_buf, call_n, plain, s)
     if (m->cfg.fp64_cancel >= 0) {   // the default: cancelling terms in FP64
         const bool small = kq == 1 || kq == 2;   // 8 queries per thread: the queue holds 2-bit slots
         if (running) return small ? GWN_BSUM(1, true, true) : GWN_BSUM(2, true, true);
@@ -983,6 +995,13 @@ static gwn_status boundary_sum_on(const gwn_mesh *m, const float *q, int64_t n, 
         default: return running ? GWN_BSUM(2, false, true) : GWN_BSUM(2, false, false);
     }
 #undef GWN_BSUM
+}
+
+int64_t boundary_parts(const gwn_mesh *m, int64_t n, bool far) {
+    if (far) return far_parts(m, n);
+    const int kq = m->cfg.queries_per_thread > 0 ? m->cfg.queries_per_thread : 4;
+    const bool cond = m->cfg.fp64_cancel >= 0;
+    return direct_parts(m, n, kq <= 2 ? 1 : (kq == 8 && !cond ? 4 : 2), cond, false);
 }
 
 gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n, const int32_t *chi, float *w,
@@ -1025,7 +1044,7 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
         GWN_CUDA_TRY(dev_alloc(&list_len, sizeof(unsigned long long), s));
         GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
     }
-    gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, -1,
+    gwn_status st = boundary_sum_on(m, q, n, chi, w, label, classify, list, list_len, listed, nullptr, n,
                                     order == SumOrder::kSpatial && far_pays(m, n), order == SumOrder::kDirect, s);
     if (st == GWN_OK && own_list) st = launch_fp64_fix_list(m, q, chi, w, nullptr, list, list_len, s);
     cudaFreeAsync(listed, s);
@@ -1038,19 +1057,18 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
 
 // The classify sequence on caller-provided scratch (allocates nothing): chi_tmp
 // [n] int32, list [n] int32, list_len one zeroed counter, listed (n + 31) / 32
-// zeroed words, partial room for partial_cap doubles (the boundary sum is split
-// into at most partial_cap / n point chunks; fewer than two means no split).
+// zeroed words, partial n times boundary_parts(m, call_n, far) doubles (unused where
+// that is 1), call_n the queries of the whole call.
 gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w,
                                       int32_t *chi_tmp, int32_t *list, unsigned long long *list_len,
-                                      unsigned *listed, double *partial, int64_t partial_cap, bool far,
+                                      unsigned *listed, double *partial, int64_t call_n, bool far,
                                       cudaStream_t s) {
     if (n <= 0) return GWN_OK;
     // (the FP64 list and w are free until the boundary sum: the long walks' list)
     gwn_status st = chi_on(m, q, n, chi_tmp, list_len, list, reinterpret_cast<int32_t *>(w), s);
     if (st != GWN_OK) return st;
     if (long_walks(m, n)) GWN_CUDA_TRY(cudaMemsetAsync(list_len, 0, sizeof(unsigned long long), s));
-    st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial, partial ? partial_cap : 0,
-                         far, false, s);
+    st = boundary_sum_on(m, q, n, chi_tmp, w, label, true, list, list_len, listed, partial, call_n, far, false, s);
     if (st != GWN_OK) return st;
     return launch_fp64_fix_list(m, q, chi_tmp, w, label, list, list_len, s);
 }

@@ -44,15 +44,23 @@ gwn_status scratch_address(int dev, unsigned char **out) {
 }
 
 
-// Queries per slice of an ordered call: 29.2 bytes of scratch each and 1 MiB of cell
-// counts (an order over fewer than 2^20 queries has at most 64^3 cells).
+// Queries per slice of an ordered call, at most: an order over fewer than 2^20 queries has
+// at most 64^3 cells.
 constexpr int64_t kSlice = (int64_t(1) << 20) - 256;
+// What a slice of n queries needs: 29.125 bytes a query and 1 MiB of cell counts (unordered
+// 12.125), with 8 bytes a query and part of the boundary, as many parts as the whole call
+// has on gwn_classify's path (so that w is the same to the bit), and the roundings.
+int64_t slice_queries(bool ordered, int64_t parts) {
+    const size_t bits = (ordered ? 29 * 8 : 12 * 8) + 1 + (parts > 1 ? 64 * (size_t)parts : 0);
+    const size_t room = kScratchBytes - kHeader - 1024 - (ordered ? gwn::order_cells_bytes(kSlice) : 0);
+    return std::min<int64_t>(kSlice, (int64_t)(room * 8 / bits));
+}
 
 // layout: [counter | chi n x int32 | list n x int32 | w n x float | listed (n + 31) / 32 x uint32 |
 //          ordered: perm n x uint32 | queries n x 12 | label n | cell counts || FP64 partials ...]
 // (the ranks of the order share the crossing numbers' place)
 gwn_status run_slice(const gwn_mesh *m, const float *q, int64_t n, uint8_t *label, float *w, bool ordered, bool far,
-                     unsigned char *base, cudaStream_t s) {
+                     int64_t call_n, int64_t parts, unsigned char *base, cudaStream_t s) {
     auto *len = reinterpret_cast<unsigned long long *>(base);
     auto *chi = reinterpret_cast<int32_t *>(base + kHeader);
     auto *list = chi + n;
@@ -65,17 +73,17 @@ gwn_status run_slice(const gwn_mesh *m, const float *q, int64_t n, uint8_t *labe
     uint8_t *ls = reinterpret_cast<uint8_t *>(cells) + (ordered ? gwn::order_cells_bytes(n) : 0);
     size_t used = ordered ? (size_t)(ls + n - base) : (size_t)(reinterpret_cast<unsigned char *>(perm) - base);
     used = (used + 255) & ~size_t(255);
-    if (used > kScratchBytes) return gwn::set_error(GWN_ERR_INVALID_ARG, "gwn_classify_static: slice beyond the scratch");
+    const size_t sums = parts > 1 ? sizeof(double) * (size_t)(parts * n) : 0;
+    if (used + sums > kScratchBytes) return gwn::set_error(GWN_ERR_INVALID_ARG, "gwn_classify_static: slice beyond the scratch");
     double *partial = reinterpret_cast<double *>(base + used);
-    const int64_t partial_cap = (int64_t)((kScratchBytes - used) / sizeof(double));
     GWN_CUDA_TRY(cudaMemsetAsync(len, 0, sizeof(unsigned long long), s));
     GWN_CUDA_TRY(cudaMemsetAsync(listed, 0, sizeof(unsigned) * words, s));
     if (!ordered)
-        return gwn::launch_classify_on_scratch(m, q, n, label, w ? w : ws, chi, list, len, listed, partial, partial_cap,
+        return gwn::launch_classify_on_scratch(m, q, n, label, w ? w : ws, chi, list, len, listed, partial, call_n,
                                                false, s);
     gwn_status st = gwn::order_queries_on(m, q, n, reinterpret_cast<uint32_t *>(chi), perm, qs, cells, s);
     if (st == GWN_OK)
-        st = gwn::launch_classify_on_scratch(m, qs, n, ls, ws, chi, list, len, listed, partial, partial_cap, far, s);
+        st = gwn::launch_classify_on_scratch(m, qs, n, ls, ws, chi, list, len, listed, partial, call_n, far, s);
     if (st == GWN_OK) st = gwn::scatter_results(perm, n, ws, w, nullptr, nullptr, ls, label, s);
     return st;
 }
@@ -116,9 +124,11 @@ extern "C" gwn_status gwn_classify_static(const gwn_mesh *m, const float *q, int
             // Large calls run in spatial order like gwn_classify's, in slices that fit the
             // scratch (an order over the slice serves as well); small ones as they come.
             const bool ordered = n >= gwn::kOrderMinQueries, far = ordered && gwn::far_pays(m, n);
-            for (int64_t at = 0; at < n && st == GWN_OK; at += kSlice)
-                st = run_slice(m, q + 3 * at, std::min<int64_t>(kSlice, n - at), label + at,
-                               w_or_null ? w_or_null + at : nullptr, ordered, far, base, s);
+            const int64_t parts = gwn::boundary_parts(m, n, far), most = slice_queries(ordered, parts);
+            const int64_t slices = (n + most - 1) / most, slice = (n + slices - 1) / slices;
+            for (int64_t at = 0; at < n && st == GWN_OK; at += slice)
+                st = run_slice(m, q + 3 * at, std::min<int64_t>(slice, n - at), label + at,
+                               w_or_null ? w_or_null + at : nullptr, ordered, far, n, parts, base, s);
         }
     }
     if (prev >= 0 && prev != m->device) cudaSetDevice(prev);
