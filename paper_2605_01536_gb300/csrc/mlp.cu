@@ -83,6 +83,15 @@ constexpr int kSmemH = kSmemX;
 constexpr int kSmemBias = kSmemX + 128 * kIn * 2;           // b1..b4, w5 (5 x 64 floats) + b5
 constexpr int kSmemFwd = kSmemBias + (5 * kHid + 4) * 4;
 
+// k_mlp_infer: the weights, the biases, then a feature buffer per group, of 112 features
+// (7 MMA steps hold the 99) and later its activations
+constexpr int kInferIn = 112;
+constexpr int kInferGroups = 6;
+constexpr int kSmemInferBias = 2048;                        // (5 x 64 + 1) floats, then to the next KB
+constexpr int kSmemGroup = 128 * kInferIn * 2;
+constexpr int kSmemInfer(int groups) { return kSmemX + kSmemInferBias + groups * kSmemGroup; }
+static_assert(kInferIn >= kFeat && kInferIn % 16 == 0 && kSmemInfer(kInferGroups) <= 227 * 1024 - 1024, "fits an SM");
+
 __device__ __forceinline__ void store_row_bf16(unsigned char *sA, int r, const float *v, int K) {
     // 8 consecutive k of row r are one 16-byte chunk of a core matrix
     for (int kc = 0; kc < K / 8; ++kc) {
@@ -105,6 +114,7 @@ __device__ __forceinline__ float2 sincos_halfturns(float t) {
 
 // Features of one query written as BF16 into row r of the core-layout matrix
 // sX, eight at a time (one 16-byte store per core-matrix row chunk).
+template <int W = kIn>
 __device__ __forceinline__ void features_to_smem(float qx, float qy, float qz, const MlpDev &P, unsigned char *sX,
                                                  int r) {
     const float x[3] = {fmaf(qx, P.scale[0], P.offset[0]), fmaf(qy, P.scale[1], P.offset[1]),
@@ -112,7 +122,7 @@ __device__ __forceinline__ void features_to_smem(float qx, float qy, float qz, c
     float buf[8];
     float2 sc = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < kIn; ++i) {
+    for (int i = 0; i < W; ++i) {
         float v = 0.f;
         if (i < 3) {
             v = x[i];
@@ -130,7 +140,7 @@ __device__ __forceinline__ void features_to_smem(float qx, float qy, float qz, c
             __nv_bfloat162 p[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) p[t] = __floats2bfloat162_rn(buf[2 * t], buf[2 * t + 1]);
-            *reinterpret_cast<uint4 *>(sX + tc::core_offset(r, i - 7, kIn)) = *reinterpret_cast<uint4 *>(p);
+            *reinterpret_cast<uint4 *>(sX + tc::core_offset(r, i - 7, W)) = *reinterpret_cast<uint4 *>(p);
         }
     }
 }
@@ -170,12 +180,9 @@ __device__ __forceinline__ bool mma_layer(uint32_t tm, unsigned char *sA, unsign
     return true;
 }
 
-// Forward pass over queries (one thread per query row, 128 per tile, persistent
-// CTAs).  mode 0: inference + gate (label where |w_hat - 1/2| > margin, the query
-// lies outside the surface band and, when chi_gate is given, |w_hat - chi| <=
-// chi_tol; else the query goes to the fallback list); mode 1: training (gathered samples, stores
-// the features and activations, the loss, delta4 = dL/dz4 (ReLU mask applied),
-// and the gradients of w5 and b5); mode 2: the raw output w_hat for every query.
+// Forward pass of a training step (one thread per sample, 128 per tile, persistent
+// CTAs) over the gathered samples: stores the features and activations, the loss,
+// delta4 = dL/dz4 (ReLU mask applied), and the gradients of w5 and b5.
 // Gradients are summed across CTAs in 64-bit fixed point (units of 2^-40):
 // integer addition does not depend on the order in which CTAs arrive, so a
 // training run is bit-reproducible for a given seed (FP32 atomics were not).
@@ -186,12 +193,7 @@ __device__ __forceinline__ void grad_add(long long *acc, float g) {
 }
 
 __global__ void __launch_bounds__(128) k_mlp_forward(
-    MlpDev P, const float *__restrict__ q, int64_t n, int mode, float margin,
-    // inference outputs
-    float *__restrict__ w_out, uint8_t *__restrict__ label, int32_t *__restrict__ fb_list,
-    unsigned long long *__restrict__ fb_len, const int32_t *__restrict__ chi_gate, float chi_tol,
-    // training
-    const int64_t *__restrict__ sample_idx, const float *__restrict__ target, __nv_bfloat16 *__restrict__ Xs,
+    MlpDev P, const float *__restrict__ q, int64_t n, const int64_t *__restrict__ sample_idx, const float *__restrict__ target, __nv_bfloat16 *__restrict__ Xs,
     __nv_bfloat16 *__restrict__ H, __nv_bfloat16 *__restrict__ D4, long long *__restrict__ grad,
     long long *__restrict__ loss,
     float inv_batch, unsigned *err) {
@@ -229,17 +231,14 @@ __global__ void __launch_bounds__(128) k_mlp_forward(
     for (int64_t tile = blockIdx.x; tile < ntiles && alive; tile += gridDim.x) {
         const int64_t row = tile * 128 + tid;
         const bool valid = row < n;
-        int64_t src = row;
-        if (mode == 1 && valid) src = sample_idx[row];
+        const int64_t src = valid ? sample_idx[row] : 0;
         const float qx = valid ? q[3 * src] : 0.f, qy = valid ? q[3 * src + 1] : 0.f,
                     qz = valid ? q[3 * src + 2] : 0.f;
-        {
-            features_to_smem(qx, qy, qz, P, sX, tid);
-            if (mode == 1 && valid)
-                for (int kc = 0; kc < kIn / 8; ++kc)
-                    *reinterpret_cast<uint4 *>(Xs + (size_t)row * kIn + kc * 8) =
-                        *reinterpret_cast<const uint4 *>(sX + tc::core_offset(tid, kc * 8, kIn));
-        }
+        features_to_smem(qx, qy, qz, P, sX, tid);
+        if (valid)
+            for (int kc = 0; kc < kIn / 8; ++kc)
+                *reinterpret_cast<uint4 *>(Xs + (size_t)row * kIn + kc * 8) =
+                    *reinterpret_cast<const uint4 *>(sX + tc::core_offset(tid, kc * 8, kIn));
         unsigned char *sW[4] = {sW1, sW2, sW3, sW4};
         float h[kHid];
         for (int l = 0; l < 4 && alive; ++l) {
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(128) k_mlp_forward(
             for (int j = 0; j < kHid; ++j) h[j] = fmaxf(h[j] + sB[l * kHid + j], 0.f);
             // the MMA that read sH has completed: overwrite it with this layer's output
             store_row_bf16(sH, tid, h, kHid);
-            if (mode == 1 && valid) {
+            if (valid) {
 #pragma unroll
                 for (int kc = 0; kc < kHid / 8; ++kc) {
                     __nv_bfloat162 p[4];
@@ -265,56 +264,161 @@ __global__ void __launch_bounds__(128) k_mlp_forward(
         float y = sB[5 * kHid];
 #pragma unroll
         for (int j = 0; j < kHid; ++j) y = fmaf(sB[4 * kHid + j], h[j], y);
-        if (mode == 2) {
-            if (valid) w_out[row] = y;
-        } else if (mode == 0) {
-            if (valid) {
-                if (fabsf(y - 0.5f) > margin && !in_band(P, qx, qy, qz) &&
-                    (!chi_gate || fabsf(y - (float)chi_gate[row]) <= chi_tol)) {
-                    w_out[row] = y;
-                    label[row] = y > 0.5f ? 1 : 0;
-                } else {
-                    const unsigned long long slot = atomicAdd(fb_len, 1ull);
-                    fb_list[slot] = (int32_t)row;
-                }
+        // dL/dy for L = mean (y - t)^2; dL/dh4 = dy * w5 (the ReLU mask of h4 is applied with h4 > 0)
+        const float dy = valid ? 2.f * (y - target[src]) * inv_batch : 0.f;
+        float d4[kHid];
+#pragma unroll
+        for (int j = 0; j < kHid; ++j) d4[j] = h[j] > 0.f ? dy * sB[4 * kHid + j] : 0.f;
+        if (valid) {
+#pragma unroll
+            for (int kc = 0; kc < kHid / 8; ++kc) {
+                __nv_bfloat162 p[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(d4[kc * 8 + 2 * i], d4[kc * 8 + 2 * i + 1]);
+                *reinterpret_cast<uint4 *>(D4 + (size_t)row * kHid + kc * 8) = *reinterpret_cast<uint4 *>(p);
             }
-        } else {
-            // dL/dy for L = mean (y - t)^2; dL/dh4 = dy * w5 (the ReLU mask of h4 is applied with h4 > 0)
-            const float dy = valid ? 2.f * (y - target[src]) * inv_batch : 0.f;
-            float d4[kHid];
-#pragma unroll
-            for (int j = 0; j < kHid; ++j) d4[j] = h[j] > 0.f ? dy * sB[4 * kHid + j] : 0.f;
-            if (valid) {
-#pragma unroll
-                for (int kc = 0; kc < kHid / 8; ++kc) {
-                    __nv_bfloat162 p[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(d4[kc * 8 + 2 * i], d4[kc * 8 + 2 * i + 1]);
-                    *reinterpret_cast<uint4 *>(D4 + (size_t)row * kHid + kc * 8) = *reinterpret_cast<uint4 *>(p);
-                }
-            }
-            // gradients of w5, b5 and the loss: warp sums, then one atomic per block
-            const float e = valid ? (y - target[src]) : 0.f;
-#pragma unroll
-            for (int j = 0; j < kHid + 2; ++j) {
-                float g = j < kHid ? dy * h[j] : (j == kHid ? dy : e * e * inv_batch);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-                if (lane == 0) red[warp][j] = g;
-            }
-            __syncthreads();
-            if (tid < kHid + 2) {
-                const float g = red[0][tid] + red[1][tid] + red[2][tid] + red[3][tid];
-                if (tid < kHid) grad_add(&grad[oW5 + tid], g);
-                else if (tid == kHid) grad_add(&grad[oB5], g);
-                else grad_add(loss, g);
-            }
-            __syncthreads();
         }
+        // gradients of w5, b5 and the loss: warp sums, then one atomic per block
+        const float e = valid ? (y - target[src]) : 0.f;
+#pragma unroll
+        for (int j = 0; j < kHid + 2; ++j) {
+            float g = j < kHid ? dy * h[j] : (j == kHid ? dy : e * e * inv_batch);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+            if (lane == 0) red[warp][j] = g;
+        }
+        __syncthreads();
+        if (tid < kHid + 2) {
+            const float g = red[0][tid] + red[1][tid] + red[2][tid] + red[3][tid];
+            if (tid < kHid) grad_add(&grad[oW5 + tid], g);
+            else if (tid == kHid) grad_add(&grad[oB5], g);
+            else grad_add(loss, g);
+        }
+        __syncthreads();
     }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tm, 64);
+}
+
+// Network outputs of queries: w_hat raw (label null), or gated (label where |w_hat - 1/2|
+// > margin, the query lies outside the surface band and, when chi_gate is given, |w_hat -
+// chi| <= chi_tol; else the query goes to the fallback list).
+//
+// A tile of 128 queries is a serial chain (features, then MMA, wait, epilogue per layer)
+// and bound by its latency, so an SM wants many tiles in flight: G groups of 128 threads
+// work on tiles of their own, each with a feature buffer, 64 TMEM columns, an mbarrier
+// and a named barrier, over one copy of the weights.  Six groups (28 KB of features each,
+// 99 of them padded to 112 = 7 MMA steps instead of 8) fit where three CTAs with the
+// weights in each did: 16.8M queries 1.74 -> 1.21 ms (0.30 of the BF16 peak), a call of 1M
+// 151 -> 125 us.  Next bound: shared-memory traffic of operands and activations (about 1.8k
+// of a tile's 2.9k cycles).
+template <int G>
+__global__ void __launch_bounds__(128 * G) k_mlp_infer(MlpDev P, const float *__restrict__ q, int64_t n, float margin,
+                                                       float *__restrict__ w_out, uint8_t *__restrict__ label,
+                                                       int32_t *__restrict__ fb_list,
+                                                       unsigned long long *__restrict__ fb_len,
+                                                       const int32_t *__restrict__ chi_gate, float chi_tol,
+                                                       unsigned *err) {
+    constexpr int kCols = G == 1 ? 64 : (G <= 4 ? 256 : 512);   // TMEM columns: a power of two
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bars[G];
+    __shared__ uint32_t tmem_base;
+    const int group = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = tid >> 5;
+    const unsigned char *sW[4] = {smem + kSmemW1, smem + kSmemW2, smem + kSmemW3, smem + kSmemW4};
+    float *sB = reinterpret_cast<float *>(smem + kSmemX);
+    unsigned char *sX = smem + kSmemX + kSmemInferBias + group * kSmemGroup;
+    stage_matrix(smem + kSmemW1, P.wbf, kHid, kIn);
+    for (int l = 0; l < 3; ++l)
+        stage_matrix(smem + kSmemW2 + l * kHid * kHid * 2, P.wbf + kHid * kIn + l * kHid * kHid, kHid, kHid);
+    for (int i = threadIdx.x; i < kHid; i += blockDim.x) {
+        sB[i] = P.params[oB1 + i];
+        sB[kHid + i] = P.params[oB2 + i];
+        sB[2 * kHid + i] = P.params[oB3 + i];
+        sB[3 * kHid + i] = P.params[oB4 + i];
+        sB[4 * kHid + i] = P.params[oW5 + i];
+    }
+    if (threadIdx.x == 0) sB[5 * kHid] = P.params[oB5];
+    if (threadIdx.x < 32) tc::tmem_alloc(&tmem_base, kCols);
+    if (tid == 0) tc::mbar_init(&bars[group], 1);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tm = tmem_base + 64u * group;
+    uint32_t phase = 0;
+    bool alive = true;
+    const int64_t ntiles = (n + 127) / 128;
+    for (int64_t tile = blockIdx.x + (int64_t)gridDim.x * group; tile < ntiles && alive; tile += (int64_t)gridDim.x * G) {
+        const int64_t row = tile * 128 + tid;
+        const bool valid = row < n;
+        const float qx = valid ? q[3 * row] : 0.f, qy = valid ? q[3 * row + 1] : 0.f, qz = valid ? q[3 * row + 2] : 0.f;
+        features_to_smem<kInferIn>(qx, qy, qz, P, sX, tid);
+        float y = sB[5 * kHid];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            tc::fence_proxy_async_smem();
+            tc::fence_before_sync();
+            tc::group_sync(group + 1);
+            tc::fence_after_sync();
+            if (tid == 0) {
+                if (l == 0) tc::gemm_128x64_steps(tm, sX, kInferIn, sW[0], kIn, kInferIn / 16);
+                else tc::gemm_128x64(tm, sX, sW[l], kHid, false);
+                tc::mma_commit(&bars[group]);
+            }
+            // the decision must be the same in every thread of the group
+            alive = tc::group_and(group + 1, tc::mbar_wait(&bars[group], phase, kWaitPolls));
+            phase ^= 1u;
+            tc::fence_after_sync();
+            if (!alive) break;
+            // the MMA that read the buffer has completed: the activations take its place
+#pragma unroll
+            for (int c = 0; c < kHid; c += 32) {
+                float h[32];
+                tc::tmem_ld32(tm + ((uint32_t)(warp * 32) << 16) + c, h);
+                const float4 *b4 = reinterpret_cast<const float4 *>(sB + l * kHid + c);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4 b = b4[j];
+                    h[4 * j] = fmaxf(h[4 * j] + b.x, 0.f);
+                    h[4 * j + 1] = fmaxf(h[4 * j + 1] + b.y, 0.f);
+                    h[4 * j + 2] = fmaxf(h[4 * j + 2] + b.z, 0.f);
+                    h[4 * j + 3] = fmaxf(h[4 * j + 3] + b.w, 0.f);
+                }
+                if (l < 3) {
+#pragma unroll
+                    for (int kc = 0; kc < 32; kc += 8) {
+                        __nv_bfloat162 p[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) p[i] = __floats2bfloat162_rn(h[kc + 2 * i], h[kc + 2 * i + 1]);
+                        *reinterpret_cast<uint4 *>(sX + tc::core_offset(tid, c + kc, kHid)) =
+                            *reinterpret_cast<uint4 *>(p);
+                    }
+                } else {   // output layer (FP32 on the CUDA cores: a 64-wide dot product per query)
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) y = fmaf(sB[4 * kHid + c + j], h[j], y);
+                }
+            }
+            tc::fence_before_sync();
+        }
+        if (!alive) {
+            if (tid == 0) atomicOr(err, 1u);
+            break;
+        }
+        if (!valid) continue;
+        if (!label) {
+            w_out[row] = y;
+        } else if (fabsf(y - 0.5f) > margin && !in_band(P, qx, qy, qz) &&
+                   (!chi_gate || fabsf(y - (float)chi_gate[row]) <= chi_tol)) {
+            w_out[row] = y;
+            label[row] = y > 0.5f ? 1 : 0;
+        } else {
+            const unsigned long long slot = atomicAdd(fb_len, 1ull);
+            fb_list[slot] = (int32_t)row;
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x < 32) tc::tmem_dealloc(tmem_base, kCols);
 }
 
 // eight BF16 values of a 16-byte chunk as FP32
@@ -650,6 +754,26 @@ int sm_count() {
     return sms > 0 ? sms : 148;
 }
 
+// Up to three tiles per SM: a CTA each (calls of 100 to 58k queries take 47-50 us either
+// way, the latency of one tile and of the call).  More: one CTA per SM, its groups loop
+// over the tiles.
+void launch_infer(const MlpDev &P, const float *q, int64_t n, float margin, float *w, uint8_t *label, int32_t *list,
+                  unsigned long long *len, const int32_t *chi_gate, float chi_tol, unsigned *err, cudaStream_t st) {
+    const int64_t ntiles = (n + 127) / 128;
+    const int sms = sm_count();
+    if (ntiles <= 3 * sms) {
+        cudaFuncSetAttribute(k_mlp_infer<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInfer(1));
+        k_mlp_infer<1><<<(unsigned)ntiles, 128, kSmemInfer(1), st>>>(P, q, n, margin, w, label, list, len, chi_gate,
+                                                                     chi_tol, err);
+    } else {
+        constexpr int G = kInferGroups;
+        cudaFuncSetAttribute(k_mlp_infer<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInfer(G));
+        const unsigned grid = (unsigned)sms;
+        k_mlp_infer<G><<<grid, 128 * G, kSmemInfer(G), st>>>(P, q, n, margin, w, label, list, len, chi_gate, chi_tol,
+                                                             err);
+    }
+}
+
 bool g_freq_set[64] = {};
 
 gwn_status set_freq_table() {
@@ -823,9 +947,7 @@ static gwn_status mlp_fwd_bwd(Surrogate *s, const float *q, const float *target,
     cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFwd);
     const int64_t ntiles = (nb + 127) / 128;
     const int grid = (int)std::min<int64_t>(ntiles, 3 * sm_count());
-    k_mlp_forward<<<grid, 128, kSmemFwd, st>>>(P, q, nb, 1, 0.f, nullptr, nullptr, nullptr, nullptr, nullptr, 0.f,
-                                               s->idx, target,
-                                               s->Xs, s->H, s->D[0], s->gacc, s->gacc + kParams, 1.f / (float)nb,
+    k_mlp_forward<<<grid, 128, kSmemFwd, st>>>(P, q, nb, s->idx, target, s->Xs, s->H, s->D[0], s->gacc, s->gacc + kParams, 1.f / (float)nb,
                                                s->err);
     // layers 4, 3, 2: delta_{l-1} and the grads of W_l, b_l
     const __nv_bfloat16 *Wbf[4] = {s->wbf, s->wbf + kHid * kIn, s->wbf + kHid * kIn + kHid * kHid,
@@ -963,14 +1085,9 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
             return r0;
         }
     }
-    cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFwd);
     {
         ProfScope prof("surrogate_forward", st);
-        const int64_t ntiles = (n + 127) / 128;
-        const int grid = (int)std::min<int64_t>(ntiles, 3 * sm_count());
-        k_mlp_forward<<<grid, 128, kSmemFwd, st>>>(P, q, n, 0, s->cfg.margin, w, label, list, len, chi_all,
-                                                   s->cfg.chi_tol, nullptr, nullptr,
-                                                   nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, s->err);
+        launch_infer(P, q, n, s->cfg.margin, w, label, list, len, chi_all, s->cfg.chi_tol, s->err, st);
     }
     unsigned long long nfb = 0;
     GWN_CUDA_TRY(cudaMemcpyAsync(&nfb, len, sizeof(nfb), cudaMemcpyDeviceToHost, st));
@@ -1122,12 +1239,7 @@ gwn_status gwn_surrogate_predict(const gwn_mesh *m, const float *q, int64_t n, f
     DeviceScope dev_scope(m->device);
     cudaStream_t st = (cudaStream_t)stream;
     Surrogate *s = m->sur;
-    cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFwd);
-    const int64_t ntiles = (n + 127) / 128;
-    const int grid = (int)std::min<int64_t>(ntiles, 3 * sm_count());
-    k_mlp_forward<<<grid, 128, kSmemFwd, st>>>(mlp_dev(s), q, n, 2, 0.f, w_hat, nullptr, nullptr, nullptr, nullptr, 0.f,
-                                               nullptr,
-                                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, s->err);
+    launch_infer(mlp_dev(s), q, n, 0.f, w_hat, nullptr, nullptr, nullptr, nullptr, 0.f, s->err, st);
     GWN_LAUNCH_CHECK("surrogate predict");
     return check_err(s, st);
 }
@@ -1276,11 +1388,7 @@ gwn_status gwn_surrogate_calibrate(gwn_mesh *m, const float *samples, int64_t n,
     GWN_CUDA_TRY(dev_alloc(&hist, sizeof(unsigned long long) * kCalibBins, st));
     cudaMemsetAsync(len, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * kCalibBins, st);
-    cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFwd);
-    const int grid = (int)std::min<int64_t>((n + 127) / 128, 3 * sm_count());
-    k_mlp_forward<<<grid, 128, kSmemFwd, st>>>(mlp_dev(s), samples, n, 2, 0.f, w_hat, nullptr, nullptr, nullptr,
-                                               nullptr, 0.f, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                               nullptr, 0.f, s->err);
+    launch_infer(mlp_dev(s), samples, n, 0.f, w_hat, nullptr, nullptr, nullptr, nullptr, 0.f, s->err, st);
     gwn_status r;
     if ((r = launch_chi(m, samples, n, chi, st)) == GWN_OK &&
         (r = launch_boundary_sum_list(m, samples, n, chi, w, lab, true, list, len, SumOrder::kCaller, st)) == GWN_OK &&

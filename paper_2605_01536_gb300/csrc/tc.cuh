@@ -107,6 +107,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// the same, 32 columns
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // D[128][64] (TMEM, FP32) = A[128][K] x B[64][K]^T (both BF16, core-matrix
 // layout in shared memory), K a multiple of 16; issued by the calling thread.
 __device__ __forceinline__ void gemm_128x64(uint32_t d_tmem, const void *a_smem, const void *b_smem, int K,
@@ -120,6 +136,28 @@ __device__ __forceinline__ void gemm_128x64(uint32_t d_tmem, const void *a_smem,
         mma_bf16(d_tmem, ad, bd, idesc, (s > 0 || accumulate_first) ? 1u : 0u);
     }
 }
+
+// The same over the first 16 `steps` of K, A stored ka wide and B kb wide
+__device__ __forceinline__ void gemm_128x64_steps(uint32_t d_tmem, const void *a_smem, int ka, const void *b_smem, int kb,
+                                                  int steps) {
+    const uint32_t a0 = smem_u32(a_smem), b0 = smem_u32(b_smem);
+    constexpr uint32_t idesc = idesc_bf16_f32(128, 64);
+    for (int s = 0; s < steps; ++s)
+        mma_bf16(d_tmem, smem_desc(a0 + 256u * s, 128u, (uint32_t)ka * 16u),
+                 smem_desc(b0 + 256u * s, 128u, (uint32_t)kb * 16u), idesc, s > 0 ? 1u : 0u);
+}
+
+// AND of a predicate over the 128 threads that share named barrier `id`
+__device__ __forceinline__ bool group_and(int id, bool p) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred a, b;\n setp.ne.u32 a, %1, 0;\n bar.red.and.pred b, %2, 128, a;\n selp.u32 %0, 1, 0, b;\n}\n"
+        : "=r"(r)
+        : "r"((uint32_t)p), "r"(id)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
 }  // namespace tc
 }  // namespace gwn
