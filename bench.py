@@ -935,7 +935,7 @@ def run_surrogate_infer(args):
                 "config": {"workload": f"surrogate_infer: {WORKLOADS['surrogate_infer']}", "n_queries": n,
                            "l2": "flushed between steps (256 MB write); inputs 201 MB > L2"},
                 "roofline": {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                             "traffic": None, "kernel": "k_mlp_forward", "flop_per_query": flop_per_q,
+                             "traffic": None, "kernel": "k_mlp_infer", "flop_per_query": flop_per_q,
                              "algorithmic_bytes_per_query": 16},
                 "gpu_launches": args.steps, "clocks": clk}
         print(json.dumps(line), flush=True)
@@ -1290,7 +1290,7 @@ def step_roofline(roof, troof, step_ms):
     """The whole step against its roofline: the boundary sum's bound (the larger
     of its FP32 issue and SFU times) plus the crossing count's byte time at the
     HBM rate, over the measured step time."""
-    if not roof or "fp32_bound_ms" not in roof or roof["frac"] is None:
+    if not roof or "fp32_bound_ms" not in roof or roof.get("frac", 0.0) is None:
         return None
     a5 = max(roof["fp32_bound_ms"], roof.get("sfu_bound_ms", 0.0))
     a4 = troof["bytes_per_launch"] / (troof["peak"] * 1e9) * 1e3 if troof else 0.0
