@@ -76,7 +76,11 @@ enum {
 
 typedef struct gwn_mesh gwn_mesh;
 
-/* Tuning knobs; zero-initialise and set what you need (0 = default). */
+/* Tuning knobs; zero-initialise and set what you need (0 = default).  A nonzero
+ * queries_per_thread or boundary_tile, chain_boundary -1 and fp64_cancel
+ * -1 keep the boundary sum on the kernel that adds every edge; by default long boundaries
+ * are summed over a hierarchy with expansions of their distant pieces (truncated at 1e-7
+ * each) and small calls in one kernel. */
 typedef struct gwn_config {
     int32_t queries_per_thread;   /* boundary-sum kernel: queries held per thread (1,2,4,8) */
     int32_t boundary_tile;        /* boundary points staged in shared memory per step */
@@ -180,7 +184,8 @@ GWN_API gwn_status gwn_mesh_destroy(gwn_mesh *mesh);
  * times in its net direction; vertices are matched by index, not welded by
  * position), its chaining into closed loops, and a linear BVH over the
  * triangles (Morton codes of centroids, radix sort, Karras hierarchy, bottom-up
- * box refit, escape links for stackless traversal).  Replaces the paper's
+ * box refit, escape links for stackless traversal), and a hierarchy over the
+ * boundary where sampled queries would profit.  Replaces the paper's
  * Embree BVH (Sec. 5).  Idempotent.  Synchronises `stream` once to read the
  * boundary size.
  */
@@ -262,8 +267,9 @@ GWN_API gwn_status gwn_query_chi_visits(const gwn_mesh *mesh, const float *q, in
  * (x[i], y[j], z[k]) for i < nx, j < ny, k < nz; outputs are indexed
  * [(k * ny + j) * nx + i] (x fastest).  x, y, z are float32 arrays in host or
  * device memory (copied by the call); z must be non-decreasing; all
- * coordinates finite; nx * ny * nz <= 2^31 - 1.  One BVH walk per (x, y)
- * column replaces nz walks; each cell's crossing decision is the same exact,
+ * coordinates finite; nx * ny * nz <= 2^31 - 1.  Each triangle is
+ * rasterised once onto the (x, y) columns, whose running sums along z give every
+ * cell its count; each cell's crossing decision is the same exact,
  * perturbed predicate the per-query path evaluates at that point, so chi is
  * bit-identical to gwn_query_chi on the same points.  Both calls synchronise
  * `stream` once and require gwn_build_accel.
@@ -307,7 +313,8 @@ GWN_API gwn_status gwn_get_counters(gwn_mesh *mesh, gwn_counters *out, int reset
  * bit-identical to gwn_classify's on a mesh without a surrogate (each query's
  * arithmetic does not depend on the rest of the batch or its order).
  *   - Scratch: one 32 MiB file-scope device array per GPU that loads the
- *     library, held until the process exits; every call uses it.
+ *     library, held until the process exits; a call that needs more runs in
+ *     slices of the queries.
  *   - Limit: n <= 2,097,152 queries per call; larger n fails with
  *     GWN_ERR_INVALID_ARG.  q, label and w_or_null must be device memory of
  *     the mesh's GPU (GWN_ERR_INVALID_ARG otherwise, with nothing launched).
