@@ -529,7 +529,10 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
 // each (random soups, whose every loop is a triangle, and small holes), and its
 // rounding is relative to the triangle's solid angle, not to the edges' steep angles.
 // With unit vectors A, B, C toward the vertices, N the triangle's normal vector:
-//   den = 1 + A.B + A.C + B.C,  det = (a . N) / (|a| |b| |c|).
+//   den = 1 + A.B + A.C + B.C,  det = (a . N) / (|a| |b| |c|) = (A . N') (h / (|b| |c|)),
+// N = h N' with h a power of two and N' of magnitude about 1: a . N and 1 / (|a| |b| |c|)
+// alone go with the cube of the coordinates, and FP32 holds neither beyond 2^42 or below
+// 2^-43 (A . N' and h / (|b| |c|) it holds wherever it holds the squared distances).
 // The term enters the group product if 0.41 den - |det| > 0.05: its angle is below
 // pi/8 (8 factors stay below pi), away from the cut at +-pi, and den > 0.12 bounds
 // the amplification of rounding.  Otherwise (the query within about an edge's length)
@@ -543,7 +546,7 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
 // against FP64 on soup8 1.3e-6 -> 5.2e-7.  Bound by the FP32 pipe (74 issue slots a term).
 struct __align__(16) TriLoop {
     float4 a, b, c;   // the vertices; a.w = max z
-    float4 n;         // (b - a) x (c - a)
+    float4 n;         // (b - a) x (c - a) = n.w (n.x, n.y, n.z), n.w a power of two
     float4 box;       // min x, max x, min y, max y
 };
 static_assert(sizeof(TriLoop) == 80, "TriLoop must be 80 bytes");
@@ -653,7 +656,7 @@ __device__ __noinline__ void tri_deferred(const unsigned *queue, int count, cons
                         ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz);
             const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
                               (bx * cx + by * cy + bz * cz) * (ib * ic);
-            const float det = (ax * T.n.x + ay * T.n.y + az * T.n.z) * (ia * ib * ic);
+            const float det = (ax * T.n.x + ay * T.n.y + az * T.n.z) * ia * (T.n.w * (ib * ic));
             if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
             else edges = true;
         }
@@ -723,10 +726,10 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
                 const float2 ab = fma2(ax, px, fma2(ay, py, mul2(az, pz)));
                 const float2 ac = fma2(ax, cx, fma2(ay, cy, mul2(az, cz)));
                 const float2 bc = fma2(px, cx, fma2(py, cy, mul2(pz, cz)));
-                const float2 iab = mul2(ia, ib);
-                den[k] = fma2(ab, iab, fma2(mul2(ac, ia), ic, fma2(mul2(bc, ib), ic, bc2(1.f))));
+                const float2 ibc = mul2(ib, ic);
+                den[k] = fma2(bc, ibc, fma2(mul2(ac, ia), ic, fma2(mul2(ab, ia), ib, bc2(1.f))));
                 const float2 dn = fma2(ax, bc2(N.x), fma2(ay, bc2(N.y), mul2(az, bc2(N.z))));
-                det[k] = mul2(dn, mul2(iab, ic));
+                det[k] = mul2(mul2(dn, ia), mul2(bc2(N.w), ibc));
                 // a NaN (a padding query past n) counts as accepted: its sum is never read
                 const float2 v = fma2(bc2(kTanGroup), den[k], neg2(make_float2(fabsf(det[k].x), fabsf(det[k].y))));
                 fail |= (v.x <= kTriAccept ? 1u : 0u) << (2 * k) | (v.y <= kTriAccept ? 2u : 0u) << (2 * k);

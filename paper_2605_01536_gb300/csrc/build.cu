@@ -428,7 +428,12 @@ __global__ void k_split_loops(const float4 *__restrict__ pts, const uint2 *__res
     T[0] = a;
     T[1] = b;
     T[2] = c;
-    T[3] = make_float4((float)(uy * vz - uz * vy), (float)(uz * vx - ux * vz), (float)(ux * vy - uy * vx), 0.f);
+    // the normal as a power of two times a vector of magnitude about 1 (0 if it vanishes)
+    const double nx = uy * vz - uz * vy, ny = uz * vx - ux * vz, nz = ux * vy - uy * vx;
+    const double top = fmax(fabs(nx), fmax(fabs(ny), fabs(nz)));
+    const int e = top > 0.0 ? ilogb(top) : 0;
+    T[3] = make_float4((float)scalbn(nx, -e), (float)scalbn(ny, -e), (float)scalbn(nz, -e),
+                       top > 0.0 ? (float)scalbn(1.0, e) : 0.f);
     T[4] = make_float4(fminf(a.x, fminf(b.x, c.x)), fmaxf(a.x, fmaxf(b.x, c.x)), fminf(a.y, fminf(b.y, c.y)),
                        fmaxf(a.y, fmaxf(b.y, c.y)));
 }
