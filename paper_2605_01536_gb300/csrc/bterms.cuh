@@ -533,10 +533,16 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
 // N = h N' with h a power of two and N' of magnitude about 1: a . N and 1 / (|a| |b| |c|)
 // alone go with the cube of the coordinates, and FP32 holds neither beyond 2^42 or below
 // 2^-43 (A . N' and h / (|b| |c|) it holds wherever it holds the squared distances).
-// The term enters the group product if 0.41 den - |det| > 0.05: its angle is below
-// pi/8 (8 factors stay below pi), away from the cut at +-pi, and den > 0.12 bounds
-// the amplification of rounding.  Otherwise (the query within about an edge's length)
-// it takes its own atan2 or, close to T, its three edges' terms.  A ray that meets the
+// The rounding of A . N' reaches det times g = h / (|b| |c|), which is large beside b or c
+// (an edge length L over the distance) and along a triangle's short edge opposite a.
+// The term enters the group product if 0.41 den - |det| - g / 8 > 0.05: its angle is below
+// pi/8 (8 factors stay below pi), away from the cut at +-pi, den > 0.12 and g < 13 bound
+// the amplification of rounding (at most 1e-7 of w a term, in an emulation over random
+// and slim triangles at 3 to 1e-5 edge lengths; without g 8e-3 at 1e-5, and 1e-4 at one
+// edge length of a triangle with one edge a thousandth of the others).  Otherwise (the
+// query within about an edge's length) it takes its own atan2, with the nearest vertex in
+// the place of a (then |N| <= 4 times the product of the two other distances, at most
+// 6e-7 of w), or, close to T, its three edges' terms.  A ray that meets the
 // triangle's box takes the crossing predicate; every other ray misses T.  Both are
 // deferred like the batched kernel's failing terms: about 3% of a warp's triangles have
 // such a lane (random soup, 100k queries), and done in place, with most lanes idle,
@@ -551,6 +557,24 @@ struct __align__(16) TriLoop {
 };
 static_assert(sizeof(TriLoop) == 80, "TriLoop must be 80 bytes");
 constexpr float kTriAccept = 0.05f;
+constexpr float kTriSpread = 0.125f;   // weight of g
+
+// det of a triangle's term from the nearest vertex; a, b, c: the relative vectors, ia, ib,
+// ic: their reciprocal lengths
+__device__ __forceinline__ float tri_det_near(float4 n, float3 a, float3 b, float3 c, float ia, float ib, float ic) {
+    if (ib >= fmaxf(ia, ic)) {
+        const float i = ia;
+        a = b;
+        ia = ib;
+        ib = i;
+    } else if (ic >= ia) {
+        const float i = ia;
+        a = c;
+        ia = ic;
+        ic = i;
+    }
+    return (a.x * n.x + a.y * n.y + a.z * n.z) * ia * (n.w * (ib * ic));
+}
 
 // The exact predicate, where the FP32 filter of tri_cross cannot decide.
 __device__ __noinline__ int tri_cross_exact(const TriLoop &T, float qx, float qy, float qz,
@@ -652,11 +676,13 @@ __device__ __noinline__ void tri_deferred(const unsigned *queue, int count, cons
         if (fail && !edges) {   // a well-conditioned angle away from the cut takes its own atan2
             const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy,
                         bz = T.b.z - qz, cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
-            const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az), ib = sfu_rsqrt(bx * bx + by * by + bz * bz),
-                        ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz);
+            // (1e-37: a coincident vertex gives a finite reciprocal length)
+            const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az + 1e-37f), ib = sfu_rsqrt(bx * bx + by * by + bz * bz + 1e-37f),
+                        ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz + 1e-37f);
             const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
                               (bx * cx + by * cy + bz * cz) * (ib * ic);
-            const float det = (ax * T.n.x + ay * T.n.y + az * T.n.z) * ia * (T.n.w * (ib * ic));
+            const float det = tri_det_near(T.n, make_float3(ax, ay, az), make_float3(bx, by, bz), make_float3(cx, cy, cz),
+                                           ia, ib, ic);
             if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
             else edges = true;
         }
@@ -729,9 +755,11 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
                 const float2 ibc = mul2(ib, ic);
                 den[k] = fma2(bc, ibc, fma2(mul2(ac, ia), ic, fma2(mul2(ab, ia), ib, bc2(1.f))));
                 const float2 dn = fma2(ax, bc2(N.x), fma2(ay, bc2(N.y), mul2(az, bc2(N.z))));
-                det[k] = mul2(mul2(dn, ia), mul2(bc2(N.w), ibc));
+                const float2 g = mul2(bc2(N.w), ibc);
+                det[k] = mul2(mul2(dn, ia), g);
                 // a NaN (a padding query past n) counts as accepted: its sum is never read
-                const float2 v = fma2(bc2(kTanGroup), den[k], neg2(make_float2(fabsf(det[k].x), fabsf(det[k].y))));
+                const float2 v = fma2(bc2(-kTriSpread), g,
+                                      fma2(bc2(kTanGroup), den[k], neg2(make_float2(fabsf(det[k].x), fabsf(det[k].y)))));
                 fail |= (v.x <= kTriAccept ? 1u : 0u) << (2 * k) | (v.y <= kTriAccept ? 2u : 0u) << (2 * k);
                 inbox |= (-nqx[k].x >= bx.x && -nqx[k].x <= bx.y && -nqy[k].x >= bx.z && -nqy[k].x <= bx.w && -nqz[k].x <= a.w ? 1u : 0u) << (2 * k) |
                          (-nqx[k].y >= bx.x && -nqx[k].y <= bx.y && -nqy[k].y >= bx.z && -nqy[k].y <= bx.w && -nqz[k].y <= a.w ? 2u : 0u) << (2 * k);
