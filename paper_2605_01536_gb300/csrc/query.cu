@@ -683,12 +683,13 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const float *__restrict
 // ------------------------------------------------------------- direct ----
 
 // Direct sum (Eq. 2, each area by Eq. 6): per triangle 2 atan2(det, den) with unit vectors
-// A, B, C toward the vertices, den = 1 + A.B + A.C + B.C and det = (a . N) / (|a| |b| |c|),
-// N the triangle's normal vector (a . N = det[a b c], without the cancellation of the
-// relative vectors' products; computed once per block when the triangle is staged).
+// A, B, C toward the vertices, den = 1 + A.B + A.C + B.C and det = (A . N') (h / (|b| |c|)),
+// N = h N' the triangle's normal vector as for triangle loops (bterms.cuh; computed once
+// per block when the triangle is staged, as accurate as the FP32 vertices allow: a slim
+// triangle's normal is small against the products it is made of).
 // Terms are multiplied into a group's complex product like the boundary sum's (one atan2
-// per 8 triangles) while 0.41 den - |det| > 0.05: an angle below pi/8, well-conditioned;
-// nearer triangles take their own.  Each thread holds 2 KP queries as float2 pairs.  The
+// per 8 triangles) under the triangle loops' test: an angle below pi/8, well-conditioned;
+// nearer triangles take their own, with the nearest vertex in the place of a.  Each thread holds 2 KP queries as float2 pairs.  The
 // triangle range is split into gridDim.y chunks so that any query count fills the GPU:
 // with one chunk the kernel writes w, otherwise FP64 partial sums [chunk][query] that
 // k_direct_reduce adds in chunk order.  Bound by the FP32 pipe: 47 paired operations a
@@ -698,7 +699,8 @@ template <int KP>
 __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, int64_t n, const float *__restrict__ tri9,
                                                    int64_t nt, int tile, int64_t chunk_len, float *__restrict__ w,
                                                    double *__restrict__ partial) {
-    extern __shared__ float4 s_dir[];   // per triangle: (a, N.x), (b, N.y), (c, N.z)
+    extern __shared__ float4 s_dir[];   // per triangle: (a, N'.x), (b, N'.y), (c, N'.z); then their h
+    float *s_h = reinterpret_cast<float *>(s_dir + 3 * tile);
     constexpr int KQ = 2 * KP;
     const int64_t base = (int64_t)blockIdx.x * blockDim.x * KQ + threadIdx.x;
     const int64_t t_begin = (int64_t)blockIdx.y * chunk_len;
@@ -736,19 +738,34 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
             const float *T = tri9 + 9 * (t0 + i);
             const float ax = __ldg(T), ay = __ldg(T + 1), az = __ldg(T + 2), bx = __ldg(T + 3), by = __ldg(T + 4),
                         bz = __ldg(T + 5), cx = __ldg(T + 6), cy = __ldg(T + 7), cz = __ldg(T + 8);
-            const float ux = bx - ax, uy = by - ay, uz = bz - az, vx = cx - ax, vy = cy - ay, vz = cz - az;
-            // x1 y2 - x2 y1 with the rounding of the second product made good
-            auto cross = [](float x1, float y2, float x2, float y1) {
-                const float m = x2 * y1;
-                return fmaf(x1, y2, -m) + fmaf(-x2, y1, m);
-            };
-            s_dir[3 * i] = make_float4(ax, ay, az, cross(uy, vz, vy, uz));
-            s_dir[3 * i + 1] = make_float4(bx, by, bz, cross(uz, vx, vz, ux));
-            s_dir[3 * i + 2] = make_float4(cx, cy, cz, cross(ux, vy, vx, uy));
+            float u[3], v[3], ul[3], vl[3], N[3];   // the edges as exact sums of two floats
+            two_diff32(bx, ax, u[0], ul[0]);
+            two_diff32(by, ay, u[1], ul[1]);
+            two_diff32(bz, az, u[2], ul[2]);
+            two_diff32(cx, ax, v[0], vl[0]);
+            two_diff32(cy, ay, v[1], vl[1]);
+            two_diff32(cz, az, v[2], vl[2]);
+            float top = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+                // u1 v2 - u2 v1 with the rounding of the second product made good, and the low parts
+                const float m = u[k2] * v[k1];
+                N[k] = (fmaf(u[k1], v[k2], -m) + fmaf(-u[k2], v[k1], m)) +
+                       (fmaf(u[k1], vl[k2], ul[k1] * v[k2]) - fmaf(u[k2], vl[k1], ul[k2] * v[k1]));
+                top = fmaxf(top, fabsf(N[k]));
+            }
+            const int e = __float_as_int(top) & 0x7f800000;   // h = 2^floor(log2 top), or 0
+            const float r = e ? __int_as_float((254 << 23) - e) : 0.f;
+            s_dir[3 * i] = make_float4(ax, ay, az, N[0] * r);
+            s_dir[3 * i + 1] = make_float4(bx, by, bz, N[1] * r);
+            s_dir[3 * i + 2] = make_float4(cx, cy, cz, N[2] * r);
+            s_h[i] = __int_as_float(e);
         }
         __syncthreads();
         for (int j = 0; j < cnt; ++j) {
             const float4 A = s_dir[3 * j], B = s_dir[3 * j + 1], C = s_dir[3 * j + 2];
+            const float h = s_h[j];
 #pragma unroll
             for (int k = 0; k < KP; ++k) {
                 const float2 ax = add2(bc2(A.x), nqx[k]), ay = add2(bc2(A.y), nqy[k]), az = add2(bc2(A.z), nqz[k]);
@@ -763,14 +780,21 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
                 const float2 ab = fma2(ax, bx, fma2(ay, by, mul2(az, bz)));
                 const float2 ac = fma2(ax, cx, fma2(ay, cy, mul2(az, cz)));
                 const float2 bc = fma2(bx, cx, fma2(by, cy, mul2(bz, cz)));
-                const float2 iab = mul2(ia, ib);
-                const float2 den = fma2(ab, iab, fma2(mul2(ac, ia), ic, fma2(mul2(bc, ib), ic, bc2(1.f))));
+                const float2 ibc = mul2(ib, ic);
+                const float2 den = fma2(bc, ibc, fma2(mul2(ac, ia), ic, fma2(mul2(ab, ia), ib, bc2(1.f))));
                 const float2 dn = fma2(ax, bc2(A.w), fma2(ay, bc2(B.w), mul2(az, bc2(C.w))));
-                const float2 det = mul2(dn, mul2(iab, ic));
-                const float2 v = fma2(bc2(kTanGroup), den, neg2(make_float2(fabsf(det.x), fabsf(det.y))));
+                const float2 g = mul2(bc2(h), ibc);
+                const float2 det = mul2(mul2(dn, ia), g);
+                const float2 v = fma2(bc2(-kTriSpread), g,
+                                      fma2(bc2(kTanGroup), den, neg2(make_float2(fabsf(det.x), fabsf(det.y)))));
                 const bool px = v.x > kTriAccept, py = v.y > kTriAccept;
-                if (!px) part[k].x += fast_atan2(det.x, den.x);
-                if (!py) part[k].y += fast_atan2(det.y, den.y);
+                const float4 N = make_float4(A.w, B.w, C.w, h);
+                if (!px)
+                    part[k].x += fast_atan2(tri_det_near(N, make_float3(ax.x, ay.x, az.x), make_float3(bx.x, by.x, bz.x),
+                                                         make_float3(cx.x, cy.x, cz.x), ia.x, ib.x, ic.x), den.x);
+                if (!py)
+                    part[k].y += fast_atan2(tri_det_near(N, make_float3(ax.y, ay.y, az.y), make_float3(bx.y, by.y, bz.y),
+                                                         make_float3(cx.y, cy.y, cz.y), ia.y, ib.y, ic.y), den.y);
                 const float2 fd = make_float2(px ? den.x : 1.f, py ? den.y : 1.f);
                 const float2 fn = make_float2(px ? det.x : 0.f, py ? det.y : 0.f);
                 const float2 r = fma2(re[k], fd, neg2(mul2(im[k], fn)));
@@ -1171,7 +1195,7 @@ gwn_status launch_direct(const gwn_mesh *m, const float *q, int64_t n, float *w,
     {
         ProfScope prof("direct_sum", s);
         dim3 grid((unsigned)qblocks, (unsigned)chunks);
-        k_direct<KP><<<grid, 256, sizeof(float4) * 3 * tile, s>>>(q, n, m->tri9, m->nt, tile, chunk_len, w, partial);
+        k_direct<KP><<<grid, 256, (sizeof(float4) * 3 + sizeof(float)) * tile, s>>>(q, n, m->tri9, m->nt, tile, chunk_len, w, partial);
         if (partial) k_direct_reduce<<<grid_for(n, 256), 256, 0, s>>>(partial, n, (int)chunks, w);
     }
     if (partial) cudaFreeAsync(partial, s);

@@ -78,3 +78,47 @@ def test_triangle_loops_beside_vertices(kind, n):
         err = np.abs(x.cpu().numpy()[sel].astype(np.float64) - ref["w_antipodal"])[ok]
         assert err.max() <= TOL, err.max()
     assert np.array_equal(lab.cpu().numpy()[sel][ok], (ref["w_antipodal"][ok] > 0.5).astype(np.uint8))
+
+
+DIRECT = {
+    "soup": lambda rng: soup(300, rng),
+    "slim": lambda rng: slim(300, rng),
+    "cap": lambda rng: (lambda m: (m.V, m.F))(gen.small_cap(4, 0.8)),
+    "closed": lambda rng: sphere(),
+}
+
+
+@pytest.mark.parametrize("kind", list(DIRECT))
+def test_direct_beside_vertices(kind):
+    """Queries close to a face's plane, compared with the distance to its vertices, are left out: the
+    solid angle jumps inside the face."""
+    import paper_2605_01536_gb300 as gwn
+    rng = np.random.default_rng(3)
+    V, F = DIRECT[kind](rng)
+    Q = beside_vertices(V, F, 4_000, rng)
+    A, B, C = (V[F[:, i]].astype(np.float64) for i in range(3))
+    N = np.cross(B - A, C - A)
+    keep = np.ones(len(Q), bool)
+    for i, p in enumerate(Q.astype(np.float64)):
+        d = np.abs(np.einsum("ij,ij->i", p - A, N)) / np.linalg.norm(N, axis=1)
+        e = np.linalg.norm(np.stack([p - A, p - B, p - C]), axis=2).min(0)
+        keep[i] = (d > np.minimum(0.03 * e, 1e-4)).all() and e.min() > 0   # (on a vertex w is undefined)
+    Q = Q[keep]
+    assert len(Q) >= 500
+    ref = oracle.direct(V, F, Q)
+    with gwn.Mesh(V, F, build=False) as m:
+        w = m.direct(torch.from_numpy(Q).cuda()).cpu().numpy().astype(np.float64)
+    assert np.abs(w - ref).max() <= TOL, np.abs(w - ref).max()
+
+
+@pytest.mark.parametrize("k", [-45, 30, 44, 58])
+def test_direct_scaled_by_a_power_of_two(k):
+    import paper_2605_01536_gb300 as gwn
+    rng = np.random.default_rng(5)
+    mesh = gen.random_soup(300, rng)
+    Q = rng.uniform(-0.6, 1.6, (2_000, 3)).astype(np.float32)
+    got = []
+    for s in (np.float32(1), np.float32(2.0 ** k)):
+        with gwn.Mesh(mesh.V * s, mesh.F, build=False) as m:
+            got.append(m.direct(torch.from_numpy(Q * s).cuda()).cpu().numpy().astype(np.float64))
+    assert np.abs(got[1] - got[0]).max() <= TOL
