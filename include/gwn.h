@@ -151,9 +151,10 @@ typedef struct gwn_counters {
                                      boundary point exactly straight above or below it) */
     uint64_t cancel_terms;        /* boundary terms evaluated in FP64 because their denominator
                                      cancels (gwn_config.fp64_cancel) */
-    uint64_t cancel_overflow;     /* cancelling terms beyond a warp's queue in the batched launch
-                                     whose query was not listed for FP64 re-evaluation (0 unless a
-                                     list could not be kept) */
+    uint64_t cancel_overflow;     /* cancelling terms taken in FP32 without an FP64 re-evaluation of
+                                     their query: always 0 (a query with more than 64 such terms in
+                                     a tile of the boundary, or 4 in a leaf of its hierarchy, is
+                                     re-evaluated in FP64 and counted in fp64_reevaluations) */
     uint64_t reserved[4];
 } gwn_counters;
 

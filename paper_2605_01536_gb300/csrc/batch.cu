@@ -38,7 +38,7 @@ struct gwn_batch {
     double *d_acc = nullptr;
     int32_t *d_chi = nullptr;
     int64_t *d_off = nullptr;              // [n_mesh + 1] query offsets
-    int32_t *d_list = nullptr;             // queries whose cancelling terms overflowed the kernel's queue
+    int32_t *d_list = nullptr;             // queries with many cancelling terms in a tile
     unsigned long long *d_list_len = nullptr;
     unsigned *d_listed = nullptr;          // one bit per query
     // the queries in (mesh, Morton) order and the results in that order
@@ -162,7 +162,7 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
 }
 
 // One run: the queries in (mesh, Morton) order, the persistent kernel and the
-// FP64 re-evaluation of overflow queries on that order, the results scattered
+// FP64 re-evaluation of the listed queries on that order, the results scattered
 // back to the caller's order.
 gwn_status enqueue_run(gwn_batch *b, const float *q, float *w, int32_t *chi, cudaStream_t s) {
     if (b->n_tiles > 0) GWN_CUDA_TRY(cudaMemsetAsync(b->d_tile_done, 0, sizeof(unsigned) * b->n_tiles, s));

@@ -274,21 +274,24 @@ __device__ double edge_angle64(float4 Pa, float4 Pb, float qx, float qy, float q
 // lane), and the warp evaluates the queue in FP64 after the tile's edges, where
 // the loop's registers are free; the results go to per-query 64-bit
 // fixed-point sums (units of 2^-40 rad) with integer atomics, exact and
-// independent of the order.  A queue that is full (more than kCancelCap such
-// terms for one warp in one tile) lists the query for a full FP64
-// re-evaluation instead (k_fp64_fix), once per query (the listed bits).
-constexpr int kCancelCap = 64;
+// independent of the order.  A queue without room for what comes next is evaluated and
+// emptied on the spot, so that a query's sum does not depend on how many terms its
+// neighbours in the warp queue.  A query with more than kCancelOwn such terms in one tile
+// is listed for a full FP64 re-evaluation (k_fp64_fix), once (the listed bits).
+constexpr int kCancelCap = 256;   // room for a warp's 128 queries' terms of one edge, twice
+constexpr int kCancelOwn = 64;
 constexpr double kFixUnit = 0x1p-40;
 constexpr double kFixScale64 = 0x1p40;
 
 struct CancelQ {
     unsigned *queue;            // this warp's queue, kCancelCap entries
     int *count;                 // this warp's entry count
+    int *own;                   // terms per query of the warp in this tile, own[32 slot + lane]
     long long *fix;             // fixed-point sums, fix[k blockDim.x + t]
     const float *q;             // the block's queries: slot k of thread t at q[3 (t + k blockDim.x)]
     int64_t qbase;              // caller's index of the block's query slot 0 of thread 0 (for the list)
-    int32_t *list;              // queries for a full FP64 re-evaluation (NULL: count the term as
-    unsigned long long *list_len;   //  an FP32 one and record it in CNT_CANCEL_OVERFLOW)
+    int32_t *list;              // queries for a full FP64 re-evaluation
+    unsigned long long *list_len;
     unsigned *listed;           // one bit per query: already listed
 };
 
@@ -300,38 +303,54 @@ __device__ __forceinline__ void list_query(int64_t idx, int32_t *list, unsigned 
     list[atomicAdd(list_len, 1ull)] = (int32_t)idx;
 }
 
-// Queue a cancelling term; false when the queue is full and the query has been
-// listed for a full FP64 re-evaluation (or there is no list).
-__device__ __forceinline__ bool cancel_enqueue(const CancelQ &cq, int j, int k, int lane) {
-    const int slot = atomicAdd(cq.count, 1);
-    if (slot < kCancelCap) {
-        cq.queue[slot] = (unsigned)j << 7 | (unsigned)k << 5 | (unsigned)lane;
-        return true;
-    }
-    if (cq.list) list_query(cq.qbase + (threadIdx.x & ~31) + lane + (int64_t)k * blockDim.x, cq.list, cq.list_len,
-                            cq.listed);
-    return false;
+// Queue a term (the caller has made sure of room).
+__device__ __forceinline__ void cancel_push(const CancelQ &cq, unsigned entry) {
+    cq.queue[atomicAdd(cq.count, 1)] = entry;
 }
 
-// FP64 evaluation of this warp's queued terms (points of the staged tile); all
-// 32 lanes of the warp call it, with the loop's registers out of use.
-__device__ __noinline__ void cancel_drain(const CancelQ &cq, const float4 *s_pts, unsigned long long *counters) {
+// The entries of the warp's queue; every lane of the warp calls it.
+__device__ __forceinline__ int cancel_count(const int *count) {
+    __syncwarp();
+    return __shfl_sync(0xffffffffu, *count, 0);
+}
+
+// Start of a tile: no terms of this tile yet.
+template <int KQ>
+__device__ __forceinline__ void cancel_tile(const CancelQ &cq) {
+#pragma unroll
+    for (int k = 0; k < KQ; ++k) cq.own[32 * k + (threadIdx.x & 31)] = 0;
+    __syncwarp();
+}
+
+// FP64 evaluation of this warp's queued terms; edge(j) gives the two points of entry j's
+// edge.  All 32 lanes of the warp call it, with the loop's registers out of use.
+template <class Edge>
+__device__ __forceinline__ void cancel_drain_edges(const CancelQ &cq, unsigned long long *counters, Edge &&edge) {
     __syncwarp();
     const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    const int count = min(*cq.count, kCancelCap);
+    const int count = *cq.count;
     for (int r = lane; r < count; r += 32) {
         const unsigned e = cq.queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
+        const int slot = (int)(e & 127u), owner = warp0 + (slot & 31), k = slot >> 5;
         const int local = owner + k * (int)blockDim.x;
-        const double t = edge_angle64(s_pts[j], s_pts[j + 1], cq.q[3 * local], cq.q[3 * local + 1],
-                                      cq.q[3 * local + 2], counters);
+        float4 Pa, Pb;
+        edge((int)(e >> 7), Pa, Pb);
+        const double t = edge_angle64(Pa, Pb, cq.q[3 * local], cq.q[3 * local + 1], cq.q[3 * local + 2], counters);
         atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
                   (unsigned long long)__double2ll_rn(t * kFixScale64));
+        if (atomicAdd(&cq.own[slot], 1) == kCancelOwn) list_query(cq.qbase + local, cq.list, cq.list_len, cq.listed);
     }
     if (lane == 0 && count > 0) atomicAdd(&counters[CNT_CANCEL], (unsigned long long)count);
     __syncwarp();
     if (lane == 0) *cq.count = 0;
     __syncwarp();
+}
+// entries: edges of the staged points
+__device__ __noinline__ void cancel_drain(const CancelQ &cq, const float4 *s_pts, unsigned long long *counters) {
+    cancel_drain_edges(cq, counters, [&](int j, float4 &Pa, float4 &Pb) {
+        Pa = s_pts[j];
+        Pb = s_pts[j + 1];
+    });
 }
 
 // A term that failed the group test and does not cancel, from the n and d the
@@ -350,32 +369,30 @@ struct BsumDefer {
 
 // The deferred terms of the batched kernel, drained by all 32 lanes.  With
 // Cond, a term whose d cancels goes on the cancellation queue (FP64 after the
-// tile) instead; if that is full it is taken in FP32 and counted.
+// tile, or as soon as the queue may be short of room) instead.
 template <bool Cond>
 __device__ __noinline__ void bsum_drain(const unsigned *queue, int count, const float4 *s_pts, const float *q,
                                         long long *fix, CancelQ cq, unsigned long long *counters) {
     const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    for (int r = lane; r < count; r += 32) {
-        const unsigned e = queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
-        const int local = owner + k * (int)blockDim.x;
-        const float4 Pa = s_pts[j], Pb = s_pts[j + 1];
-        const float qx = q[3 * local], qy = q[3 * local + 1], qz = q[3 * local + 2];
-        const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
-        const float n = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
-        const float d = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
-        if (Cond && cancels(n, d, A.h, B.h)) {
-            const int slot = atomicAdd(cq.count, 1);
-            if (slot < kCancelCap) {
-                cq.queue[slot] = (unsigned)j << 7 | (unsigned)k << 5 | (unsigned)(e & 31u);
-                continue;
+    for (int r0 = 0; r0 < count; r0 += 32) {
+        if (r0 + lane < count) {
+            const unsigned e = queue[r0 + lane];
+            const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
+            const int local = owner + k * (int)blockDim.x;
+            const float4 Pa = s_pts[j], Pb = s_pts[j + 1];
+            const float qx = q[3 * local], qy = q[3 * local + 1], qz = q[3 * local + 2];
+            const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
+            const float n = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
+            const float d = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
+            if (Cond && cancels(n, d, A.h, B.h)) {
+                cancel_push(cq, e);
+            } else {
+                const float t = edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
+                atomicAdd(reinterpret_cast<unsigned long long *>(fix + (k * (int)blockDim.x + owner)),
+                          (unsigned long long)__float2ll_rn(t * kFixScale));
             }
-            if (cq.list) list_query(cq.qbase + local, cq.list, cq.list_len, cq.listed);
-            else atomicAdd(&counters[CNT_CANCEL_OVERFLOW], 1ull);
         }
-        const float t = edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
-        atomicAdd(reinterpret_cast<unsigned long long *>(fix + (k * (int)blockDim.x + owner)),
-                  (unsigned long long)__float2ll_rn(t * kFixScale));
+        if (Cond && cancel_count(cq.count) > kCancelCap - 32) cancel_drain(cq, s_pts, counters);
     }
     __syncwarp();
 }
@@ -610,10 +627,9 @@ __device__ __forceinline__ int tri_cross(const TriLoop &T, float qx, float qy, f
 
 __device__ __forceinline__ float4 tri_vertex(const TriLoop &T, int e) { return e == 0 ? T.a : e == 1 ? T.b : T.c; }
 
-// The three edge terms of triangle j (of the staged tile) for query slot k of a lane
-// (the block's query local); ill-conditioned ones go on the warp's FP64 queue (entry
-// 3 j + edge), or list the query when that is full.
-__device__ __noinline__ float tri_edges(const TriLoop &T, int j, int k, int lane, int local, float qx, float qy, float qz, const CancelQ &cq,
+// The three edge terms of triangle j (of the staged tile) for the query of slot (32 k +
+// lane); ill-conditioned ones go on the warp's FP64 queue (entry 3 j + edge).
+__device__ __noinline__ float tri_edges(const TriLoop &T, int j, unsigned slot, float qx, float qy, float qz, const CancelQ &cq,
                                         unsigned long long *counters) {
     float sum = 0.f;
     for (int e = 0; e < 3; ++e) {
@@ -621,39 +637,19 @@ __device__ __noinline__ float tri_edges(const TriLoop &T, int j, int k, int lane
         const PointRel A = point_rel_twin(Pa, qx, qy, qz), B = point_rel_twin(Pb, qx, qy, qz);
         const float n = __fmaf_rn(A.ay, B.ax, -__fmul_rn(A.ax, B.ay));
         const float d = __fmaf_rn(A.h, B.h, __fmaf_rn(A.ax, B.ax, __fmul_rn(A.ay, B.ay)));
-        if (cancels(n, d, A.h, B.h)) {
-            const int slot = atomicAdd(cq.count, 1);
-            if (slot < kCancelCap) {
-                cq.queue[slot] = (unsigned)(3 * j + e) << 7 | (unsigned)k << 5 | (unsigned)lane;
-                continue;
-            }
-            if (cq.list) list_query(cq.qbase + local, cq.list, cq.list_len, cq.listed);
-            else atomicAdd(&counters[CNT_CANCEL_OVERFLOW], 1ull);
-        }
-        sum += edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
+        if (cancels(n, d, A.h, B.h)) cancel_push(cq, (unsigned)(3 * j + e) << 7 | slot);
+        else sum += edge_term(n, d, A, B, Pa, Pb, qx, qy, qz, counters);
     }
     return sum;
 }
 
-// FP64 evaluation of the warp's queued edges of the staged triangles (cancel_drain).
+// entries: edges of the staged triangles
 __device__ __noinline__ void tri_drain(const CancelQ &cq, const TriLoop *s_tri, unsigned long long *counters) {
-    __syncwarp();
-    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    const int count = min(*cq.count, kCancelCap);
-    for (int r = lane; r < count; r += 32) {
-        const unsigned e = cq.queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7);
-        const int local = owner + k * (int)blockDim.x, ed = j % 3;
+    cancel_drain_edges(cq, counters, [&](int j, float4 &Pa, float4 &Pb) {
         const TriLoop &T = s_tri[j / 3];
-        const double t = edge_angle64(tri_vertex(T, ed), tri_vertex(T, ed == 2 ? 0 : ed + 1), cq.q[3 * local],
-                                      cq.q[3 * local + 1], cq.q[3 * local + 2], counters);
-        atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
-                  (unsigned long long)__double2ll_rn(t * kFixScale64));
-    }
-    if (lane == 0 && count > 0) atomicAdd(&counters[CNT_CANCEL], (unsigned long long)count);
-    __syncwarp();
-    if (lane == 0) *cq.count = 0;
-    __syncwarp();
+        Pa = tri_vertex(T, j % 3);
+        Pb = tri_vertex(T, j % 3 == 2 ? 0 : j % 3 + 1);
+    });
 }
 
 // The warp's deferred triangle terms, drained by all 32 lanes: entry
@@ -662,35 +658,38 @@ __device__ __noinline__ void tri_drain(const CancelQ &cq, const TriLoop *s_tri, 
 __device__ __noinline__ void tri_deferred(const unsigned *queue, int count, const TriLoop *s_tri, const CancelQ &cq,
                                           unsigned long long *counters) {
     const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
-    for (int r = lane; r < count; r += 32) {
-        const unsigned e = queue[r];
-        const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7 & 0xffffffu);
-        const bool fail = e >> 31;
-        const int local = owner + k * (int)blockDim.x;
-        const float qx = cq.q[3 * local], qy = cq.q[3 * local + 1], qz = cq.q[3 * local + 2];
-        const TriLoop &T = s_tri[j];
-        bool edges = false;
-        const bool inbox = qx >= T.box.x && qx <= T.box.y && qy >= T.box.z && qy <= T.box.w && qz <= T.a.w;
-        const int cr = inbox ? tri_cross(T, qx, qy, qz, &edges, counters) : 0;
-        float t = 0.f;
-        if (fail && !edges) {   // a well-conditioned angle away from the cut takes its own atan2
-            const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy,
-                        bz = T.b.z - qz, cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
-            // (1e-37: a coincident vertex gives a finite reciprocal length)
-            const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az + 1e-37f), ib = sfu_rsqrt(bx * bx + by * by + bz * bz + 1e-37f),
-                        ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz + 1e-37f);
-            const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
-                              (bx * cx + by * cy + bz * cz) * (ib * ic);
-            const float det = tri_det_near(T.n, make_float3(ax, ay, az), make_float3(bx, by, bz), make_float3(cx, cy, cz),
-                                           ia, ib, ic);
-            if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
-            else edges = true;
+    for (int r0 = 0; r0 < count; r0 += 32) {
+        if (r0 + lane < count) {
+            const unsigned e = queue[r0 + lane];
+            const int owner = warp0 + (int)(e & 31u), k = (int)(e >> 5 & 3u), j = (int)(e >> 7 & 0xffffffu);
+            const bool fail = e >> 31;
+            const int local = owner + k * (int)blockDim.x;
+            const float qx = cq.q[3 * local], qy = cq.q[3 * local + 1], qz = cq.q[3 * local + 2];
+            const TriLoop &T = s_tri[j];
+            bool edges = false;
+            const bool inbox = qx >= T.box.x && qx <= T.box.y && qy >= T.box.z && qy <= T.box.w && qz <= T.a.w;
+            const int cr = inbox ? tri_cross(T, qx, qy, qz, &edges, counters) : 0;
+            float t = 0.f;
+            if (fail && !edges) {   // a well-conditioned angle away from the cut takes its own atan2
+                const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy,
+                            bz = T.b.z - qz, cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
+                // (1e-37: a coincident vertex gives a finite reciprocal length)
+                const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az + 1e-37f), ib = sfu_rsqrt(bx * bx + by * by + bz * bz + 1e-37f),
+                            ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz + 1e-37f);
+                const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
+                                  (bx * cx + by * cy + bz * cz) * (ib * ic);
+                const float det = tri_det_near(T.n, make_float3(ax, ay, az), make_float3(bx, by, bz), make_float3(cx, cy, cz),
+                                               ia, ib, ic);
+                if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
+                else edges = true;
+            }
+            const double sum = edges ? (double)tri_edges(T, j, e & 127u, qx, qy, qz, cq, counters)
+                                     : (double)t - 6.28318530717958647693 * cr;
+            if (sum != 0.0)
+                atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
+                          (unsigned long long)__double2ll_rn(sum * kFixScale64));
         }
-        const double sum = edges ? (double)tri_edges(T, j, k, (int)(e & 31u), local, qx, qy, qz, cq, counters)
-                                 : (double)t - 6.28318530717958647693 * cr;
-        if (sum != 0.0)
-            atomicAdd(reinterpret_cast<unsigned long long *>(cq.fix + (k * (int)blockDim.x + owner)),
-                      (unsigned long long)__double2ll_rn(sum * kFixScale64));
+        if (cancel_count(cq.count) > kCancelCap - 96) tri_drain(cq, s_tri, counters);   // 3 edges a lane
     }
     __syncwarp();
 }
@@ -733,6 +732,7 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
         __syncthreads();
         const float4 *src = reinterpret_cast<const float4 *>(tris + t0);
         for (int i = threadIdx.x; i < 5 * cnt; i += blockDim.x) reinterpret_cast<float4 *>(s_tri)[i] = __ldg(src + i);
+        cancel_tile<KQ>(cq);
         __syncthreads();
         for (int j = 0; j < cnt; ++j) {
             const float4 a = s_tri[j].a, b = s_tri[j].b, c = s_tri[j].c, N = s_tri[j].n, bx = s_tri[j].box;
@@ -798,7 +798,7 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
             tri_deferred(queue, q_count, s_tri, cq, counters);
             q_count = 0;
         }
-        if (*cq.count > 0) tri_drain(cq, s_tri, counters);
+        if (cancel_count(cq.count) > 0) tri_drain(cq, s_tri, counters);
 #pragma unroll
         for (int k = 0; k < KP; ++k) {
             s_acc[(2 * k) * blockDim.x + threadIdx.x] += (double)part[k].x + (double)comp[k].x;

@@ -107,7 +107,7 @@ enum CounterSlot {
     CNT_SUR_FALLBACK = 8,
     CNT_GRAD_SKIPPED = 9,
     CNT_CANCEL = 10,
-    CNT_CANCEL_OVERFLOW = 11,
+    CNT_CANCEL_OVERFLOW = 11,   // never counted: every such query is listed
     CNT_SLOTS = 16
 };
 
@@ -298,8 +298,8 @@ struct BatchItem {      // kind 0: crossing numbers of the tile; 1: points, 2: t
     int32_t kind;
     int64_t p_begin, p_end;   // queries of the tile, edge start points, or triangle loops
 };
-// list / list_len / listed: queries whose cancelling boundary terms overflow the
-// kernel's queue, for launch_batch_fp64_fix (listed: zeroed bits, one per query)
+// list / list_len / listed: queries with many cancelling boundary terms in a tile,
+// for launch_batch_fp64_fix (listed: zeroed bits, one per query)
 gwn_status launch_batch_kernel(int kp, int grid, int tile_pts, const BatchMesh *meshes, const BatchTile *tiles,
                                const BatchItem *items, int64_t n_items, const float *q, int32_t *chi, double *acc,
                                float *w, unsigned *tile_done, unsigned long long *head, int32_t *list,

@@ -234,7 +234,7 @@ __device__ __forceinline__ void bsum_accumulate(const float4 *__restrict__ pts, 
                     q_count = 0;
                 }
             }
-        } else if (fail) {   // rare: the failing terms one by one
+        } else if (C ? __any_sync(0xffffffffu, fail) : fail != 0) {   // rare: the failing terms one by one
             const float4 Pa = s_pts[j], Pb = s_pts[j + 1];
 #pragma unroll
             for (int k = 0; k < KQ; ++k) {
@@ -248,15 +248,18 @@ __device__ __forceinline__ void bsum_accumulate(const float4 *__restrict__ pts, 
                 const float qx = -(hi ? nqx[kp].y : nqx[kp].x), qy = -(hi ? nqy[kp].y : nqy[kp].x),
                             qz = -(hi ? nqz[kp].y : nqz[kp].x);
                 const float nk = hi ? en[kp].y : en[kp].x, dk = hi ? ed[kp].y : ed[kp].x;
-                // a queued ill-conditioned term is added after the tile, in FP64.  Only
+                // a queued ill-conditioned term is added later, in FP64.  Only
                 // the loop for warps near the tile tests: no query outside the
                 // tile's widened box has such a term, so a query's terms do not
                 // depend on its warp
                 float t = 0.f;
-                if (!(C && cancels(nk, dk, a.h, b.h) && cancel_enqueue(cq, j, k, (int)(threadIdx.x & 31))))
-                    t = fallback_term(nk, dk, a, b, Pa, Pb, qx, qy, qz, counters);
+                if (C && cancels(nk, dk, a.h, b.h)) cancel_push(cq, (unsigned)j << 7 | (unsigned)k << 5 | (threadIdx.x & 31u));
+                else t = fallback_term(nk, dk, a, b, Pa, Pb, qx, qy, qz, counters);
                 if (hi) two_sum_acc(st.part[kp].y, st.comp[kp].y, t);
                 else two_sum_acc(st.part[kp].x, st.comp[kp].x, t);
+            }
+            if constexpr (C) {   // (the whole warp is here)
+                if (cancel_count(cq.count) > kCancelCap - 32 * KQ) cancel_drain(cq, s_pts, counters);
             }
         }
         if (++g_count == GROUP) finalize();
@@ -300,6 +303,7 @@ __device__ __forceinline__ void bsum_accumulate(const float4 *__restrict__ pts, 
                 near |= in_box(box, -nqx[k].x, -nqy[k].x, -nqz[k].x) || in_box(box, -nqx[k].y, -nqy[k].y, -nqz[k].y);
             }
             near = __any_sync(0xffffffffu, near);
+            if (near) cancel_tile<KQ>(cq);
         }
         if (near) run_edges(std::true_type{}, cnt);
         else run_edges(std::false_type{}, cnt);
@@ -312,8 +316,7 @@ __device__ __forceinline__ void bsum_accumulate(const float4 *__restrict__ pts, 
             }
         }
         if constexpr (Cond) {   // the queued cancelling terms of this tile, in FP64
-            __syncwarp();
-            if (*cq.count > 0) cancel_drain(cq, s_pts, counters);
+            if (cancel_count(cq.count) > 0) cancel_drain(cq, s_pts, counters);
         }
 #pragma unroll
         for (int k = 0; k < KP; ++k) {
@@ -353,7 +356,7 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
                                                       unsigned long long *__restrict__ counters) {
     // dynamic shared memory (bsum_smem): tile + 1 points | 2 KP x blockDim FP64 sums |
     // (Cond) 2 KP x blockDim fixed-point sums, per warp kCancelCap queue entries, per warp
-    // a count
+    // a count per query, per warp a count
     extern __shared__ float4 s_pts[];
     double *s_acc = reinterpret_cast<double *>(s_pts + tile + 1);
     constexpr int KQ = 2 * KP;
@@ -367,11 +370,12 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
     unsigned *tri_queue = nullptr;   // with triangle loops, after the counts: per warp 64 KQ entries
     if constexpr (Cond) {
         const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-        tri_queue = reinterpret_cast<unsigned *>(s_acc + 2 * KQ * blockDim.x) + nwarps * (kCancelCap + 1) + warp * 64 * KQ;
         cq.fix = reinterpret_cast<long long *>(s_acc + KQ * blockDim.x);
         unsigned *queues = reinterpret_cast<unsigned *>(cq.fix + KQ * blockDim.x);
         cq.queue = queues + warp * kCancelCap;
-        cq.count = reinterpret_cast<int *>(queues + nwarps * kCancelCap) + warp;
+        cq.own = reinterpret_cast<int *>(queues + nwarps * kCancelCap) + warp * 32 * KQ;
+        cq.count = reinterpret_cast<int *>(queues + nwarps * (kCancelCap + 32 * KQ)) + warp;
+        tri_queue = queues + nwarps * (kCancelCap + 32 * KQ + 1) + warp * 64 * KQ;
         cq.q = q + 3 * qblock;
         cq.qbase = qblock;
         cq.list = list;
@@ -410,7 +414,7 @@ __global__ void __launch_bounds__(kBsumThreads, 4) k_boundary_sum(const float *_
 static size_t bsum_smem(int kp, int tile, bool cond, bool tris) {
     const size_t kq = 2 * (size_t)kp, threads = kBsumThreads;
     size_t b = sizeof(float4) * (tile + 1) + sizeof(double) * kq * threads;
-    if (cond) b += sizeof(long long) * kq * threads + (sizeof(unsigned) * kCancelCap + sizeof(int)) * (threads / 32);
+    if (cond) b += sizeof(long long) * kq * threads + sizeof(unsigned) * (kCancelCap + 32 * kq + 1) * (threads / 32);
     if (tris) b += sizeof(unsigned) * 64 * kq * (threads / 32);
     return b;
 }
@@ -481,7 +485,8 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
             CancelQ cq;
             cq.fix = dq.fix;
             cq.queue = queues + nwarps * (64 * KQ) + warp * kCancelCap;
-            cq.count = reinterpret_cast<int *>(queues + nwarps * (64 * KQ + kCancelCap)) + warp;
+            cq.own = reinterpret_cast<int *>(queues + nwarps * (64 * KQ + kCancelCap)) + warp * 32 * KQ;
+            cq.count = reinterpret_cast<int *>(queues + nwarps * (96 * KQ + kCancelCap)) + warp;
             cq.q = dq.q;
             cq.qbase = tl.q_begin;
             cq.list = list;
@@ -567,8 +572,8 @@ __global__ void __launch_bounds__(256) k_fp64_fix(const float *__restrict__ q, c
     }
 }
 
-// The batched launch's FP64 re-evaluation: one block per listed query (its
-// cancelling terms overflowed the kernel's queue); the mesh is found by binary
+// The batched launch's FP64 re-evaluation: one block per listed query (more than
+// kCancelOwn cancelling terms in a tile); the mesh is found by binary
 // search in the meshes' query offsets.
 __global__ void __launch_bounds__(256) k_batch_fp64_fix(const BatchMesh *__restrict__ meshes,
                                                         const int64_t *__restrict__ mesh_off, int n_mesh,
@@ -1060,8 +1065,8 @@ gwn_status launch_boundary_sum_list(const gwn_mesh *m, const float *q, int64_t n
     unsigned *listed = nullptr;
     GWN_CUDA_TRY(dev_alloc(&listed, sizeof(unsigned) * words, s));
     GWN_CUDA_TRY(cudaMemsetAsync(listed, 0, sizeof(unsigned) * words, s));
-    // without a caller list (no labels wanted), queries whose cancelling terms
-    // overflow the kernel's queue still need their FP64 re-evaluation
+    // without a caller list (no labels wanted), queries with more cancelling terms in
+    // a tile than kCancelOwn still need their FP64 re-evaluation
     const bool own_list = list == nullptr;
     if (own_list) {
         GWN_CUDA_TRY(dev_alloc(&list, sizeof(int32_t) * n, s));
@@ -1099,11 +1104,11 @@ gwn_status launch_classify_on_scratch(const gwn_mesh *m, const float *q, int64_t
 
 // k_batch's dynamic shared memory: tile + 1 points, then per query slot an FP64
 // sum and a fixed-point sum, then per warp one deferred-term queue of 64 KQ
-// entries, then per warp a cancelling-term queue and its count.
+// entries, then per warp a cancelling-term queue, its queries' counts and its own.
 static size_t batch_smem(int kp, int tile_pts) {
     const size_t kq = 2 * (size_t)kp, threads = 256, warps = threads / 32;
     return sizeof(float4) * (tile_pts + 1) + (sizeof(double) + sizeof(long long)) * kq * threads +
-           sizeof(unsigned) * (64 * kq + kCancelCap) * warps + sizeof(int) * warps;
+           sizeof(unsigned) * (96 * kq + kCancelCap + 1) * warps;
 }
 
 template <int KP>
