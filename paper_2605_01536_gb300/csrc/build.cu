@@ -129,8 +129,8 @@ __global__ void k_emit_edges(const int32_t *__restrict__ mult, const uint64_t *_
 }
 
 // Boundary edges by buckets of the smaller vertex: half-edges are counted and placed
-// per vertex (entry: larger vertex << 1 | direction), and one thread nets out each
-// vertex's few entries.  A vertex with more than kBucketMax entries sets *overflow and
+// per vertex (entry: larger vertex << 1 | direction), and each vertex's few entries are
+// netted out against one another.  A vertex with more than kBucketMax entries sets *overflow and
 // the sort below takes over.  A half-edge from a vertex to itself (repeated index in a
 // degenerate face) is a zero chain and contributes nothing.
 constexpr uint32_t kBucketMax = 128;
@@ -171,35 +171,63 @@ __device__ __forceinline__ int bucket_net(const uint32_t *__restrict__ entry, ui
     return m;
 }
 
-// emit = 0: edges of each vertex into n_out; else the edges themselves, each vertex's
-// from out[v] on in ascending order of the other vertex
+// The copies of entry i's edge (net[i] != 0) at their place: after the copies of the vertex's
+// edges with a smaller other vertex, which begin at base
+__device__ __forceinline__ void bucket_emit(const uint32_t *__restrict__ entry, const int32_t *__restrict__ net, uint32_t b,
+                                            uint32_t e, uint32_t i, int32_t v, uint32_t base, int32_t *__restrict__ edges) {
+    const int m = net[i];
+    if (m == 0) return;
+    const int32_t hi = (int32_t)(entry[i] >> 1);
+    for (uint32_t j = b; j < e; ++j)
+        if ((int32_t)(entry[j] >> 1) < hi) base += (uint32_t)abs(net[j]);
+    for (int r = 0; r < abs(m); ++r) {
+        edges[2 * (base + r)] = m > 0 ? v : hi;
+        edges[2 * (base + r) + 1] = m > 0 ? hi : v;
+    }
+}
+
+// edges NULL: every entry's net multiplicity into net and each vertex's number of edges
+// into out; else the edges themselves, each vertex's from out[v] on in ascending order of
+// the other vertex.  A thread per vertex; buckets of more than kBucketSerial entries, whose
+// cost goes with the square of their size, are taken by the warp together (one thread and
+// nothing kept between the passes: a vertex of 126 unmatched half-edges 55 ms).
+constexpr uint32_t kBucketSerial = 16;
 __global__ void k_bucket_net(const uint32_t *__restrict__ entry, const uint32_t *__restrict__ first,
-                             const uint32_t *__restrict__ count, int64_t nv, uint32_t *__restrict__ out,
-                             int32_t *__restrict__ edges, const uint32_t *__restrict__ overflow) {
+                             const uint32_t *__restrict__ count, int64_t nv, int32_t *__restrict__ net,
+                             uint32_t *__restrict__ out, int32_t *__restrict__ edges,
+                             const uint32_t *__restrict__ overflow) {
+    if (*overflow) return;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nv || *overflow) return;
-    const uint32_t b = first[v], e = b + count[v];
+    const int lane = threadIdx.x & 31;
+    const uint32_t b = v < nv ? first[v] : 0u, e = v < nv ? b + count[v] : 0u;
     uint32_t total = 0;
-    for (uint32_t i = b; i < e; ++i) {
-        const int m = bucket_net(entry, b, e, i);
-        if (m == 0) continue;
-        const uint32_t c = (uint32_t)(m < 0 ? -m : m);
-        if (edges) {
-            uint32_t before = out[v];   // copies of this vertex's edges with a smaller other vertex
-            for (uint32_t j = b; j < e; ++j)
-                if (entry[j] >> 1 < entry[i] >> 1) {
-                    const int mj = bucket_net(entry, b, e, j);
-                    before += (uint32_t)(mj < 0 ? -mj : mj);
-                }
-            const int32_t hi = (int32_t)(entry[i] >> 1);
-            for (uint32_t r = 0; r < c; ++r) {
-                edges[2 * (before + r)] = m > 0 ? (int32_t)v : hi;
-                edges[2 * (before + r) + 1] = m > 0 ? hi : (int32_t)v;
+    if (e - b <= kBucketSerial) {
+        for (uint32_t i = b; i < e; ++i) {
+            if (edges) {
+                bucket_emit(entry, net, b, e, i, (int32_t)v, out[v], edges);
+            } else {
+                net[i] = bucket_net(entry, b, e, i);
+                total += (uint32_t)abs(net[i]);
             }
         }
-        total += c;
     }
-    if (!edges) out[v] = total;
+    for (unsigned big = __ballot_sync(0xffffffffu, e - b > kBucketSerial); big; big &= big - 1) {
+        const int src = __ffs(big) - 1;
+        const uint32_t wb = __shfl_sync(0xffffffffu, b, src), we = __shfl_sync(0xffffffffu, e, src);
+        const int64_t wv = v - lane + src;
+        uint32_t sum = 0;
+        for (uint32_t i = wb + lane; i < we; i += 32) {
+            if (edges) {
+                bucket_emit(entry, net, wb, we, i, (int32_t)wv, out[wv], edges);
+            } else {
+                net[i] = bucket_net(entry, wb, we, i);
+                sum += (uint32_t)abs(net[i]);
+            }
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == src) total = sum;
+    }
+    if (!edges && v < nv) out[v] = total;
 }
 
 // keys for sorting edges by start (which = 0) or end (which = 1) vertex
@@ -776,7 +804,8 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
         k_bucket_count<<<grid_for(nh, TB), TB, 0, s>>>(m->F, nh, count, rank, tot + 2);
         if ((st = exclusive_scan_u32(count, first, m->nv, nullptr, s)) != GWN_OK) return st;
         k_bucket_place<<<grid_for(nh, TB), TB, 0, s>>>(m->F, nh, first, rank, entry);
-        k_bucket_net<<<grid_for(m->nv, TB), TB, 0, s>>>(entry, first, count, m->nv, out, nullptr, tot + 2);
+        int32_t *net = reinterpret_cast<int32_t *>(rank);   // the ranks are not needed any more
+        k_bucket_net<<<grid_for(m->nv, TB), TB, 0, s>>>(entry, first, count, m->nv, net, out, nullptr, tot + 2);
         if ((st = exclusive_scan_u32(out, out, m->nv, tot + 1, s)) != GWN_OK) return st;
         uint32_t tot_h[3] = {0, 0, 0};
         GWN_CUDA_TRY(cudaMemcpyAsync(tot_h, tot, sizeof(tot_h), cudaMemcpyDeviceToHost, s));
@@ -786,7 +815,8 @@ gwn_status build_boundary(gwn_mesh *m, cudaStream_t s) {
             m->nb = tot_h[1];
             if (m->nb > 0) {
                 GWN_CUDA_TRY(dev_alloc(&m->bedges, sizeof(int32_t) * 2 * m->nb, s));
-                k_bucket_net<<<grid_for(m->nv, TB), TB, 0, s>>>(entry, first, count, m->nv, out, m->bedges, tot + 2);
+                k_bucket_net<<<grid_for(m->nv, TB), TB, 0, s>>>(entry, first, count, m->nv, net, out, m->bedges,
+                                                                tot + 2);
             }
         }
         for (uint32_t *p : {count, first, rank, entry, out}) cudaFreeAsync(p, s);
