@@ -37,6 +37,11 @@
  *     `stream`), copies the results back and synchronises `stream` before
  *     returning.  Caller-owned memory is
  *     never retained after a call returns.
+ *   - Device memory: scratch and mesh arrays come from one stream-ordered pool per
+ *     device, which keeps up to 1 GiB that is not in use while a mesh, batch or
+ *     parametric surface of the device lives, and gives all of it back when the last
+ *     one is destroyed.  A call's scratch is at most 128 MiB of partial sums, 8 MiB of
+ *     cell counts and about 60 bytes a query or grid cell, besides staged host buffers.
  *   - Layouts: points are float32 [n][3] (x, y, z interleaved, 12 bytes per
  *     point, 4-byte aligned); faces are int32 [nt][3] (counter-clockwise seen
  *     from the side the normal points to); per-query outputs are dense arrays

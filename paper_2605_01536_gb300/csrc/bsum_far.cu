@@ -127,7 +127,7 @@ __device__ __noinline__ void far_drain(const FarQueue fq, const float4 *__restri
 
 template <bool Running>
 __global__ void __launch_bounds__(kFarThreads, 5)
-    k_boundary_far(const float *__restrict__ q, int64_t n, const FarNode *__restrict__ nodes,
+    k_boundary_far(const float *__restrict__ q, int64_t first, int64_t n, const FarNode *__restrict__ nodes,
                    const int32_t *__restrict__ roots, int nroots, double *__restrict__ partial,
                    const float *__restrict__ coef, const float4 *__restrict__ pts, const int32_t *__restrict__ chi,
                    float *__restrict__ w, uint8_t *__restrict__ label, int classify, float margin,
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kFarThreads, 5)
     __shared__ unsigned s_queue[kWarps][32 * KQ * kFarOwn];
     __shared__ int s_count[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t qbase = ((int64_t)blockIdx.x * kWarps + warp) * (32 * KQ);
+    const int64_t qbase = first + ((int64_t)blockIdx.x * kWarps + warp) * (32 * KQ);   // queries [first, n)
     if (qbase >= n) return;
     const FarQueue fq{s_queue[warp], &s_count[warp], s_fix[warp]};
     float2 nqx[KP], nqy[KP], nqz[KP], part[KP], comp[KP];
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kFarThreads, 5)
         if (idx >= n) continue;
         const double sum = acc[k] + (double)fq.fix[32 * k + lane] * kFixUnit;
         if (partial) {
-            partial[(int64_t)blockIdx.y * n + idx] = sum;
+            partial[(int64_t)blockIdx.y * (n - first) + (idx - first)] = sum;
             continue;
         }
         const double wv = (double)chi[idx] + sum * kInv2Pi;
@@ -396,24 +396,27 @@ gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, con
                                unsigned long long *list_len, unsigned *listed, double *partial_buf,
                                int64_t call_n, cudaStream_t s) {
     const float margin = m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f;
-    const int64_t blocks = (n + kFarThreads * 2 - 1) / (kFarThreads * 2);
     const int64_t split = far_parts(m, call_n);
     double *partial = split > 1 ? partial_buf : nullptr;
     const bool own = split > 1 && !partial_buf;
-    if (own) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * split * n, s));
-    const dim3 grid((unsigned)blocks, (unsigned)split);
+    const int64_t slice = own ? query_slice(n, sizeof(double) * split) : n;
+    if (own) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * split * slice, s));
 #define GWN_FAR(R)                                                                                                    \
-    k_boundary_far<R><<<grid, kFarThreads, 0, s>>>(q, n, m->far_nodes, m->far_roots, m->far_nroots, partial,           \
+    k_boundary_far<R><<<grid, kFarThreads, 0, s>>>(q, at, end, m->far_nodes, m->far_roots, m->far_nroots, partial,           \
                                                    m->far_coef, m->far_pts, chi, w, label, classify ? 1 : 0, margin,   \
                                                    list, list_len, listed, m->counters)
-    if (running) GWN_FAR(true);
-    else GWN_FAR(false);
-#undef GWN_FAR
-    note_launches(1);
-    if (partial) {
-        launch_boundary_combine(partial, n, (int)split, chi, w, label, classify, margin, list, list_len, listed, s);
-        if (own) cudaFreeAsync(partial, s);
+    for (int64_t at = 0; at < n; at += slice) {
+        const int64_t end = std::min(n, at + slice);
+        const dim3 grid((unsigned)((end - at + kFarThreads * 2 - 1) / (kFarThreads * 2)), (unsigned)split);
+        if (running) GWN_FAR(true);
+        else GWN_FAR(false);
+        note_launches(1);
+        if (partial)
+            launch_boundary_combine(partial, at, end - at, (int)split, chi, w, label, classify, margin, list, list_len,
+                                    listed, s);
     }
+#undef GWN_FAR
+    if (own) cudaFreeAsync(partial, s);
     GWN_LAUNCH_CHECK("k_boundary_far");
     return GWN_OK;
 }

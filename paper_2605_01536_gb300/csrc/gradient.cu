@@ -167,13 +167,15 @@ __global__ void __launch_bounds__(kGradThreads) k_gradient(const float *__restri
     }
 }
 
-__global__ void k_gradient_combine(const double *__restrict__ partial, int64_t n, int chunks, double scale,
-                                   float *__restrict__ grad) {
+// place: the queries' places in grad, or NULL: as they come
+__global__ void k_gradient_combine(const double *__restrict__ partial, const uint32_t *__restrict__ place, int64_t n,
+                                   int chunks, double scale, float *__restrict__ grad) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * n) return;
     double s = 0.0;
     for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * 3 * n + i];
-    grad[i] = (float)(s * scale);
+    const int64_t o = place ? 3 * (int64_t)place[i / 3] + i % 3 : i;
+    grad[o] = (float)(s * scale);
 }
 
 // Gradient of a node's expansion for two queries at (x, y, z) from its centre in
@@ -248,18 +250,18 @@ __device__ __forceinline__ void two_sum2(float2 &part, float2 &comp, float2 x) {
 // mesh's longest side (gpad): Algorithm 3's terms lose up to u h / rho^2 where a
 // boundary point h above the query stands rho beside its ray, and inside that margin
 // the terms are kept, so that the results differ from the direct sum's by rounding
-// everywhere.  perm: the queries' places in the output.
+// everywhere.  perm: the queries' places in the output; partial sums are in the queries' order.
 // Bound by issue (an expansion's gradient is about 560 instructions for two queries per
 // lane).  soup8, 200k queries: 59.3 -> 5.4 ms; soup6 (12k points), 100k: 1.98 -> 1.04 ms;
 // median error against FP64 on soup8 1.9e-5 -> 5.6e-6.  A truncation bound of 4e-6
 // instead of 2e-6: 5% faster.
 __global__ void __launch_bounds__(kGradThreads, 4)
-    k_gradient_far(const float *__restrict__ q, const uint32_t *__restrict__ perm, int64_t n,
+    k_gradient_far(const float *__restrict__ q, const uint32_t *__restrict__ perm, int64_t first, int64_t n,
                    const FarNode *__restrict__ nodes, const int32_t *__restrict__ roots, int nroots,
                    double *__restrict__ partial, const float *__restrict__ gcoef, const float4 *__restrict__ pts,
                    float *__restrict__ grad, unsigned long long *__restrict__ counters) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t qbase = ((int64_t)blockIdx.x * (kGradThreads / 32) + warp) * 64;
+    const int64_t qbase = first + ((int64_t)blockIdx.x * (kGradThreads / 32) + warp) * 64;   // queries [first, n)
     if (qbase >= n) return;
     const int64_t i0 = qbase + lane, i1 = i0 + 32;
     const bool ok0 = i0 < n, ok1 = i1 < n;
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(kGradThreads, 4)
         const int64_t o = perm[i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if (partial) partial[((int64_t)blockIdx.y * n + o) * 3 + c] = acc[3 * h + c];
+            if (partial) partial[((int64_t)blockIdx.y * (n - first) + (i - first)) * 3 + c] = acc[3 * h + c];
             else grad[3 * o + c] = (float)acc[3 * h + c];
         }
     }
@@ -384,19 +386,26 @@ gwn_status launch_gradient(const gwn_mesh *m, const float *q, int64_t n, float *
         double *partial = nullptr;
         const int64_t blocks = (n + 2 * kGradThreads - 1) / (2 * kGradThreads);
         const int64_t split = std::max<int64_t>(1, std::min<int64_t>((320 * (int64_t)sms + blocks - 1) / blocks, m->far_nroots));
+        const int64_t slice = split > 1 ? query_slice(n, sizeof(double) * 3 * split) : n;
         gwn_status st = [&]() -> gwn_status {
             GWN_CUDA_TRY(dev_alloc(&keys, sizeof(uint32_t) * n, s));
             GWN_CUDA_TRY(dev_alloc(&perm, sizeof(uint32_t) * n, s));
             GWN_CUDA_TRY(dev_alloc(&qs, sizeof(float) * 3 * n, s));
-            if (split > 1) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * 3 * split * n, s));
+            if (split > 1) GWN_CUDA_TRY(dev_alloc(&partial, sizeof(double) * 3 * split * slice, s));
             return order_queries(m, q, n, keys, perm, qs, s);
         }();
         if (st == GWN_OK) {
             ProfScope prof("gradient", s);
-            k_gradient_far<<<dim3((unsigned)blocks, (unsigned)split), kGradThreads, 0, s>>>(
-                qs, perm, n, m->far_nodes, m->far_roots, m->far_nroots, partial, m->far_gcoef, m->far_pts, grad,
-                m->counters);
-            if (partial) k_gradient_combine<<<grid_for(3 * n, 256), 256, 0, s>>>(partial, n, (int)split, 1.0, grad);
+            for (int64_t at = 0; at < n; at += slice) {
+                const int64_t end = std::min(n, at + slice), count = end - at;
+                const dim3 grid((unsigned)((count + 2 * kGradThreads - 1) / (2 * kGradThreads)), (unsigned)split);
+                k_gradient_far<<<grid, kGradThreads, 0, s>>>(qs, perm, at, end, m->far_nodes, m->far_roots, m->far_nroots,
+                                                             partial, m->far_gcoef, m->far_pts, grad, m->counters);
+                note_launches(1);
+                if (!partial) continue;
+                k_gradient_combine<<<grid_for(3 * count, 256), 256, 0, s>>>(partial, perm + at, count, (int)split, 1.0, grad);
+                note_launches(1);
+            }
         }
         for (void *p : {(void *)keys, (void *)perm, (void *)qs, (void *)partial})
             if (p) cudaFreeAsync(p, s);
@@ -422,7 +431,8 @@ gwn_status launch_gradient(const gwn_mesh *m, const float *q, int64_t n, float *
         dim3 grid((unsigned)qblocks, (unsigned)chunks);
         k_gradient<KP><<<grid, kGradThreads, smem, s>>>(q, n, m->bpts, m->npts, tile, chunk_len, partial, grad,
                                                         m->counters);
-        if (partial) k_gradient_combine<<<grid_for(3 * n, 256), 256, 0, s>>>(partial, n, (int)chunks, kInv4Pi, grad);
+        if (partial)
+            k_gradient_combine<<<grid_for(3 * n, 256), 256, 0, s>>>(partial, nullptr, n, (int)chunks, kInv4Pi, grad);
     }
     if (partial) cudaFreeAsync(partial, s);
     GWN_LAUNCH_CHECK("k_gradient");

@@ -239,8 +239,18 @@ gwn_status launch_boundary_far(const gwn_mesh *m, const float *q, int64_t n, con
 // Parts a call of n queries splits the boundary into (partial sums: n doubles a part)
 int64_t far_parts(const gwn_mesh *m, int64_t n);
 int64_t boundary_parts(const gwn_mesh *m, int64_t n, bool far);
-// query.cu: w = chi + (sum over chunks, in order) / 2pi of partial [chunks][n], then the labels
-void launch_boundary_combine(const double *partial, int64_t n, int chunks, const int32_t *chi, float *w,
+// Partial sums of a walk split into parts take at most this much at a time: more queries
+// run in slices of query_slice(n, bytes of one query's partial sums), multiples of 256.
+// (The boundary sum's take 100 MB at most and stay whole; 64 MiB cost 2M queries on soup8 4%
+// for the end of one more launch.  The gradient's would take 300 MB.)
+constexpr int64_t kPartialBytes = int64_t(128) << 20;
+inline int64_t query_slice(int64_t n, int64_t bytes) {
+    const int64_t most = (kPartialBytes / bytes) & ~int64_t(255), slices = (n + most - 1) / most;
+    return ((n + slices - 1) / slices + 255) & ~int64_t(255);
+}
+// query.cu: w = chi + (sum over chunks, in order) / 2pi of partial [chunks][n] for the
+// queries from first on, then the labels
+void launch_boundary_combine(const double *partial, int64_t first, int64_t n, int chunks, const int32_t *chi, float *w,
                              uint8_t *label, bool classify, float margin, int32_t *list,
                              unsigned long long *list_len, unsigned *listed, cudaStream_t s);
 // quant.cu: the fixed-point frame of the mesh (quantize_bits), written into the

@@ -523,15 +523,15 @@ __global__ void __launch_bounds__(256, 2) k_batch(const BatchMesh *__restrict__ 
 }
 
 // w = chi + (sum over chunks, in chunk order) / 2pi, then the labels
-__global__ void k_boundary_combine(const double *__restrict__ partial, int64_t n, int chunks,
+__global__ void k_boundary_combine(const double *__restrict__ partial, int64_t first, int64_t n, int chunks,
                                    const int32_t *__restrict__ chi, float *__restrict__ w,
                                    uint8_t *__restrict__ label, int classify, float margin,
                                    int32_t *__restrict__ list, unsigned long long *__restrict__ list_len,
                                    unsigned *__restrict__ listed) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, idx = first + i;
+    if (i >= n) return;
     double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * n + idx];
+    for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * n + i];
     const double wv = (double)chi[idx] + s * kInv2Pi;
     w[idx] = (float)wv;
     if (classify) {
@@ -910,10 +910,10 @@ gwn_status launch_chi_visits(const gwn_mesh *m, const float *q, int64_t n, int32
     return GWN_OK;
 }
 
-void launch_boundary_combine(const double *partial, int64_t n, int chunks, const int32_t *chi, float *w,
+void launch_boundary_combine(const double *partial, int64_t first, int64_t n, int chunks, const int32_t *chi, float *w,
                              uint8_t *label, bool classify, float margin, int32_t *list,
                              unsigned long long *list_len, unsigned *listed, cudaStream_t s) {
-    k_boundary_combine<<<grid_for(n, 256), 256, 0, s>>>(partial, n, chunks, chi, w, label, classify ? 1 : 0, margin,
+    k_boundary_combine<<<grid_for(n, 256), 256, 0, s>>>(partial, first, n, chunks, chi, w, label, classify ? 1 : 0, margin,
                                                         list, list_len, listed);
     note_launches(1);
 }
@@ -981,7 +981,7 @@ static gwn_status launch_bsum_kp(const gwn_mesh *m, const float *q, int64_t n, c
                                                                       margin, list, list_len, listed, m->counters);
     note_launches(1);
     if (partial) {
-        launch_boundary_combine(partial, n, (int)chunks, chi, w, label, classify, margin, list, list_len, listed, s);
+        launch_boundary_combine(partial, 0, n, (int)chunks, chi, w, label, classify, margin, list, list_len, listed, s);
         if (own) cudaFreeAsync(partial, s);
     }
     GWN_LAUNCH_CHECK("k_boundary_sum");
