@@ -85,7 +85,8 @@ typedef struct gwn_mesh gwn_mesh;
  * queries_per_thread or boundary_tile, chain_boundary -1 and fp64_cancel
  * -1 keep the boundary sum on the kernel that adds every edge; by default long boundaries
  * are summed over a hierarchy with expansions of their distant pieces (truncated at 1e-7
- * each) and small calls in one kernel. */
+ * each, or less where those of one query would add up to more than half of
+ * classify_margin) and small calls in one kernel. */
 typedef struct gwn_config {
     int32_t queries_per_thread;   /* boundary-sum kernel: queries held per thread (1,2,4,8) */
     int32_t boundary_tile;        /* boundary points staged in shared memory per step */

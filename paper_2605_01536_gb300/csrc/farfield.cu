@@ -65,7 +65,7 @@ constexpr int kFarWideLevel = 7;   // 128 leaves, about 2048 points
 template <int Threads>
 __global__ void __launch_bounds__(Threads) k_far_geom(FarShape sh, int64_t t0, const int32_t *__restrict__ cut,
                                                   const uint2 *__restrict__ ends, const float4 *__restrict__ pts,
-                                                  int64_t npts, const float *__restrict__ mesh_box,
+                                                  int64_t npts, const float *__restrict__ mesh_box, float eps,
                                                   FarNode *__restrict__ nodes) {
     constexpr int kWarps = Threads / 32;
     __shared__ float s_red[kWarps][8];
@@ -146,17 +146,17 @@ __global__ void __launch_bounds__(Threads) k_far_geom(FarShape sh, int64_t t0, c
     e *= 1.001f * 0.0795774715f;
     FarNode nd;
     nd.cx = cx; nd.cy = cy; nd.cz = cz;
-    // smallest x = r / s in [1.5, 2^14] with the truncation bound <= kFarEps
+    // smallest x = r / s in [1.5, 2^14] with the truncation bound <= eps
     auto bound = [&](float x) {
         const float y = 1.f / x, g = 1.f / (1.f - y);
         return e * exp2f(-(P + 2) * log2f(x)) * ((P + 1) * g + y * g * g);
     };
     float lo = 1.5f, hi = 16384.f;
-    if (bound(lo) <= kFarEps) hi = lo;
+    if (bound(lo) <= eps) hi = lo;
     else
         for (int it = 0; it < 30; ++it) {
             const float mid = sqrtf(lo * hi);
-            if (bound(mid) <= kFarEps) hi = mid;
+            if (bound(mid) <= eps) hi = mid;
             else lo = mid;
         }
     const bool leaf = l == 0;
@@ -494,19 +494,22 @@ __global__ void k_far_roots(FarShape sh, int l, int32_t *__restrict__ roots) {
 }
 
 // Cost of the hierarchical sum at sample points of the mesh's box (a fixed hash
-// sequence), in the operation counts of the query kernel, summed into *cost.
+// sequence), in the operation counts of the query kernel, summed into *cost, and the
+// expansions each sample takes, added to taken[sample].
 __device__ __forceinline__ float far_hash(uint32_t x) {
     x ^= x >> 16; x *= 0x7feb352du; x ^= x >> 15; x *= 0x846ca68bu; x ^= x >> 16;
     return (float)(x >> 8) * (1.0f / 16777216.0f);
 }
 constexpr int kFarVisitCost = 15, kFarEvalCost = 280, kFarChordCost = 80, kFarEdgeCost = 32;
 __global__ void k_far_sample(const FarNode *__restrict__ nodes, const int32_t *__restrict__ roots, int nroots,
-                             const float *__restrict__ box, int nsample, unsigned long long *__restrict__ cost) {
+                             const float *__restrict__ box, int nsample, unsigned long long *__restrict__ cost,
+                             uint32_t *__restrict__ taken) {
     // one thread per (sample, subtree): a whole walk is a serial chain of hundreds of loads
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t / nroots;
     unsigned long long c = 0;
     if (i < nsample) {
+        uint32_t expansions = 0;
         const float x = box[0] + (box[3] - box[0]) * far_hash(3u * i + 1u),
                     y = box[1] + (box[4] - box[1]) * far_hash(3u * i + 2u),
                     z = box[2] + (box[5] - box[2]) * far_hash(3u * i + 3u);
@@ -519,12 +522,14 @@ __global__ void k_far_sample(const FarNode *__restrict__ nodes, const int32_t *_
             c += kFarVisitCost;
             if (dx * dx + dy * dy + dz * dz > nd.r2acc && !hit) {
                 c += kFarEvalCost + kFarChordCost * nd.nchord;
+                ++expansions;
                 node = nd.skip;
             } else {
                 if (nd.skip == node + 1) c += kFarEdgeCost * nd.count;
                 ++node;
             }
         }
+        if (expansions) atomicAdd(&taken[i], expansions);
     }
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(cost, c);
@@ -549,23 +554,39 @@ gwn_status build_far(gwn_mesh *m, float4 *pts, const uint2 *ends, cudaStream_t s
     Cplx *raw = nullptr;
     FarNode *nodes = nullptr;
     float *coef = nullptr;
-    unsigned long long *cost = nullptr, cost_h = 0;
+    struct Sample {
+        unsigned long long cost;
+        uint32_t taken[kSamples];
+    } *sample = nullptr, sample_h;
     GWN_CUDA_TRY(dev_alloc(&cut, sizeof(int32_t) * (sh.nleaf + 1), s));
-    GWN_CUDA_TRY(dev_alloc(&cost, sizeof(unsigned long long), s));
+    GWN_CUDA_TRY(dev_alloc(&sample, sizeof(Sample), s));
     GWN_CUDA_TRY(dev_alloc(&nodes, sizeof(FarNode) * sh.total, s));
     GWN_CUDA_TRY(dev_alloc(&roots, sizeof(int32_t) * (nroots + 1), s));
-    GWN_CUDA_TRY(cudaMemsetAsync(cost, 0, sizeof(unsigned long long), s));
     k_far_cuts<<<grid_for(sh.nleaf + 1, 256), 256, 0, s>>>(ends, npts, sh.nleaf, cut);
     const int64_t wide = sh.top >= kFarWideLevel ? sh.off[kFarWideLevel] : sh.total;   // first wide node
-    if (wide < sh.total)
-        k_far_geom<1024><<<(unsigned)(sh.total - wide), 1024, 0, s>>>(sh, wide, cut, ends, pts, npts, m->box, nodes);
-    k_far_geom<64><<<(unsigned)wide, 64, 0, s>>>(sh, 0, cut, ends, pts, npts, m->box, nodes);
     k_far_roots<<<1, kFarRoots + 32, 0, s>>>(sh, rl, roots);
-    k_far_sample<<<grid_for((int64_t)kSamples * nroots, 128), 128, 0, s>>>(nodes, roots, nroots, m->box, kSamples, cost);
-    GWN_CUDA_TRY(cudaMemcpyAsync(&cost_h, cost, sizeof(cost_h), cudaMemcpyDeviceToHost, s));
-    GWN_CUDA_TRY(cudaStreamSynchronize(s));
-    m->far_cost = (double)cost_h / kSamples;
-    if (m->far_cost <= kFarWorth * 28.0 * (double)npts) {
+    const double budget = 0.5 * (m->cfg.classify_margin > 0.f ? m->cfg.classify_margin : 1e-4f);
+    double eps = kFarEps, first_cost = 0.0;
+    bool held = false;   // the expansions' bounds add up to no more than the budget
+    for (int round = 0; round < 4 && !held && eps >= kFarEpsMin; ++round) {
+        if (wide < sh.total)
+            k_far_geom<1024><<<(unsigned)(sh.total - wide), 1024, 0, s>>>(sh, wide, cut, ends, pts, npts, m->box, (float)eps,
+                                                                         nodes);
+        k_far_geom<64><<<(unsigned)wide, 64, 0, s>>>(sh, 0, cut, ends, pts, npts, m->box, (float)eps, nodes);
+        GWN_CUDA_TRY(cudaMemsetAsync(sample, 0, sizeof(Sample), s));
+        k_far_sample<<<grid_for((int64_t)kSamples * nroots, 128), 128, 0, s>>>(nodes, roots, nroots, m->box, kSamples,
+                                                                              &sample->cost, sample->taken);
+        GWN_CUDA_TRY(cudaMemcpyAsync(&sample_h, sample, sizeof(Sample), cudaMemcpyDeviceToHost, s));
+        GWN_CUDA_TRY(cudaStreamSynchronize(s));
+        m->far_cost = (double)sample_h.cost / kSamples;
+        if (round == 0) first_cost = m->far_cost;
+        if (m->far_cost > kFarWorth * 28.0 * (double)npts) break;
+        const double most = *std::max_element(sample_h.taken, sample_h.taken + kSamples);
+        held = most * eps <= budget;
+        if (!held) eps *= 0.9 * std::pow(budget / (most * eps), 1.25);   // (expansions grow like eps^-0.2)
+    }
+    // (the gradient's radii have a bound of their own: first_cost decides whether it gets the hierarchy)
+    if (first_cost <= kFarWorth * 28.0 * (double)npts) {
         GWN_CUDA_TRY(dev_alloc(&raw, sizeof(Cplx) * kFarRaw * sh.total, s));
         GWN_CUDA_TRY(dev_alloc(&coef, sizeof(float) * kFarCoef * sh.total, s));
         k_far_leaf_moments<<<grid_for(sh.nleaf, 2), 64, 0, s>>>(sh, nodes, pts, raw);
@@ -581,14 +602,14 @@ gwn_status build_far(gwn_mesh *m, float4 *pts, const uint2 *ends, cudaStream_t s
         m->far_nn = sh.total;
         m->far_roots = roots;
         m->far_nroots = nroots;
-        m->far_sum = m->far_cost <= kFarWorth * direct_cost(m);
+        m->far_sum = held && m->far_cost <= kFarWorth * direct_cost(m);
     } else {
         cudaFreeAsync(nodes, s);
         cudaFreeAsync(pts, s);
         cudaFreeAsync(roots, s);
     }
     cudaFreeAsync(cut, s);
-    cudaFreeAsync(cost, s);
+    cudaFreeAsync(sample, s);
     GWN_LAUNCH_CHECK("boundary hierarchy");
     return GWN_OK;
 }
