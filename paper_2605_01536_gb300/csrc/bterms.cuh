@@ -576,9 +576,16 @@ static_assert(sizeof(TriLoop) == 80, "TriLoop must be 80 bytes");
 constexpr float kTriAccept = 0.05f;
 constexpr float kTriSpread = 0.125f;   // weight of g
 
-// det of a triangle's term from the nearest vertex; a, b, c: the relative vectors, ia, ib,
-// ic: their reciprocal lengths
-__device__ __forceinline__ float tri_det_near(float4 n, float3 a, float3 b, float3 c, float ia, float ib, float ic) {
+// A triangle's term by itself, det from the nearest vertex; a, b, c: the relative vectors.
+// The unit vectors are exact down to lengths of 3e-19 (a distance that something is added
+// to, as the edge terms' 1e-37, is no harm there, where n and d shrink alike, but den
+// is 1 plus products of unit vectors: w off by 0.1 at 1e-18).  Returns the smallest squared length.
+__device__ __forceinline__ float tri_own(float4 n, float3 a, float3 b, float3 c, float &det, float &den) {
+    const float la = a.x * a.x + a.y * a.y + a.z * a.z, lb = b.x * b.x + b.y * b.y + b.z * b.z,
+                lc = c.x * c.x + c.y * c.y + c.z * c.z;
+    float ia = sfu_rsqrt(fmaxf(la, 1e-37f)), ib = sfu_rsqrt(fmaxf(lb, 1e-37f)), ic = sfu_rsqrt(fmaxf(lc, 1e-37f));
+    den = 1.f + (a.x * b.x + a.y * b.y + a.z * b.z) * (ia * ib) + (a.x * c.x + a.y * c.y + a.z * c.z) * (ia * ic) +
+          (b.x * c.x + b.y * c.y + b.z * c.z) * (ib * ic);
     if (ib >= fmaxf(ia, ic)) {
         const float i = ia;
         a = b;
@@ -590,7 +597,8 @@ __device__ __forceinline__ float tri_det_near(float4 n, float3 a, float3 b, floa
         ia = ic;
         ic = i;
     }
-    return (a.x * n.x + a.y * n.y + a.z * n.z) * ia * (n.w * (ib * ic));
+    det = (a.x * n.x + a.y * n.y + a.z * n.z) * ia * (n.w * (ib * ic));
+    return fminf(la, fminf(lb, lc));
 }
 
 // The exact predicate, where the FP32 filter of tri_cross cannot decide.
@@ -671,16 +679,11 @@ __device__ __noinline__ void tri_deferred(const unsigned *queue, int count, cons
             const int cr = inbox ? tri_cross(T, qx, qy, qz, &edges, counters) : 0;
             float t = 0.f;
             if (fail && !edges) {   // a well-conditioned angle away from the cut takes its own atan2
-                const float ax = T.a.x - qx, ay = T.a.y - qy, az = T.a.z - qz, bx = T.b.x - qx, by = T.b.y - qy,
-                            bz = T.b.z - qz, cx = T.c.x - qx, cy = T.c.y - qy, cz = T.c.z - qz;
-                // (1e-37: a coincident vertex gives a finite reciprocal length)
-                const float ia = sfu_rsqrt(ax * ax + ay * ay + az * az + 1e-37f), ib = sfu_rsqrt(bx * bx + by * by + bz * bz + 1e-37f),
-                            ic = sfu_rsqrt(cx * cx + cy * cy + cz * cz + 1e-37f);
-                const float den = 1.f + (ax * bx + ay * by + az * bz) * (ia * ib) + (ax * cx + ay * cy + az * cz) * (ia * ic) +
-                                  (bx * cx + by * cy + bz * cz) * (ib * ic);
-                const float det = tri_det_near(T.n, make_float3(ax, ay, az), make_float3(bx, by, bz), make_float3(cx, cy, cz),
-                                               ia, ib, ic);
-                if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f)) t = fast_atan2(det, den);
+                float det, den;
+                const float least = tri_own(T.n, make_float3(T.a.x - qx, T.a.y - qy, T.a.z - qz),
+                                            make_float3(T.b.x - qx, T.b.y - qy, T.b.z - qz),
+                                            make_float3(T.c.x - qx, T.c.y - qy, T.c.z - qz), det, den);
+                if (den * den + det * det > 0.01f && (den > 0.f || fabsf(det) > 0.1f) && least > 1e-37f) t = fast_atan2(det, den);
                 else edges = true;
             }
             const double sum = edges ? (double)tri_edges(T, j, e & 127u, qx, qy, qz, cq, counters)
@@ -710,6 +713,10 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
     if ((threadIdx.x & 31) == 0) *cq.count = 0;
     __syncwarp();
     float2 re[KP], im[KP], part[KP], comp[KP];
+    unsigned live = 0;   // query slots that are not padding past n (NaN), whose sums are never read
+#pragma unroll
+    for (int k = 0; k < KP; ++k)
+        live |= (nqx[k].x == nqx[k].x ? 1u : 0u) << (2 * k) | (nqx[k].y == nqx[k].y ? 2u : 0u) << (2 * k);
     int q_count = 0;   // entries in the warp's queue
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
@@ -743,10 +750,9 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
                 const float2 ax = add2(bc2(a.x), nqx[k]), ay = add2(bc2(a.y), nqy[k]), az = add2(bc2(a.z), nqz[k]);
                 const float2 px = add2(bc2(b.x), nqx[k]), py = add2(bc2(b.y), nqy[k]), pz = add2(bc2(b.z), nqz[k]);
                 const float2 cx = add2(bc2(c.x), nqx[k]), cy = add2(bc2(c.y), nqy[k]), cz = add2(bc2(c.z), nqz[k]);
-                // (1e-37: a coincident vertex gives a finite reciprocal length)
-                const float2 la = fma2(ax, ax, fma2(ay, ay, fma2(az, az, bc2(1e-37f))));
-                const float2 lb = fma2(px, px, fma2(py, py, fma2(pz, pz, bc2(1e-37f))));
-                const float2 lc = fma2(cx, cx, fma2(cy, cy, fma2(cz, cz, bc2(1e-37f))));
+                const float2 la = fma2(ax, ax, fma2(ay, ay, mul2(az, az)));
+                const float2 lb = fma2(px, px, fma2(py, py, mul2(pz, pz)));
+                const float2 lc = fma2(cx, cx, fma2(cy, cy, mul2(cz, cz)));
                 const float2 ia = make_float2(sfu_rsqrt(la.x), sfu_rsqrt(la.y)), ib = make_float2(sfu_rsqrt(lb.x), sfu_rsqrt(lb.y)),
                              ic = make_float2(sfu_rsqrt(lc.x), sfu_rsqrt(lc.y));
                 const float2 ab = fma2(ax, px, fma2(ay, py, mul2(az, pz)));
@@ -757,13 +763,14 @@ __device__ __forceinline__ void tri_accumulate(const TriLoop *__restrict__ tris,
                 const float2 dn = fma2(ax, bc2(N.x), fma2(ay, bc2(N.y), mul2(az, bc2(N.z))));
                 const float2 g = mul2(bc2(N.w), ibc);
                 det[k] = mul2(mul2(dn, ia), g);
-                // a NaN (a padding query past n) counts as accepted: its sum is never read
+                // (an infinite reciprocal length, at a vertex, makes v NaN or -infinity: not accepted)
                 const float2 v = fma2(bc2(-kTriSpread), g,
                                       fma2(bc2(kTanGroup), den[k], neg2(make_float2(fabsf(det[k].x), fabsf(det[k].y)))));
-                fail |= (v.x <= kTriAccept ? 1u : 0u) << (2 * k) | (v.y <= kTriAccept ? 2u : 0u) << (2 * k);
+                fail |= (v.x > kTriAccept ? 0u : 1u) << (2 * k) | (v.y > kTriAccept ? 0u : 2u) << (2 * k);
                 inbox |= (-nqx[k].x >= bx.x && -nqx[k].x <= bx.y && -nqy[k].x >= bx.z && -nqy[k].x <= bx.w && -nqz[k].x <= a.w ? 1u : 0u) << (2 * k) |
                          (-nqx[k].y >= bx.x && -nqx[k].y <= bx.y && -nqy[k].y >= bx.z && -nqy[k].y <= bx.w && -nqz[k].y <= a.w ? 2u : 0u) << (2 * k);
             }
+            fail &= live;
             // near the triangle, or below its box (every lane of the warp is here)
             if (__any_sync(0xffffffffu, fail | inbox)) {
                 const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;

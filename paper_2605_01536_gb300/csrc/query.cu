@@ -776,10 +776,9 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
                 const float2 ax = add2(bc2(A.x), nqx[k]), ay = add2(bc2(A.y), nqy[k]), az = add2(bc2(A.z), nqz[k]);
                 const float2 bx = add2(bc2(B.x), nqx[k]), by = add2(bc2(B.y), nqy[k]), bz = add2(bc2(B.z), nqz[k]);
                 const float2 cx = add2(bc2(C.x), nqx[k]), cy = add2(bc2(C.y), nqy[k]), cz = add2(bc2(C.z), nqz[k]);
-                // (1e-37: a coincident vertex gives a finite reciprocal length)
-                const float2 la = fma2(ax, ax, fma2(ay, ay, fma2(az, az, bc2(1e-37f))));
-                const float2 lb = fma2(bx, bx, fma2(by, by, fma2(bz, bz, bc2(1e-37f))));
-                const float2 lc = fma2(cx, cx, fma2(cy, cy, fma2(cz, cz, bc2(1e-37f))));
+                const float2 la = fma2(ax, ax, fma2(ay, ay, mul2(az, az)));
+                const float2 lb = fma2(bx, bx, fma2(by, by, mul2(bz, bz)));
+                const float2 lc = fma2(cx, cx, fma2(cy, cy, mul2(cz, cz)));
                 const float2 ia = make_float2(sfu_rsqrt(la.x), sfu_rsqrt(la.y)), ib = make_float2(sfu_rsqrt(lb.x), sfu_rsqrt(lb.y)),
                              ic = make_float2(sfu_rsqrt(lc.x), sfu_rsqrt(lc.y));
                 const float2 ab = fma2(ax, bx, fma2(ay, by, mul2(az, bz)));
@@ -792,14 +791,17 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
                 const float2 det = mul2(mul2(dn, ia), g);
                 const float2 v = fma2(bc2(-kTriSpread), g,
                                       fma2(bc2(kTanGroup), den, neg2(make_float2(fabsf(det.x), fabsf(det.y)))));
-                const bool px = v.x > kTriAccept, py = v.y > kTriAccept;
+                const bool px = v.x > kTriAccept, py = v.y > kTriAccept;   // (not if NaN, at a vertex)
                 const float4 N = make_float4(A.w, B.w, C.w, h);
-                if (!px)
-                    part[k].x += fast_atan2(tri_det_near(N, make_float3(ax.x, ay.x, az.x), make_float3(bx.x, by.x, bz.x),
-                                                         make_float3(cx.x, cy.x, cz.x), ia.x, ib.x, ic.x), den.x);
-                if (!py)
-                    part[k].y += fast_atan2(tri_det_near(N, make_float3(ax.y, ay.y, az.y), make_float3(bx.y, by.y, bz.y),
-                                                         make_float3(cx.y, cy.y, cz.y), ia.y, ib.y, ic.y), den.y);
+                float od, oe;
+                if (!px) {
+                    tri_own(N, make_float3(ax.x, ay.x, az.x), make_float3(bx.x, by.x, bz.x), make_float3(cx.x, cy.x, cz.x), od, oe);
+                    part[k].x += fast_atan2(od, oe);
+                }
+                if (!py) {
+                    tri_own(N, make_float3(ax.y, ay.y, az.y), make_float3(bx.y, by.y, bz.y), make_float3(cx.y, cy.y, cz.y), od, oe);
+                    part[k].y += fast_atan2(od, oe);
+                }
                 const float2 fd = make_float2(px ? den.x : 1.f, py ? den.y : 1.f);
                 const float2 fn = make_float2(px ? det.x : 0.f, py ? det.y : 0.f);
                 const float2 r = fma2(re[k], fd, neg2(mul2(im[k], fn)));

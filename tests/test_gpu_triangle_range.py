@@ -52,3 +52,22 @@ def test_scaled_by_a_power_of_two(k, nt):
     assert np.array_equal(out[1][clear], ref[1][clear]) and np.array_equal(out[2][clear], ref[2][clear])
     for a, b in zip(out[3:], ref[3:]):
         assert np.isfinite(a).all() and np.abs(a.astype(np.float64) - b).max() <= TOL
+
+
+@pytest.mark.parametrize("k", [-40, -44])
+def test_below_vertices_at_small_scales(k):
+    """Queries straight below vertices at 1e-4 to 1 edge lengths, down to distances of 1e-18, where 1e-37
+    beside the squared distance shortens a unit vector by far more than rounding.  (Beside a vertex the
+    edges' own terms are off there; straight below it n and d shrink alike, down to 2^-44.)"""
+    import paper_2605_01536_gb300 as gwn
+    rng = np.random.default_rng(3)
+    mesh = gen.random_soup(400, rng)
+    p = mesh.V[rng.integers(0, len(mesh.V), 17_000)]
+    Q = (p - np.float32([0, 0, 1]) * (0.2 * 10.0 ** rng.uniform(-4, 0, (len(p), 1)))).astype(np.float32)
+    got = []
+    for s in (np.float32(1), np.float32(2.0 ** k)):
+        q = torch.from_numpy(Q * s).cuda()
+        with gwn.Mesh(mesh.V * s, mesh.F) as m, gwn.Batch([m], [len(Q)]) as b:
+            got.append([x.cpu().numpy().astype(np.float64) for x in (m.query(q)[0], m.classify(q, want_w=True)[1], b.run(q)[0])])
+    for a, b in zip(got[1], got[0]):
+        assert np.abs(a - b).max() <= TOL, np.abs(a - b).max()
