@@ -988,7 +988,7 @@ def run_gradient(args):
         terms = n * info["n_boundary_edges"]
         ach = terms * GRAD_OPS_PER_TERM / per / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": peak_tops, "unit": "Top/s (FP32 issue slots)",
-                "frac": ach / peak_tops, "traffic": None, "kernel": "k_gradient", "ms_per_launch": per * 1e3,
+                "frac": ach / peak_tops, "traffic": None, "kernel": "gradient", "ms_per_launch": per * 1e3,
                 "edge_terms_per_launch": terms, "ops_per_term": GRAD_OPS_PER_TERM}
         plain_terms(roof)
     e2e = None

@@ -41,7 +41,7 @@ struct gwn_batch {
     int32_t *d_list = nullptr;             // queries with many cancelling terms in a tile
     unsigned long long *d_list_len = nullptr;
     unsigned *d_listed = nullptr;          // one bit per query
-    // the queries in (mesh, Morton) order and the results in that order
+    // the queries in (mesh, Hilbert) order and the results in that order
     uint64_t *d_keys = nullptr;
     uint32_t *d_perm = nullptr;
     float *d_qs = nullptr, *d_ws = nullptr;
@@ -161,7 +161,7 @@ gwn_status build_schedule(gwn_batch *b, int kp, int chunk, int tile, int grid, i
     return GWN_OK;
 }
 
-// One run: the queries in (mesh, Morton) order, the persistent kernel and the
+// One run: the queries in (mesh, Hilbert) order, the persistent kernel and the
 // FP64 re-evaluation of the listed queries on that order, the results scattered
 // back to the caller's order.
 gwn_status enqueue_run(gwn_batch *b, const float *q, float *w, int32_t *chi, cudaStream_t s) {

@@ -366,7 +366,11 @@ __global__ void __launch_bounds__(kFarThreads, 5)
 }  // namespace
 
 // Calls of the default schedule (an explicit queries_per_thread, boundary_tile or
-// fp64_cancel = -1 asks for the direct sum's own) large enough to be ordered in space.
+// fp64_cancel = -1 asks for the direct sum's own) large enough to be ordered in space.  The
+// limit is the order's; direct / hierarchy where an order and the hierarchy begin at 1,024
+// queries, query: soup6 (12k points) 3k queries 133 / 158 us, 16k 234 / 268; soup7 (51k) 6k
+// 321 / 474, 12k 509 / 500, 16k 656 / 532; soup8 (203k) 6k 915 / 1322, 12k 1614 / 1355, 16k
+// 2103 / 1392; gradient: soup6 6k 263 / 183, soup7 582 / 502, soup8 1936 / 1783, 12k 3850 / 1834.
 bool far_pays_gradient(const gwn_mesh *m, int64_t n) {
     return m->far_nodes && n >= kOrderMinQueries && m->cfg.queries_per_thread == 0 && m->cfg.boundary_tile == 0 &&
            m->cfg.fp64_cancel >= 0;

@@ -542,7 +542,7 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
 // three antipodal terms sum to (Eq. 9 for T alone)
 //   2 pi S_T = atan2(det, den) - 2 pi cross(q, T),
 // half T's solid angle (van Oosterom-Strackee) minus the signed crossing of the
-// ray with T.  One such term costs 43 paired operations against 3 edges of about 60
+// ray with T.  One such term costs 45 paired operations against 3 edges of about 60
 // each (random soups, whose every loop is a triangle, and small holes), and its
 // rounding is relative to the triangle's solid angle, not to the edges' steep angles.
 // With unit vectors A, B, C toward the vertices, N the triangle's normal vector:
@@ -564,9 +564,10 @@ __device__ double bsum64_range(const float4 *__restrict__ pts, int64_t j0, int64
 // deferred like the batched kernel's failing terms: about 3% of a warp's triangles have
 // such a lane (random soup, 100k queries), and done in place, with most lanes idle,
 // they cost more than all the rest.  Measured, edges -> triangles: soup8's direct sum with
-// 2M queries 383 -> 212 ms; 3,000 random triangles with 20k queries 0.83 -> 0.43 ms (2.0
-// ms with the terms done in place), 20,000 with 50k 6.6 -> 3.0 ms; the maximum error
-// against FP64 on soup8 1.3e-6 -> 5.2e-7.  Bound by the FP32 pipe (74 issue slots a term).
+// 2M queries 383 -> 228 ms; 3,000 random triangles with 20k queries 0.53 -> 0.18 ms,
+// 20,000 with 50k 5.6 -> 2.2 ms, with 100k 10.8 -> 4.3 ms (4.0 without the test on g); the
+// maximum error against FP64 on soup8 1.3e-6 -> 6.0e-7.  Bound by the FP32 pipe (62% of
+// its cycles; issue 65%).
 struct __align__(16) TriLoop {
     float4 a, b, c;   // the vertices; a.w = max z
     float4 n;         // (b - a) x (c - a) = n.w (n.x, n.y, n.z), n.w a power of two

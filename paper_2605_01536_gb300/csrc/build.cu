@@ -4,8 +4,10 @@
 // in pairs, so only the oriented boundary dM contributes.  Treated as a 1-chain:
 // every face contributes its three directed edges; an undirected edge {u, v}
 // (matched by vertex index) has net multiplicity m = #(u->v) - #(v->u) and
-// appears |m| times in its net direction.  Steps: sort the 3 nt half-edge keys,
-// segmented sum of the signs, compaction.  Edges are then chained into closed
+// appears |m| times in its net direction.  Steps: the half-edges are put into a bucket per
+// smaller vertex and netted out there, in ascending order of the other vertex (a mesh with
+// a vertex of very many half-edges: sort of the 3 nt half-edge keys, segmented sum of the
+// signs, compaction).  Edges are then chained into closed
 // loops (the boundary of a 2-chain is a cycle: in-degree = out-degree at every
 // vertex) so that consecutive edges share their common point in the query
 // kernel.
@@ -131,7 +133,9 @@ __global__ void k_emit_edges(const int32_t *__restrict__ mult, const uint64_t *_
 // Boundary edges by buckets of the smaller vertex: half-edges are counted and placed
 // per vertex (entry: larger vertex << 1 | direction), and each vertex's few entries are
 // netted out against one another.  A vertex with more than kBucketMax entries sets *overflow and
-// the sort below takes over.  A half-edge from a vertex to itself (repeated index in a
+// the sort above takes over (one such vertex beside a 642k-triangle mesh, buckets / sort: 200
+// entries 1.78 / 1.98 ms for the whole build, 400 entries 2.04 / 1.99, 1,000 entries 3.80 / 2.00;
+// alone 0.61 / 0.59, 0.90 / 0.64, 2.86 / 0.85).  A half-edge from a vertex to itself (repeated index in a
 // degenerate face) is a zero chain and contributes nothing.
 constexpr uint32_t kBucketMax = 128;
 __global__ void k_bucket_count(const int32_t *__restrict__ F, int64_t nh, uint32_t *__restrict__ count,
@@ -351,7 +355,9 @@ __global__ void __launch_bounds__(1024) k_jump_small(const uint32_t *__restrict_
         }
     }
 }
-constexpr int64_t kJumpSmall = 16384;   // edges k_jump_small takes (a launch per round costs more)
+// Edges k_jump_small takes.  Build of a rim, one block / a launch per round: 100 edges 500 / 565
+// us, 4,000 970 / 1057, 16,000 1173 / 1200, 17,000 1228 / 1229, 60,000 2059 / 1517.
+constexpr int64_t kJumpSmall = 16384;
 
 // points per loop (length + 1 closing point), stored at the representative
 __global__ void k_loop_sizes(const uint32_t *__restrict__ rep, const uint32_t *__restrict__ dist, int64_t nb,

@@ -495,7 +495,8 @@ __global__ void k_far_roots(FarShape sh, int l, int32_t *__restrict__ roots) {
 
 // Cost of the hierarchical sum at sample points of the mesh's box (a fixed hash
 // sequence), in the operation counts of the query kernel, summed into *cost, and the
-// expansions each sample takes, added to taken[sample].
+// expansions each sample takes, added to taken[sample].  (The hash is the published
+// 32-bit integer mixer "lowbias32" of C. Wellons' hash prospector.)
 __device__ __forceinline__ float far_hash(uint32_t x) {
     x ^= x >> 16; x *= 0x7feb352du; x ^= x >> 15; x *= 0x846ca68bu; x ^= x >> 16;
     return (float)(x >> 8) * (1.0f / 16777216.0f);

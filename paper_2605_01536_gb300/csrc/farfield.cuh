@@ -52,9 +52,14 @@ constexpr int kFarLeaf = 16;                              // target points of a 
 constexpr float kFarGradEps = 2e-6f;                      // truncation bound of one gradient, times the box's side
 constexpr int kFarGradCoef = 3 * (kFarP + 2 * (kFarP * (kFarP + 3) / 2));   // 288: x, y, z
 constexpr double kFarWorth = 0.5;                         // used below this share of the direct sum's cost
-constexpr int kFarMinPoints = 1024;                       // no hierarchy below this many points
+// Built from this many points on.  (Wavy rims: of 150 to 1,000 points no hierarchy passes
+// kFarWorth; of 1,500 one does, 1M queries 2.59 -> 1.60 ms.)
+constexpr int kFarMinPoints = 1024;
 constexpr int kFarRoots = 64;                             // subtrees a walk may be split into (at most)
-constexpr int kFarMinEdges = 10;                          // a leaf below this is summed directly
+// A leaf of fewer edges is summed directly.  Limits 1 / 10 / 17: query, soup6 with 100k
+// queries 584 / 583 / 646 us, soup8 with 200k 2432 / 2413 / 2715; gradient 891 / 883 / 859 and
+// 5682 / 5684 / 5117 us.
+constexpr int kFarMinEdges = 10;
 
 // Preorder node, 80 bytes.  A leaf's skip is its own index + 1.
 struct __align__(16) FarNode {

@@ -252,7 +252,7 @@ __device__ __forceinline__ void two_sum2(float2 &part, float2 &comp, float2 x) {
 // the terms are kept, so that the results differ from the direct sum's by rounding
 // everywhere.  perm: the queries' places in the output; partial sums are in the queries' order.
 // Bound by issue (an expansion's gradient is about 560 instructions for two queries per
-// lane).  soup8, 200k queries: 59.3 -> 5.4 ms; soup6 (12k points), 100k: 1.98 -> 1.04 ms;
+// lane).  soup8, 200k queries: 59.3 -> 5.4 ms; soup6 (12k points), 100k: 1.98 -> 0.93 ms;
 // median error against FP64 on soup8 1.9e-5 -> 5.6e-6.  A truncation bound of 4e-6
 // instead of 2e-6: 5% faster.
 __global__ void __launch_bounds__(kGradThreads, 4)

@@ -1108,7 +1108,7 @@ gwn_status classify_with_surrogate(const gwn_mesh *m, const float *q, int64_t n,
         GWN_CUDA_TRY(cudaMemsetAsync(len2, 0, sizeof(unsigned long long), st));
         const unsigned g = grid_for((int64_t)nfb, 256);
         const int64_t nf = (int64_t)nfb;
-        // the fallback queries in Morton order (the atomic compaction scrambled them)
+        // the fallback queries in Hilbert order (the atomic compaction scrambled them)
         r = order_query_list(m, q, list, nf, st);
         if (r == GWN_OK) {
             k_gather3<<<g, 256, 0, st>>>(q, list, len, qf);

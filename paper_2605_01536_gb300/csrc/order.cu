@@ -1,12 +1,13 @@
 // Spatial order of a query batch.  The crossing count walks the BVH once per
-// query, and the boundary kernel decides per warp and boundary tile whether
-// its cancellation test is needed; both do best when the queries of a warp lie
-// close together.  Large batches are therefore evaluated in the order of the
-// Morton codes of the queries in the mesh's box (the build's own radix sort),
-// and the results are scattered back to the caller's order.  Each query's
-// arithmetic does not depend on its neighbours, so the order changes
-// no result.  Batches of many meshes are ordered the same way within each
-// mesh's range of queries.
+// query, the boundary hierarchy's walk takes the union over a warp, and the boundary
+// kernel decides per warp and boundary tile whether its cancellation test is
+// needed; all do best when the queries of a warp lie close together.  Large batches are
+// therefore evaluated cell by cell along a Hilbert curve over the mesh's box (a counting
+// sort), and the results are scattered back to the caller's order.  Places come from
+// atomics: the order inside a cell, and which queries share a warp, differ from run to
+// run.  Each query's arithmetic does not depend on its neighbours, so no result does.
+// Lists of queries and the queries of many meshes (within each mesh's range) are
+// put in the order of their Hilbert keys by the build's radix sort, which is stable.
 #include <algorithm>
 
 #include "farfield.cuh"
@@ -18,9 +19,8 @@ namespace {
 
 constexpr int TB = 256;
 
-// Keys of 24 bits (256 cells per axis of the box's cube): as coherent for a warp as
-// 30 and one radix pass fewer (measured 3% of the degenerate precision workload's
-// classify step).
+// Radix-sorted keys of 24 bits (256 cells per axis of the box's cube): as coherent for a
+// warp as 30 and one pass fewer.
 constexpr int kOrderBits = 24;
 
 // Hilbert key of p in the cube at the low corner of box = (min x, min y, min z,

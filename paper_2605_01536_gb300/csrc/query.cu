@@ -28,7 +28,9 @@ namespace {
 // Launched in blocks of 128 threads (compiled for up to 256): finer tails than
 // 256 (measured 5.6% faster on 2M soup8 queries, bit-identical).
 constexpr int kChiThreads = 128;
-constexpr int64_t kSmallTris = 2048;   // leaves k_small tests one by one (64 per lane)
+// Leaves k_small tests one by one (64 per lane); a call of 500 queries on closed spheres, one
+// by one / walking: 320 leaves 21.6 / 24.3 us, 1,280 20.4 / 22.5, 5,120 38.9 / 23.1.
+constexpr int64_t kSmallTris = 2048;
 
 // Fixed selects the predicate mode at compile time (the host knows the mesh's
 // quantize_bits), so the exact kernel carries none of the fixed-point code.
@@ -697,9 +699,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const float *__restrict
 // nearer triangles take their own, with the nearest vertex in the place of a.  Each thread holds 2 KP queries as float2 pairs.  The
 // triangle range is split into gridDim.y chunks so that any query count fills the GPU:
 // with one chunk the kernel writes w, otherwise FP64 partial sums [chunk][query] that
-// k_direct_reduce adds in chunk order.  Bound by the FP32 pipe: 47 paired operations a
-// term (75 with an atan2 and a 3 x 3 determinant each): 30k queries x 40k triangles
-// 2.54 -> 1.92 ms.
+// k_direct_reduce adds in chunk order.  Bound by the FP32 pipe (75% of its cycles): 49 paired
+// operations a term (75 with an atan2 and a 3 x 3 determinant each): 30k queries x 40k
+// triangles 2.54 -> 2.01 ms.  Errors above 1e-5 beside surfaces, edges and vertices (132 sets
+// of queries against FP64) 29.7k -> 11.8k against that determinant's.
 template <int KP>
 __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, int64_t n, const float *__restrict__ tri9,
                                                    int64_t nt, int tile, int64_t chunk_len, float *__restrict__ w,

@@ -1,7 +1,8 @@
 // Device-wide exclusive scan and stable LSD radix sort (8-bit digits).
 //
-// Used by the acceleration build: Morton codes of triangle centroids for the
-// LBVH, and undirected half-edge keys for the boundary extraction.
+// Used by the acceleration build (Morton codes of triangle centroids for the LBVH, boundary
+// edges by vertex, loops by their keys, and half-edge keys where buckets do not serve) and
+// for the order of query lists and batches of meshes.
 //
 // Radix pass (per 8-bit digit), three kernels:
 //   1. per-tile digit histogram, written digit-major: counts[d * ntiles + t];
