@@ -696,12 +696,16 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const float *__restrict
 // triangle's normal is small against the products it is made of).
 // Terms are multiplied into a group's complex product like the boundary sum's (one atan2
 // per 8 triangles) under the triangle loops' test: an angle below pi/8, well-conditioned;
-// nearer triangles take their own, with the nearest vertex in the place of a.  Each thread holds 2 KP queries as float2 pairs.  The
+// nearer triangles take their own, for the pair of queries at once and with the determinant
+// of the unit vectors, which is as accurate beside every vertex (the nearest vertex against
+// N' for each query that failed: 200k queries beside the 200 slim triangles of a fan 196
+// us, now 149; every term by itself 139).  a is the vertex opposite the longest edge, so
+// that b and c are far apart and few terms of slim triangles fail.  Each thread holds 2 KP queries as float2 pairs.  The
 // triangle range is split into gridDim.y chunks so that any query count fills the GPU:
 // with one chunk the kernel writes w, otherwise FP64 partial sums [chunk][query] that
 // k_direct_reduce adds in chunk order.  Bound by the FP32 pipe (75% of its cycles): 49 paired
 // operations a term (75 with an atan2 and a 3 x 3 determinant each): 30k queries x 40k
-// triangles 2.54 -> 2.01 ms.  Errors above 1e-5 beside surfaces, edges and vertices (132 sets
+// triangles 2.54 -> 1.97 ms.  Errors above 1e-5 beside surfaces, edges and vertices (132 sets
 // of queries against FP64) 29.7k -> 11.8k against that determinant's.
 template <int KP>
 __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, int64_t n, const float *__restrict__ tri9,
@@ -744,8 +748,23 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
         __syncthreads();
         for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
             const float *T = tri9 + 9 * (t0 + i);
-            const float ax = __ldg(T), ay = __ldg(T + 1), az = __ldg(T + 2), bx = __ldg(T + 3), by = __ldg(T + 4),
-                        bz = __ldg(T + 5), cx = __ldg(T + 6), cy = __ldg(T + 7), cz = __ldg(T + 8);
+            float ax = __ldg(T), ay = __ldg(T + 1), az = __ldg(T + 2), bx = __ldg(T + 3), by = __ldg(T + 4),
+                  bz = __ldg(T + 5), cx = __ldg(T + 6), cy = __ldg(T + 7), cz = __ldg(T + 8);
+            auto len2 = [](float x, float y, float z) { return x * x + y * y + z * z; };
+            auto turn = [](float &x, float &y, float &z) {   // (x, y, z) -> (y, z, x)
+                const float t = x;
+                x = y;
+                y = z;
+                z = t;
+            };
+            // a opposite the longest edge
+            const float la = len2(cx - bx, cy - by, cz - bz), lb = len2(ax - cx, ay - cy, az - cz),
+                        lc = len2(bx - ax, by - ay, bz - az);
+            for (int turns = lb > fmaxf(la, lc) ? 1 : lc > la ? 2 : 0; turns > 0; --turns) {
+                turn(ax, bx, cx);
+                turn(ay, by, cy);
+                turn(az, bz, cz);
+            }
             float u[3], v[3], ul[3], vl[3], N[3];   // the edges as exact sums of two floats
             two_diff32(bx, ax, u[0], ul[0]);
             two_diff32(by, ay, u[1], ul[1]);
@@ -795,15 +814,21 @@ __global__ void __launch_bounds__(256, 2) k_direct(const float *__restrict__ q, 
                 const float2 v = fma2(bc2(-kTriSpread), g,
                                       fma2(bc2(kTanGroup), den, neg2(make_float2(fabsf(det.x), fabsf(det.y)))));
                 const bool px = v.x > kTriAccept, py = v.y > kTriAccept;   // (not if NaN, at a vertex)
-                const float4 N = make_float4(A.w, B.w, C.w, h);
-                float od, oe;
-                if (!px) {
-                    tri_own(N, make_float3(ax.x, ay.x, az.x), make_float3(bx.x, by.x, bz.x), make_float3(cx.x, cy.x, cz.x), od, oe);
-                    part[k].x += fast_atan2(od, oe);
-                }
-                if (!py) {
-                    tri_own(N, make_float3(ax.y, ay.y, az.y), make_float3(bx.y, by.y, bz.y), make_float3(cx.y, cy.y, cz.y), od, oe);
-                    part[k].y += fast_atan2(od, oe);
+                if (!(px && py)) {   // an atan2 of the pair's own, by the determinant of the unit vectors
+                    float2 ja = ia, jb = ib, jc = ic, oe = den;
+                    if (!(v.x > -1e30f && v.y > -1e30f)) {   // at a vertex: finite reciprocal lengths
+                        auto finite = [](float2 i) { return make_float2(fminf(i.x, 3.1e18f), fminf(i.y, 3.1e18f)); };
+                        ja = finite(ia);
+                        jb = finite(ib);
+                        jc = finite(ic);
+                        oe = fma2(bc, mul2(jb, jc), fma2(mul2(ac, ja), jc, fma2(mul2(ab, ja), jb, bc2(1.f))));
+                    }
+                    const float2 Ax = mul2(ax, ja), Ay = mul2(ay, ja), Az = mul2(az, ja), Bx = mul2(bx, jb),
+                                 By = mul2(by, jb), Bz = mul2(bz, jb), Cx = mul2(cx, jc), Cy = mul2(cy, jc), Cz = mul2(cz, jc);
+                    const float2 od = fma2(Ax, fma2(By, Cz, neg2(mul2(Bz, Cy))),
+                                           fma2(Ay, fma2(Bz, Cx, neg2(mul2(Bx, Cz))), mul2(Az, fma2(Bx, Cy, neg2(mul2(By, Cx))))));
+                    const float2 t = fast_atan2_2(od, oe);
+                    part[k] = add2(part[k], make_float2(px ? 0.f : t.x, py ? 0.f : t.y));
                 }
                 const float2 fd = make_float2(px ? den.x : 1.f, py ? den.y : 1.f);
                 const float2 fn = make_float2(px ? det.x : 0.f, py ? det.y : 0.f);
