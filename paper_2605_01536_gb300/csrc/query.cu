@@ -703,7 +703,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const float *__restrict
 // that b and c are far apart and few terms of slim triangles fail.  Each thread holds 2 KP queries as float2 pairs.  The
 // triangle range is split into gridDim.y chunks so that any query count fills the GPU:
 // with one chunk the kernel writes w, otherwise FP64 partial sums [chunk][query] that
-// k_direct_reduce adds in chunk order.  Bound by the FP32 pipe (75% of its cycles): 49 paired
+// k_direct_reduce adds in chunk order.  Bound by the FP32 pipe (77% of its cycles): 49 paired
 // operations a term (75 with an atan2 and a 3 x 3 determinant each): 30k queries x 40k
 // triangles 2.54 -> 1.97 ms.  Errors above 1e-5 beside surfaces, edges and vertices (132 sets
 // of queries against FP64) 29.7k -> 11.8k against that determinant's.
