@@ -691,7 +691,7 @@ __global__ void k_gather3(const float *__restrict__ q, const int32_t *__restrict
                           const unsigned long long *__restrict__ len, float *__restrict__ out) {
     const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= *len) return;
-    const int32_t j = list[i];
+    const int64_t j = list[i];
     out[3 * i] = q[3 * j];
     out[3 * i + 1] = q[3 * j + 1];
     out[3 * i + 2] = q[3 * j + 2];

@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(256) k_fp64_fix(const float *__restrict__ q, c
     __shared__ double red[256];
     const unsigned long long len = *list_len;
     for (unsigned long long li = blockIdx.x; li < len; li += gridDim.x) {
-        const int32_t idx = list[li];
+        const int64_t idx = list[li];
         const float qx = q[3 * idx], qy = q[3 * idx + 1], qz = q[3 * idx + 2];
         // thread t: the edges starting at points [t c, (t + 1) c), c = ceil((npts - 1) / blockDim)
         const int64_t nstart = npts > 0 ? npts - 1 : 0, per = (nstart + blockDim.x - 1) / blockDim.x;
